@@ -27,8 +27,9 @@ struct AttParams {
   float *lse;
   int32_t *status;
   int32_t *done;   // [batch*Hkv] split-arrival counters (zero between launches)
-  int batch, Hq, Hkv, G, Pmax, kbud, num_blocks, splits, pages_per_cta;
-  int B;             // tokens per page (the bf16 kernels: 16 only)
+  int batch, Hq, Hkv, G, Pmax, kbud, num_blocks, splits;
+  int B;             // tokens per page
+  int sub_shift;     // bf16 kernel: a page is 2^sub_shift tiles of 16 tokens (0, 1, 2 for pages of 16, 32, 64 tokens)
   int kvdiv;         // the KV head of problem h is h / kvdiv (1; per-head page tables: G, with G = 1 and Hkv = Hq here)
   int fused_merge;   // 1: the last CTA of a problem merges its splits; 0: a separate merge kernel follows
   int cluster;       // 1: the splits of a problem form one thread-block cluster and merge through its shared memory
@@ -45,6 +46,19 @@ constexpr int kTile = LOCKS_B * LOCKS_D * 2;                 // 4096 B: one K or
 constexpr int kAttStage = 2 * kTile;                         // K + V
 constexpr int kAttStages = LOCKS_ATT_STAGES;                  // ring depth per warp
 constexpr int kAttSmem = LOCKS_ATT_WARPS * kAttStages * kAttStage;
+// A single CTA merging many splits of many heads is a serial tail: beyond 64 (head, split) pairs the splits of a problem
+// go to the parallel merge kernel.
+constexpr int kFusedMerge = 64;
+
+// Slice `part` of `parts` nearly equal slices of n list entries.  Taken from the length the device sees: the table's
+// row (what the host could slice) is usually longer than the sequence, and equal slices of the row leave the last CTAs
+// of a problem idle: dense attention over 16 requests of 3K .. 12K tokens in rows of 32K 144.5 us, 3.6 TB/s; sliced by
+// length 94.2 us, 5.55 TB/s (0.86 of the copy bandwidth).
+__device__ __forceinline__ void slice_of(int n, int part, int parts, int &lo, int &hi) {
+  const int per = (n + parts - 1) / parts;
+  lo = min(part * per, n);
+  hi = min(lo + per, n);
+}
 
 // Resolve the idx-th page of this problem's list: logical page, physical block, valid tokens.
 __device__ __forceinline__ bool resolve_page(const AttParams &p, int b, int64_t prob, int idx, int T, int &block,
@@ -68,8 +82,12 @@ __device__ __forceinline__ uint32_t movm_trans_b16(uint32_t v) {
 //   O^T[128 dims x 8 heads]  += V^T[128 x 16] . P^T[16 x 8]          (8 row tiles, A = V via ldmatrix.trans,
 //                                                                   B = P^T after an 8x8 movmatrix transpose)
 // so both products use all 16 rows of the tile and the accumulator is 32 registers per 8 heads.
+//
+// Pages of 32 and 64 tokens are two and four such tiles; the list of pages is walked tile by tile.
+// Pages of 32 and 64 tokens are two and four such tiles: the page list is walked tile by tile (32-token pages, 4 requests
+// x 128 pages of 32 tokens: 71 + 6 us on the fp32 kernel that reads the pages once per query head, 15 us here).
 template <int NH, bool CONTIG>
-__global__ void __launch_bounds__(LOCKS_ATT_WARPS * 32) attend_bf16_kernel(AttParams p) {
+__global__ void __launch_bounds__(LOCKS_ATT_WARPS * 32, LOCKS_ATT_CTAS_PER_SM) attend_bf16_kernel(AttParams p) {
   extern __shared__ __align__(128) uint8_t smem[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int x = lane >> 2, t = lane & 3;
@@ -99,14 +117,13 @@ __global__ void __launch_bounds__(LOCKS_ATT_WARPS * 32) attend_bf16_kernel(AttPa
   const float c2 = p.sm_scale * kLog2e;
   pdl_wait();   // page table from the selector, appended K/V rows, sequence lengths
   const int T = p.seq_lens[b];
-  const int P = (T + LOCKS_B - 1) / LOCKS_B;
-  int npages = p.ids ? p.cnt[prob] : P;
+  int npages = p.ids ? p.cnt[prob] : (T + p.B - 1) / p.B;
   if (p.ids && (npages < 0 || npages > p.kbud)) {   // a count beyond the table's row: use the row, report it
     if (threadIdx.x == 0) set_status(p.status, LOCKS_ERR_BAD_BLOCK);
     npages = npages < 0 ? 0 : p.kbud;
   }
-  const int lo = split * p.pages_per_cta;
-  const int hi = min(lo + p.pages_per_cta, npages);
+  int lo, hi;
+  slice_of(npages << p.sub_shift, split, p.splits, lo, hi);
 
   float oacc[8][NH][4];
 #pragma unroll
@@ -127,12 +144,17 @@ __global__ void __launch_bounds__(LOCKS_ATT_WARPS * 32) attend_bf16_kernel(AttPa
 
   // page ids and physical blocks of this warp's pages are resolved 32 at a time, one lane each, so the
   // two dependent global loads are paid once per batch instead of once per page
-  const int first = lo + warp;
+  const int first = lo + warp, sub_mask = (1 << p.sub_shift) - 1;
   auto resolve_batch = [&](int jb, int &blk, int &nt) {
     const int idx = first + (jb + lane) * LOCKS_ATT_WARPS;
     blk = 0;
     nt = 0;
-    if (idx < hi && !resolve_page(p, b, prob, idx, T, blk, nt)) nt = 0;
+    if (idx < hi) {
+      if (resolve_page(p, b, prob, idx >> p.sub_shift, T, blk, nt))
+        nt = min(LOCKS_B, nt - (idx & sub_mask) * LOCKS_B);   // tokens of this tile (none past the sequence's end)
+      else
+        blk = nt = 0;
+    }
   };
   int blk_cur, nt_cur, blk_nxt = 0, nt_nxt = 0;
   resolve_batch(0, blk_cur, nt_cur);
@@ -142,7 +164,8 @@ __global__ void __launch_bounds__(LOCKS_ATT_WARPS * 32) attend_bf16_kernel(AttPa
     const int block = __shfl_sync(0xffffffffu, blk_cur, j & 31);
     const int ntok = __shfl_sync(0xffffffffu, nt_cur, j & 31);
     uint8_t *kt = ring + stage * kAttStage, *vt = kt + kTile;
-    const int64_t base = ((int64_t)block * p.sb + (int64_t)hkv * p.sh) * 2 + goff0;
+    const int sub = (first + j * LOCKS_ATT_WARPS) & sub_mask;   // tile within its page
+    const int64_t base = ((int64_t)block * p.sb + (int64_t)hkv * p.sh + (int64_t)(sub * LOCKS_B) * p.st) * 2 + goff0;
     const uint8_t *kp = Kb + base, *vp = Vb + base;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
@@ -451,7 +474,8 @@ __global__ void __launch_bounds__(128) attend_generic_kernel(AttParams p) {
     if (threadIdx.x == 0) set_status(p.status, LOCKS_ERR_BAD_BLOCK);
     npages = npages < 0 ? 0 : p.kbud;
   }
-  const int lo = split * p.pages_per_cta, hi = min(lo + p.pages_per_cta, npages);
+  int lo, hi;
+  slice_of(npages, split, p.splits, lo, hi);
   const T *K = reinterpret_cast<const T *>(p.k), *V = reinterpret_cast<const T *>(p.v), *Q = reinterpret_cast<const T *>(p.q);
   float qv[4], o[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
@@ -600,26 +624,25 @@ int locks_launch_attend(locks_ctx *c, const void *q, const locks_kv *kv, int bat
     p.kvdiv = p.G; p.Hkv = p.Hq; p.G = 1;
   }
   const bool dense = ids == nullptr;
-  // one wave: as many splits per problem as resident CTA slots allow, at least one page per warp
-  const int npages = dense ? c->Pmax : c->k;
+  const bool bf = c->cfg.kv_dtype == LOCKS_BF16;   // tensor-core kernel
+  p.sub_shift = !bf ? 0 : (c->B == 64 ? 2 : (c->B == 32 ? 1 : 0));
+  // one wave: as many splits per problem as resident CTA slots allow, at least one tile (generic kernel: page) per warp
+  const int ntiles = (dense ? c->Pmax : c->k) << p.sub_shift;
   int slots = c->num_sms * LOCKS_ATT_CTAS_PER_SM;
   if (slots > LOCKS_ATT_SLOT_BOUND) slots = LOCKS_ATT_SLOT_BOUND;
   int splits = slots / (batch * p.Hkv);
-  const int most = (npages + LOCKS_ATT_WARPS - 1) / LOCKS_ATT_WARPS;
+  const int most = (ntiles + LOCKS_ATT_WARPS - 1) / LOCKS_ATT_WARPS;
   if (splits > most) splits = most;
   if (splits > LOCKS_ATT_MAX_SPLITS) splits = LOCKS_ATT_MAX_SPLITS;
   if (splits < 1) splits = 1;
   // With clearly more problems than SMs every SM streams for several CTAs already: splitting a problem in
   // two only adds the merge (config 2, 256 problems: -1.5 to -2 us per step with one CTA per problem)
   if (!dense && 2 * batch * p.Hkv >= 3 * c->num_sms) splits = 1;
-  p.pages_per_cta = (npages + splits - 1) / splits;
-  p.splits = (npages + p.pages_per_cta - 1) / p.pages_per_cta;
+  p.splits = splits;
   p.done = c->att_done;
-  // a single CTA merging many splits of many heads is a serial tail: beyond 64 (head, split) pairs use the
-  // parallel merge kernel instead
-  p.fused_merge = (p.G * p.splits <= 64) ? 1 : 0;
+  p.fused_merge = (p.G * p.splits <= kFusedMerge) ? 1 : 0;
   // Preferred: the splits of a problem as one thread-block cluster (2, 4, 8 or 16 CTAs) that merges through
-  // distributed shared memory, as long as a CTA then has at most 8 pages per warp to stream.
+  // distributed shared memory, as long as a CTA then has at most 8 tiles per warp to stream.
   p.cluster = 0;
   if (c->att_cluster_max < 0) {   // largest cluster of this kernel the device can place (probed once)
     c->att_cluster_max = 0;
@@ -641,59 +664,44 @@ int locks_launch_attend(locks_ctx *c, const void *q, const locks_kv *kv, int bat
     }
     (void)cudaGetLastError();   // a refused probe is not an error of this call
   }
-  if (c->cfg.kv_dtype == LOCKS_BF16 && c->B == LOCKS_B && splits >= 2 && c->att_cluster_max >= 2) {
+  if (bf && splits >= 2 && c->att_cluster_max >= 2) {
     int cs = 2;
     while (cs * 2 <= splits && cs * 2 <= c->att_cluster_max) cs *= 2;
-    const int ppc = (npages + cs - 1) / cs;
-    if (ppc <= 8 * LOCKS_ATT_WARPS && (npages + ppc - 1) / ppc == cs) {
+    if ((ntiles + cs - 1) / cs <= 8 * LOCKS_ATT_WARPS) {
       p.cluster = 1;
-      p.pages_per_cta = ppc;
       p.splits = cs;
       p.fused_merge = 1;   // no merge launch follows
     }
   }
-  const bool bf = c->cfg.kv_dtype == LOCKS_BF16 && c->B == LOCKS_B;   // tensor-core kernel: bf16 cache, 16-token pages
   if (bf) {
-    if (locks_attrs_needed(LOCKS_ATTR_ATTEND)) {
-      cudaFuncSetAttribute(attend_bf16_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmem);
-      cudaFuncSetAttribute(attend_bf16_kernel<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmem);
-      cudaFuncSetAttribute(attend_bf16_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmem);
-      cudaFuncSetAttribute(attend_bf16_kernel<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmem);
-      cudaFuncSetAttribute(attend_bf16_kernel<1, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-      cudaFuncSetAttribute(attend_bf16_kernel<2, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-      cudaFuncSetAttribute(attend_bf16_kernel<1, false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-      cudaFuncSetAttribute(attend_bf16_kernel<2, false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    }
-    dim3 grid(p.splits, p.Hkv, batch);
     const bool contig = kv->stride_token == LOCKS_D;
-    const dim3 blk(LOCKS_ATT_WARPS * 32);
-    if (p.cluster) {
-      if (p.G <= 8) {
-        if (contig) locks_launch_pdl_cluster(attend_bf16_kernel<1, true>, grid, blk, kAttSmem, p.splits, st, p);
-        else locks_launch_pdl_cluster(attend_bf16_kernel<1, false>, grid, blk, kAttSmem, p.splits, st, p);
-      } else {
-        if (contig) locks_launch_pdl_cluster(attend_bf16_kernel<2, true>, grid, blk, kAttSmem, p.splits, st, p);
-        else locks_launch_pdl_cluster(attend_bf16_kernel<2, false>, grid, blk, kAttSmem, p.splits, st, p);
-      }
-    } else if (p.G <= 8) {
-      if (contig) locks_launch_pdl(attend_bf16_kernel<1, true>, grid, blk, kAttSmem, st, p);
-      else locks_launch_pdl(attend_bf16_kernel<1, false>, grid, blk, kAttSmem, st, p);
-    } else {
-      if (contig) locks_launch_pdl(attend_bf16_kernel<2, true>, grid, blk, kAttSmem, st, p);
-      else locks_launch_pdl(attend_bf16_kernel<2, false>, grid, blk, kAttSmem, st, p);
-    }
+    const dim3 grid(p.splits, p.Hkv, batch), blk(LOCKS_ATT_WARPS * 32);
+    const bool attrs = locks_attrs_needed(LOCKS_ATTR_ATTEND);
+#define LOCKS_ATT_CASE(NH_, CONTIG_)                                                                                  \
+  do {                                                                                                               \
+    if (attrs) {                                                                                                     \
+      cudaFuncSetAttribute(attend_bf16_kernel<NH_, CONTIG_>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmem); \
+      cudaFuncSetAttribute(attend_bf16_kernel<NH_, CONTIG_>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);     \
+    }                                                                                                                \
+    if ((p.G > 8) != (NH_ == 2) || contig != CONTIG_) break;                                                         \
+    if (p.cluster) locks_launch_pdl_cluster(attend_bf16_kernel<NH_, CONTIG_>, grid, blk, kAttSmem, p.splits, st, p); \
+    else locks_launch_pdl(attend_bf16_kernel<NH_, CONTIG_>, grid, blk, kAttSmem, st, p);                             \
+  } while (0)
+    LOCKS_ATT_CASE(1, true);
+    LOCKS_ATT_CASE(1, false);
+    LOCKS_ATT_CASE(2, true);
+    LOCKS_ATT_CASE(2, false);
+#undef LOCKS_ATT_CASE
   } else {
-    dim3 grid(p.splits, p.Hq, batch);
-    if (c->cfg.kv_dtype == LOCKS_BF16) locks_launch_pdl(attend_generic_kernel<__nv_bfloat16>, grid, dim3(128), 0, st, p);
-    else locks_launch_pdl(attend_generic_kernel<float>, grid, dim3(128), 0, st, p);
+    locks_launch_pdl(attend_generic_kernel<float>, dim3(p.splits, p.Hq, batch), dim3(128), 0, st, p);
   }
   int rc = locks_check_launch(c);
   if (rc != LOCKS_OK || p.splits == 1 || (bf && p.fused_merge)) return rc;
-  dim3 mg(p.Hq, batch);
-  if (c->cfg.kv_dtype == LOCKS_BF16) locks_launch_pdl(attend_merge_kernel<__nv_bfloat16>, mg, dim3(128), 0, st, (const float *)c->att_o,
-                           (const float *)c->att_lse, p.splits, reinterpret_cast<__nv_bfloat16 *>(out), lse, p.Hq);
-  else locks_launch_pdl(attend_merge_kernel<float>, mg, dim3(128), 0, st, (const float *)c->att_o,
-                        (const float *)c->att_lse, p.splits, reinterpret_cast<float *>(out), lse, p.Hq);
+  const dim3 mg(c->cfg.num_q_heads, batch);
+  if (bf) locks_launch_pdl(attend_merge_kernel<__nv_bfloat16>, mg, dim3(128), 0, st, (const float *)c->att_o, (const float *)c->att_lse,
+                           p.splits, reinterpret_cast<__nv_bfloat16 *>(out), lse, p.Hq);
+  else locks_launch_pdl(attend_merge_kernel<float>, mg, dim3(128), 0, st, (const float *)c->att_o, (const float *)c->att_lse, p.splits,
+                        reinterpret_cast<float *>(out), lse, p.Hq);
   return locks_check_launch(c);
 }
 
@@ -777,8 +785,8 @@ extern "C" int locks_sparse_attend_noalloc(const locks_config *cfg, const void *
   if (splits > most) splits = most;
   if (splits > kNoAllocMaxSplits) splits = kNoAllocMaxSplits;
   if (splits < 1) splits = 1;
-  p.pages_per_cta = (npages + splits - 1) / splits;
-  p.splits = (npages + p.pages_per_cta - 1) / p.pages_per_cta;
+  p.splits = splits;
+  p.sub_shift = 0;
   p.fused_merge = 1;
   p.cluster = 0;
   // the array keeps whatever the last call left: the arrival counters and the status word must start at zero
