@@ -1,6 +1,7 @@
 """Sizes at which the kernels' partitions and variants change: edges of tiles, remainders, the ends of their ranges."""
 import numpy as np
 import pytest
+import torch
 
 import locks_synth
 import oracle
@@ -24,3 +25,65 @@ def test_dense_attention_ragged_rows(lens, Hq, Hkv, B, layout):
     assert np.abs(out - oout).max() <= 2e-2
     assert np.abs(lse - olse).max() <= 1e-3 * max(1.0, np.abs(olse).max() / 10)
     assert gc.status() == 0
+
+
+def _page_keys(kind, B, rng):
+    """[B, 128] keys: the workloads' structure, and pages whose Gram matrix has close, equal, few or no eigenvalues."""
+    d = 128
+    if kind == "identical":
+        return np.tile(rng.standard_normal(d), (B, 1))
+    if kind == "rank1":
+        return rng.standard_normal(d) + np.outer(rng.standard_normal(B), rng.standard_normal(d))
+    if kind == "orthogonal":     # B - 1 equal eigenvalues
+        return np.eye(B, d) * 3.0
+    if kind == "two_keys":       # one eigenvalue
+        return np.where((np.arange(B) % 2 == 0)[:, None], rng.standard_normal(d), rng.standard_normal(d))
+    if kind == "blocks":         # equal pairs of eigenvalues in decoupled blocks
+        k = np.zeros((B, d))
+        for i in range(B):
+            k[i, (i // 4) * 8 + i % 4] = 2.0
+        return k
+    dirs = rng.standard_normal((6, d))
+    dirs /= np.linalg.norm(dirs, axis=1, keepdims=True)
+    k = 3.0 * rng.standard_normal(d) + (3.0 * rng.standard_normal((B, 6))) @ dirs + 0.1 * rng.standard_normal((B, d))
+    return k * {"large": 2.0 ** 30, "small": 2.0 ** -50}.get(kind, 1.0)
+
+
+# The page that a decode step has just filled, at every page size and rank.  What is compared does not depend on the
+# basis inside a (near-)degenerate eigenspace: the singular values, the residual of the rank-r summary, orthonormal
+# rows.  The fp32 Gram matrix is off by 2^-24 x sqrt(128 B) of its largest eigenvalue (1e-5 at B = 64).
+@pytest.mark.parametrize("B", [16, 32, 64])
+@pytest.mark.parametrize("kind", ["structured", "identical", "rank1", "orthogonal", "two_keys", "blocks", "large", "small"])
+def test_step_build_of_a_filled_page(B, kind):
+    from gpu_util import GpuCase
+    for r in (1, 2, 8, 16):
+        w = locks_synth.Workload("fill", [3 * B, 2 * B - 1, 5 * B], Hq=2, Hkv=2, B=B, dtype="f32", fmt="f32", rank=r, budget=2 * B, seed=B + r)
+        gc = GpuCase(w)
+        rng = np.random.default_rng(B * 100 + r)
+        keys = {}
+        for b in (0, 2):
+            blk = int(gc.case.block_table[b, w.seq_lens[b] // B - 1])
+            for h in range(2):
+                keys[b, h] = (blk, _page_keys(kind, B, rng).astype(np.float32))
+                gc.case.k[blk, h] = torch.from_numpy(keys[b, h][1])
+        summ = gc.ctx.new_summaries(gc.case.num_blocks)
+        out = torch.empty(w.n, w.Hq, w.d, device="cuda:0")
+        gc.ctx.locks_build_summaries(gc.kv, w.n, summ, torch.zeros(3, dtype=torch.int32, device="cuda:0"),
+                                     torch.tensor([2, 1, 4], dtype=torch.int32, device="cuda:0"))   # all but the filled pages
+        gc.ctx.locks_decode_step(gc.case.q, None, None, gc.kv, summ, w.n, out)
+        assert gc.status() == 0
+        got = summ.cpu().numpy()
+        for (b, h), (blk, k) in keys.items():
+            mu, V, Cc = oracle.unpack(gc.fmt, r, got[blk, h], B, w.d)
+            D = k.astype(np.float64) - k.astype(np.float64).mean(0)
+            sv = np.linalg.svd(D, compute_uv=False)[:r]
+            top = max(float(sv[0]), 1e-30)
+            keep = (sv ** 2 > 4e-6 * sv[0] ** 2) & (sv > 1e-4 * np.linalg.norm(k))   # clearly above the zero-mode thresholds
+            assert np.abs(mu - k.astype(np.float64).mean(0)).max() <= 1e-6 * max(np.abs(k).max(), 1e-30)
+            assert np.abs(np.linalg.norm(Cc, axis=0) - sv)[keep].max(initial=0.0) <= 1e-4 * top, (r, b, h)
+            n = int(keep.sum())
+            assert np.abs(V[:n] @ V[:n].T - np.eye(n)).max(initial=0.0) <= 2e-4, (r, b, h)
+            res = np.linalg.norm(D - Cc @ V)
+            best = np.sqrt(max((D ** 2).sum() - (sv[:n] ** 2).sum(), 0.0))
+            assert res <= best + 2e-3 * top, (r, b, h, res, best)
+        del gc
