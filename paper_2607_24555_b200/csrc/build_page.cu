@@ -10,9 +10,9 @@
 // stop test that looks only at pairs with one of the r modes that are kept (emulated in fp32 on this repository's
 // synthetic pages: 7.7 -> 4.9 sweeps at B = 16 and r = 8, 3.0 at r = 2, 8.5 -> 5.1 at B = 32; worst eigenvector entry
 // 1e-4 -> 4e-5 from fp64).  Measured beside a running selector and attention, from the launch to the last store: B = 16,
-r = 8 31 -> 22 us, of it the Jacobi sweeps 19 -> 10 (226 cycles a step), the factorisation 3, the basis 3.5; r = 2 27 -> 18
-us; B = 32 400 -> 47 us.  Steps that a page fills: 8 x 32K 64.5 -> 59.2 us, 32 x 16K at r = 2 75.3 -> 62.4, 4 x 16K with
-32-token pages 497 -> 176.
+// r = 8 31 -> 22 us, of it the Jacobi sweeps 19 -> 10 (226 cycles a step), the factorisation 3, the basis 3.5; r = 2 27 -> 18
+// us; B = 32 400 -> 47 us.  Steps that a page fills: 8 x 32K 64.5 -> 59.2 us, 32 x 16K at r = 2 75.3 -> 62.4, 4 x 16K with
+// 32-token pages 497 -> 176.
 //
 // The other phases use all of the page's threads (keys and centroid: one or two dimensions each; Gram matrix: dimensions
 // dealt to the warps; basis and quantisation: a warp per mode), in short loops: a freshly filled page finds this code in
