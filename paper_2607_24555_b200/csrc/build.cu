@@ -1,59 +1,75 @@
-// Summary build (Sec. 4 "Build (once, when a page completes)").
+// Summary build (Sec. 4 "Build (once, when a page completes)"), bulk, 16-token pages (build_page.cu has the rest).
 //
-// build_kernel (bulk, 16-token pages; build_page.cu has the rest): one warp takes 8 (page, KV head) items through three phases.
-//   1. per item, all lanes: load the page's 16 keys (lane owns 4 consecutive dims of every key), centroid mu,
-//      deviations D, and the Gram matrix M = D D^T (16 x 16) on the tensor cores; M goes to shared memory
-//   2. all 8 items at once: eigendecomposition of M by one-sided Jacobi in fp32.  Four lanes hold one item's
-//      matrix (4 columns of 16 entries each, in registers); columns are rotated in pairs until they are mutually
-//      orthogonal, which leaves M W = U Lambda: column norms are the eigenvalues, normalised columns the
-//      eigenvectors.  Pairing by odd-even transposition (16 steps per sweep meet every two columns once; a
-//      rotated pair swaps places), so only the pairs that straddle two lanes need shuffles.
-//   3. per item, all lanes: reload the keys, rank the modes by eigenvalue, keep r_eff <= min(r, 15) modes above
-//      the zero-mode thresholds, V = D^T U_r Sigma_r^-1 (lane's 4 dims), C = U_r Sigma_r, sign: largest |V| entry
-//      positive; store fp32 (F32 format) or quantise: symmetric abs-max, fp16 scale, round-half-even codes
-//      (int4 basis per column, int8 coefficients per row, int8 centroid) packed in the blob layout
+// One warp takes 8 (page, KV head) items through three phases:
+//   1. per item, all lanes: centre the page's 16 keys and form the Gram matrix M = D D^T (16 x 16) on the tensor cores; M
+//      goes to shared memory
+//   2. all 8 items at once: eigendecomposition of M by one-sided Jacobi in fp32.  Four lanes hold one item's matrix (4
+//      columns of 16 entries each, in registers).  A QR factorisation with column pivoting comes first; the columns of
+//      R^T are then rotated in pairs until they are mutually orthogonal: column norms are the eigenvalues, normalised
+//      columns the eigenvectors.
+//   3. per item, all lanes: modes above the zero-mode thresholds, V = D^T U_r Sigma_r^-1, C = U_r Sigma_r, sign: largest
+//      |V| entry positive; store or quantise: symmetric abs-max, fp16 scale, round-half-even codes (int4 basis per column,
+//      int8 coefficients per row, int8 centroid) packed in the blob layout
+// build_i4_kernel: bf16 keys, int4 summaries.  build_kernel: everything else (fp32 keys, the other formats).
+//
+// Bound by instruction issue and its latencies, not by bytes: an eigenproblem per 4 KB page.  131 008 page-heads of 8 x 32K
+// tokens: 1347 us with 8.2 Jacobi sweeps and all phases through shared memory (6 960 warp instructions per page-head), 908
+// us with the factorisation in front (5.0 sweeps) and build_i4_kernel's phases 1 and 3 (3 930).
 #include "build_common.cuh"
 
 namespace {
 
 constexpr int kBuildWarps = 2;
 constexpr int kBuildItems = 8;                                   // (page, KV head) items per warp
-constexpr int kBuildCtasPerSm = 8;                // 16 warps per SM
+constexpr int kBuildCtasPerSm = 8;                               // 16 warps per SM
 constexpr int kBuildScratch = 2 * LOCKS_B * 128;                 // 4096 B: bf16 half-tiles of D (hi | lo); later the blob
-constexpr int kBuildMat = kBuildItems * LOCKS_B * LOCKS_B * 4;   // 8192 B: Gram matrices; later the leading eigenvectors, every entry twice
+constexpr int kMat = LOCKS_B * LOCKS_B + 16;                     // floats per item's matrix: items on different banks
+constexpr int kBuildMat = kBuildItems * kMat * 4;                // 8704 B: Gram matrices, then R^T, then the leading eigenvectors
 constexpr int kBuildSmemPerWarp = kBuildScratch + kBuildMat + 64 + kBuildItems * LOCKS_B * 4;   // + key norms, eigenvalues
+constexpr int kUs = 20;                                          // build_i4_kernel: floats per eigenvector
+constexpr int kPiv = 2 * kBuildItems * LOCKS_B;                  // floats: pivot columns of two steps; later an item's centroid
+constexpr int kBuildI4SmemPerWarp = kPiv * 4 + kBuildMat + kBuildItems * LOCKS_B * 4;
 
-// One-sided Jacobi on 32 / LPI matrices at once, LPI = 16 / CPL lanes per matrix.  Lane (item = lane / LPI,
-// j = lane % LPI) holds columns CPL j .. CPL j + CPL - 1 of its item's matrix W (initially M, symmetric: the
-// columns are read as rows), w[c][i] = rows 2i, 2i+1 of column CPL j + c as a packed pair, and their squared
-// norms.  A sweep is 8 x (even step, odd step):
-//   even: the pairs (0,1), (2,3) .. of the lane;   odd: the pairs (1,2) .. of the lane and the pair (last column of
-//   lane j, first column of lane j+1),
+__device__ __forceinline__ float rcp_approx(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// One-sided Jacobi on 8 matrices at once.  Lane (item = lane / 4, j = lane % 4) holds columns 4 j .. 4 j + 3 of its item's
+// matrix W, w[c][i] = rows 2i, 2i+1 of column 4 j + c as a packed pair, and their squared norms.  A sweep is 8 x (even
+// step, odd step):
+//   even: the pairs (0,1), (2,3) of the lane;   odd: the pair (1,2) of the lane and the pair (last column of lane j, first
+//   column of lane j+1),
 // every pair rotated and then swapped in place.  The straddling pair is computed by both lanes (each from the
 // other's column, fetched by shuffle) and each keeps its own half of the result; the outer lanes' columns 0 and
-// 15 sit the odd step out.  CPL = 4 (8 matrices per warp) costs the fewest instructions per matrix; CPL = 2
-// (4 matrices) has the shorter instruction stream per sweep, for a decode step's few freshly filled pages.
-// Result: the columns ranked by norm (descending, ties to the lower position); unit eigenvectors of the leading
-// min(r, 8) modes to us[item][token][mode] as pairs (u, u) (r > 8: all 16, plain entries, [token][16]), the 16
-// eigenvalues to lam_s[item][mode].
-template <int CPL>
-__device__ __forceinline__ void jacobi_phase(const float *mat, float2 *us, float *lam_s, uint32_t live, int r, int lane) {
-  constexpr int LPI = LOCKS_B / CPL;
+// 15 sit the odd step out.
+// W starts as R^T of M's QR factorisation with column pivoting (modified Gram-Schmidt, only R kept: Drmac and Veselic's
+// preconditioning; R^T's left singular vectors are M's eigenvectors): half a sweep's work that saves three of eight
+// (emulated in fp32 on this repository's synthetic pages, worst of 8 items: 8.2 -> 5.0 sweeps; the worst eigenvector
+// entry falls from 1.1e-4 to 3.5e-5 from fp64).
+// Result: the columns ranked by norm (descending, ties to the lower position), the 16 eigenvalues to lam_s[item][mode],
+// unit eigenvectors of the leading min(r, 8) modes to us: PAIRS = false us[item][mode][token], kUs floats per mode; PAIRS =
+// true [item][token][mode] as pairs (u, u) (r > 8: all 16, plain entries, [token][16]).
+template <bool PAIRS>
+__device__ __forceinline__ void jacobi_phase(float *mat, float *piv, float *us, float *lam_s, uint32_t live, int r, int lane) {
+  constexpr int CPL = 4, LPI = LOCKS_B / CPL;
   const int item = lane / LPI, j = lane % LPI;
   const bool item_live = (live >> item) & 1u;   // lanes of an absent item compute on zeros
+  float *mine = mat + item * kMat;
   float2 w[CPL][8];
-  {
-    const float4 *src = reinterpret_cast<const float4 *>(mat + item * LOCKS_B * LOCKS_B + CPL * j * LOCKS_B);
+  auto load = [&](bool live_item) {
+    const float4 *src = reinterpret_cast<const float4 *>(mine + CPL * j * LOCKS_B);
 #pragma unroll
     for (int c = 0; c < CPL; ++c)
 #pragma unroll
       for (int q4 = 0; q4 < 4; ++q4) {
-        const float4 f = item_live ? src[c * 4 + q4] : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 f = live_item ? src[c * 4 + q4] : make_float4(0.f, 0.f, 0.f, 0.f);
         w[c][2 * q4] = make_float2(f.x, f.y);
         w[c][2 * q4 + 1] = make_float2(f.z, f.w);
       }
-  }
-  __syncwarp();   // every lane holds its columns: the matrices' shared memory may be overwritten from here on
+  };
+  load(item_live);
   auto seg_max = [&](float v) {   // maximum over the lanes of the item
 #pragma unroll
     for (int o = 1; o < LPI; o <<= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
@@ -98,11 +114,74 @@ __device__ __forceinline__ void jacobi_phase(const float *mat, float2 *us, float
     for (int i = 2; i < 8; i += 2) { acc0 = fma2(a[i], b[i], acc0); acc1 = fma2(a[i + 1], b[i + 1], acc1); }
     return (acc0.x + acc1.x) + (acc0.y + acc1.y);
   };
-  const float tol2 = LOCKS_BUILD_COS_TOL * LOCKS_BUILD_COS_TOL;
+  norms();
+  // ---- QR with column pivoting.  The norms that choose the pivot are downdated; the pivot's own is exact.
+  {
+    uint32_t used = 0u;
+#pragma unroll 1
+    for (int k = 0; k < LOCKS_B; ++k) {
+      // largest remaining column: the norm's bits with the column in the lowest four; + 16 so that 0 means "used"
+      uint32_t best = 0u;
+#pragma unroll
+      for (int c = 0; c < CPL; ++c) {
+        const uint32_t key = ((__float_as_uint(fmaxf(n[c], 0.f)) & ~15u) + 16u) | (uint32_t)(CPL * j + c);
+        best = max(best, ((used >> c) & 1u) ? 0u : key);
+      }
+      best = max(best, __shfl_xor_sync(0xffffffffu, best, 1));
+      best = max(best, __shfl_xor_sync(0xffffffffu, best, 2));
+      float4 *pb = reinterpret_cast<float4 *>(piv + ((k & 1) * kBuildItems + item) * LOCKS_B);
+      const int pc = (int)(best & 15u) - CPL * j;   // this lane's column of that number, if 0 .. 3
+#pragma unroll
+      for (int c = 0; c < CPL; ++c)
+        if (c == pc) {
+#pragma unroll
+          for (int q4 = 0; q4 < 4; ++q4) pb[q4] = make_float4(w[c][2 * q4].x, w[c][2 * q4].y, w[c][2 * q4 + 1].x, w[c][2 * q4 + 1].y);
+        }
+      __syncwarp();   // (the buffer of step k - 1 is not written before every lane has passed here)
+      float2 pv[8];
+#pragma unroll
+      for (int q4 = 0; q4 < 4; ++q4) {
+        const float4 f = pb[q4];
+        pv[2 * q4] = make_float2(f.x, f.y);
+        pv[2 * q4 + 1] = make_float2(f.z, f.w);
+      }
+      const float pp = dot(pv, pv), ir = pp > 1e-37f ? rsqrt_approx(pp) : 0.f;
+      float rk[CPL];
+#pragma unroll
+      for (int c = 0; c < CPL; ++c) {
+        rk[c] = ((used >> c) & 1u) ? 0.f : (c == pc ? pp : dot(w[c], pv)) * ir;
+        const float f = -rk[c] * ir;
+        const float2 f2 = make_float2(f, f);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) w[c][i] = fma2(f2, pv[i], w[c][i]);
+        n[c] = fmaf(-rk[c], rk[c], n[c]);
+      }
+      if (pc >= 0 && pc < CPL) used |= 1u << pc;
+      *reinterpret_cast<float4 *>(mine + k * LOCKS_B + CPL * j) = make_float4(rk[0], rk[1], rk[2], rk[3]);   // column k of R^T
+    }
+    __syncwarp();
+    load(true);
+  }
+  // The stop test: no pair above the tolerance in a whole sweep.  With few modes kept only pairs with one of the r largest
+  // columns count (r = 2: 5.4 -> 3.3 sweeps); with 8 the others add a fifth of a sweep, less than finding the r-th norm.
+  const float tol = r >= 8 ? 3.f * LOCKS_BUILD_COS_TOL : LOCKS_BUILD_COS_TOL, tol2 = tol * tol;
   int bad = 0;
-  float floor_n = 0.f;
+  float floor_n = 0.f, top = 0.f;
+  int rank[CPL];
+  auto ranks = [&]() {
+#pragma unroll
+    for (int c = 0; c < CPL; ++c) rank[c] = 0;
+#pragma unroll
+    for (int jj = 0; jj < LPI; ++jj)
+#pragma unroll
+      for (int cc = 0; cc < CPL; ++cc) {
+        const float o = __shfl_sync(0xffffffffu, n[cc], (lane & ~(LPI - 1)) + jj);
+#pragma unroll
+        for (int c = 0; c < CPL; ++c) rank[c] += (int)(o > n[c]) | ((int)(o == n[c]) & (int)(jj * CPL + cc < j * CPL + c));
+      }
+  };
   // columns whose norm is rounding noise beside the largest (null directions) do not hold up convergence
-  auto check = [&](float a, float b, float g) { bad |= (int)(g * g > tol2 * a * b) & (int)(fminf(a, b) > floor_n); };
+  auto check = [&](float a, float b, float g) { bad |= (int)(g * g > tol2 * a * b) & (int)(fminf(a, b) > floor_n) & (int)(fmaxf(a, b) >= top); };
   // rotate columns P, Q of this lane and swap them
   auto pair_in_lane = [&](float2 (&wp)[8], float2 (&wq)[8], float &np, float &nq) {
     const float g = dot(wp, wq);
@@ -128,6 +207,13 @@ __device__ __forceinline__ void jacobi_phase(const float *mat, float2 *us, float
 #pragma unroll
       for (int c = 1; c < CPL; ++c) nm = fmaxf(nm, n[c]);
       floor_n = 1e-11f * seg_max(nm);   // squared norm = squared eigenvalue: modes below 3e-6 of the largest
+    }
+    if (r < 8) {
+      ranks();
+      float least = INFINITY;
+#pragma unroll
+      for (int c = 0; c < CPL; ++c) least = rank[c] < r ? fminf(least, n[c]) : least;
+      top = -0.999f * seg_max(-least);
     }
     bad = 0;
 #pragma unroll 1
@@ -173,27 +259,24 @@ __device__ __forceinline__ void jacobi_phase(const float *mat, float2 *us, float
     if (!__any_sync(0xffffffffu, bad != 0)) break;
   }
   norms();
-  int rank[CPL];
-#pragma unroll
-  for (int c = 0; c < CPL; ++c) rank[c] = 0;
-#pragma unroll
-  for (int jj = 0; jj < LPI; ++jj)
-#pragma unroll
-    for (int cc = 0; cc < CPL; ++cc) {
-      const float o = __shfl_sync(0xffffffffu, n[cc], (lane & ~(LPI - 1)) + jj);
-#pragma unroll
-      for (int c = 0; c < CPL; ++c) rank[c] += (o > n[c]) || (o == n[c] && (jj * CPL + cc) < (j * CPL + c));
-    }
+  ranks();
 #pragma unroll
   for (int c = 0; c < CPL; ++c) {
     lam_s[item * LOCKS_B + rank[c]] = sqrtf(n[c]) * unscale;
     const float inv = n[c] > 0.f ? rsqrtf(n[c]) : 0.f;
-    if (r > 8) {   // ranks above 8 (fp32 summaries): all 16 modes, plain entries
-      float *dst = reinterpret_cast<float *>(us) + item * LOCKS_B * LOCKS_B + rank[c];
+    if (!PAIRS) {
+      if (rank[c] < 8) {
+        float4 *dst = reinterpret_cast<float4 *>(us + (item * 8 + rank[c]) * kUs);
+#pragma unroll
+        for (int q4 = 0; q4 < 4; ++q4)
+          dst[q4] = make_float4(w[c][2 * q4].x * inv, w[c][2 * q4].y * inv, w[c][2 * q4 + 1].x * inv, w[c][2 * q4 + 1].y * inv);
+      }
+    } else if (r > 8) {   // ranks above 8 (fp32 summaries): all 16 modes, plain entries
+      float *dst = us + item * LOCKS_B * LOCKS_B + rank[c];
 #pragma unroll
       for (int i = 0; i < 8; ++i) { dst[(2 * i) * LOCKS_B] = w[c][i].x * inv; dst[(2 * i + 1) * LOCKS_B] = w[c][i].y * inv; }
     } else if (rank[c] < 8) {
-      float2 *dst = us + item * LOCKS_B * 8 + rank[c];
+      float2 *dst = reinterpret_cast<float2 *>(us) + item * LOCKS_B * 8 + rank[c];
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         const float u0 = w[c][i].x * inv, u1 = w[c][i].y * inv;
@@ -205,28 +288,290 @@ __device__ __forceinline__ void jacobi_phase(const float *mat, float2 *us, float
   __syncwarp();
 }
 
+// Physical block of item `lane` (< 8) of this warp, -1 if there is none; page ranges as locks_build_summaries has them.
+__device__ __forceinline__ int item_block(const BuildParams &p, int warp, int lane) {
+  if (lane >= kBuildItems) return -1;
+  const int b = blockIdx.z % p.batch;
+  const int complete = p.seq_lens[b] / LOCKS_B;
+  const int p0 = p.page_begin ? p.page_begin[b] : 0;
+  const int p1 = min(p.page_end ? p.page_end[b] : complete, complete);
+  const int page = p0 + (blockIdx.x * kBuildWarps + warp) * kBuildItems + lane;
+  if (page < 0 || page >= p1 || page >= p.Pmax) return -1;
+  const int block = p.block_table[(int64_t)b * p.Pmax + page];
+  if (block >= 0 && block < p.num_blocks) return block;
+  set_status(p.status, LOCKS_ERR_BAD_BLOCK);
+  return -1;
+}
+
+__device__ __forceinline__ uint32_t bf16x2_add(uint32_t a, uint32_t b) {
+  const __nv_bfloat162 d = __hadd2_rn(*reinterpret_cast<__nv_bfloat162 *>(&a), *reinterpret_cast<__nv_bfloat162 *>(&b));
+  return *reinterpret_cast<const uint32_t *>(&d);
+}
+__device__ __forceinline__ uint32_t bf16x2_sub(uint32_t a, uint32_t b) {
+  const __nv_bfloat162 d = __hsub2_rn(*reinterpret_cast<__nv_bfloat162 *>(&a), *reinterpret_cast<__nv_bfloat162 *>(&b));
+  return *reinterpret_cast<const uint32_t *>(&d);
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  float2 d;
+  asm("add.rn.f32x2 %0, %1, %2;"
+      : "=l"(*reinterpret_cast<unsigned long long *>(&d))
+      : "l"(*reinterpret_cast<unsigned long long *>(&a)), "l"(*reinterpret_cast<unsigned long long *>(&b)));
+  return d;
+}
+// fp16 scale of codes -qmax .. qmax for values up to `best`, and its reciprocal (0 for a zero scale: all codes 0)
+__device__ __forceinline__ __half code_scale(float best, float inv_qmax, float &inv) {
+  const __half s = __float2half_rn(best * inv_qmax);
+  const float f = __half2float(s);
+  inv = f == 0.f ? 0.f : rcp_approx(f);
+  return s;
+}
+
+// bf16 keys, int4 summaries.  Neither phase 1 nor phase 3 touches shared memory for the keys: a lane loads from global
+// memory the 16-byte chunks that are its own MMA fragments (any assignment of dimensions to fragment positions will do in
+// phase 1, where they are summed over; in phase 3 it decides which dimensions of the basis a lane receives).
+//   Phase 1: the keys minus c = bf16(mean) split exactly into two bf16 terms H + L (Knuth's TwoSum in bf16 pairs), M' =
+//   (H + L)(H + L)^T, and M = M' centred in both directions (c is not quite the mean).
+//   Phase 3: V Sigma = U^T D = (U - mean U)^T K, U in three bf16 terms (24 bits, rows 0-7 and 8-15 of one A operand and rows
+//   0-7 of another whose rows 8-15 are 1/16 and give the centroid), K as stored: products exact, sums fp32.
+__global__ void __launch_bounds__(kBuildWarps * 32, kBuildCtasPerSm) build_i4_kernel(BuildParams p) {
+  extern __shared__ __align__(16) uint8_t smem_raw[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int x = lane >> 2, t = lane & 3, h = blockIdx.y, r = p.r;
+  const int it_block = item_block(p, warp, lane);
+  const uint32_t live = __ballot_sync(0xffffffffu, it_block >= 0);
+  if (!live) return;
+  const int layer = blockIdx.z / p.batch;
+  const __nv_bfloat16 *kbase = reinterpret_cast<const __nv_bfloat16 *>(p.k_layers ? p.k_layers[layer] : p.k);
+  uint8_t *sbase = p.summ_layers ? reinterpret_cast<uint8_t *>(p.summ_layers[layer]) : p.summ;
+  float *piv = reinterpret_cast<float *>(smem_raw + warp * kBuildI4SmemPerWarp), *mat = piv + kPiv, *lam_s = mat + kBuildItems * kMat;
+  auto page_keys = [&](int s) {
+    return kbase + (int64_t)__shfl_sync(0xffffffffu, it_block, s) * p.sb + (int64_t)h * p.sh;
+  };
+
+  // ---- 1. Gram matrices: lane (x, t) holds dimensions 8t .. 8t+7 (+ 32 j) of tokens x and x + 8
+#pragma unroll 1
+  for (int s = 0; s < kBuildItems; ++s) {
+    if (!((live >> s) & 1u)) continue;
+    const __nv_bfloat16 *K = page_keys(s) + (int64_t)x * p.st + 8 * t;
+    uint32_t ka[16], kb[16], nc[16];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const uint4 a = *reinterpret_cast<const uint4 *>(K + 32 * j), b = *reinterpret_cast<const uint4 *>(K + 8 * p.st + 32 * j);
+      ka[4 * j] = a.x; ka[4 * j + 1] = a.y; ka[4 * j + 2] = a.z; ka[4 * j + 3] = a.w;
+      kb[4 * j] = b.x; kb[4 * j + 1] = b.y; kb[4 * j + 2] = b.z; kb[4 * j + 3] = b.w;
+    }
+#pragma unroll
+    for (int i = 0; i < 16; ++i) nc[i] = bf16x2_add(ka[i], kb[i]);
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1)
+#pragma unroll
+      for (int i = 0; i < 16; ++i) nc[i] = bf16x2_add(nc[i], __shfl_xor_sync(0xffffffffu, nc[i], o));
+    float X0[4] = {0.f, 0.f, 0.f, 0.f}, X1[4] = {0.f, 0.f, 0.f, 0.f}, Y0[4] = {0.f, 0.f, 0.f, 0.f}, Y1[4] = {0.f, 0.f, 0.f, 0.f};
+    auto split = [&](uint32_t k, uint32_t n, uint32_t &hi, uint32_t &lo) {   // k + n = hi + lo exactly
+      hi = bf16x2_add(k, n);
+      const uint32_t bb = bf16x2_sub(hi, k);
+      lo = bf16x2_add(bf16x2_sub(k, bf16x2_sub(hi, bb)), bf16x2_sub(n, bb));
+    };
+#pragma unroll
+    for (int i = 0; i < 16; i += 2) {   // one k-step: registers i, i + 1 of both tokens are the A and the B operand
+      uint32_t H[4], L[4];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const __nv_bfloat162 m = __hmul2(*reinterpret_cast<__nv_bfloat162 *>(&nc[i + u]), __floats2bfloat162_rn(-1.f / LOCKS_B, -1.f / LOCKS_B));
+        const uint32_t n = *reinterpret_cast<const uint32_t *>(&m);
+        split(ka[i + u], n, H[2 * u], L[2 * u]);
+        split(kb[i + u], n, H[2 * u + 1], L[2 * u + 1]);
+      }
+      mma_bf16(X0, H[0], H[1], H[2], H[3], H[0], H[2]);
+      mma_bf16(X1, H[0], H[1], H[2], H[3], H[1], H[3]);
+      mma_bf16(Y0, H[0], H[1], H[2], H[3], L[0], L[2]);
+      mma_bf16(Y1, H[0], H[1], H[2], H[3], L[1], L[3]);
+      mma_bf16(X0, L[0], L[1], L[2], L[3], L[0], L[2]);
+      mma_bf16(X1, L[0], L[1], L[2], L[3], L[1], L[3]);
+      mma_bf16(Y0, L[0], L[1], L[2], L[3], H[0], H[2]);
+      mma_bf16(Y1, L[0], L[1], L[2], L[3], H[1], H[3]);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) { X0[i] += Y0[i]; X1[i] += Y1[i]; }   // [0..1]: row x, columns 2t, 2t+1 (X1: + 8); [2..3]: row x + 8
+    float r0 = (X0[0] + X0[1]) + (X1[0] + X1[1]), r1 = (X0[2] + X0[3]) + (X1[2] + X1[3]);
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1) { r0 += __shfl_xor_sync(0xffffffffu, r0, o); r1 += __shfl_xor_sync(0xffffffffu, r1, o); }
+    r0 *= 1.f / LOCKS_B;   // means of rows x and x + 8; by symmetry also of those columns
+    r1 *= 1.f / LOCKS_B;
+    float c0 = __shfl_sync(0xffffffffu, r0, 8 * t), c1 = __shfl_sync(0xffffffffu, r0, 8 * t + 4);
+    float c8 = __shfl_sync(0xffffffffu, r1, 8 * t), c9 = __shfl_sync(0xffffffffu, r1, 8 * t + 4);
+    float g = (c0 + c1) + (c8 + c9);
+    g += __shfl_xor_sync(0xffffffffu, g, 1);
+    g += __shfl_xor_sync(0xffffffffu, g, 2);
+    g *= 1.f / LOCKS_B;
+    r0 -= g;
+    r1 -= g;
+    float *dst = mat + s * kMat + x * LOCKS_B + 2 * t;
+    *reinterpret_cast<float2 *>(dst) = make_float2(X0[0] - (r0 + c0), X0[1] - (r0 + c1));
+    *reinterpret_cast<float2 *>(dst + 8) = make_float2(X1[0] - (r0 + c8), X1[1] - (r0 + c9));
+    *reinterpret_cast<float2 *>(dst + 8 * LOCKS_B) = make_float2(X0[2] - (r1 + c0), X0[3] - (r1 + c1));
+    *reinterpret_cast<float2 *>(dst + 8 * LOCKS_B + 8) = make_float2(X1[2] - (r1 + c8), X1[3] - (r1 + c9));
+  }
+  __syncwarp();
+
+  // ---- 2. eigenvectors and eigenvalues of all the warp's items at once
+  jacobi_phase<false>(mat, piv, mat, lam_s, live, r, lane);
+
+  // ---- 3. basis, coefficients, centroid.  Lane (x, t) receives mode x, dimensions 16 t .. 16 t + 15 (+ 64)
+#pragma unroll 1
+  for (int s = 0; s < kBuildItems; ++s) {
+    if (!((live >> s) & 1u)) continue;
+    const __nv_bfloat16 *K = page_keys(s) + (int64_t)(2 * t) * p.st + 8 * x;
+    uint4 kk[2][4];   // tokens 2t, 2t + 1, 2t + 8, 2t + 9; dimensions 8 x .. 8 x + 7 (+ 64)
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int hc = 0; hc < 2; ++hc) kk[hc][i] = *reinterpret_cast<const uint4 *>(K + (int64_t)((i & 1) + 8 * (i >> 1)) * p.st + 64 * hc);
+    const float *U = mat + s * 8 * kUs, *lam = lam_s + s * LOCKS_B;
+    uint32_t A[4], Lo[2];
+    {
+      const float2 ua = *reinterpret_cast<const float2 *>(U + x * kUs + 2 * t), ub = *reinterpret_cast<const float2 *>(U + x * kUs + 8 + 2 * t);
+      float m = (ua.x + ua.y) + (ub.x + ub.y);
+      m += __shfl_xor_sync(0xffffffffu, m, 1);
+      m += __shfl_xor_sync(0xffffffffu, m, 2);
+      m *= 1.f / LOCKS_B;
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        float a = (i ? ub.x : ua.x) - m, b = (i ? ub.y : ua.y) - m;
+        if (x >= r) a = b = 0.f;
+        A[2 * i] = pack_bf16(a, b);
+        a -= __uint_as_float(A[2 * i] << 16);
+        b -= __uint_as_float(A[2 * i] & 0xFFFF0000u);
+        A[2 * i + 1] = pack_bf16(a, b);
+        a -= __uint_as_float(A[2 * i + 1] << 16);
+        b -= __uint_as_float(A[2 * i + 1] & 0xFFFF0000u);
+        Lo[i] = pack_bf16(a, b);
+      }
+    }
+    const uint32_t kOne = 0x3D803D80u;   // 1/16
+    float2 v[2][8];   // [hc][j]: dimensions 64 hc + 16 t + j and + 8
+    float *mu_s = piv;
+#pragma unroll
+    for (int hc = 0; hc < 2; ++hc) {
+      float2 mu[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        auto word = [&](const uint4 &q) { return j < 2 ? q.x : (j < 4 ? q.y : (j < 6 ? q.z : q.w)); };
+        const uint32_t sel = (j & 1) ? 0x7632u : 0x5410u;
+        const uint32_t b0 = __byte_perm(word(kk[hc][0]), word(kk[hc][1]), sel), b1 = __byte_perm(word(kk[hc][2]), word(kk[hc][3]), sel);
+        float C1[4] = {0.f, 0.f, 0.f, 0.f}, C2[4] = {0.f, 0.f, 0.f, 0.f};
+        mma_bf16(C1, A[0], A[1], A[2], A[3], b0, b1);
+        mma_bf16(C2, Lo[0], kOne, Lo[1], kOne, b0, b1);
+        v[hc][j] = add2(add2(make_float2(C2[0], C2[1]), make_float2(C1[2], C1[3])), make_float2(C1[0], C1[1]));
+        mu[j] = make_float2(C2[2], C2[3]);
+      }
+      if (x == 0) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          *reinterpret_cast<float4 *>(mu_s + 64 * hc + 16 * t + 4 * q) = make_float4(mu[4 * q].x, mu[4 * q + 1].x, mu[4 * q + 2].x, mu[4 * q + 3].x);
+          *reinterpret_cast<float4 *>(mu_s + 64 * hc + 16 * t + 8 + 4 * q) = make_float4(mu[4 * q].y, mu[4 * q + 1].y, mu[4 * q + 2].y, mu[4 * q + 3].y);
+        }
+      }
+    }
+    __syncwarp();
+    uint8_t *gout = sbase + ((int64_t)__shfl_sync(0xffffffffu, it_block, s) * p.Hkv + h) * p.S;
+    // ---- centroid: dimensions 4 lane .. + 3
+    const float4 mu4 = *reinterpret_cast<const float4 *>(mu_s + 4 * lane);
+    {
+      const float mx = fmaxf(fmaxf(fabsf(mu4.x), fabsf(mu4.y)), fmaxf(fabsf(mu4.z), fabsf(mu4.w)));
+      float inv;
+      const __half sh = code_scale(__uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(mx))), 1.f / 127.f, inv);
+      auto code = [&](float v) { return (uint32_t)((int)round_code(v, inv, 127.f) + 128); };
+      // dim offset c = 2*half + e -> byte e*2 + half
+      *reinterpret_cast<uint32_t *>(gout + i4_off_mu(r) + lane * 4) = code(mu4.x) | (code(mu4.z) << 8) | (code(mu4.y) << 16) | (code(mu4.w) << 24);
+      if (lane == 0) *reinterpret_cast<__half *>(gout + i4_off_smu(r)) = sh;
+      if (lane < 16 && i4_off_smu(r) + 2 + lane < p.S) gout[i4_off_smu(r) + 2 + lane] = 0;   // bytes between the payload and the stride
+    }
+    // ---- the mode's place among those above the zero-mode thresholds (eigenvalues descend: no gaps)
+    const float knorm2 = warp_sum((float)LOCKS_B * (mu4.x * mu4.x + mu4.y * mu4.y + mu4.z * mu4.z + mu4.w * mu4.w) +
+                                  (lane < LOCKS_B ? lam[lane] : 0.f));
+    const float lam0 = lam[0], lx = lam[x];
+    const bool keep = x < r && lam0 > 0.f && lx > 1e-6f * lam0 && lx > 1e-10f * knorm2;
+    // ---- basis: largest magnitude and its sign (lowest dimension on ties)
+    float mx = v[0][0].x, mn = v[0][0].x;
+#pragma unroll
+    for (int hc = 0; hc < 2; ++hc)
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        mx = fmaxf(mx, fmaxf(v[hc][j].x, v[hc][j].y));
+        mn = fminf(mn, fminf(v[hc][j].x, v[hc][j].y));
+      }
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1) {
+      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+    }
+    bool neg = -mn > mx;
+    if (__any_sync(0xffffffffu, keep && mx == -mn)) {   // opposite entries of the same magnitude
+      int at = LOCKS_D << 1;   // 2 * dimension + (negative)
+#pragma unroll
+      for (int hc = 1; hc >= 0; --hc)
+#pragma unroll
+        for (int i = 15; i >= 0; --i) {
+          const float y = i < 8 ? v[hc][i & 7].x : v[hc][i & 7].y;
+          if (fabsf(y) == mx) at = 2 * (64 * hc + 16 * t + i) + (y < 0.f ? 1 : 0);
+        }
+      at = min(at, __shfl_xor_sync(0xffffffffu, at, 1));
+      at = min(at, __shfl_xor_sync(0xffffffffu, at, 2));
+      if (mx == -mn) neg = at & 1;
+    }
+    const float isig = keep ? rsqrtf(lx) : 0.f;
+    float inv;
+    const __half sv = code_scale(fmaxf(mx, -mn) * isig, 1.f / 7.f, inv);
+    inv *= neg ? -isig : isig;   // (a unit vector's largest entry is at least 0.088: the scale is a normal fp16, no code leaves -7 .. 7)
+    // code + 8 in the low bits of 1.5 * 2^23 + code + 8; a word's nibbles from the top: dimensions 7 5 3 1 6 4 2 0
+    if (x < r) {
+#pragma unroll
+      for (int hc = 0; hc < 2; ++hc) {
+        uint32_t wx = 0u, wy = 0u;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const int j = q < 4 ? 7 - 2 * q : 14 - 2 * q;
+          wx = wx * 16u + __float_as_uint(fmaf(v[hc][j].x, inv, 12582920.f));
+          wy = wy * 16u + __float_as_uint(fmaf(v[hc][j].y, inv, 12582920.f));
+        }
+        *reinterpret_cast<uint2 *>(gout + x * 64 + 32 * hc + 8 * t) = make_uint2(wx - 0x3F400000u, wy - 0x3F400000u);
+      }
+      if (t == 0) *reinterpret_cast<__half *>(gout + i4_off_sv(r) + 2 * x) = sv;
+    }
+    // ---- coefficients C = U Sigma: tokens x and x + 8, modes 2t and 2t + 1
+    const float sg = keep ? (neg ? -sqrtf(lx) : sqrtf(lx)) : 0.f;
+    const float g0 = __shfl_sync(0xffffffffu, sg, 8 * t), g1 = __shfl_sync(0xffffffffu, sg, 8 * t + 4);
+    const float *Ut = U + 2 * t * kUs + x;
+    const float ca = g0 * Ut[0], cb = g1 * Ut[kUs], cc = g0 * Ut[8], cd = g1 * Ut[kUs + 8];
+    float ma = fmaxf(fabsf(ca), fabsf(cb)), mb = fmaxf(fabsf(cc), fabsf(cd));
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1) {
+      ma = fmaxf(ma, __shfl_xor_sync(0xffffffffu, ma, o));
+      mb = fmaxf(mb, __shfl_xor_sync(0xffffffffu, mb, o));
+    }
+    float ia, ib;
+    const __half sa = code_scale(ma, 1.f / 127.f, ia), sb = code_scale(mb, 1.f / 127.f, ib);
+    if (t < r / 2) {
+      auto code = [&](float v, float inv) { return (uint32_t)((int)round_code(v, inv, 127.f) + 128); };
+      *reinterpret_cast<uint32_t *>(gout + i4_off_coef(r) + (x * (r / 2) + t) * 4) =
+          code(ca, ia) | (code(cb, ia) << 8) | (code(cc, ib) << 16) | (code(cd, ib) << 24);
+    }
+    if (t == 0) {
+      __half *dst = reinterpret_cast<__half *>(gout + i4_off_sc(r)) + (x >> 1) * 4 + (x & 1);
+      dst[0] = sa;
+      dst[2] = sb;
+    }
+    __syncwarp();   // the centroid's shared memory is written again for the next item
+  }
+}
+
 template <typename T, int FMT>
 __global__ void __launch_bounds__(kBuildWarps * 32, kBuildCtasPerSm) build_kernel(BuildParams p) {
   extern __shared__ __align__(16) uint8_t smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  // ---- the warp's items: lane s < 8 works out item s
-  int it_block = -1;
-  const int it_b = blockIdx.z % p.batch, h = blockIdx.y;
-  if (lane < kBuildItems) {
-    const int complete = p.seq_lens[it_b] / LOCKS_B;
-    const int p0 = p.page_begin ? p.page_begin[it_b] : 0;
-    const int p1 = min(p.page_end ? p.page_end[it_b] : complete, complete);
-    int page = p0 + (blockIdx.x * kBuildWarps + warp) * kBuildItems + lane;
-    if (page < 0 || page >= p1) page = -1;
-    if (page >= p.Pmax) page = -1;
-    if (page >= 0) {
-      it_block = p.block_table[(int64_t)it_b * p.Pmax + page];
-      if (it_block < 0 || it_block >= p.num_blocks) {
-        set_status(p.status, LOCKS_ERR_BAD_BLOCK);
-        it_block = -1;
-      }
-    }
-  }
+  const int h = blockIdx.y;
+  const int it_block = item_block(p, warp, lane);   // the warp's items: lane s < 8 works out item s
   const uint32_t live = __ballot_sync(0xffffffffu, it_block >= 0);
   if (!live) return;
 
@@ -235,7 +580,7 @@ __global__ void __launch_bounds__(kBuildWarps * 32, kBuildCtasPerSm) build_kerne
   uint8_t *sbase = p.summ_layers ? reinterpret_cast<uint8_t *>(p.summ_layers[layer]) : p.summ;
   uint8_t *scratch = smem_raw + warp * kBuildSmemPerWarp;                        // D half-tiles; phase 3: the blob
   float *mat = reinterpret_cast<float *>(scratch + kBuildScratch);              // [8][16][16] Gram; then [8][16][8] pairs (u, u) of U_r
-  float *kn_s = mat + kBuildItems * LOCKS_B * LOCKS_B;                          // [8] squared norm of the page's keys
+  float *kn_s = mat + kBuildItems * kMat;                          // [8] squared norm of the page's keys
   float *lam_s = kn_s + 16;                                                     // [8][16] eigenvalues, descending
   float2 *us = reinterpret_cast<float2 *>(mat);
   const int r = p.r;
@@ -347,7 +692,7 @@ __global__ void __launch_bounds__(kBuildWarps * 32, kBuildCtasPerSm) build_kerne
         const int j = j0 + jj;
         g[jj] = 0.5f * (XA[i * 17 + j] + XA[j * 17 + i]) + YA[i * 17 + j] + YA[j * 17 + i];
       }
-      float4 *dst = reinterpret_cast<float4 *>(mat + s * LOCKS_B * LOCKS_B + i * LOCKS_B + j0);
+      float4 *dst = reinterpret_cast<float4 *>(mat + s * kMat + i * LOCKS_B + j0);
       dst[0] = make_float4(g[0], g[1], g[2], g[3]);
       dst[1] = make_float4(g[4], g[5], g[6], g[7]);
       __syncwarp();
@@ -355,7 +700,7 @@ __global__ void __launch_bounds__(kBuildWarps * 32, kBuildCtasPerSm) build_kerne
   }
 
   // ---- 2. eigenvectors and eigenvalues of all the warp's items at once
-  jacobi_phase<4>(mat, us, lam_s, live, r, lane);
+  jacobi_phase<true>(mat, reinterpret_cast<float *>(scratch), mat, lam_s, live, r, lane);
 
   // ---- 3. per item: modes, basis, coefficients, quantisation
   uint8_t *blob = scratch;
@@ -551,7 +896,10 @@ int locks_launch_build(locks_ctx *c, const locks_kv *kv, int batch, const int32_
     else build_kernel<float, F_><<<grid, kBuildWarps * 32, smem, st>>>(p);                                                 \
   } while (0)
   switch (c->cfg.summary_fmt) {
-    case LOCKS_FMT_I4: LOCKS_BUILD_CASE(LOCKS_FMT_I4); break;
+    case LOCKS_FMT_I4:
+      if (bf) build_i4_kernel<<<grid, kBuildWarps * 32, kBuildWarps * kBuildI4SmemPerWarp, st>>>(p);
+      else build_kernel<float, LOCKS_FMT_I4><<<grid, kBuildWarps * 32, smem, st>>>(p);
+      break;
     case LOCKS_FMT_I8: LOCKS_BUILD_CASE(LOCKS_FMT_I8); break;
     case LOCKS_FMT_BF16: LOCKS_BUILD_CASE(LOCKS_FMT_BF16); break;
     default: LOCKS_BUILD_CASE(LOCKS_FMT_F32); break;
