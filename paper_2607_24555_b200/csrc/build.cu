@@ -14,7 +14,8 @@
 //
 // Bound by instruction issue and its latencies, not by bytes: an eigenproblem per 4 KB page.  131 008 page-heads of 8 x 32K
 // tokens: 1347 us with 8.2 Jacobi sweeps and all phases through shared memory (6 960 warp instructions per page-head), 908
-// us with the factorisation in front (5.0 sweeps) and build_i4_kernel's phases 1 and 3 (3 930).
+// us with the factorisation in front (5.0 sweeps) and build_i4_kernel's phases 1 and 3 (3 930), 870 us with every pair
+// rotated in one lane, by shears.  10 CTAs of 96 registers per SM instead of 8 of 128: 957 us (spills).
 #include "build_common.cuh"
 
 namespace {
@@ -37,13 +38,9 @@ __device__ __forceinline__ float rcp_approx(float x) {
 }
 
 // One-sided Jacobi on 8 matrices at once.  Lane (item = lane / 4, j = lane % 4) holds columns 4 j .. 4 j + 3 of its item's
-// matrix W, w[c][i] = rows 2i, 2i+1 of column 4 j + c as a packed pair, and their squared norms.  A sweep is 8 x (even
-// step, odd step):
-//   even: the pairs (0,1), (2,3) of the lane;   odd: the pair (1,2) of the lane and the pair (last column of lane j, first
-//   column of lane j+1),
-// every pair rotated and then swapped in place.  The straddling pair is computed by both lanes (each from the
-// other's column, fetched by shuffle) and each keeps its own half of the result; the outer lanes' columns 0 and
-// 15 sit the odd step out.
+// matrix W, w[c][i] = rows 2i, 2i+1 of column 4 j + c as a packed pair, and their squared norms: two pairs of columns.
+// Odd-even transposition (16 steps per sweep meet every two columns once): every step rotates all pairs and passes one
+// column of each to a neighbour, half of the time within the lane.
 // W starts as R^T of M's QR factorisation with column pivoting (modified Gram-Schmidt, only R kept: Drmac and Veselic's
 // preconditioning; R^T's left singular vectors are M's eigenvectors): half a sweep's work that saves three of eight
 // (emulated in fp32 on this repository's synthetic pages, worst of 8 items: 8.2 -> 5.0 sweeps; the worst eigenvector
@@ -180,26 +177,35 @@ __device__ __forceinline__ void jacobi_phase(float *mat, float *piv, float *us, 
         for (int c = 0; c < CPL; ++c) rank[c] += (int)(o > n[c]) | ((int)(o == n[c]) & (int)(jj * CPL + cc < j * CPL + c));
       }
   };
-  // columns whose norm is rounding noise beside the largest (null directions) do not hold up convergence
-  auto check = [&](float a, float b, float g) { bad |= (int)(g * g > tol2 * a * b) & (int)(fminf(a, b) > floor_n) & (int)(fmaxf(a, b) >= top); };
-  // rotate columns P, Q of this lane and swap them
-  auto pair_in_lane = [&](float2 (&wp)[8], float2 (&wq)[8], float &np, float &nq) {
-    const float g = dot(wp, wq);
-    check(np, nq, g);
-    float c, sn, tn;
-    jacobi_angle(np, nq, g, c, sn, tn);
-    const float2 C2 = make_float2(c, c), S2 = make_float2(sn, sn), nS2 = make_float2(-sn, -sn);
+  // A pair holds a column that it kept from the step before (a) and one that it has been passed (b).  Which of the two is the
+  // lower position alternates from step to step, and so do the signs of the rotation and of the swap that follows it,
+  // which leaves one formula: passed on c a + s b (in a), kept c b - s a (in b).
+  struct Angle { float c, s; };
+  auto angle = [&](const float2 (&a)[8], const float2 (&b)[8], float &na, float &nb, bool there) {
+    const float g = dot(a, b);
+    // columns whose norm is rounding noise beside the largest (null directions) do not hold up convergence
+    bad |= (int)there & (int)(g * g > tol2 * na * nb) & (int)(fminf(na, nb) > floor_n) & (int)(fmaxf(na, nb) >= top);
+    Angle r;
+    float tn;
+    jacobi_angle(nb, na, g, r.c, r.s, tn);
+    tn = there ? tn * g : nb - na;   // (no pair: the two change places)
+    na = fmaxf(na + tn, 0.f);
+    nb = fmaxf(nb - tn, 0.f);
+    return r;
+  };
+  // as three shears (tau = tan(angle / 2) = s / (1 + c)): three packed operations per row instead of four
+  auto rotate = [&](float2 (&a)[8], float2 (&b)[8], float &na, float &nb) {
+    const Angle r = angle(a, b, na, nb, true);
+    const float tau = r.s * rcp_approx(1.f + r.c);
+    const float2 T2 = make_float2(tau, tau), S2 = make_float2(-r.s, -r.s);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      const float2 pp = fma2(C2, wp[i], mul2(nS2, wq[i]));
-      const float2 qq = fma2(S2, wp[i], mul2(C2, wq[i]));
-      wp[i] = qq;
-      wq[i] = pp;
+      a[i] = fma2(T2, b[i], a[i]);
+      b[i] = fma2(S2, a[i], b[i]);
+      a[i] = fma2(T2, b[i], a[i]);
     }
-    const float na = fmaxf(fmaf(-tn, g, np), 0.f);
-    np = fmaxf(fmaf(tn, g, nq), 0.f);
-    nq = na;
   };
+  const int up = (lane & ~(LPI - 1)) | ((j + 1) & (LPI - 1)), down = (lane & ~(LPI - 1)) | ((j - 1) & (LPI - 1));
   for (int sweep = 0; sweep < LOCKS_BUILD_SWEEPS; ++sweep) {
     norms();
     {
@@ -216,45 +222,42 @@ __device__ __forceinline__ void jacobi_phase(float *mat, float *piv, float *us, 
       top = -0.999f * seg_max(-least);
     }
     bad = 0;
-#pragma unroll 1
+#pragma unroll 2
     for (int st2 = 0; st2 < 8; ++st2) {
-#pragma unroll
-      for (int c = 0; c + 1 < CPL; c += 2) pair_in_lane(w[c], w[c + 1], n[c], n[c + 1]);
-      // odd step: the straddling pairs first (they read the lane's outer columns, which its inner pairs do not touch)
-      float2 qr[8], pr[8];
+      // even step: the lane's pairs (w[1], w[0]) and (w[3], w[2])
+      rotate(w[1], w[0], n[1], n[0]);
+      rotate(w[3], w[2], n[3], n[2]);
+      // a pair passes to the one before it: w[3] to w[0]'s, w[1] to the lane below
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
-        qr[i].x = __shfl_down_sync(0xffffffffu, w[0][i].x, 1, LPI);
-        qr[i].y = __shfl_down_sync(0xffffffffu, w[0][i].y, 1, LPI);
-        pr[i].x = __shfl_up_sync(0xffffffffu, w[CPL - 1][i].x, 1, LPI);
-        pr[i].y = __shfl_up_sync(0xffffffffu, w[CPL - 1][i].y, 1, LPI);
+        w[1][i].x = __shfl_sync(0xffffffffu, w[1][i].x, up);
+        w[1][i].y = __shfl_sync(0xffffffffu, w[1][i].y, up);
       }
-      const float nqr = __shfl_down_sync(0xffffffffu, n[0], 1, LPI), npr = __shfl_up_sync(0xffffffffu, n[CPL - 1], 1, LPI);
-      // pair A: p = own last column, q = next lane's column 0; this lane's last column becomes q' = s p + c q
+      n[1] = __shfl_sync(0xffffffffu, n[1], up);
+      // odd step: (w[0], w[3]) and (w[2], w[1]); the item's last pair has the two ends of the row, which do not meet
+      rotate(w[0], w[3], n[0], n[3]);
       {
-        const float g = dot(w[CPL - 1], qr);
-        float c, sn, tn;
-        jacobi_angle(n[CPL - 1], nqr, g, c, sn, tn);
-        check(n[CPL - 1], j == LPI - 1 ? 0.f : nqr, g);   // (the outer lane's pair does not exist: norm 0 never counts)
-        c = j == LPI - 1 ? 0.f : c; sn = j == LPI - 1 ? 1.f : sn;
-        const float2 C2 = make_float2(c, c), S2 = make_float2(sn, sn);
+        Angle r = angle(w[2], w[1], n[2], n[1], j != LPI - 1);
+        if (j == LPI - 1) { r.c = 0.f; r.s = 1.f; }
+        const float2 C2 = make_float2(r.c, r.c), S2 = make_float2(r.s, r.s), nS2 = make_float2(-r.s, -r.s);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) w[CPL - 1][i] = fma2(S2, w[CPL - 1][i], mul2(C2, qr[i]));
-        n[CPL - 1] = j == LPI - 1 ? n[CPL - 1] : fmaxf(fmaf(tn, g, nqr), 0.f);
+        for (int i = 0; i < 8; ++i) {
+          const float2 a = fma2(C2, w[2][i], mul2(S2, w[1][i]));
+          w[1][i] = fma2(C2, w[1][i], mul2(nS2, w[2][i]));
+          w[2][i].x = __shfl_sync(0xffffffffu, a.x, down);   // a pair passes to the one after it: w[0] to w[1]'s, w[2] to the lane above
+          w[2][i].y = __shfl_sync(0xffffffffu, a.y, down);
+        }
+        n[2] = __shfl_sync(0xffffffffu, n[2], down);
       }
-      // pair B: p = previous lane's last column, q = own column 0; this lane's column 0 becomes p' = c p - s q
-      {
-        const float g = dot(pr, w[0]);
-        float c, sn, tn;
-        jacobi_angle(npr, n[0], g, c, sn, tn);
-        c = j == 0 ? 0.f : c; sn = j == 0 ? -1.f : sn;
-        const float2 C2 = make_float2(c, c), nS2 = make_float2(-sn, -sn);
+      // the lane's pairs are now (w[3], w[2]) and (w[1], w[0]), in this order: exchange the names
 #pragma unroll
-        for (int i = 0; i < 8; ++i) w[0][i] = fma2(C2, pr[i], mul2(nS2, w[0][i]));
-        n[0] = j == 0 ? n[0] : fmaxf(fmaf(-tn, g, npr), 0.f);
+      for (int c = 0; c < 2; ++c) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) { const float2 y = w[c][i]; w[c][i] = w[c + 2][i]; w[c + 2][i] = y; }
+        const float y = n[c];
+        n[c] = n[c + 2];
+        n[c + 2] = y;
       }
-#pragma unroll
-      for (int c = 1; c + 1 < CPL; c += 2) pair_in_lane(w[c], w[c + 1], n[c], n[c + 1]);
     }
     if (!__any_sync(0xffffffffu, bad != 0)) break;
   }
