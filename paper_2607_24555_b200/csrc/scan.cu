@@ -257,6 +257,59 @@ __device__ __forceinline__ void mma_f16_z(float (&d)[4], uint32_t a0, uint32_t a
                : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.f));
 }
 
+// A query head as MMA operand registers: lane (.., t) holds dims 32 t .. 32 t + 31 of `row`; a0[s] dims 4 s, 4 s + 1, a2[s]
+// dims 4 s + 2, 4 s + 3 divided by 16 (see "Numerics").  inv = 1 / the power of two that the row was scaled by, sum8 = 8 times
+// the sum of the scaled row.  All four lanes of a row take part.
+__device__ __forceinline__ void load_q_row(const __nv_bfloat16 *row, int t, bool valid, uint32_t (&a0)[8], uint32_t (&a2)[8],
+                                           float &inv, float &sum8) {
+  uint4 v[4] = {};
+  if (valid) {
+    const uint4 *qp = reinterpret_cast<const uint4 *>(row + 32 * t);
+#pragma unroll
+    for (int m = 0; m < 4; ++m) v[m] = __ldg(qp + m);
+  }
+  const uint32_t *w = reinterpret_cast<const uint32_t *>(v);
+  uint32_t mx = 0u;  // largest |q| of the row as a bf16 bit pattern (orders like the value)
+#pragma unroll
+  for (int i = 0; i < 16; ++i) mx = __vmaxu2(mx, w[i] & 0x7FFF7FFFu);
+  mx = max(mx & 0xFFFFu, mx >> 16);
+  mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+  mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+  const float fm = __uint_as_float(mx << 16);
+  float s = 1.f;
+  if (fm > 0.f && fm < INFINITY) {
+    int e;
+    (void)frexpf(fm, &e);        // fm = f 2^e, f in [0.5, 1)
+    s = ldexpf(1.f, -(e + 1));   // max |q| s < 0.5
+  }
+  inv = 1.f / s;
+  float acc = 0.f;
+#pragma unroll
+  for (int ks = 0; ks < 8; ++ks) {
+    const uint32_t u0 = w[2 * ks], u1 = w[2 * ks + 1];
+    const uint32_t h0 = pack_f16(__uint_as_float(u0 << 16) * s, __uint_as_float(u0 & 0xFFFF0000u) * s);
+    const uint32_t h1 = pack_f16(__uint_as_float(u1 << 16) * s, __uint_as_float(u1 & 0xFFFF0000u) * s);
+    const float2 f0 = h2f2(h0), f1 = h2f2(h1);
+    acc += (f0.x + f0.y) + (f1.x + f1.y);     // sum of the fp16 values actually multiplied
+    a0[ks] = h0;
+    a2[ks] = pack_f16(f1.x * 0.0625f, f1.y * 0.0625f);
+  }
+  acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+  acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+  sum8 = 8.f * acc;
+}
+
+// the running log-sum-exp of a head's candidate pages, one exp per value
+__device__ __forceinline__ void lse_accumulate(float &m, float &sacc, float v) {
+  // branch-free: a value of -inf (masked page) adds nothing, whatever m is (also -inf at the start)
+  const bool live = v > -INFINITY;
+  const float d = v - m;                                    // NaN only if both are -inf: not live then
+  const float e = live ? __expf(-fabsf(d)) : 0.f;           // m = -inf, v finite: exp(-inf) = 0
+  const bool up = live && d > 0.f;
+  sacc = up ? fmaf(sacc, e, 1.f) : sacc + e;
+  m = up ? v : m;
+}
+
 struct Cursor {
   int prob, grp, nsc, b, h;   // (request, KV head) of prob are refreshed only when prob changes
   const int32_t *bt;          // block-table row of request b
@@ -519,46 +572,6 @@ __global__ void __launch_bounds__(kScanWarps * 32, kScanCtasPerSm) scan_i4_kerne
   const __nv_bfloat16 *q = reinterpret_cast<const __nv_bfloat16 *>(p.q);
   const float c2 = p.sm_scale * kLog2e;
 
-  auto load_q_row = [&](int b, int hq, bool valid, uint32_t (&a0)[8], uint32_t (&a2)[8], float &inv, float &sum8) {
-    uint4 v[4] = {};
-    if (valid) {
-      const uint4 *qp = reinterpret_cast<const uint4 *>(q + ((int64_t)b * p.Hq + hq) * LOCKS_D + 32 * t);
-#pragma unroll
-      for (int m = 0; m < 4; ++m) v[m] = __ldg(qp + m);
-    }
-    const uint32_t *w = reinterpret_cast<const uint32_t *>(v);
-    uint32_t mx = 0u;  // largest |q| of the row as a bf16 bit pattern (orders like the value)
-#pragma unroll
-    for (int i = 0; i < 16; ++i) mx = __vmaxu2(mx, w[i] & 0x7FFF7FFFu);
-    mx = max(mx & 0xFFFFu, mx >> 16);
-    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-    const float fm = __uint_as_float(mx << 16);
-    float s = 1.f;
-    if (fm > 0.f && fm < INFINITY) {
-      int e;
-      (void)frexpf(fm, &e);        // fm = f 2^e, f in [0.5, 1)
-      s = ldexpf(1.f, -(e + 1));   // max |q| s < 0.5
-    }
-    inv = 1.f / s;
-    const float s16 = s * 0.0625f;
-    float acc = 0.f;
-#pragma unroll
-    for (int ks = 0; ks < 8; ++ks) {
-      const uint32_t u0 = w[2 * ks], u1 = w[2 * ks + 1];
-      const uint32_t h0 = pack_f16(__uint_as_float(u0 << 16) * s, __uint_as_float(u0 & 0xFFFF0000u) * s);
-      const uint32_t h1 = pack_f16(__uint_as_float(u1 << 16) * s, __uint_as_float(u1 & 0xFFFF0000u) * s);
-      const float2 f0 = h2f2(h0), f1 = h2f2(h1);
-      acc += (f0.x + f0.y) + (f1.x + f1.y);     // sum of the fp16 values actually multiplied
-      a0[ks] = h0;
-      a2[ks] = pack_f16(f1.x * 0.0625f, f1.y * 0.0625f);
-    }
-    (void)s16;
-    acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-    acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-    sum8 = 8.f * acc;
-  };
-
   // candidate partial (max, sum exp) of the current problem, kept per lane and reduced across the warp
   // only when the warp moves on: one (head, warp) partial per problem instead of one per group
   float pm[NH], ps[NH];
@@ -568,15 +581,6 @@ __global__ void __launch_bounds__(kScanWarps * 32, kScanCtasPerSm) scan_i4_kerne
   float *srow[NH];                              // score row(s) of this lane's head(s) of the current problem
 #pragma unroll
   for (int hh = 0; hh < NH; ++hh) srow[hh] = p.shat;
-  auto accumulate = [&](float &m, float &sacc, float v) {   // online log-sum-exp, one exp per value
-    // branch-free: a value of -inf (masked page) adds nothing, whatever m is (also -inf at the start)
-    const bool live = v > -INFINITY;
-    const float d = v - m;                                    // NaN only if both are -inf: not live then
-    const float e = live ? __expf(-fabsf(d)) : 0.f;           // m = -inf, v finite: exp(-inf) = 0
-    const bool up = live && d > 0.f;
-    sacc = up ? fmaf(sacc, e, 1.f) : sacc + e;
-    m = up ? v : m;
-  };
   float2 *red = reinterpret_cast<float2 *>(smem + kScanWarps * (kScanStages * kStageBytes + 64));   // [warp][16]
   auto flush = [&](bool to_smem, bool finished) {
     const int pslot = cur_pslot;
@@ -623,7 +627,7 @@ __global__ void __launch_bounds__(kScanWarps * 32, kScanCtasPerSm) scan_i4_kerne
       for (int hh = 0; hh < NH; ++hh) {
         float s8;
         const int gx = PK ? (x & 3) : x + 8 * hh;   // head held by this lane's column
-        load_q_row(b, h * p.G + gx, gx < p.G, qb0[hh], qb2[hh], inv_s[hh], s8);
+        load_q_row(q + ((int64_t)b * p.Hq + h * p.G + gx) * LOCKS_D, t, gx < p.G, qb0[hh], qb2[hh], inv_s[hh], s8);
         // lane (x, t) owns head gx; the column fragment needs the heads of columns 2t, 2t+1
         ksum[2 * hh] = __shfl_sync(0xffffffffu, s8, (2 * t) * 4);
         ksum[2 * hh + 1] = __shfl_sync(0xffffffffu, s8, (2 * t + 1) * 4);
@@ -916,7 +920,7 @@ __global__ void __launch_bounds__(kScanWarps * 32, kScanCtasPerSm) scan_i4_kerne
       const float v = res[0] * kLn2;
       const bool in = t < LOCKS_GROUP / 2 && page < cc.nsc;
       if (g < p.G && in) store_score(srow[0] + page, v);
-      accumulate(pm[0], ps[0], (in && page >= 1) ? v : -INFINITY);
+      lse_accumulate(pm[0], ps[0], (in && page >= 1) ? v : -INFINITY);
     } else {
     const int page0 = cc.grp * LOCKS_GROUP + 2 * t;
 #pragma unroll
@@ -930,8 +934,8 @@ __global__ void __launch_bounds__(kScanWarps * 32, kScanCtasPerSm) scan_i4_kerne
         if (in0) store_score(dst, v0);
         if (in1) store_score(dst + 1, v1);
       }
-      accumulate(pm[hh], ps[hh], (in0 && page0 >= 1) ? v0 : -INFINITY);
-      accumulate(pm[hh], ps[hh], in1 ? v1 : -INFINITY);
+      lse_accumulate(pm[hh], ps[hh], (in0 && page0 >= 1) ? v0 : -INFINITY);
+      lse_accumulate(pm[hh], ps[hh], in1 ? v1 : -INFINITY);
     }
     }
     advance(cc, it + 1 < n_units);
@@ -961,6 +965,164 @@ __global__ void __launch_bounds__(kScanWarps * 32, kScanCtasPerSm) scan_i4_kerne
     for (int s = 0; s < inflight && s < kScanStages; ++s) {
       const int st = (it + s) % kScanStages;
       (void)mbar_wait(&full[st], ((it + s) / kScanStages) & 1);
+    }
+  }
+}
+
+// ------------------------------------------------------------------------------------------------
+// int4 summaries of 32- and 64-token pages (B = 8 NT), bf16 queries.  The arithmetic of scan_i4_kernel with the query heads
+// as MMA rows and the codes as the other operand: the projection then comes out as the operand of the logits MMA, with no
+// transpose, and the centroid dots come out in the lanes that finish the pages.  With 8 heads or fewer half of the rows are
+// idle, which these page sizes can afford: half or a quarter as many summaries for the same context.  A warp takes groups
+// of 8 pages in strides; no staging, the loads of a summary (1 .. 1.3 KB) go straight to fragments and other warps cover
+// their latency.  4 x 16K tokens, 32-token pages, 4 heads per KV head (floor 2.4 us): 137 us in the plain kernel, which passes
+// over a summary once per head; the whole step 176 -> 65 us.
+// ------------------------------------------------------------------------------------------------
+constexpr int kWideWarps = 4;
+
+template <int R, int NT, int NH>
+__global__ void __launch_bounds__(kWideWarps * 32) scan_wide_kernel(ScanParams p) {
+  constexpr int B = 8 * NT, S = i4_stride(R, B);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, x = lane >> 2, t = lane & 3, h = blockIdx.y, b = blockIdx.z;
+  pdl_trigger();
+  pdl_wait();
+  publish_lengths(p, (blockIdx.x | blockIdx.y | blockIdx.z) == 0, threadIdx.x, kWideWarps * 32);
+  const int P = (step_len(p, b) + B - 1) / B;
+  if (P <= p.k) return;               // every page is kept: nothing to rank
+  const int nsc = P - 1;              // pages 0 .. P-2 are scored
+  int grp = blockIdx.x * kWideWarps + warp;
+  if (grp * LOCKS_GROUP >= nsc) return;
+
+  uint32_t qb0[2][8], qb2[2][8];
+  float inv_s[NH], ksum[NH];
+#pragma unroll
+  for (int hh = 0; hh < 2; ++hh) {
+    if (hh < NH) {
+      const int g = x + 8 * hh;
+      load_q_row(reinterpret_cast<const __nv_bfloat16 *>(p.q) + ((int64_t)b * p.Hq + h * p.G + g) * LOCKS_D, t, g < p.G, qb0[hh],
+                 qb2[hh], inv_s[hh], ksum[hh]);
+      inv_s[hh] *= p.sm_scale * kLog2e;   // turns a scaled dot product into a log2-domain logit
+    } else {
+#pragma unroll
+      for (int s = 0; s < 8; ++s) qb0[hh][s] = qb2[hh][s] = 0u;
+    }
+  }
+  const int32_t *bt = p.block_table + (int64_t)b * p.Pmax;
+  const uint8_t *summ = p.summ + (int64_t)h * S;
+  const int64_t page_stride = (int64_t)p.Hkv * S;
+  for (; grp * LOCKS_GROUP < nsc; grp += gridDim.x * kWideWarps) {
+    const int page_of_lane = grp * LOCKS_GROUP + (lane & 7);
+    int block = page_of_lane < nsc ? bt[page_of_lane] : -1;
+    bool have = page_of_lane < nsc;
+    if (have && (block < 0 || block >= p.num_blocks)) {
+      set_status(p.status, LOCKS_ERR_BAD_BLOCK);
+      have = false;
+    }
+    const uint32_t valid = __ballot_sync(0xffffffffu, have) & 0xffu;   // pages of the group that are scored
+    if (!have) block = 0;
+    // ---- centroid dots: columns = pages.  cen: heads x (+ 8), pages 2t, 2t + 1
+    float cen[4] = {0.f, 0.f, 0.f, 0.f};
+    float smu;
+    {
+      const uint8_t *pb = summ + (int64_t)__shfl_sync(0xffffffffu, block, x) * page_stride;
+      const uint4 *mp = reinterpret_cast<const uint4 *>(pb + i4_off_mu(R, B) + 32 * t);
+      const uint4 m0 = mp[0], m1 = mp[1];
+      smu = __half2float(*reinterpret_cast<const __half *>(pb + i4_off_smu(R, B)));
+      const uint32_t mw[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
+#pragma unroll
+      for (int s = 0; s < 8; ++s) {
+        const uint32_t b0 = f16x2_sub(and_or(mw[s], 0x00FF00FFu, 0x64006400u), 0x64806480u);                    // code
+        const uint32_t b1 = f16x2_fma(and_or(mw[s] >> 8, 0x00FF00FFu, 0x64006400u), 0x4C004C00u, 0xF480F480u);   // 16 * code
+        mma_f16(cen, qb0[0][s], qb0[1][s], qb2[0][s], qb2[1][s], b0, b1);
+      }
+    }
+    float res[NH][2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const float sm = __shfl_sync(0xffffffffu, smu, (2 * t + e) * 4);
+#pragma unroll
+      for (int hh = 0; hh < NH; ++hh) res[hh][e] = cen[2 * hh + e] * sm * inv_s[hh];
+    }
+#pragma unroll 2
+    for (int pg = 0; pg < LOCKS_GROUP; ++pg) {
+      const uint8_t *pb = summ + (int64_t)__shfl_sync(0xffffffffu, block, pg) * page_stride;
+      // lane (x, t): basis of rank x, quarter t; coefficients of tokens 8 n + x, ranks 2t, 2t + 1; scales of tokens 8 n + 2t, + 1
+      const uint4 w4 = (R == 8 || x < R) ? *reinterpret_cast<const uint4 *>(pb + lane * 16) : make_uint4(0u, 0u, 0u, 0u);
+      uint32_t cw[NT], sc[NT];
+#pragma unroll
+      for (int n = 0; n < NT; ++n) {
+        cw[n] = (t < R / 2) ? *reinterpret_cast<const uint16_t *>(pb + i4_off_coef(R) + (8 * n + x) * R + 2 * t) : 0x8080u;
+        sc[n] = *reinterpret_cast<const uint32_t *>(pb + i4_off_sc(R, B) + 2 * (8 * n + 2 * t));
+      }
+      const float2 sv = (t < R / 2) ? h2f2(*reinterpret_cast<const uint32_t *>(pb + i4_off_sv(R, B) + 4 * t)) : make_float2(0.f, 0.f);
+      // ---- projection: rows = heads, columns = ranks
+      float c[4];
+      const uint32_t wd[4] = {w4.x, w4.y, w4.z, w4.w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const uint32_t u = wd[j], u8 = u >> 8;
+        if (j == 0) mma_f16_z(c, qb0[0][0], qb0[1][0], qb2[0][0], qb2[1][0], u & 0x000F000Fu, u & 0x00F000F0u);
+        else mma_f16(c, qb0[0][2 * j], qb0[1][2 * j], qb2[0][2 * j], qb2[1][2 * j], u & 0x000F000Fu, u & 0x00F000F0u);
+        mma_f16(c, qb0[0][2 * j + 1], qb0[1][2 * j + 1], qb2[0][2 * j + 1], qb2[1][2 * j + 1], u8 & 0x000F000Fu, u8 & 0x00F000F0u);
+      }
+      uint32_t hi[2] = {0u, 0u}, lo[2] = {0u, 0u};
+#pragma unroll
+      for (int hh = 0; hh < NH; ++hh) {   // undo 2^-24, remove the + 8 offset, apply the column scale
+        const float p0 = fmaf(c[2 * hh], 16777216.f, -ksum[hh]) * sv.x, p1 = fmaf(c[2 * hh + 1], 16777216.f, -ksum[hh]) * sv.y;
+        hi[hh] = pack_f16(p0, p1);
+        const float2 hf = h2f2(hi[hh]);
+        lo[hh] = pack_f16(p0 - hf.x, p1 - hf.y);
+      }
+      // ---- logits: rows = heads, k = ranks (hi | lo), columns = tokens
+      float y[NT][4];
+#pragma unroll
+      for (int n = 0; n < NT; ++n) {
+        const uint32_t cf = f16x2_sub(__byte_perm(cw[n], 0x64646464u, 0x4140), 0x64806480u);
+        mma_f16_z(y[n], hi[0], hi[1], lo[0], lo[1], cf, cf);
+      }
+#pragma unroll
+      for (int hh = 0; hh < NH; ++hh) {
+        float my = -INFINITY;
+#pragma unroll
+        for (int n = 0; n < NT; ++n) {
+          const float2 s2 = h2f2(sc[n]);
+          y[n][2 * hh] *= s2.x;
+          y[n][2 * hh + 1] *= s2.y;
+          my = fmaxf(my, fmaxf(y[n][2 * hh], y[n][2 * hh + 1]));
+        }
+        my = fmaxf(my, __shfl_xor_sync(0xffffffffu, my, 1));
+        my = fmaxf(my, __shfl_xor_sync(0xffffffffu, my, 2));
+        const float iv = inv_s[hh], m = my * iv;
+        float e = 0.f;
+#pragma unroll
+        for (int n = 0; n < NT; ++n) e += fast_ex2(fmaf(y[n][2 * hh], iv, -m)) + fast_ex2(fmaf(y[n][2 * hh + 1], iv, -m));
+        e += __shfl_xor_sync(0xffffffffu, e, 1);
+        e += __shfl_xor_sync(0xffffffffu, e, 2);
+        const float v = m + fast_lg2(e);
+        if (t == (pg >> 1)) {
+          if (pg & 1) res[hh][1] += v; else res[hh][0] += v;
+        }
+      }
+    }
+    // ---- write s^ and the group's candidate partial
+#pragma unroll
+    for (int hh = 0; hh < NH; ++hh) {
+      const int g = x + 8 * hh, page0 = grp * LOCKS_GROUP + 2 * t;
+      float pm = -INFINITY, ps = 0.f;
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const float v = res[hh][e] * kLn2;
+        const bool in = (valid >> (2 * t + e)) & 1u;
+        if (g < p.G && in) p.shat[((int64_t)b * p.Hq + h * p.G + g) * p.Pmax + page0 + e] = v;
+        lse_accumulate(pm, ps, in && page0 + e >= 1 ? v : -INFINITY);
+      }
+#pragma unroll
+      for (int o = 1; o < 4; o <<= 1) {
+        const float om = __shfl_xor_sync(0xffffffffu, pm, o), os = __shfl_xor_sync(0xffffffffu, ps, o);
+        const float nm = fmaxf(pm, om);
+        if (nm > -INFINITY) { ps = ps * __expf(pm - nm) + os * __expf(om - nm); pm = nm; }
+      }
+      if (t == 0 && g < p.G) p.part[((int64_t)b * p.Hq + h * p.G + g) * p.max_groups + grp] = make_float2(pm, ps);
     }
   }
 }
@@ -1077,6 +1239,21 @@ int locks_launch_scan(locks_ctx *c, const void *q, const void *summaries, const 
     else if (balanced) LOCKS_SCAN_LAUNCH(2, false, true);
     else LOCKS_SCAN_LAUNCH(2, false, false);
 #undef LOCKS_SCAN_LAUNCH
+  } else if (c->cfg.summary_fmt == LOCKS_FMT_I4 && c->cfg.q_dtype == LOCKS_BF16 && c->scorer == LOCKS_SCORER_SUMMARY) {
+    // 32- and 64-token pages: about four CTAs of four warps per SM, each warp striding a problem's groups
+    const int most = (c->max_groups + kWideWarps - 1) / kWideWarps, want = (4 * c->num_sms + batch * p.Hkv - 1) / (batch * p.Hkv);
+    const dim3 grid(most < want ? most : want, p.Hkv, batch), blk(kWideWarps * 32);
+#define LOCKS_WIDE_LAUNCH(R_)                                                                                \
+  do {                                                                                                      \
+    if (c->B == 32 && c->G <= 8) locks_launch_pdl(scan_wide_kernel<R_, 4, 1>, grid, blk, 0, st, p);         \
+    else if (c->B == 32) locks_launch_pdl(scan_wide_kernel<R_, 4, 2>, grid, blk, 0, st, p);                 \
+    else if (c->G <= 8) locks_launch_pdl(scan_wide_kernel<R_, 8, 1>, grid, blk, 0, st, p);                  \
+    else locks_launch_pdl(scan_wide_kernel<R_, 8, 2>, grid, blk, 0, st, p);                                 \
+  } while (0)
+    if (p.r == 8) LOCKS_WIDE_LAUNCH(8);
+    else if (p.r == 4) LOCKS_WIDE_LAUNCH(4);
+    else LOCKS_WIDE_LAUNCH(2);
+#undef LOCKS_WIDE_LAUNCH
   } else {
     dim3 grid((c->max_groups + 3) / 4, p.Hkv, batch);
     const bool qbf = c->cfg.q_dtype == LOCKS_BF16;

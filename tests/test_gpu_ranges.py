@@ -133,3 +133,15 @@ def test_bulk_build_partial_warps_and_degenerate_pages(rank, layout):
             total += got[blk].size
             differ += int((got[blk] != want[blk]).sum())
     assert differ <= 2e-3 * total, (differ, total)
+
+
+# The scan of int4 summaries at 32- and 64-token pages: every rank, one and two tiles of query heads, group sizes that fill
+# neither, sequences that end inside a group of eight pages, more groups than warps (strides), extreme logits.
+@pytest.mark.parametrize("B", [32, 64])
+@pytest.mark.parametrize("lens,Hq,Hkv,rank,qs", [([40, 9, 17.5], 8, 2, 8, 1.0), ([33, 8.2], 32, 2, 8, 2.0), ([41], 12, 1, 4, 1.0),
+                                                 ([25, 24, 18], 6, 3, 2, 1.0), ([900], 16, 1, 8, 4.0), ([60, 3], 2, 2, 4, 0.0)])
+def test_wide_page_scan(B, lens, Hq, Hkv, rank, qs):
+    from gpu_util import GpuCase, check_select_and_attend
+    w = locks_synth.Workload("wide", [max(1, int(n * B)) for n in lens], Hq=Hq, Hkv=Hkv, B=B, rank=rank, budget=6 * B, seed=B + rank, q_scale=qs)
+    gc = GpuCase(w)
+    check_select_and_attend(gc, gc.oracle_summaries(), out_tol=2e-2)
