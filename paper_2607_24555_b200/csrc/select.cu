@@ -2,13 +2,13 @@
 //   log Z_g   = log sum_{j in 1..P-2} exp s^_j(q_g)                       (candidates only)
 //   log m_bar_j = log( (1/G) sum_g exp(s^_j(q_g) - log Z_g) )
 //   S = {0, P-1}  U  top-(k-2) candidates by log m_bar_j (ties: lower page index), ids ascending.
-// One 512-thread CTA ranks a chunk of 2048 / 4096 / 8192 pages of a (request, KV head): it turns the
-// chunk's scores into order-preserving 32-bit keys in shared memory, finds the (k-2)-th largest with an
-// exact 4-pass radix select and compacts the winners in page order.  With one chunk per problem that is
-// the final table.  With several, each chunk emits its own top-(k-2) (value, page) list, and the CTA of a
-// problem that finishes last ranks the lists the same way in the same launch (a chunk's local top-(k-2)
-// always contains the chunk's share of the global top-(k-2), ties included, because both rounds use the
-// same lower-index tie rule and lists stay in page order).
+// One 512-thread CTA ranks a chunk of 512 .. 8192 pages of a (request, KV head): it turns the chunk's scores into
+// order-preserving 32-bit keys in shared memory and emits the K = k-2 largest in page order (select_emit: a histogram that
+// finds the bin of the K-th largest key, an exact ranking of that bin's few keys, and a bit map of the winners, whose prefix
+// counts are the output positions).  With one chunk per problem that is the final table.  With several, each chunk emits
+// its own top-(k-2) (key, page) list, and the CTA of a problem that finishes last ranks the lists the same way in the same
+// launch (a chunk's local top-(k-2) always contains the chunk's share of the global top-(k-2), ties included, because both
+// rounds use the same lower-index tie rule and lists stay in page order).
 // Pages are dealt to threads round-robin (element i of thread t is page i*512 + t), so loads are
 // coalesced and every thread is busy whatever the context length.
 // The kernel runs once through its code on at most a few dozen SMs, so instruction fetch is a visible part
@@ -73,15 +73,20 @@ __device__ __forceinline__ void append_token(const locks_append &a, int batch, i
   }
 }
 
+constexpr int kListMax = 256;    // keys of the threshold bin that are ranked pair by pair
+constexpr int kElemBits = 13;    // kMaxKeys = 2^13 elements
+
 struct SelShared {
-  uint32_t key[kMaxKeys];             // order-preserving keys, element i of thread t at i*512 + t
+  uint32_t key[kMaxKeys];             // order-preserving keys, element i of thread t at i*512 + t; 0 = not a candidate
   int hist[3 * 256];                  // radix histograms, rotating
-  __align__(16) int cnt[256];         // per (slab, warp) winner counts for the ordered compaction
-  int misc[16];                       // per-pass result (double-buffered), arrival flag
+  __align__(16) uint32_t gt[256];     // winners, one bit per element in element order
+  __align__(16) uint32_t eq[256];     // elements of the threshold bin, where it holds equal keys or wins whole
+  __align__(16) uint32_t list[kListMax];
+  int nlist;
+  int misc[16];                       // arrival flag
   float lz2[16];                      // log2-domain log Z_g
   float lzm[kNW], lzs[kNW];           // per-warp (max, sum) of the log Z reduction
-  uint32_t red[2 * kNW];              // per-warp AND / OR of the keys
-  int win[kMaxWin];                   // final round: entry index of winner number pos
+  uint32_t red[2 * kNW];              // per-warp smallest and largest valid key
 };
 
 extern __shared__ __align__(16) uint8_t sel_smem[];
@@ -104,51 +109,57 @@ __device__ __forceinline__ uint32_t order_key(float f) {
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-// K-th largest of the keys sh.key[i*512 + t], i < nslab (invalid elements hold key 0; 1 <= K <= number of
-// valid keys).  Returns (key, how many of the keys equal to it belong to the top K).
-// Radix passes of up to 8 bits from the top over the keys' offsets from the smallest valid key (one MIN / MAX
-// reduction first).  A pass costs one barrier: all warps count into
-// one 256-bin histogram, then every warp scans it on its own (lane l owns bins 8 (31 - l) .. + 7, so
-// lane order is descending digit order) while the histogram of the next pass -- three rotate -- is
-// already being filled by warps that are ahead.
-__device__ __noinline__ uint2 radix_select(int nslab, int K) {
+// smallest and largest valid key of this thread -> sh.red (read by select_emit after its first barrier)
+__device__ __forceinline__ void publish_range(SelShared &sh, uint32_t kmin, uint32_t kmax) {
+  kmin = __reduce_min_sync(0xffffffffu, kmin);
+  kmax = __reduce_max_sync(0xffffffffu, kmax);
+  if ((threadIdx.x & 31) == 0) { sh.red[threadIdx.x >> 5] = kmin; sh.red[kNW + (threadIdx.x >> 5)] = kmax; }
+}
+
+// The K largest of the keys sh.key[i*512 + t], i < nslab (1 <= K <= number of valid keys; the range of the keys is in
+// sh.red), in element order and with ties to the lower element.  Winner number pos of element e is written as
+//   kEmitIds:   ids[1 + pos] = c0 + e                         (final table of a single-chunk problem)
+//   kEmitList:  list_key[pos] = key, list_idx[pos] = c0 + e   (a chunk's candidate list)
+//   kEmitFinal: ids[1 + pos] = page of entry e                (final table from the problem's lists; pages at sh.key[4096 + e]
+//                                                              if there are at most 4096 entries, else in list_idx)
+// The keys' offsets from the smallest one need far fewer than 32 bits (page masses lie within a few units of each other),
+// and one pass over their leading 8 bits usually leaves a few dozen keys in the bin of the K-th largest: these are ranked
+// pair by pair.  A fuller bin is divided again; a bin of equal keys, or one that wins whole, needs no ranking.
+// What bounds this is the chain of barriers, shuffles and instruction fetches (every phase runs once, on few SMs), not the
+// keys: four barriers here, where three 8-bit radix passes and an ordered compaction by ballots and a scan of counts took
+// eleven.  Steps, before and after: 1 x 8K tokens 27.8 -> 26.6 us, 8 x 32K 59.3 -> 57.1, 32 x 16K with a budget of 16 pages
+// 62.0 -> 58.1, 24 chat requests 59.4 -> 57.1, 1 x 128K (lists of 9 chunks, ranked twice) 42.4 -> 41.2.  Running this code
+// once on made-up keys before the wait for the scan, to have it in the instruction caches, costs 1 .. 6 us: the selector's
+// CTAs become resident only when the scan is nearly over.
+enum { kEmitIds = 0, kEmitList = 1, kEmitFinal = 2 };
+constexpr int kFinalPages = kMaxKeys / 2;
+
+__device__ __noinline__ void select_emit(int nslab, int K, int mode, int c0, int32_t *ids, uint32_t *list_key, int32_t *list_idx) {
   SelShared &sh = shared_state();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (tid < 256) sh.hist[tid] = 0;
-  uint32_t kmin = 0xFFFFFFFFu, kmax = 0u;
-#pragma unroll 4
-  for (int i = 0; i < nslab; ++i) {
-    const uint32_t k = sh.key[i * LOCKS_SEL_THREADS + tid];
-    if (k) { kmin = min(kmin, k); kmax = max(kmax, k); }
-  }
-  kmin = __reduce_min_sync(0xffffffffu, kmin);
-  kmax = __reduce_max_sync(0xffffffffu, kmax);
-  if (lane == 0) { sh.red[warp] = kmin; sh.red[kNW + warp] = kmax; }
+  if (tid == 0) sh.nlist = 0;
   __syncthreads();
-  kmin = __reduce_min_sync(0xffffffffu, sh.red[lane & (kNW - 1)]);
-  kmax = __reduce_max_sync(0xffffffffu, sh.red[kNW + (lane & (kNW - 1))]);
-  // The passes rank the keys' offsets from the smallest valid key: page masses lie within a few units of each
-  // other, so the offsets need far fewer than 32 bits (typically 24: three passes), and the first pass already
-  // works on bits in which the keys differ, which spreads them over the bins (hundreds of atomics on two or
-  // three counters would serialise); the later passes see only the few keys of the threshold bin.
-  const int bits = 32 - __clz(kmax - kmin);   // 0: all valid keys are equal (kmax >= kmin: K >= 1 valid keys)
-  uint32_t mask = 0u, prefix = 0u;            // decided leading bits of the offset of the K-th largest key
-  int remaining = K;
-  int cur = 0;
+  const uint32_t kmin = __reduce_min_sync(0xffffffffu, sh.red[lane & (kNW - 1)]);
+  const uint32_t kmax = __reduce_max_sync(0xffffffffu, sh.red[kNW + (lane & (kNW - 1))]);
+  int left = 32 - __clz(kmax - kmin);   // undecided bits of the offsets (0: all valid keys are equal)
+  uint32_t prefix = 0u;                 // decided leading bits of the offset of the K-th largest key, in place
+  int remaining = K;                    // of the keys with that prefix, how many win
+  bool rank = false;                    // they are to be ranked (else: all of them equal, or all of them win)
 #pragma unroll 1
-  for (int left = bits; left > 0;) {   // bits not yet decided
+  for (int cur = 0; left > 0;) {
     const int width = min(8, left), shift = left - width;
-    const uint32_t dmask = (1u << width) - 1u;
-    left = shift;
     const int nxt = cur == 2 ? 0 : cur + 1;
     int *hc = sh.hist + cur * 256;
     if (tid < 256) sh.hist[nxt * 256 + tid] = 0;   // last read two passes ago
+    const uint32_t above = left < 32 ? prefix >> left : 0u;
 #pragma unroll 4
     for (int i = 0; i < nslab; ++i) {
       const uint32_t k = sh.key[i * LOCKS_SEL_THREADS + tid], d = k - kmin;
-      if (k && (d & mask) == prefix) atomicAdd(&hc[(d >> shift) & dmask], 1);
+      if (k && (left < 32 ? d >> left : 0u) == above) atomicAdd(&hc[(d >> shift) & ((1u << width) - 1u)], 1);
     }
     __syncthreads();
+    // every warp: lane l owns bins 8 (31 - l) .. + 7, so lane order is descending digit order
     const int base = 8 * (31 - lane);
     const int4 lo = *reinterpret_cast<const int4 *>(hc + base), hi = *reinterpret_cast<const int4 *>(hc + base + 4);
     const int c[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
@@ -160,89 +171,125 @@ __device__ __noinline__ uint2 radix_select(int nslab, int K) {
       if (lane >= o) incl += v;
     }
     const bool hit = incl - tot < remaining && remaining <= incl;   // the K-th largest falls in this lane's bins
-    int digit = 0, rem = 0, acc = incl - tot;
+    uint32_t found = 0u;   // digit (8 bits), count in its bin (12), rank wanted within it (12; at most the count)
+    int acc = incl - tot;
 #pragma unroll
     for (int j = 7; j >= 0; --j) {
-      if (hit && acc < remaining && remaining <= acc + c[j]) { digit = base + j; rem = remaining - acc; }
+      if (hit && acc < remaining && remaining <= acc + c[j]) found = (uint32_t)(base + j) << 24 | (uint32_t)min(c[j], 4095) << 12 | (uint32_t)min(remaining - acc, 4095);
       acc += c[j];
     }
     const uint32_t who = __ballot_sync(0xffffffffu, hit);
-    const int src = who ? __ffs(who) - 1 : 0;
-    digit = __shfl_sync(0xffffffffu, digit, src);
-    remaining = __shfl_sync(0xffffffffu, rem, src);
-    prefix |= (uint32_t)digit << shift;
-    mask |= dmask << shift;
+    found = __shfl_sync(0xffffffffu, found, who ? __ffs(who) - 1 : 0);
+    const int count = (int)((found >> 12) & 4095u);
+    remaining = (int)(found & 4095u);   // (K is below 4096)
+    prefix |= (found >> 24) << shift;
+    left = shift;
     cur = nxt;
+    if (count == remaining && count < 4095) break;
+    rank = count <= kListMax && left + kElemBits <= 32;
+    if (rank) break;
   }
-  return make_uint2(kmin + prefix, (uint32_t)remaining);
-}
-
-enum { kEmitIds = 0, kEmitList = 1, kEmitFinal = 2 };
-
-// Winners = keys above `prefix` plus the first `remaining` keys equal to it, in element order.  Winner
-// number `pos` (< cap) of element e is written as
-//   kEmitIds:   ids[1 + pos] = c0 + e                         (final table of a single-chunk problem)
-//   kEmitList:  list_key[pos] = key, list_idx[pos] = c0 + e   (a chunk's candidate list)
-//   kEmitFinal: ids[1 + pos] = list_idx[e]                    (final table from the problem's lists)
-__device__ __noinline__ void compact_emit(int nslab, uint32_t prefix, int remaining, int cap, int mode,
-                                          int c0, int32_t *ids, uint32_t *list_key, int32_t *list_idx) {
-  SelShared &sh = shared_state();
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (mode == kEmitFinal)
-    for (int j = tid; j < cap; j += LOCKS_SEL_THREADS) sh.win[j] = 0;   // a slot no winner fills still names a real entry
-  __syncthreads();   // the previous user of sh.cnt is done
+  if (left == 0) rank = false;
+  // ---- winners above the bin, and the bin's own keys
+  const uint32_t at = left < 32 ? prefix >> left : 0u;
 #pragma unroll 2
   for (int i = 0; i < nslab; ++i) {
-    const uint32_t k = sh.key[i * LOCKS_SEL_THREADS + tid];
-    const uint32_t bg = __ballot_sync(0xffffffffu, k > prefix), be = __ballot_sync(0xffffffffu, k == prefix);
-    if (lane == 0) sh.cnt[i * kNW + warp] = (__popc(bg) << 16) | __popc(be);
+    const int e = i * LOCKS_SEL_THREADS + tid;
+    const uint32_t k = sh.key[e], d = k - kmin, top = left < 32 ? d >> left : 0u;
+    const uint32_t g = __ballot_sync(0xffffffffu, k && top > at), q = __ballot_sync(0xffffffffu, k && top == at);
+    if (lane == 0) { sh.gt[i * kNW + warp] = g; sh.eq[i * kNW + warp] = q; }
+    if (rank && k && top == at)   // the rest of the offset, then the element: larger is better, no two alike
+      sh.list[min(atomicAdd(&sh.nlist, 1), kListMax - 1)] = (d & ((1u << left) - 1u)) << kElemBits | (uint32_t)(kMaxKeys - 1 - e);
   }
   __syncthreads();
-  if (warp == 0) {   // exclusive scan of the nslab * kNW (<= 256) counts in (slab, warp) order, 8 per lane
-    const int n = nslab * kNW;
-    int4 *q = reinterpret_cast<int4 *>(sh.cnt + lane * 8);
-    int4 lo = q[0], hi = q[1];
-    int c[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
-    int tot = 0;
+  if (rank) {
+    const int n = min(sh.nlist, kListMax);
+    if (tid < n) {
+      const uint32_t mine = sh.list[tid];
+      int better = 0;
+      for (int j = 0; j < n; j += 4) {
+        const uint4 o = *reinterpret_cast<const uint4 *>(sh.list + j);
+        better += (int)(o.x > mine) + (int)(o.y > mine && j + 1 < n) + (int)(o.z > mine && j + 2 < n) + (int)(o.w > mine && j + 3 < n);
+      }
+      const int e = kMaxKeys - 1 - (int)(mine & (kMaxKeys - 1));
+      if (better < remaining) atomicOr(&sh.gt[e >> 5], 1u << (e & 31));
+    }
+    __syncthreads();
+  }
+  const int nw = nslab * kNW;
+  if (K < 24 * nslab) {
+    // ---- few winners: a thread per 32 elements finds the position of its first winner and walks its winners (8192 pages, 126
+    // winners: 0.7 us, the other way 2.4)
+    if (warp * 32 >= nw) return;
+    int before = 0, eq_before = 0;   // winners, and unranked keys of the bin, in the words of the warps before this one
 #pragma unroll
-    for (int j = 0; j < 8; ++j) { if (lane * 8 + j >= n) c[j] = 0; tot += c[j]; }
-    int incl = tot;
+    for (int u = 0; u < 8; ++u) {
+      const int w = u * 32 + lane;
+      if (w < warp * 32) { before += __popc(sh.gt[w]); eq_before += __popc(sh.eq[w]); }
+    }
+    const int w = warp * 32 + lane;
+    uint32_t won = w < nw ? sh.gt[w] : 0u, q = w < nw && !rank ? sh.eq[w] : 0u;
+    int incl = __popc(won) | __popc(q) << 16;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int v = __shfl_up_sync(0xffffffffu, incl, o);
       if (lane >= o) incl += v;
     }
-    int run = incl - tot;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) { const int v = c[j]; c[j] = run; run += v; }
-    q[0] = make_int4(c[0], c[1], c[2], c[3]);
-    q[1] = make_int4(c[4], c[5], c[6], c[7]);
+    before = __reduce_add_sync(0xffffffffu, before);
+    eq_before = __reduce_add_sync(0xffffffffu, eq_before);
+    int pos = before + (incl & 0xffff) - __popc(won);
+    if (!rank) {
+      eq_before += (incl >> 16) - __popc(q);
+      pos += min(eq_before, remaining);
+      for (int take = remaining - eq_before; q && take > 0; --take) { won |= q & -q; q &= q - 1; }
+    }
+    for (; won; won &= won - 1, ++pos) {
+      const int e = w * 32 + __ffs(won) - 1;
+      if (mode == kEmitIds) ids[1 + pos] = c0 + e;
+      else if (mode == kEmitList) { list_key[pos] = sh.key[e]; list_idx[pos] = c0 + e; }
+      else ids[1 + pos] = list_key ? (int32_t)sh.key[kFinalPages + e] : __ldcg(list_idx + e);
+    }
+    return;
   }
-  __syncthreads();
+  // ---- positions: every warp counts the winners (and the bin's unranked keys) before each of its words; lane l owns words
+  // 8 l .. 8 l + 7, and word i * kNW + warp is the same one of lane 2 i or 2 i + 1 for every i (512 pages, 126 winners: 0.8 us,
+  // the other way 1.4)
+  const int mine = warp & 7, half = warp >> 3;
+  uint32_t g8[8], q8[8];
+  {
+    const uint4 *gp = reinterpret_cast<const uint4 *>(sh.gt + 8 * lane), *qp = reinterpret_cast<const uint4 *>(sh.eq + 8 * lane);
+    const bool in = 8 * lane < nw;
+    const uint4 z = make_uint4(0u, 0u, 0u, 0u), a = in ? gp[0] : z, b = in ? gp[1] : z, c = in && !rank ? qp[0] : z, d = in && !rank ? qp[1] : z;
+    g8[0] = a.x; g8[1] = a.y; g8[2] = a.z; g8[3] = a.w; g8[4] = b.x; g8[5] = b.y; g8[6] = b.z; g8[7] = b.w;
+    q8[0] = c.x; q8[1] = c.y; q8[2] = c.z; q8[3] = c.w; q8[4] = d.x; q8[5] = d.y; q8[6] = d.z; q8[7] = d.w;
+  }
+  int before = 0, total = 0;   // packed: winners | unranked keys << 16; before this lane's word `mine`, and in all of its words
+  uint32_t g = 0u, q = 0u;
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    if (u == mine) { before = total; g = g8[u]; q = q8[u]; }
+    total += __popc(g8[u]) | __popc(q8[u]) << 16;
+  }
+  int incl = total;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += v;
+  }
+  before += incl - total;
   const uint32_t lt = (1u << lane) - 1u;
 #pragma unroll 2
   for (int i = 0; i < nslab; ++i) {
-    const int e = i * LOCKS_SEL_THREADS + tid;
-    const uint32_t k = sh.key[e];
-    const bool gt = k > prefix, eq = k == prefix;
-    const uint32_t bg = __ballot_sync(0xffffffffu, gt), be = __ballot_sync(0xffffffffu, eq);
-    const int base = sh.cnt[i * kNW + warp];
-    const int gt_before = (base >> 16) + __popc(bg & lt), eq_before = (base & 0xffff) + __popc(be & lt);
-    const int pos = gt_before + min(eq_before, remaining);
-    if ((gt || (eq && eq_before < remaining)) && pos < cap) {
+    const int src = 2 * i + half;
+    const uint32_t gw = __shfl_sync(0xffffffffu, g, src), qw = __shfl_sync(0xffffffffu, q, src);
+    const int pre = __shfl_sync(0xffffffffu, before, src);
+    const int eq_before = (pre >> 16) + __popc(qw & lt);
+    const bool won = ((gw >> lane) & 1u) || (((qw >> lane) & 1u) && eq_before < remaining);
+    if (won) {
+      const int e = i * LOCKS_SEL_THREADS + tid, pos = (pre & 0xffff) + __popc(gw & lt) + min(eq_before, remaining);
       if (mode == kEmitIds) ids[1 + pos] = c0 + e;
-      else if (mode == kEmitList) { list_key[pos] = k; list_idx[pos] = c0 + e; }
-      else sh.win[pos] = e;   // the page of entry e is fetched below, all winners at once
-    }
-  }
-  if (mode == kEmitFinal) {
-    __syncthreads();
-    for (int j0 = tid; j0 < cap; j0 += 4 * LOCKS_SEL_THREADS) {
-      int v[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) { const int j = j0 + u * LOCKS_SEL_THREADS; v[u] = j < cap ? __ldcg(list_idx + sh.win[j]) : 0; }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) { const int j = j0 + u * LOCKS_SEL_THREADS; if (j < cap) ids[1 + j] = v[u]; }
+      else if (mode == kEmitList) { list_key[pos] = sh.key[e]; list_idx[pos] = c0 + e; }
+      else ids[1 + pos] = list_key ? (int32_t)sh.key[kFinalPages + e] : __ldcg(list_idx + e);
     }
   }
 }
@@ -277,9 +324,8 @@ __device__ __noinline__ void group_logz(const float2 *part0, int G, int max_grou
           m = nm;
         }
       }
-      float M = m;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+      const uint32_t top = __reduce_max_sync(0xffffffffu, order_key(m));
+      const float M = __uint_as_float((top & 0x80000000u) ? top & 0x7FFFFFFFu : ~top);
       s = M > -INFINITY ? s * ex2f((m - M) * kLog2e) : 0.f;
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
@@ -339,6 +385,7 @@ __device__ __noinline__ void chunk_keys(const float *shat0, const float2 *part0,
     __syncthreads();
   }
   const float logG = combine == LOCKS_COMBINE_SHARE_AVG ? __logf((float)G) : 0.f;
+  uint32_t kmin = 0xFFFFFFFFu, kmax = 0u;
   float m[SB], s[SB];
 #pragma unroll
   for (int sl = 0; sl < SB; ++sl) { m[sl] = -INFINITY; s[sl] = 0.f; }
@@ -370,8 +417,13 @@ __device__ __noinline__ void chunk_keys(const float *shat0, const float2 *part0,
         if (i < nslab) {
           const bool valid = page >= 1 && page <= P - 2;
           const float val = (combine == LOCKS_COMBINE_GROUP_MAX ? m[sl] : m[sl] + lg2f(s[sl])) * kLn2 - logG;
-          sh.key[i * LOCKS_SEL_THREADS + tid] = valid ? order_key(val) : 0u;
-          if (valid && logshare0) logshare0[page] = val;
+          const uint32_t key = order_key(val);
+          sh.key[i * LOCKS_SEL_THREADS + tid] = valid ? key : 0u;
+          if (valid) {
+            kmin = min(kmin, key);
+            kmax = max(kmax, key);
+            if (logshare0) logshare0[page] = val;
+          }
         }
         m[sl] = -INFINITY;
         s[sl] = 0.f;
@@ -384,6 +436,7 @@ __device__ __noinline__ void chunk_keys(const float *shat0, const float2 *part0,
     i0 = i1;
     g0 = g1;
   }
+  publish_range(sh, kmin, kmax);
 }
 
 // Several chunks per problem: the chunk that arrives last ranks the problem's candidate lists.
@@ -406,15 +459,19 @@ __device__ __noinline__ void select_finish(int32_t *done, int chunks, int kc, in
   // entries in list order (chunk, position) = page order; element i of thread t is entry i*512 + t
   const int N = chunks * kc;
   const int nslab = (N + LOCKS_SEL_THREADS - 1) / LOCKS_SEL_THREADS;
+  const bool pages_too = N <= kFinalPages;
+  uint32_t kmin = 0xFFFFFFFFu, kmax = 0u;
 #pragma unroll 4
   for (int i = 0; i < nslab; ++i) {
     const int e = i * LOCKS_SEL_THREADS + tid;
-    sh.key[e] = e < N ? __ldcg(ck + e) : 0u;
+    const uint32_t key = e < N ? __ldcg(ck + e) : 0u;
+    sh.key[e] = key;
+    if (pages_too) sh.key[kFinalPages + e] = e < N ? (uint32_t)__ldcg(ci + e) : 0u;
+    if (key) { kmin = min(kmin, key); kmax = max(kmax, key); }
   }
-  if (K2 > 0) {
-    const uint2 r = radix_select(nslab, K2);
-    compact_emit(nslab, r.x, (int)r.y, K2, kEmitFinal, 0, ids, nullptr, const_cast<int32_t *>(ci));
-  }
+  publish_range(sh, kmin, kmax);
+  if (K2 > 0)
+    select_emit(nslab, K2, kEmitFinal, 0, ids, pages_too ? sh.key : nullptr, const_cast<int32_t *>(ci));
   if (tid == 0) {
     ids[0] = 0;
     ids[k - 1] = P - 1;
@@ -464,10 +521,8 @@ __global__ void __launch_bounds__(LOCKS_SEL_THREADS, 2) select_kernel(SelParams 
   }
   const int cand_in_chunk = min(P - 2, c0 + p.chunk_pages - 1) - max(1, c0) + 1;
   const int K = min(p.k - 2, cand_in_chunk);
-  uint2 kth = make_uint2(0xFFFFFFFFu, 0u);
-  if (K > 0) kth = radix_select(nslab, K);
   if (p.chunks == 1) {
-    if (K > 0) compact_emit(nslab, kth.x, (int)kth.y, K, kEmitIds, c0, ids, nullptr, nullptr);
+    if (K > 0) select_emit(nslab, K, kEmitIds, c0, ids, nullptr, nullptr);
     if (tid == 0) {
       ids[0] = 0;
       ids[p.k - 1] = P - 1;
@@ -476,7 +531,7 @@ __global__ void __launch_bounds__(LOCKS_SEL_THREADS, 2) select_kernel(SelParams 
   } else {
     uint32_t *lk = p.cand_key + (prob * p.chunks + chunk) * p.kc;
     for (int j = K + tid; j < p.kc; j += LOCKS_SEL_THREADS) lk[j] = 0u;   // fewer candidates than list slots
-    if (K > 0) compact_emit(nslab, kth.x, (int)kth.y, K, kEmitList, c0, nullptr, lk, p.cand_idx + (prob * p.chunks + chunk) * p.kc);
+    if (K > 0) select_emit(nslab, K, kEmitList, c0, nullptr, lk, p.cand_idx + (prob * p.chunks + chunk) * p.kc);
     select_finish(p.sel_done + prob, p.chunks, p.kc, p.k, ids, p.cnt + prob, p.cand_key + prob * p.chunks * p.kc,
                   p.cand_idx + prob * p.chunks * p.kc, P);
   }
@@ -529,23 +584,29 @@ __global__ void __launch_bounds__(LOCKS_SEL_THREADS) merge_selection_kernel(cons
   if (tid == 0) s_valid = 0;
   __syncthreads();
   int mine = 0;
+  uint32_t kmin = 0xFFFFFFFFu, kmax = 0u;
   for (int i = 0; i < nslab; ++i) {
     const int e = i * LOCKS_SEL_THREADS + tid;
     uint32_t key = 0u;
     if (e < N) {
       const int r = e / kc, j = e - r * kc;
       const int64_t at = ((int64_t)r * nprob + prob) * kc + j;
-      if (cand_page[at] >= 0) { key = order_key(cand_key[at]); ++mine; }
+      if (cand_page[at] >= 0) {
+        key = order_key(cand_key[at]);
+        kmin = min(kmin, key);
+        kmax = max(kmax, key);
+        ++mine;
+      }
     }
     sh.key[e] = key;
   }
   for (int j = tid; j < kc; j += LOCKS_SEL_THREADS) out[j] = -1;
   if (mine) atomicAdd(&s_valid, mine);
+  publish_range(sh, kmin, kmax);
   __syncthreads();
   const int K = min(kc, s_valid);
   if (K > 0) {
-    const uint2 r = radix_select(nslab, K);
-    compact_emit(nslab, r.x, (int)r.y, K, kEmitIds, 0, out - 1, nullptr, nullptr);   // out[pos] = winning entry, in list order
+    select_emit(nslab, K, kEmitIds, 0, out - 1, nullptr, nullptr);   // out[pos] = winning entry, in list order
     __syncthreads();
     int page[(kMaxWin + LOCKS_SEL_THREADS - 1) / LOCKS_SEL_THREADS];
 #pragma unroll

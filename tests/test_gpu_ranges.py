@@ -145,3 +145,37 @@ def test_wide_page_scan(B, lens, Hq, Hkv, rank, qs):
     w = locks_synth.Workload("wide", [max(1, int(n * B)) for n in lens], Hq=Hq, Hkv=Hkv, B=B, rank=rank, budget=6 * B, seed=B + rank, q_scale=qs)
     gc = GpuCase(w)
     check_select_and_attend(gc, gc.oracle_summaries(), out_tol=2e-2)
+
+
+# The K largest of up to 8192 keys in list order, ties to the earlier entry (exact: whole numbers against a sort).  Keys that
+# leave the first histogram's threshold bin empty, full or crowded: all equal, two values, a crowd beside far outliers (a
+# range of 32 bits), equal keys across the threshold, a smooth spread; as few as one winner, as many as there are entries.
+@pytest.mark.parametrize("parts,kc", [(1, 1), (3, 1), (2, 30), (9, 126), (33, 126), (16, 510), (4, 2046), (8, 700)])
+@pytest.mark.parametrize("kind", ["equal", "two", "outliers", "ties", "spread", "holes"])
+def test_ranking_of_candidate_lists(parts, kc, kind):
+    import paper_2607_24555_b200 as locks
+    from paper_2607_24555_b200.binding import make_config
+    if parts * kc > 8192:
+        pytest.skip("more entries than a ranking takes")
+    rng = np.random.default_rng(parts * 31 + kc)
+    ctx = locks.Context(make_config(2, 2, 8, "i4", "bf16", 2, 8000, (kc + 2) * 16))
+    shape = (parts, 2, 2, kc)
+    key = {"equal": np.full(shape, -3.25), "two": rng.choice([-1.0, -2.0], shape), "spread": -8.0 + 3.0 * rng.standard_normal(shape),
+           "outliers": np.where(rng.random(shape) < 0.01, rng.choice([3e38, -3e38], shape), -5.0 + 1e-5 * rng.standard_normal(shape)),
+           "ties": np.round(-6.0 + 2.0 * rng.standard_normal(shape), 1), "holes": -8.0 + 3.0 * rng.standard_normal(shape)}[kind].astype(np.float32)
+    page = np.tile(np.arange(parts * kc, dtype=np.int32).reshape(parts, 1, 1, kc) * 7 + 1, (1, 2, 2, 1))
+    if kind == "holes":
+        page[rng.random(shape) < 0.9] = -1
+    ids = torch.full((2, 2, kc), -7, dtype=torch.int32, device="cuda:0")
+    cnt = torch.full((2, 2), -7, dtype=torch.int32, device="cuda:0")
+    for _ in range(2):
+        ctx.locks_merge_selection(torch.from_numpy(key).cuda(), torch.from_numpy(page).cuda(), 2, ids, cnt)
+    ids, cnt = ids.cpu().numpy(), cnt.cpu().numpy()
+    for b in range(2):
+        for h in range(2):
+            k, p = key[:, b, h].reshape(-1), page[:, b, h].reshape(-1)
+            there = np.flatnonzero(p >= 0)
+            best = np.sort(there[np.argsort(-k[there], kind="stable")[:kc]])
+            assert cnt[b, h] == len(best)
+            assert np.array_equal(ids[b, h, :len(best)], p[best])
+            assert np.all(ids[b, h, len(best):] == -1)
