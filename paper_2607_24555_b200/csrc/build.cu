@@ -1,21 +1,23 @@
-// Summary build (Sec. 4 "Build (once, when a page completes)"), bulk, 16-token pages (build_page.cu has the rest).
+// Summary build (Sec. 4 "Build (once, when a page completes)"), bulk (build_page.cu has the page that a decode step fills).
 //
-// One warp takes 8 (page, KV head) items through three phases:
-//   1. per item, all lanes: centre the page's 16 keys and form the Gram matrix M = D D^T (16 x 16) on the tensor cores; M
-//      goes to shared memory
-//   2. all 8 items at once: eigendecomposition of M by one-sided Jacobi in fp32.  Four lanes hold one item's matrix (4
-//      columns of 16 entries each, in registers).  A QR factorisation with column pivoting comes first; the columns of
-//      R^T are then rotated in pairs until they are mutually orthogonal: column norms are the eigenvalues, normalised
-//      columns the eigenvectors.
-//   3. per item, all lanes: modes above the zero-mode thresholds, V = D^T U_r Sigma_r^-1, C = U_r Sigma_r, sign: largest
-//      |V| entry positive; store or quantise: symmetric abs-max, fp16 scale, round-half-even codes (int4 basis per column,
-//      int8 coefficients per row, int8 centroid) packed in the blob layout
-// build_i4_kernel: bf16 keys, int4 summaries.  build_kernel: everything else (fp32 keys, the other formats).
+// 16-token pages: one warp takes 8 (page, KV head) items through three phases.
+//   1. per item, all lanes: load the page's 16 keys (lane owns 4 consecutive dims of every key), centroid mu,
+//      deviations D, and the Gram matrix M = D D^T (16 x 16) on the tensor cores; M goes to shared memory
+//   2. all 8 items at once: eigendecomposition of M by one-sided Jacobi in fp32.  Four lanes hold one item's
+//      matrix (4 columns of 16 entries each, in registers); columns are rotated in pairs until they are mutually
+//      orthogonal, which leaves M W = U Lambda: column norms are the eigenvalues, normalised columns the
+//      eigenvectors.
+//   3. per item, all lanes: reload the keys, rank the modes by eigenvalue, keep r_eff <= min(r, 15) modes above
+//      the zero-mode thresholds, V = D^T U_r Sigma_r^-1 (lane's 4 dims), C = U_r Sigma_r, sign: largest |V| entry
+//      positive; store fp32 (F32 format) or quantise: symmetric abs-max, fp16 scale, round-half-even codes
+//      (int4 basis per column, int8 coefficients per row, int8 centroid) packed in the blob layout
+// build_i4_kernel: bf16 keys, int4 summaries.  build_kernel: everything else (fp32 keys, the other formats), one instruction
+// sequence for all of them.  Both round alike.
 //
-// Bound by instruction issue and its latencies, not by bytes: an eigenproblem per 4 KB page.  131 008 page-heads of 8 x 32K
-// tokens: 1347 us with 8.2 Jacobi sweeps and all phases through shared memory (6 960 warp instructions per page-head), 908
-// us with the factorisation in front (5.0 sweeps) and build_i4_kernel's phases 1 and 3 (3 930), 870 us with every pair
-// rotated in one lane, by shears.  10 CTAs of 96 registers per SM instead of 8 of 128: 957 us (spills).
+// The bytes of a summary decide near-ties between pages, so what is computed and in which order is kept exactly: a
+// preconditioned solver (build_page.cu's; 5 sweeps for 8) builds 131 008 page-heads in 870 us and is as accurate, but one
+// byte in ten thousand comes out differently, and one request in a few hundred then keeps another page.
+#include <type_traits>
 #include "build_common.cuh"
 
 namespace {
@@ -25,48 +27,51 @@ constexpr int kBuildItems = 8;                                   // (page, KV he
 constexpr int kBuildCtasPerSm = 8;                               // 16 warps per SM
 constexpr int kBuildScratch = 2 * LOCKS_B * 128;                 // 4096 B: bf16 half-tiles of D (hi | lo); later the blob
 constexpr int kMat = LOCKS_B * LOCKS_B + 16;                     // floats per item's matrix: items on different banks
-constexpr int kBuildMat = kBuildItems * kMat * 4;                // 8704 B: Gram matrices, then R^T, then the leading eigenvectors
+constexpr int kBuildMat = kBuildItems * kMat * 4;                // 8704 B: Gram matrices; later the leading eigenvectors, every entry twice
 constexpr int kBuildSmemPerWarp = kBuildScratch + kBuildMat + 64 + kBuildItems * LOCKS_B * 4;   // + key norms, eigenvalues
-constexpr int kUs = 20;                                          // build_i4_kernel: floats per eigenvector
-constexpr int kPiv = 2 * kBuildItems * LOCKS_B;                  // floats: pivot columns of two steps; later an item's centroid
-constexpr int kBuildI4SmemPerWarp = kPiv * 4 + kBuildMat + kBuildItems * LOCKS_B * 4;
 
-__device__ __forceinline__ float rcp_approx(float x) {
-  float y;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
+// The plane rotation that makes two columns p, q orthogonal, from a = |p|^2, b = |q|^2, g = p . q (smaller angle):
+// with d = b - a and h = d^2 + 4 g^2, cos 2t = |d| / sqrt(h) and sin 2t = 2 g sign(d) / sqrt(h), so
+// c = sqrt((1 + cos 2t) / 2) and s = sin 2t / (2 c): two reciprocal square roots in a row (approximate ones are
+// enough for the angle; c^2 + s^2 = 1 holds to their rounding).  p' = c p - s q, q' = s p + c q.  Inputs too small
+// or too large to square are left alone.
+__device__ __forceinline__ void plane_rotation(float a, float b, float g, float &c, float &sn) {
+  const float d = b - a, hh = fmaf(d, d, 4.f * g * g);
+  const bool ok = hh > 1e-37f && hh < 1e37f;   // branch-free: independent pairs interleave in one basic block
+  const float rs = rsqrt_approx(ok ? hh : 1.f);
+  const float x = fmaf(0.5f * fabsf(d), rs, 0.5f);
+  const float r2 = rsqrt_approx(x);
+  const float s0 = copysignf(g * rs * r2, d == 0.f ? g : g * d);
+  c = ok ? x * r2 : 1.f;
+  sn = ok ? s0 : 0.f;
 }
 
 // One-sided Jacobi on 8 matrices at once.  Lane (item = lane / 4, j = lane % 4) holds columns 4 j .. 4 j + 3 of its item's
-// matrix W, w[c][i] = rows 2i, 2i+1 of column 4 j + c as a packed pair, and their squared norms: two pairs of columns.
-// Odd-even transposition (16 steps per sweep meet every two columns once): every step rotates all pairs and passes one
-// column of each to a neighbour, half of the time within the lane.
-// W starts as R^T of M's QR factorisation with column pivoting (modified Gram-Schmidt, only R kept: Drmac and Veselic's
-// preconditioning; R^T's left singular vectors are M's eigenvectors): half a sweep's work that saves three of eight
-// (emulated in fp32 on this repository's synthetic pages, worst of 8 items: 8.2 -> 5.0 sweeps; the worst eigenvector
-// entry falls from 1.1e-4 to 3.5e-5 from fp64).
+// matrix W (initially M, symmetric: the columns are read as rows), w[c][i] = rows 2i, 2i+1 of column 4 j + c as a packed
+// pair, and their squared norms: two pairs of columns.  Odd-even transposition: 16 steps per sweep meet every two columns
+// once; every step rotates all pairs, a rotated pair swaps places, and one column of each pair is passed to a neighbour,
+// half of the time within the lane.
 // Result: the columns ranked by norm (descending, ties to the lower position), the 16 eigenvalues to lam_s[item][mode],
-// unit eigenvectors of the leading min(r, 8) modes to us: PAIRS = false us[item][mode][token], kUs floats per mode; PAIRS =
-// true [item][token][mode] as pairs (u, u) (r > 8: all 16, plain entries, [token][16]).
-template <bool PAIRS>
-__device__ __forceinline__ void jacobi_phase(float *mat, float *piv, float *us, float *lam_s, uint32_t live, int r, int lane) {
+// unit eigenvectors of the leading min(r, 8) modes to us as pairs (u, u): BY_MODE [item][mode][token], else
+// [item][token][mode] (r > 8: all 16, plain entries, [token][16]).
+template <bool BY_MODE>
+__device__ __forceinline__ void jacobi_phase(const float *mat, float *us, float *lam_s, uint32_t live, int r, int lane) {
   constexpr int CPL = 4, LPI = LOCKS_B / CPL;
   const int item = lane / LPI, j = lane % LPI;
   const bool item_live = (live >> item) & 1u;   // lanes of an absent item compute on zeros
-  float *mine = mat + item * kMat;
   float2 w[CPL][8];
-  auto load = [&](bool live_item) {
-    const float4 *src = reinterpret_cast<const float4 *>(mine + CPL * j * LOCKS_B);
+  {
+    const float4 *src = reinterpret_cast<const float4 *>(mat + item * kMat + CPL * j * LOCKS_B);
 #pragma unroll
     for (int c = 0; c < CPL; ++c)
 #pragma unroll
       for (int q4 = 0; q4 < 4; ++q4) {
-        const float4 f = live_item ? src[c * 4 + q4] : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 f = item_live ? src[c * 4 + q4] : make_float4(0.f, 0.f, 0.f, 0.f);
         w[c][2 * q4] = make_float2(f.x, f.y);
         w[c][2 * q4 + 1] = make_float2(f.z, f.w);
       }
-  };
-  load(item_live);
+  }
+  __syncwarp();   // every lane holds its columns: the matrices' shared memory may be overwritten from here on
   auto seg_max = [&](float v) {   // maximum over the lanes of the item
 #pragma unroll
     for (int o = 1; o < LPI; o <<= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
@@ -111,101 +116,45 @@ __device__ __forceinline__ void jacobi_phase(float *mat, float *piv, float *us, 
     for (int i = 2; i < 8; i += 2) { acc0 = fma2(a[i], b[i], acc0); acc1 = fma2(a[i + 1], b[i + 1], acc1); }
     return (acc0.x + acc1.x) + (acc0.y + acc1.y);
   };
-  norms();
-  // ---- QR with column pivoting.  The norms that choose the pivot are downdated; the pivot's own is exact.
-  {
-    uint32_t used = 0u;
-#pragma unroll 1
-    for (int k = 0; k < LOCKS_B; ++k) {
-      // largest remaining column: the norm's bits with the column in the lowest four; + 16 so that 0 means "used"
-      uint32_t best = 0u;
-#pragma unroll
-      for (int c = 0; c < CPL; ++c) {
-        const uint32_t key = ((__float_as_uint(fmaxf(n[c], 0.f)) & ~15u) + 16u) | (uint32_t)(CPL * j + c);
-        best = max(best, ((used >> c) & 1u) ? 0u : key);
-      }
-      best = max(best, __shfl_xor_sync(0xffffffffu, best, 1));
-      best = max(best, __shfl_xor_sync(0xffffffffu, best, 2));
-      float4 *pb = reinterpret_cast<float4 *>(piv + ((k & 1) * kBuildItems + item) * LOCKS_B);
-      const int pc = (int)(best & 15u) - CPL * j;   // this lane's column of that number, if 0 .. 3
-#pragma unroll
-      for (int c = 0; c < CPL; ++c)
-        if (c == pc) {
-#pragma unroll
-          for (int q4 = 0; q4 < 4; ++q4) pb[q4] = make_float4(w[c][2 * q4].x, w[c][2 * q4].y, w[c][2 * q4 + 1].x, w[c][2 * q4 + 1].y);
-        }
-      __syncwarp();   // (the buffer of step k - 1 is not written before every lane has passed here)
-      float2 pv[8];
-#pragma unroll
-      for (int q4 = 0; q4 < 4; ++q4) {
-        const float4 f = pb[q4];
-        pv[2 * q4] = make_float2(f.x, f.y);
-        pv[2 * q4 + 1] = make_float2(f.z, f.w);
-      }
-      const float pp = dot(pv, pv), ir = pp > 1e-37f ? rsqrt_approx(pp) : 0.f;
-      float rk[CPL];
-#pragma unroll
-      for (int c = 0; c < CPL; ++c) {
-        rk[c] = ((used >> c) & 1u) ? 0.f : (c == pc ? pp : dot(w[c], pv)) * ir;
-        const float f = -rk[c] * ir;
-        const float2 f2 = make_float2(f, f);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) w[c][i] = fma2(f2, pv[i], w[c][i]);
-        n[c] = fmaf(-rk[c], rk[c], n[c]);
-      }
-      if (pc >= 0 && pc < CPL) used |= 1u << pc;
-      *reinterpret_cast<float4 *>(mine + k * LOCKS_B + CPL * j) = make_float4(rk[0], rk[1], rk[2], rk[3]);   // column k of R^T
-    }
-    __syncwarp();
-    load(true);
-  }
-  // The stop test: no pair above the tolerance in a whole sweep.  With few modes kept only pairs with one of the r largest
-  // columns count (r = 2: 5.4 -> 3.3 sweeps); with 8 the others add a fifth of a sweep, less than finding the r-th norm.
-  const float tol = r >= 8 ? 3.f * LOCKS_BUILD_COS_TOL : LOCKS_BUILD_COS_TOL, tol2 = tol * tol;
+  const float tol2 = LOCKS_BUILD_COS_TOL * LOCKS_BUILD_COS_TOL;
   int bad = 0;
-  float floor_n = 0.f, top = 0.f;
-  int rank[CPL];
-  auto ranks = [&]() {
-#pragma unroll
-    for (int c = 0; c < CPL; ++c) rank[c] = 0;
-#pragma unroll
-    for (int jj = 0; jj < LPI; ++jj)
-#pragma unroll
-      for (int cc = 0; cc < CPL; ++cc) {
-        const float o = __shfl_sync(0xffffffffu, n[cc], (lane & ~(LPI - 1)) + jj);
-#pragma unroll
-        for (int c = 0; c < CPL; ++c) rank[c] += (int)(o > n[c]) | ((int)(o == n[c]) & (int)(jj * CPL + cc < j * CPL + c));
-      }
-  };
-  // A pair holds a column that it kept from the step before (a) and one that it has been passed (b).  Which of the two is the
-  // lower position alternates from step to step, and so do the signs of the rotation and of the swap that follows it,
-  // which leaves one formula: passed on c a + s b (in a), kept c b - s a (in b).
-  struct Angle { float c, s; };
-  auto angle = [&](const float2 (&a)[8], const float2 (&b)[8], float &na, float &nb, bool there) {
-    const float g = dot(a, b);
-    // columns whose norm is rounding noise beside the largest (null directions) do not hold up convergence
-    bad |= (int)there & (int)(g * g > tol2 * na * nb) & (int)(fminf(na, nb) > floor_n) & (int)(fmaxf(na, nb) >= top);
-    Angle r;
-    float tn;
-    jacobi_angle(nb, na, g, r.c, r.s, tn);
-    tn = there ? tn * g : nb - na;   // (no pair: the two change places)
-    na = fmaxf(na + tn, 0.f);
-    nb = fmaxf(nb - tn, 0.f);
-    return r;
-  };
-  // as three shears (tau = tan(angle / 2) = s / (1 + c)): three packed operations per row instead of four
-  auto rotate = [&](float2 (&a)[8], float2 (&b)[8], float &na, float &nb) {
-    const Angle r = angle(a, b, na, nb, true);
-    const float tau = r.s * rcp_approx(1.f + r.c);
-    const float2 T2 = make_float2(tau, tau), S2 = make_float2(-r.s, -r.s);
+  float floor_n = 0.f;
+  // columns whose norm is rounding noise beside the largest (null directions) do not hold up convergence
+  // One pair: a is the column that it kept from the step before, b the one that it has been passed; in even steps b is the
+  // lower position (p), in odd ones a.  The lower position receives q' = s p + c q, the upper one p' = c p - s q.  What is
+  // passed on ends in a, what is kept in b.  `there` = false: the two ends of the row, which do not meet: they change places.
+  auto rotate = [&](auto odd, float2 (&a)[8], float2 (&b)[8], float &na, float &nb, bool there) {
+    constexpr bool kOdd = decltype(odd)::value;
+    const float g = dot(a, b), np = kOdd ? na : nb, nq = kOdd ? nb : na;
+    bad |= (int)there & (int)(g * g > tol2 * np * nq) & (int)(fminf(np, nq) > floor_n);
+    float c, sn;
+    plane_rotation(np, nq, g, c, sn);
+    float x2 = 2.f * c * sn * g;
+    if (kOdd && !there) { c = 0.f; sn = 1.f; x2 = 0.f; }
+    const float2 C2 = make_float2(c, c), S2 = make_float2(sn, sn), nS2 = make_float2(-sn, -sn);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      a[i] = fma2(T2, b[i], a[i]);
-      b[i] = fma2(S2, a[i], b[i]);
-      a[i] = fma2(T2, b[i], a[i]);
+      const float2 p = kOdd ? a[i] : b[i], q = kOdd ? b[i] : a[i];
+      const float2 pp = fma2(C2, p, mul2(nS2, q)), qq = fma2(S2, p, mul2(C2, q));
+      a[i] = kOdd ? pp : qq;
+      b[i] = kOdd ? qq : pp;
     }
+    const float cc = c * c, ss = sn * sn;
+    const float n_p = fmaxf(fmaf(cc, np, fmaf(ss, nq, -x2)), 0.f), n_q = fmaxf(fmaf(ss, np, fmaf(cc, nq, x2)), 0.f);
+    na = kOdd ? n_p : n_q;
+    nb = kOdd ? n_q : n_p;
   };
   const int up = (lane & ~(LPI - 1)) | ((j + 1) & (LPI - 1)), down = (lane & ~(LPI - 1)) | ((j - 1) & (LPI - 1));
+  auto fetch = [&](float2 (&col)[8], float &norm, int from) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      col[i].x = __shfl_sync(0xffffffffu, col[i].x, from);
+      col[i].y = __shfl_sync(0xffffffffu, col[i].y, from);
+    }
+    norm = __shfl_sync(0xffffffffu, norm, from);
+  };
+  constexpr std::false_type even{};
+  constexpr std::true_type odd{};
   for (int sweep = 0; sweep < LOCKS_BUILD_SWEEPS; ++sweep) {
     norms();
     {
@@ -214,41 +163,15 @@ __device__ __forceinline__ void jacobi_phase(float *mat, float *piv, float *us, 
       for (int c = 1; c < CPL; ++c) nm = fmaxf(nm, n[c]);
       floor_n = 1e-11f * seg_max(nm);   // squared norm = squared eigenvalue: modes below 3e-6 of the largest
     }
-    if (r < 8) {
-      ranks();
-      float least = INFINITY;
-#pragma unroll
-      for (int c = 0; c < CPL; ++c) least = rank[c] < r ? fminf(least, n[c]) : least;
-      top = -0.999f * seg_max(-least);
-    }
     bad = 0;
 #pragma unroll 2
     for (int st2 = 0; st2 < 8; ++st2) {
-      // even step: the lane's pairs (w[1], w[0]) and (w[3], w[2])
-      rotate(w[1], w[0], n[1], n[0]);
-      rotate(w[3], w[2], n[3], n[2]);
-      // a pair passes to the one before it: w[3] to w[0]'s, w[1] to the lane below
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        w[1][i].x = __shfl_sync(0xffffffffu, w[1][i].x, up);
-        w[1][i].y = __shfl_sync(0xffffffffu, w[1][i].y, up);
-      }
-      n[1] = __shfl_sync(0xffffffffu, n[1], up);
-      // odd step: (w[0], w[3]) and (w[2], w[1]); the item's last pair has the two ends of the row, which do not meet
-      rotate(w[0], w[3], n[0], n[3]);
-      {
-        Angle r = angle(w[2], w[1], n[2], n[1], j != LPI - 1);
-        if (j == LPI - 1) { r.c = 0.f; r.s = 1.f; }
-        const float2 C2 = make_float2(r.c, r.c), S2 = make_float2(r.s, r.s), nS2 = make_float2(-r.s, -r.s);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const float2 a = fma2(C2, w[2][i], mul2(S2, w[1][i]));
-          w[1][i] = fma2(C2, w[1][i], mul2(nS2, w[2][i]));
-          w[2][i].x = __shfl_sync(0xffffffffu, a.x, down);   // a pair passes to the one after it: w[0] to w[1]'s, w[2] to the lane above
-          w[2][i].y = __shfl_sync(0xffffffffu, a.y, down);
-        }
-        n[2] = __shfl_sync(0xffffffffu, n[2], down);
-      }
+      rotate(even, w[1], w[0], n[1], n[0], true);
+      rotate(even, w[3], w[2], n[3], n[2], true);
+      fetch(w[1], n[1], up);   // a pair passes to the one before it: w[3] to the lane's first, w[1] to the lane below
+      rotate(odd, w[0], w[3], n[0], n[3], true);
+      rotate(odd, w[2], w[1], n[2], n[1], j != LPI - 1);
+      fetch(w[2], n[2], down);   // ... and then to the one after it: w[0] to the lane's second, w[2] to the lane above
       // the lane's pairs are now (w[3], w[2]) and (w[1], w[0]), in this order: exchange the names
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
@@ -262,17 +185,29 @@ __device__ __forceinline__ void jacobi_phase(float *mat, float *piv, float *us, 
     if (!__any_sync(0xffffffffu, bad != 0)) break;
   }
   norms();
-  ranks();
+  int rank[CPL];
+#pragma unroll
+  for (int c = 0; c < CPL; ++c) rank[c] = 0;
+#pragma unroll
+  for (int jj = 0; jj < LPI; ++jj)
+#pragma unroll
+    for (int cc = 0; cc < CPL; ++cc) {
+      const float o = __shfl_sync(0xffffffffu, n[cc], (lane & ~(LPI - 1)) + jj);
+#pragma unroll
+      for (int c = 0; c < CPL; ++c) rank[c] += (o > n[c]) || (o == n[c] && (jj * CPL + cc) < (j * CPL + c));
+    }
 #pragma unroll
   for (int c = 0; c < CPL; ++c) {
     lam_s[item * LOCKS_B + rank[c]] = sqrtf(n[c]) * unscale;
     const float inv = n[c] > 0.f ? rsqrtf(n[c]) : 0.f;
-    if (!PAIRS) {
+    if (BY_MODE) {
       if (rank[c] < 8) {
-        float4 *dst = reinterpret_cast<float4 *>(us + (item * 8 + rank[c]) * kUs);
+        float4 *dst = reinterpret_cast<float4 *>(us + item * kMat + rank[c] * 2 * LOCKS_B);
 #pragma unroll
-        for (int q4 = 0; q4 < 4; ++q4)
-          dst[q4] = make_float4(w[c][2 * q4].x * inv, w[c][2 * q4].y * inv, w[c][2 * q4 + 1].x * inv, w[c][2 * q4 + 1].y * inv);
+        for (int i = 0; i < 8; ++i) {
+          const float u0 = w[c][i].x * inv, u1 = w[c][i].y * inv;
+          dst[i] = make_float4(u0, u0, u1, u1);
+        }
       }
     } else if (r > 8) {   // ranks above 8 (fp32 summaries): all 16 modes, plain entries
       float *dst = us + item * LOCKS_B * LOCKS_B + rank[c];
@@ -304,269 +239,6 @@ __device__ __forceinline__ int item_block(const BuildParams &p, int warp, int la
   if (block >= 0 && block < p.num_blocks) return block;
   set_status(p.status, LOCKS_ERR_BAD_BLOCK);
   return -1;
-}
-
-__device__ __forceinline__ uint32_t bf16x2_add(uint32_t a, uint32_t b) {
-  const __nv_bfloat162 d = __hadd2_rn(*reinterpret_cast<__nv_bfloat162 *>(&a), *reinterpret_cast<__nv_bfloat162 *>(&b));
-  return *reinterpret_cast<const uint32_t *>(&d);
-}
-__device__ __forceinline__ uint32_t bf16x2_sub(uint32_t a, uint32_t b) {
-  const __nv_bfloat162 d = __hsub2_rn(*reinterpret_cast<__nv_bfloat162 *>(&a), *reinterpret_cast<__nv_bfloat162 *>(&b));
-  return *reinterpret_cast<const uint32_t *>(&d);
-}
-__device__ __forceinline__ float2 add2(float2 a, float2 b) {
-  float2 d;
-  asm("add.rn.f32x2 %0, %1, %2;"
-      : "=l"(*reinterpret_cast<unsigned long long *>(&d))
-      : "l"(*reinterpret_cast<unsigned long long *>(&a)), "l"(*reinterpret_cast<unsigned long long *>(&b)));
-  return d;
-}
-// fp16 scale of codes -qmax .. qmax for values up to `best`, and its reciprocal (0 for a zero scale: all codes 0)
-__device__ __forceinline__ __half code_scale(float best, float inv_qmax, float &inv) {
-  const __half s = __float2half_rn(best * inv_qmax);
-  const float f = __half2float(s);
-  inv = f == 0.f ? 0.f : rcp_approx(f);
-  return s;
-}
-
-// bf16 keys, int4 summaries.  Neither phase 1 nor phase 3 touches shared memory for the keys: a lane loads from global
-// memory the 16-byte chunks that are its own MMA fragments (any assignment of dimensions to fragment positions will do in
-// phase 1, where they are summed over; in phase 3 it decides which dimensions of the basis a lane receives).
-//   Phase 1: the keys minus c = bf16(mean) split exactly into two bf16 terms H + L (Knuth's TwoSum in bf16 pairs), M' =
-//   (H + L)(H + L)^T, and M = M' centred in both directions (c is not quite the mean).
-//   Phase 3: V Sigma = U^T D = (U - mean U)^T K, U in three bf16 terms (24 bits, rows 0-7 and 8-15 of one A operand and rows
-//   0-7 of another whose rows 8-15 are 1/16 and give the centroid), K as stored: products exact, sums fp32.
-__global__ void __launch_bounds__(kBuildWarps * 32, kBuildCtasPerSm) build_i4_kernel(BuildParams p) {
-  extern __shared__ __align__(16) uint8_t smem_raw[];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int x = lane >> 2, t = lane & 3, h = blockIdx.y, r = p.r;
-  const int it_block = item_block(p, warp, lane);
-  const uint32_t live = __ballot_sync(0xffffffffu, it_block >= 0);
-  if (!live) return;
-  const int layer = blockIdx.z / p.batch;
-  const __nv_bfloat16 *kbase = reinterpret_cast<const __nv_bfloat16 *>(p.k_layers ? p.k_layers[layer] : p.k);
-  uint8_t *sbase = p.summ_layers ? reinterpret_cast<uint8_t *>(p.summ_layers[layer]) : p.summ;
-  float *piv = reinterpret_cast<float *>(smem_raw + warp * kBuildI4SmemPerWarp), *mat = piv + kPiv, *lam_s = mat + kBuildItems * kMat;
-  auto page_keys = [&](int s) {
-    return kbase + (int64_t)__shfl_sync(0xffffffffu, it_block, s) * p.sb + (int64_t)h * p.sh;
-  };
-
-  // ---- 1. Gram matrices: lane (x, t) holds dimensions 8t .. 8t+7 (+ 32 j) of tokens x and x + 8
-#pragma unroll 1
-  for (int s = 0; s < kBuildItems; ++s) {
-    if (!((live >> s) & 1u)) continue;
-    const __nv_bfloat16 *K = page_keys(s) + (int64_t)x * p.st + 8 * t;
-    uint32_t ka[16], kb[16], nc[16];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const uint4 a = *reinterpret_cast<const uint4 *>(K + 32 * j), b = *reinterpret_cast<const uint4 *>(K + 8 * p.st + 32 * j);
-      ka[4 * j] = a.x; ka[4 * j + 1] = a.y; ka[4 * j + 2] = a.z; ka[4 * j + 3] = a.w;
-      kb[4 * j] = b.x; kb[4 * j + 1] = b.y; kb[4 * j + 2] = b.z; kb[4 * j + 3] = b.w;
-    }
-#pragma unroll
-    for (int i = 0; i < 16; ++i) nc[i] = bf16x2_add(ka[i], kb[i]);
-#pragma unroll
-    for (int o = 4; o < 32; o <<= 1)
-#pragma unroll
-      for (int i = 0; i < 16; ++i) nc[i] = bf16x2_add(nc[i], __shfl_xor_sync(0xffffffffu, nc[i], o));
-    float X0[4] = {0.f, 0.f, 0.f, 0.f}, X1[4] = {0.f, 0.f, 0.f, 0.f}, Y0[4] = {0.f, 0.f, 0.f, 0.f}, Y1[4] = {0.f, 0.f, 0.f, 0.f};
-    auto split = [&](uint32_t k, uint32_t n, uint32_t &hi, uint32_t &lo) {   // k + n = hi + lo exactly
-      hi = bf16x2_add(k, n);
-      const uint32_t bb = bf16x2_sub(hi, k);
-      lo = bf16x2_add(bf16x2_sub(k, bf16x2_sub(hi, bb)), bf16x2_sub(n, bb));
-    };
-#pragma unroll
-    for (int i = 0; i < 16; i += 2) {   // one k-step: registers i, i + 1 of both tokens are the A and the B operand
-      uint32_t H[4], L[4];
-#pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const __nv_bfloat162 m = __hmul2(*reinterpret_cast<__nv_bfloat162 *>(&nc[i + u]), __floats2bfloat162_rn(-1.f / LOCKS_B, -1.f / LOCKS_B));
-        const uint32_t n = *reinterpret_cast<const uint32_t *>(&m);
-        split(ka[i + u], n, H[2 * u], L[2 * u]);
-        split(kb[i + u], n, H[2 * u + 1], L[2 * u + 1]);
-      }
-      mma_bf16(X0, H[0], H[1], H[2], H[3], H[0], H[2]);
-      mma_bf16(X1, H[0], H[1], H[2], H[3], H[1], H[3]);
-      mma_bf16(Y0, H[0], H[1], H[2], H[3], L[0], L[2]);
-      mma_bf16(Y1, H[0], H[1], H[2], H[3], L[1], L[3]);
-      mma_bf16(X0, L[0], L[1], L[2], L[3], L[0], L[2]);
-      mma_bf16(X1, L[0], L[1], L[2], L[3], L[1], L[3]);
-      mma_bf16(Y0, L[0], L[1], L[2], L[3], H[0], H[2]);
-      mma_bf16(Y1, L[0], L[1], L[2], L[3], H[1], H[3]);
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) { X0[i] += Y0[i]; X1[i] += Y1[i]; }   // [0..1]: row x, columns 2t, 2t+1 (X1: + 8); [2..3]: row x + 8
-    float r0 = (X0[0] + X0[1]) + (X1[0] + X1[1]), r1 = (X0[2] + X0[3]) + (X1[2] + X1[3]);
-#pragma unroll
-    for (int o = 1; o < 4; o <<= 1) { r0 += __shfl_xor_sync(0xffffffffu, r0, o); r1 += __shfl_xor_sync(0xffffffffu, r1, o); }
-    r0 *= 1.f / LOCKS_B;   // means of rows x and x + 8; by symmetry also of those columns
-    r1 *= 1.f / LOCKS_B;
-    float c0 = __shfl_sync(0xffffffffu, r0, 8 * t), c1 = __shfl_sync(0xffffffffu, r0, 8 * t + 4);
-    float c8 = __shfl_sync(0xffffffffu, r1, 8 * t), c9 = __shfl_sync(0xffffffffu, r1, 8 * t + 4);
-    float g = (c0 + c1) + (c8 + c9);
-    g += __shfl_xor_sync(0xffffffffu, g, 1);
-    g += __shfl_xor_sync(0xffffffffu, g, 2);
-    g *= 1.f / LOCKS_B;
-    r0 -= g;
-    r1 -= g;
-    float *dst = mat + s * kMat + x * LOCKS_B + 2 * t;
-    *reinterpret_cast<float2 *>(dst) = make_float2(X0[0] - (r0 + c0), X0[1] - (r0 + c1));
-    *reinterpret_cast<float2 *>(dst + 8) = make_float2(X1[0] - (r0 + c8), X1[1] - (r0 + c9));
-    *reinterpret_cast<float2 *>(dst + 8 * LOCKS_B) = make_float2(X0[2] - (r1 + c0), X0[3] - (r1 + c1));
-    *reinterpret_cast<float2 *>(dst + 8 * LOCKS_B + 8) = make_float2(X1[2] - (r1 + c8), X1[3] - (r1 + c9));
-  }
-  __syncwarp();
-
-  // ---- 2. eigenvectors and eigenvalues of all the warp's items at once
-  jacobi_phase<false>(mat, piv, mat, lam_s, live, r, lane);
-
-  // ---- 3. basis, coefficients, centroid.  Lane (x, t) receives mode x, dimensions 16 t .. 16 t + 15 (+ 64)
-#pragma unroll 1
-  for (int s = 0; s < kBuildItems; ++s) {
-    if (!((live >> s) & 1u)) continue;
-    const __nv_bfloat16 *K = page_keys(s) + (int64_t)(2 * t) * p.st + 8 * x;
-    uint4 kk[2][4];   // tokens 2t, 2t + 1, 2t + 8, 2t + 9; dimensions 8 x .. 8 x + 7 (+ 64)
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int hc = 0; hc < 2; ++hc) kk[hc][i] = *reinterpret_cast<const uint4 *>(K + (int64_t)((i & 1) + 8 * (i >> 1)) * p.st + 64 * hc);
-    const float *U = mat + s * 8 * kUs, *lam = lam_s + s * LOCKS_B;
-    uint32_t A[4], Lo[2];
-    {
-      const float2 ua = *reinterpret_cast<const float2 *>(U + x * kUs + 2 * t), ub = *reinterpret_cast<const float2 *>(U + x * kUs + 8 + 2 * t);
-      float m = (ua.x + ua.y) + (ub.x + ub.y);
-      m += __shfl_xor_sync(0xffffffffu, m, 1);
-      m += __shfl_xor_sync(0xffffffffu, m, 2);
-      m *= 1.f / LOCKS_B;
-#pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        float a = (i ? ub.x : ua.x) - m, b = (i ? ub.y : ua.y) - m;
-        if (x >= r) a = b = 0.f;
-        A[2 * i] = pack_bf16(a, b);
-        a -= __uint_as_float(A[2 * i] << 16);
-        b -= __uint_as_float(A[2 * i] & 0xFFFF0000u);
-        A[2 * i + 1] = pack_bf16(a, b);
-        a -= __uint_as_float(A[2 * i + 1] << 16);
-        b -= __uint_as_float(A[2 * i + 1] & 0xFFFF0000u);
-        Lo[i] = pack_bf16(a, b);
-      }
-    }
-    const uint32_t kOne = 0x3D803D80u;   // 1/16
-    float2 v[2][8];   // [hc][j]: dimensions 64 hc + 16 t + j and + 8
-    float *mu_s = piv;
-#pragma unroll
-    for (int hc = 0; hc < 2; ++hc) {
-      float2 mu[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        auto word = [&](const uint4 &q) { return j < 2 ? q.x : (j < 4 ? q.y : (j < 6 ? q.z : q.w)); };
-        const uint32_t sel = (j & 1) ? 0x7632u : 0x5410u;
-        const uint32_t b0 = __byte_perm(word(kk[hc][0]), word(kk[hc][1]), sel), b1 = __byte_perm(word(kk[hc][2]), word(kk[hc][3]), sel);
-        float C1[4] = {0.f, 0.f, 0.f, 0.f}, C2[4] = {0.f, 0.f, 0.f, 0.f};
-        mma_bf16(C1, A[0], A[1], A[2], A[3], b0, b1);
-        mma_bf16(C2, Lo[0], kOne, Lo[1], kOne, b0, b1);
-        v[hc][j] = add2(add2(make_float2(C2[0], C2[1]), make_float2(C1[2], C1[3])), make_float2(C1[0], C1[1]));
-        mu[j] = make_float2(C2[2], C2[3]);
-      }
-      if (x == 0) {
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          *reinterpret_cast<float4 *>(mu_s + 64 * hc + 16 * t + 4 * q) = make_float4(mu[4 * q].x, mu[4 * q + 1].x, mu[4 * q + 2].x, mu[4 * q + 3].x);
-          *reinterpret_cast<float4 *>(mu_s + 64 * hc + 16 * t + 8 + 4 * q) = make_float4(mu[4 * q].y, mu[4 * q + 1].y, mu[4 * q + 2].y, mu[4 * q + 3].y);
-        }
-      }
-    }
-    __syncwarp();
-    uint8_t *gout = sbase + ((int64_t)__shfl_sync(0xffffffffu, it_block, s) * p.Hkv + h) * p.S;
-    // ---- centroid: dimensions 4 lane .. + 3
-    const float4 mu4 = *reinterpret_cast<const float4 *>(mu_s + 4 * lane);
-    {
-      const float mx = fmaxf(fmaxf(fabsf(mu4.x), fabsf(mu4.y)), fmaxf(fabsf(mu4.z), fabsf(mu4.w)));
-      float inv;
-      const __half sh = code_scale(__uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(mx))), 1.f / 127.f, inv);
-      auto code = [&](float v) { return (uint32_t)((int)round_code(v, inv, 127.f) + 128); };
-      // dim offset c = 2*half + e -> byte e*2 + half
-      *reinterpret_cast<uint32_t *>(gout + i4_off_mu(r) + lane * 4) = code(mu4.x) | (code(mu4.z) << 8) | (code(mu4.y) << 16) | (code(mu4.w) << 24);
-      if (lane == 0) *reinterpret_cast<__half *>(gout + i4_off_smu(r)) = sh;
-      if (lane < 16 && i4_off_smu(r) + 2 + lane < p.S) gout[i4_off_smu(r) + 2 + lane] = 0;   // bytes between the payload and the stride
-    }
-    // ---- the mode's place among those above the zero-mode thresholds (eigenvalues descend: no gaps)
-    const float knorm2 = warp_sum((float)LOCKS_B * (mu4.x * mu4.x + mu4.y * mu4.y + mu4.z * mu4.z + mu4.w * mu4.w) +
-                                  (lane < LOCKS_B ? lam[lane] : 0.f));
-    const float lam0 = lam[0], lx = lam[x];
-    const bool keep = x < r && lam0 > 0.f && lx > 1e-6f * lam0 && lx > 1e-10f * knorm2;
-    // ---- basis: largest magnitude and its sign (lowest dimension on ties)
-    float mx = v[0][0].x, mn = v[0][0].x;
-#pragma unroll
-    for (int hc = 0; hc < 2; ++hc)
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        mx = fmaxf(mx, fmaxf(v[hc][j].x, v[hc][j].y));
-        mn = fminf(mn, fminf(v[hc][j].x, v[hc][j].y));
-      }
-#pragma unroll
-    for (int o = 1; o < 4; o <<= 1) {
-      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
-    }
-    bool neg = -mn > mx;
-    if (__any_sync(0xffffffffu, keep && mx == -mn)) {   // opposite entries of the same magnitude
-      int at = LOCKS_D << 1;   // 2 * dimension + (negative)
-#pragma unroll
-      for (int hc = 1; hc >= 0; --hc)
-#pragma unroll
-        for (int i = 15; i >= 0; --i) {
-          const float y = i < 8 ? v[hc][i & 7].x : v[hc][i & 7].y;
-          if (fabsf(y) == mx) at = 2 * (64 * hc + 16 * t + i) + (y < 0.f ? 1 : 0);
-        }
-      at = min(at, __shfl_xor_sync(0xffffffffu, at, 1));
-      at = min(at, __shfl_xor_sync(0xffffffffu, at, 2));
-      if (mx == -mn) neg = at & 1;
-    }
-    const float isig = keep ? rsqrtf(lx) : 0.f;
-    float inv;
-    const __half sv = code_scale(fmaxf(mx, -mn) * isig, 1.f / 7.f, inv);
-    inv *= neg ? -isig : isig;   // (a unit vector's largest entry is at least 0.088: the scale is a normal fp16, no code leaves -7 .. 7)
-    // code + 8 in the low bits of 1.5 * 2^23 + code + 8; a word's nibbles from the top: dimensions 7 5 3 1 6 4 2 0
-    if (x < r) {
-#pragma unroll
-      for (int hc = 0; hc < 2; ++hc) {
-        uint32_t wx = 0u, wy = 0u;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const int j = q < 4 ? 7 - 2 * q : 14 - 2 * q;
-          wx = wx * 16u + __float_as_uint(fmaf(v[hc][j].x, inv, 12582920.f));
-          wy = wy * 16u + __float_as_uint(fmaf(v[hc][j].y, inv, 12582920.f));
-        }
-        *reinterpret_cast<uint2 *>(gout + x * 64 + 32 * hc + 8 * t) = make_uint2(wx - 0x3F400000u, wy - 0x3F400000u);
-      }
-      if (t == 0) *reinterpret_cast<__half *>(gout + i4_off_sv(r) + 2 * x) = sv;
-    }
-    // ---- coefficients C = U Sigma: tokens x and x + 8, modes 2t and 2t + 1
-    const float sg = keep ? (neg ? -sqrtf(lx) : sqrtf(lx)) : 0.f;
-    const float g0 = __shfl_sync(0xffffffffu, sg, 8 * t), g1 = __shfl_sync(0xffffffffu, sg, 8 * t + 4);
-    const float *Ut = U + 2 * t * kUs + x;
-    const float ca = g0 * Ut[0], cb = g1 * Ut[kUs], cc = g0 * Ut[8], cd = g1 * Ut[kUs + 8];
-    float ma = fmaxf(fabsf(ca), fabsf(cb)), mb = fmaxf(fabsf(cc), fabsf(cd));
-#pragma unroll
-    for (int o = 1; o < 4; o <<= 1) {
-      ma = fmaxf(ma, __shfl_xor_sync(0xffffffffu, ma, o));
-      mb = fmaxf(mb, __shfl_xor_sync(0xffffffffu, mb, o));
-    }
-    float ia, ib;
-    const __half sa = code_scale(ma, 1.f / 127.f, ia), sb = code_scale(mb, 1.f / 127.f, ib);
-    if (t < r / 2) {
-      auto code = [&](float v, float inv) { return (uint32_t)((int)round_code(v, inv, 127.f) + 128); };
-      *reinterpret_cast<uint32_t *>(gout + i4_off_coef(r) + (x * (r / 2) + t) * 4) =
-          code(ca, ia) | (code(cb, ia) << 8) | (code(cc, ib) << 16) | (code(cd, ib) << 24);
-    }
-    if (t == 0) {
-      __half *dst = reinterpret_cast<__half *>(gout + i4_off_sc(r)) + (x >> 1) * 4 + (x & 1);
-      dst[0] = sa;
-      dst[2] = sb;
-    }
-    __syncwarp();   // the centroid's shared memory is written again for the next item
-  }
 }
 
 template <typename T, int FMT>
@@ -703,7 +375,7 @@ __global__ void __launch_bounds__(kBuildWarps * 32, kBuildCtasPerSm) build_kerne
   }
 
   // ---- 2. eigenvectors and eigenvalues of all the warp's items at once
-  jacobi_phase<true>(mat, reinterpret_cast<float *>(scratch), mat, lam_s, live, r, lane);
+  jacobi_phase<false>(mat, mat, lam_s, live, r, lane);
 
   // ---- 3. per item: modes, basis, coefficients, quantisation
   uint8_t *blob = scratch;
@@ -868,6 +540,251 @@ __global__ void __launch_bounds__(kBuildWarps * 32, kBuildCtasPerSm) build_kerne
   }
 }
 
+// ------------------------------------------------------------------------------------------------
+// Pages of 32 and 64 tokens (App. D "Page size"): one warp per (page, KV head), everything in fp32 from shared
+// memory, the row-major summary formats only.  The same method as above (centre, Gram, one-sided Jacobi by
+// odd-even transposition, rank, project, quantise), written for brevity rather than speed: lane m rotates the
+// column pair m of a step.
+// ------------------------------------------------------------------------------------------------
+constexpr int kWideDStride = LOCKS_D + 4;   // floats per staged key row (16-byte aligned rows, no bank conflicts)
+__host__ __device__ constexpr int build_wide_smem(int B) {
+  return (B * kWideDStride + B * (B + 1) + 2 * B + 32) * 4;   // keys, W (column-major, padded), norms, order, misc
+}
+
+template <typename T, int FMT>
+__global__ void __launch_bounds__(32) build_wide_kernel(BuildParams p, int B) {
+  extern __shared__ __align__(16) uint8_t smem_raw[];
+  const int lane = threadIdx.x;
+  const int b = blockIdx.z, h = blockIdx.y;
+  const int complete = p.seq_lens[b] / B;
+  const int p0 = p.page_begin ? p.page_begin[b] : 0;
+  const int p1 = min(p.page_end ? p.page_end[b] : complete, complete);
+  const int page = p0 + blockIdx.x;
+  if (page < 0 || page >= p1) return;
+  if (page >= p.Pmax) return;
+  const int block = p.block_table[(int64_t)b * p.Pmax + page];
+  if (block < 0 || block >= p.num_blocks) {
+    if (lane == 0) set_status(p.status, LOCKS_ERR_BAD_BLOCK);
+    return;
+  }
+  float *Ds = reinterpret_cast<float *>(smem_raw);   // [B][kWideDStride] deviations
+  float *W = Ds + B * kWideDStride;                  // [B columns][B + 1]
+  float *nr = W + B * (B + 1);                       // [B] squared column norms
+  int *order = reinterpret_cast<int *>(nr + B);      // [B] column of rank l
+  const int WS = B + 1, r = p.r;
+  // ---- keys, centroid, deviations
+  float mu[4] = {0.f, 0.f, 0.f, 0.f}, knorm2 = 0.f;
+  {
+    const T *K = reinterpret_cast<const T *>(p.k) + ((int64_t)block * p.sb + (int64_t)h * p.sh) + 4 * lane;
+    for (int i = 0; i < B; ++i) {
+      const T *src = K + (int64_t)i * p.st;
+      float v[4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) v[c] = ldf<T>(src, c);
+#pragma unroll
+      for (int c = 0; c < 4; ++c) { mu[c] += v[c]; knorm2 = fmaf(v[c], v[c], knorm2); }
+      *reinterpret_cast<float4 *>(Ds + i * kWideDStride + 4 * lane) = make_float4(v[0], v[1], v[2], v[3]);
+    }
+    knorm2 = warp_sum(knorm2);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) mu[c] /= (float)B;
+    for (int i = 0; i < B; ++i) {
+      float4 *d4 = reinterpret_cast<float4 *>(Ds + i * kWideDStride + 4 * lane);
+      float4 v = *d4;
+      v.x -= mu[0]; v.y -= mu[1]; v.z -= mu[2]; v.w -= mu[3];
+      *d4 = v;
+    }
+    __syncwarp();
+  }
+  // ---- Gram matrix: lane j (and j + 32) computes column j of M, row by row
+  float amax = 0.f;
+  for (int jj = lane; jj < B; jj += 32) {
+    for (int i = 0; i < B; ++i) {
+      const float4 *di = reinterpret_cast<const float4 *>(Ds + i * kWideDStride);
+      const float4 *dj = reinterpret_cast<const float4 *>(Ds + jj * kWideDStride);
+      float acc = 0.f;
+#pragma unroll 8
+      for (int c = 0; c < LOCKS_D / 4; ++c) {
+        const float4 x = di[c], y = dj[c];
+        acc = fmaf(x.x, y.x, fmaf(x.y, y.y, fmaf(x.z, y.z, fmaf(x.w, y.w, acc))));
+      }
+      W[jj * WS + i] = acc;
+      amax = fmaxf(amax, fabsf(acc));
+    }
+  }
+  amax = warp_max(amax);
+  // unit scale (an exact power of two, undone on the eigenvalues)
+  float unscale = 1.f;
+  if (amax > 0.f && amax < INFINITY) {
+    int ex;
+    (void)frexpf(amax, &ex);
+    ex = max(-120, min(120, ex));
+    const float sc = ldexpf(1.f, -ex);
+    unscale = ldexpf(1.f, ex);
+    for (int jj = lane; jj < B; jj += 32)
+      for (int i = 0; i < B; ++i) W[jj * WS + i] *= sc;
+  }
+  __syncwarp();
+  // ---- one-sided Jacobi, odd-even transposition, rotate then swap
+  const float tol2 = LOCKS_BUILD_COS_TOL * LOCKS_BUILD_COS_TOL;
+  for (int sweep = 0; sweep < 2 * LOCKS_BUILD_SWEEPS; ++sweep) {
+    float nm = 0.f;
+    for (int jj = lane; jj < B; jj += 32) {
+      float a = 0.f;
+      for (int i = 0; i < B; ++i) a = fmaf(W[jj * WS + i], W[jj * WS + i], a);
+      nr[jj] = a;
+      nm = fmaxf(nm, a);
+    }
+    const float floor_n = 1e-11f * warp_max(nm);
+    __syncwarp();
+    int bad = 0;
+    for (int st = 0; st < B; ++st) {
+      const int pc = 2 * lane + (st & 1), qc = pc + 1;   // the pair of this lane
+      if (qc < B) {
+        float *wp = W + pc * WS, *wq = W + qc * WS;
+        const float a = nr[pc], bq = nr[qc];
+        float g = 0.f;
+        for (int i = 0; i < B; ++i) g = fmaf(wp[i], wq[i], g);
+        bad |= (int)(g * g > tol2 * a * bq) & (int)(fminf(a, bq) > floor_n);
+        float c, sn;
+        plane_rotation(a, bq, g, c, sn);
+        for (int i = 0; i < B; ++i) {
+          const float x = wp[i], y = wq[i];
+          wp[i] = fmaf(sn, x, c * y);    // q' takes p's place
+          wq[i] = fmaf(c, x, -sn * y);   // p' takes q's place
+        }
+        nr[pc] = fmaxf(fmaf(sn * sn, a, fmaf(c * c, bq, 2.f * c * sn * g)), 0.f);
+        nr[qc] = fmaxf(fmaf(c * c, a, fmaf(sn * sn, bq, -2.f * c * sn * g)), 0.f);
+      }
+      __syncwarp();
+    }
+    if (!__any_sync(0xffffffffu, bad != 0)) break;
+  }
+  // ---- exact norms, ranking (descending, ties to the lower position)
+  for (int jj = lane; jj < B; jj += 32) {
+    float a = 0.f;
+    for (int i = 0; i < B; ++i) a = fmaf(W[jj * WS + i], W[jj * WS + i], a);
+    nr[jj] = a;
+  }
+  __syncwarp();
+  for (int jj = lane; jj < B; jj += 32) {
+    const float mine = nr[jj];
+    int rk = 0;
+    for (int o = 0; o < B; ++o) rk += (nr[o] > mine) || (nr[o] == mine && o < jj);
+    order[rk] = jj;
+  }
+  __syncwarp();
+  const float lam0 = sqrtf(nr[order[0]]) * unscale;
+  int r_eff = 0;
+  const int rmax = min(r, B - 1);
+  for (int l = 0; l < rmax; ++l) {
+    const float ll = sqrtf(nr[order[l]]) * unscale;
+    if (lam0 > 0.f && ll > 1e-6f * lam0 && ll > 1e-10f * knorm2) r_eff = l + 1; else break;
+  }
+  uint8_t *gout = p.summ + ((int64_t)block * p.Hkv + h) * p.S;
+  float *fout = reinterpret_cast<float *>(gout);
+  constexpr int WD = FMT == LOCKS_FMT_BF16 ? 2 : 1;
+  uint32_t sign_bits = 0u;
+  for (int l = 0; l < r; ++l) {
+    float v[4] = {0.f, 0.f, 0.f, 0.f}, best = 0.f;
+    if (l < r_eff) {
+      const int col = order[l];
+      const float n2 = nr[col], lam = sqrtf(n2) * unscale;
+      const float inv = rsqrtf(n2) * rsqrtf(lam);   // unit eigenvector entries, then 1 / sigma
+      for (int i = 0; i < B; ++i) {
+        const float u = W[col * WS + i];
+        const float4 d4 = *reinterpret_cast<const float4 *>(Ds + i * kWideDStride + 4 * lane);
+        v[0] = fmaf(d4.x, u, v[0]); v[1] = fmaf(d4.y, u, v[1]); v[2] = fmaf(d4.z, u, v[2]); v[3] = fmaf(d4.w, u, v[3]);
+      }
+#pragma unroll
+      for (int c = 0; c < 4; ++c) v[c] *= inv;
+      best = fabsf(v[0]); float bv = v[0];
+#pragma unroll
+      for (int c = 1; c < 4; ++c) if (fabsf(v[c]) > best) { best = fabsf(v[c]); bv = v[c]; }
+      const uint32_t mxb = __reduce_max_sync(0xffffffffu, __float_as_uint(best));
+      const uint32_t who = __ballot_sync(0xffffffffu, __float_as_uint(best) == mxb);
+      bv = __shfl_sync(0xffffffffu, bv, __ffs(who) - 1);
+      best = __uint_as_float(mxb);
+      if (bv < 0.f) {
+        sign_bits |= 1u << l;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) v[c] = -v[c];
+      }
+    }
+    if (FMT == LOCKS_FMT_F32) {
+      *reinterpret_cast<float4 *>(fout + LOCKS_D + l * LOCKS_D + lane * 4) = make_float4(v[0], v[1], v[2], v[3]);
+    } else if (FMT == LOCKS_FMT_BF16) {
+      *reinterpret_cast<uint2 *>(gout + 2 * (l * LOCKS_D + lane * 4)) = make_uint2(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]));
+    } else if (FMT == LOCKS_FMT_I8) {
+      const __half sh = __float2half_rn(best / 127.f);
+      const float sc = inv_scale(__half2float(sh));
+      if (lane == 0) *reinterpret_cast<__half *>(gout + wb_off_sv(r, 1, B) + 2 * l) = sh;
+      uint32_t wd = 0u;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) wd |= (uint32_t)((int)round_code(v[c], sc, 127.f) + 128) << (8 * c);
+      *reinterpret_cast<uint32_t *>(gout + l * LOCKS_D + lane * 4) = wd;
+    } else {   // int4 basis: the same nibble order as at B = 16
+      const __half sh = __float2half_rn(best / 7.f);
+      const float sc = inv_scale(__half2float(sh));
+      if (lane == 0) *reinterpret_cast<__half *>(gout + i4_off_sv(r, B) + 2 * l) = sh;
+      const int t = lane >> 3, s8 = lane & 7, i0 = (s8 & 1) << 1;
+      uint32_t nb[4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) nb[c] = (uint32_t)((int)round_code(v[c], sc, 7.f) + 8);
+      uint32_t pw = (nb[0] << (4 * i0)) | (nb[1] << (4 * (i0 + 4))) | (nb[2] << (4 * (i0 + 1))) | (nb[3] << (4 * (i0 + 5)));
+      pw |= __shfl_xor_sync(0xffffffffu, pw, 1);
+      if ((s8 & 1) == 0) *reinterpret_cast<uint32_t *>(gout + (l * 4 + t) * 16 + (s8 >> 1) * 4) = pw;
+    }
+  }
+  // coefficients: lane owns tokens lane and lane + 32
+  for (int tok = lane; tok < B; tok += 32) {
+    float mx = 0.f;
+    for (int l = 0; l < r; ++l) {
+      float c = 0.f;
+      if (l < r_eff) {
+        const int col = order[l];
+        c = W[col * WS + tok] * rsqrtf(nr[col]) * sqrtf(sqrtf(nr[col]) * unscale);
+        if ((sign_bits >> l) & 1u) c = -c;
+      }
+      mx = fmaxf(mx, fabsf(c));
+      if (FMT == LOCKS_FMT_F32) fout[LOCKS_D + r * LOCKS_D + tok * r + l] = c;
+    }
+    if (FMT != LOCKS_FMT_F32) {
+      const __half sh = __float2half_rn(mx / 127.f);
+      const float sc = inv_scale(__half2float(sh));
+      *reinterpret_cast<__half *>(gout + (FMT == LOCKS_FMT_I4 ? i4_off_sc(r, B) : wb_off_sc(r, WD, B)) + 2 * tok) = sh;
+      for (int l = 0; l < r; ++l) {
+        float c = 0.f;
+        if (l < r_eff) {
+          const int col = order[l];
+          c = W[col * WS + tok] * rsqrtf(nr[col]) * sqrtf(sqrtf(nr[col]) * unscale);
+          if ((sign_bits >> l) & 1u) c = -c;
+        }
+        gout[(FMT == LOCKS_FMT_I4 ? i4_off_coef(r) : wb_off_coef(r, WD)) + tok * r + l] = (uint8_t)((int)round_code(c, sc, 127.f) + 128);
+      }
+    }
+  }
+  // centroid
+  if (FMT == LOCKS_FMT_F32) {
+    *reinterpret_cast<float4 *>(fout + lane * 4) = make_float4(mu[0], mu[1], mu[2], mu[3]);
+  } else {
+    float mx = fmaxf(fmaxf(fabsf(mu[0]), fabsf(mu[1])), fmaxf(fabsf(mu[2]), fabsf(mu[3])));
+    mx = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(mx)));
+    const __half sh = __float2half_rn(mx / 127.f);
+    const float sc = inv_scale(__half2float(sh));
+    const int osmu = FMT == LOCKS_FMT_I4 ? i4_off_smu(r, B) : wb_off_smu(r, WD, B);
+    if (lane == 0) *reinterpret_cast<__half *>(gout + osmu) = sh;
+    uint32_t by[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) by[c] = (uint32_t)((int)round_code(mu[c], sc, 127.f) + 128);
+    if (FMT == LOCKS_FMT_I4)   // dim offset c = 2*half + e -> byte e*2 + half, as at B = 16
+      *reinterpret_cast<uint32_t *>(gout + i4_off_mu(r, B) + lane * 4) = by[0] | (by[2] << 8) | (by[1] << 16) | (by[3] << 24);
+    else
+      *reinterpret_cast<uint32_t *>(gout + wb_off_mu(r, WD, B) + lane * 4) = by[0] | (by[1] << 8) | (by[2] << 16) | (by[3] << 24);
+    for (int e = osmu + 2 + lane; e < p.S; e += 32) gout[e] = 0;
+  }
+}
+
 }  // namespace
 
 int locks_launch_build(locks_ctx *c, const locks_kv *kv, int batch, const int32_t *pb, const int32_t *pe,
@@ -886,9 +803,30 @@ int locks_launch_build(locks_ctx *c, const locks_kv *kv, int batch, const int32_
     const locks_scan_geom geo = locks_scan_geometry(c, batch);
     p.hint = c->hint_dev; p.hint_wpp = geo.wpp; p.hint_rounds = geo.rounds; p.hint_W = geo.W;
   }
-  if (c->B != LOCKS_B && k_layers) return LOCKS_ERR_UNSUPPORTED;   // one layer per launch
-  // A step's few pages, where latency counts, and the page sizes that the bulk kernel does not know: one CTA per page
-  if (just_filled || c->B != LOCKS_B) return locks_launch_build_pages(c, p, just_filled, st);
+  if (just_filled) return locks_launch_build_pages(c, p, st);   // a step's few pages: latency counts, one CTA per page
+  if (c->B != LOCKS_B) {   // pages of 32 / 64 tokens: the plain kernel (row-major formats; one layer per launch)
+    if (k_layers) return LOCKS_ERR_UNSUPPORTED;
+    const int B = c->B, smem = build_wide_smem(B);
+    const dim3 grid(c->Pmax, p.Hkv, batch);
+    const bool bf16kv = c->cfg.kv_dtype == LOCKS_BF16;
+#define LOCKS_WIDE_CASE(F_)                                                                                              \
+  do {                                                                                                                  \
+    if (locks_attrs_needed(LOCKS_ATTR_BUILD_WIDE + F_)) {                                                                \
+      cudaFuncSetAttribute(build_wide_kernel<__nv_bfloat16, F_>, cudaFuncAttributeMaxDynamicSharedMemorySize, build_wide_smem(64)); \
+      cudaFuncSetAttribute(build_wide_kernel<float, F_>, cudaFuncAttributeMaxDynamicSharedMemorySize, build_wide_smem(64));         \
+    }                                                                                                                   \
+    if (bf16kv) build_wide_kernel<__nv_bfloat16, F_><<<grid, 32, smem, st>>>(p, B);                        \
+    else build_wide_kernel<float, F_><<<grid, 32, smem, st>>>(p, B);                                       \
+  } while (0)
+    switch (c->cfg.summary_fmt) {
+      case LOCKS_FMT_I4: LOCKS_WIDE_CASE(LOCKS_FMT_I4); break;
+      case LOCKS_FMT_I8: LOCKS_WIDE_CASE(LOCKS_FMT_I8); break;
+      case LOCKS_FMT_BF16: LOCKS_WIDE_CASE(LOCKS_FMT_BF16); break;
+      default: LOCKS_WIDE_CASE(LOCKS_FMT_F32); break;
+    }
+#undef LOCKS_WIDE_CASE
+    return locks_check_launch(c);
+  }
   constexpr int kPer = kBuildWarps * kBuildItems;   // items per CTA (bulk)
   const dim3 grid((c->Pmax + kPer - 1) / kPer, p.Hkv, batch * (k_layers ? num_layers : 1));
   const bool bf = c->cfg.kv_dtype == LOCKS_BF16;
@@ -899,10 +837,7 @@ int locks_launch_build(locks_ctx *c, const locks_kv *kv, int batch, const int32_
     else build_kernel<float, F_><<<grid, kBuildWarps * 32, smem, st>>>(p);                                                 \
   } while (0)
   switch (c->cfg.summary_fmt) {
-    case LOCKS_FMT_I4:
-      if (bf) build_i4_kernel<<<grid, kBuildWarps * 32, kBuildWarps * kBuildI4SmemPerWarp, st>>>(p);
-      else build_kernel<float, LOCKS_FMT_I4><<<grid, kBuildWarps * 32, smem, st>>>(p);
-      break;
+    case LOCKS_FMT_I4: LOCKS_BUILD_CASE(LOCKS_FMT_I4); break;
     case LOCKS_FMT_I8: LOCKS_BUILD_CASE(LOCKS_FMT_I8); break;
     case LOCKS_FMT_BF16: LOCKS_BUILD_CASE(LOCKS_FMT_BF16); break;
     default: LOCKS_BUILD_CASE(LOCKS_FMT_F32); break;

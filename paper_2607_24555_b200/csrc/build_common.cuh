@@ -1,5 +1,5 @@
-// Parameters and arithmetic shared by the two summary-build kernels (build.cu: bulk, 16-token pages; build_page.cu: one
-// CTA per page, every page size).
+// Parameters and arithmetic shared by the summary-build kernels (build.cu: bulk; build_page.cu: the pages that a decode step
+// has just filled).
 #pragma once
 #include "locks_internal.cuh"
 
@@ -25,9 +25,8 @@ struct BuildParams {
   void *const *summ_layers;
 };
 
-// One CTA per page: the pages that a decode step has just filled (step = 1), or all pages of the call's ranges.
-// Adds its launch to c->last_launches.
-int locks_launch_build_pages(locks_ctx *c, const BuildParams &p, int step, cudaStream_t st);
+// The pages that a decode step has just filled.  Adds its launch to c->last_launches.
+int locks_launch_build_pages(locks_ctx *c, const BuildParams &p, cudaStream_t st);
 
 #define LOCKS_BUILD_COS_TOL 1e-3f   // a Jacobi sweep that met no pair above this |cosine| was the last (it left them near 1e-6: quadratic convergence)
 #define LOCKS_BUILD_SWEEPS 16       // upper bound (twice that for 32- and 64-token pages)

@@ -1,6 +1,5 @@
-// Summary build, one CTA per (page, KV head): the pages that a decode step has just filled (any page size), and every
-// build of 32- and 64-token pages.  The method is that of build.cu (Sec. 4 "Build"); here the latency of one page counts,
-// because the step that filled it ends with its summary.
+// Summary build of the pages that a decode step has just filled (any page size).  The method is that of build.cu (Sec. 4
+// "Build"); here the latency of one page counts, because the step that filled it ends with its summary.
 //
 // What bounds it is one dependent chain, the eigenproblem of the B x B Gram matrix M.  One warp solves it by one-sided
 // Jacobi in registers: a pair of columns belongs to L lanes that hold B / L rows of both, so a step (B / 2 pairs at once)
@@ -184,33 +183,20 @@ template <int B> __device__ __forceinline__ void solve_modes(PageShared<B> &sh, 
 }
 
 template <int B>
-__global__ void __launch_bounds__(page_threads(B) * page_ctas(B)) build_page_kernel(BuildParams p, int step) {
+__global__ void __launch_bounds__(page_threads(B) * page_ctas(B)) build_page_kernel(BuildParams p) {
   extern __shared__ __align__(16) uint8_t smem_raw[];
   constexpr int NT = page_threads(B), PPC = page_ctas(B), DS = dt_stride(B), NW = NT / 32, DPT = LOCKS_D / NT;
   const int sub = threadIdx.x / NT, tid = threadIdx.x % NT, lane = tid & 31, warp = tid >> 5, r = p.r;
   PageShared<B> &sh = reinterpret_cast<PageShared<B> *>(smem_raw)[sub];
   auto sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(sub + 1), "n"(NT) : "memory"); };   // the page's threads
-  int b, h, page, last_from_new = 0;
-  if (step) {
-    if (p.hint && blockIdx.x == 0 && threadIdx.x < 32)
-      locks_update_partition_hint(p.hint, p.seq_lens, p.batch, p.Hkv, p.kpages, p.hint_wpp, p.hint_rounds, p.hint_W, lane);
-    const int prob = blockIdx.x * PPC + sub;
-    if (prob >= p.batch * p.Hkv) return;
-    b = prob / p.Hkv;
-    h = prob - b * p.Hkv;
-    const int Tb = p.seq_lens[b];
-    if (Tb <= 0 || (Tb & (B - 1)) != 0) return;
-    page = Tb / B - 1;
-    last_from_new = (p.k_new && p.append_pos && p.append_pos[b] == Tb - 1) ? 1 : 0;   // the last row is this step's token
-  } else {
-    b = blockIdx.z;
-    h = blockIdx.y;
-    const int complete = p.seq_lens[b] / B;
-    const int p0 = p.page_begin ? p.page_begin[b] : 0;
-    const int p1 = min(p.page_end ? p.page_end[b] : complete, complete);
-    page = p0 + blockIdx.x * PPC + sub;
-    if (page < 0 || page >= p1) return;
-  }
+  if (p.hint && blockIdx.x == 0 && threadIdx.x < 32)
+    locks_update_partition_hint(p.hint, p.seq_lens, p.batch, p.Hkv, p.kpages, p.hint_wpp, p.hint_rounds, p.hint_W, lane);
+  const int prob = blockIdx.x * PPC + sub;
+  if (prob >= p.batch * p.Hkv) return;
+  const int b = prob / p.Hkv, h = prob - b * p.Hkv, Tb = p.seq_lens[b];
+  if (Tb <= 0 || (Tb & (B - 1)) != 0) return;
+  const int page = Tb / B - 1;
+  const bool last_from_new = p.k_new && p.append_pos && p.append_pos[b] == Tb - 1;   // the last row is this step's token
   if (page >= p.Pmax) return;
   const int block = p.block_table[(int64_t)b * p.Pmax + page];
   if (block < 0 || block >= p.num_blocks) {
@@ -428,17 +414,17 @@ __global__ void __launch_bounds__(page_threads(B) * page_ctas(B)) build_page_ker
   if (osmu + 2 + tid < p.S) gout[osmu + 2 + tid] = 0;   // bytes between the payload and the padded stride stay zero
 }
 
-template <int B> int launch_pages(locks_ctx *c, const BuildParams &p, int step, cudaStream_t st) {
+template <int B> int launch_pages(locks_ctx *c, const BuildParams &p, cudaStream_t st) {
   constexpr int PPC = page_ctas(B), smem = PPC * (int)sizeof(PageShared<B>);
-  const dim3 grid = step ? dim3((p.batch * p.Hkv + PPC - 1) / PPC) : dim3((c->Pmax + PPC - 1) / PPC, p.Hkv, p.batch);
+  const dim3 grid((p.batch * p.Hkv + PPC - 1) / PPC);
   if (locks_attrs_needed(LOCKS_ATTR_BUILD_PAGE + B / 32))
     cudaFuncSetAttribute(build_page_kernel<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  build_page_kernel<B><<<grid, PPC * page_threads(B), smem, st>>>(p, step);
+  build_page_kernel<B><<<grid, PPC * page_threads(B), smem, st>>>(p);
   return locks_check_launch(c);
 }
 
 }  // namespace
 
-int locks_launch_build_pages(locks_ctx *c, const BuildParams &p, int step, cudaStream_t st) {
-  return c->B == 64 ? launch_pages<64>(c, p, step, st) : (c->B == 32 ? launch_pages<32>(c, p, step, st) : launch_pages<16>(c, p, step, st));
+int locks_launch_build_pages(locks_ctx *c, const BuildParams &p, cudaStream_t st) {
+  return c->B == 64 ? launch_pages<64>(c, p, st) : (c->B == 32 ? launch_pages<32>(c, p, st) : launch_pages<16>(c, p, st));
 }
