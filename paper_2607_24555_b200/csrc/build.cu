@@ -241,6 +241,243 @@ __device__ __forceinline__ int item_block(const BuildParams &p, int warp, int la
   return -1;
 }
 
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  float2 d;
+  asm("add.rn.f32x2 %0, %1, %2;"
+      : "=l"(*reinterpret_cast<unsigned long long *>(&d))
+      : "l"(*reinterpret_cast<unsigned long long *>(&a)), "l"(*reinterpret_cast<unsigned long long *>(&b)));
+  return d;
+}
+
+// bf16 keys, int4 summaries: build_kernel's arithmetic with its phases 1 and 3 arranged for the common case.  Packed fp32
+// pairs; M leaves the MMA accumulators through one transposed array instead of two; all modes' basis vectors are formed
+// before any is quantised, so that their scales (a division, an fp16 rounding and a reciprocal each) are worked out by a
+// lane per mode, once; codes go straight to global memory.
+constexpr int kBuildI4SmemPerWarp = kBuildScratch + kBuildMat + 64 + kBuildItems * LOCKS_B * 4;
+__global__ void __launch_bounds__(kBuildWarps * 32, kBuildCtasPerSm) build_i4_kernel(BuildParams p) {
+  extern __shared__ __align__(16) uint8_t smem_raw[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int h = blockIdx.y, r = p.r;
+  const int it_block = item_block(p, warp, lane);   // the warp's items: lane s < 8 works out item s
+  const uint32_t live = __ballot_sync(0xffffffffu, it_block >= 0);
+  if (!live) return;
+  const int layer = blockIdx.z / p.batch;
+  const __nv_bfloat16 *kbase = reinterpret_cast<const __nv_bfloat16 *>(p.k_layers ? p.k_layers[layer] : p.k);
+  uint8_t *sbase = p.summ_layers ? reinterpret_cast<uint8_t *>(p.summ_layers[layer]) : p.summ;
+  uint8_t *scratch = smem_raw + warp * kBuildI4SmemPerWarp;          // D half-tiles, then Y
+  float *mat = reinterpret_cast<float *>(scratch + kBuildScratch);   // [8][16][16] Gram; then [8][8][16] pairs (u, u) of U_r by mode
+  float *kn_s = mat + kBuildItems * kMat;                            // [8] squared norm of the page's keys
+  float *lam_s = kn_s + 16;                                          // [8][16] eigenvalues, descending
+  // deviations of item s: v[i][e] = key i minus the centroid, dims 4 lane + 2 e, + 1; knorm2: this lane's share
+  auto load_centred = [&](int s, float2 (&v)[LOCKS_B][2], float2 (&mu)[2], bool want_norm, float &knorm2) {
+    const __nv_bfloat16 *K = kbase + (int64_t)__shfl_sync(0xffffffffu, it_block, s) * p.sb + (int64_t)h * p.sh + 4 * lane;
+#pragma unroll
+    for (int i = 0; i < LOCKS_B; ++i) {
+      const uint2 w = *reinterpret_cast<const uint2 *>(K + (int64_t)i * p.st);
+      v[i][0] = make_float2(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xFFFF0000u));
+      v[i][1] = make_float2(__uint_as_float(w.y << 16), __uint_as_float(w.y & 0xFFFF0000u));
+    }
+    if (want_norm) {
+      float2 n0 = make_float2(0.f, 0.f), n1 = n0;
+#pragma unroll
+      for (int i = 0; i < LOCKS_B; ++i) { n0 = fma2(v[i][0], v[i][0], n0); n1 = fma2(v[i][1], v[i][1], n1); }
+      knorm2 = (n0.x + n0.y) + (n1.x + n1.y);
+    }
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      mu[e] = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int i = 0; i < LOCKS_B; ++i) mu[e] = add2(mu[e], v[i][e]);
+      mu[e] = mul2(mu[e], make_float2(1.f / LOCKS_B, 1.f / LOCKS_B));
+      const float2 neg = make_float2(-mu[e].x, -mu[e].y);
+#pragma unroll
+      for (int i = 0; i < LOCKS_B; ++i) v[i][e] = add2(v[i][e], neg);
+    }
+  };
+
+  // ---- 1. Gram matrices (see build_kernel)
+#pragma unroll 1
+  for (int s = 0; s < kBuildItems; ++s) {
+    if (!((live >> s) & 1u)) continue;
+    uint32_t hl[LOCKS_B][4];   // h01, h23, l01, l23 of this lane's 4 dims, per key
+    {
+      float2 v[LOCKS_B][2], mu[2];
+      float knorm2 = 0.f;
+      load_centred(s, v, mu, true, knorm2);
+      knorm2 = warp_sum(knorm2);
+      if (lane == 0) kn_s[s] = knorm2;
+#pragma unroll
+      for (int i = 0; i < LOCKS_B; ++i)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const uint32_t hh = pack_bf16(v[i][e].x, v[i][e].y);
+          const float2 lo = add2(v[i][e], make_float2(-__uint_as_float(hh << 16), -__uint_as_float(hh & 0xFFFF0000u)));
+          hl[i][e] = hh;
+          hl[i][2 + e] = pack_bf16(lo.x, lo.y);
+        }
+    }
+    float X0[4] = {0.f, 0.f, 0.f, 0.f}, X1[4] = {0.f, 0.f, 0.f, 0.f}, Y0[4] = {0.f, 0.f, 0.f, 0.f}, Y1[4] = {0.f, 0.f, 0.f, 0.f};
+    const int c16 = lane & 15;                                          // writer: dims 4 c16 .. + 3 of the half
+    const int mq = lane >> 3, rr = lane & 7, tok = (mq & 1) * 8 + rr;   // reader (ldmatrix address lanes)
+#pragma unroll
+    for (int hf = 0; hf < 2; ++hf) {
+      if ((lane >> 4) == hf) {
+#pragma unroll
+        for (int row = 0; row < LOCKS_B; ++row) {
+          uint8_t *dst = scratch + row * 128 + ((((c16 >> 1) ^ (row & 7)) << 4) | ((c16 & 1) << 3));
+          *reinterpret_cast<uint2 *>(dst) = make_uint2(hl[row][0], hl[row][1]);
+          *reinterpret_cast<uint2 *>(dst + 2048) = make_uint2(hl[row][2], hl[row][3]);
+        }
+      }
+      __syncwarp();
+#pragma unroll
+      for (int s4 = 0; s4 < 4; ++s4) {
+        uint32_t Hf[4], Lf[4];
+        const uint8_t *src = scratch + tok * 128 + (((2 * s4 + (mq >> 1)) ^ (tok & 7)) << 4);
+        ldsm_x4(Hf, src);
+        ldsm_x4(Lf, src + 2048);
+        mma_bf16(X0, Hf[0], Hf[1], Hf[2], Hf[3], Hf[0], Hf[2]);
+        mma_bf16(X1, Hf[0], Hf[1], Hf[2], Hf[3], Hf[1], Hf[3]);
+        mma_bf16(X0, Lf[0], Lf[1], Lf[2], Lf[3], Lf[0], Lf[2]);
+        mma_bf16(X1, Lf[0], Lf[1], Lf[2], Lf[3], Lf[1], Lf[3]);
+        mma_bf16(Y0, Hf[0], Hf[1], Hf[2], Hf[3], Lf[0], Lf[2]);
+        mma_bf16(Y1, Hf[0], Hf[1], Hf[2], Hf[3], Lf[1], Lf[3]);
+      }
+      __syncwarp();
+    }
+    // accumulator (x = lane / 4, t = lane % 4): [0..1] = row x, columns 2t, 2t+1 (X1: + 8); [2..3] = row x + 8.  X is symmetric
+    // as computed; M = X + Y + Y^T, the transpose through a padded 16 x 17 array in the (now free) scratch
+    {
+      float *YA = reinterpret_cast<float *>(scratch);
+      const int x = lane >> 2, t = lane & 3;
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        YA[x * 17 + 2 * t + e] = Y0[e]; YA[(x + 8) * 17 + 2 * t + e] = Y0[2 + e];
+        YA[x * 17 + 8 + 2 * t + e] = Y1[e]; YA[(x + 8) * 17 + 8 + 2 * t + e] = Y1[2 + e];
+      }
+      __syncwarp();
+      float *dst = mat + s * kMat + x * LOCKS_B + 2 * t;
+      const float *yt = YA + 2 * t * 17 + x;   // column 2t of Y^T's row x
+      *reinterpret_cast<float2 *>(dst) = make_float2(X0[0] + Y0[0] + yt[0], X0[1] + Y0[1] + yt[17]);
+      *reinterpret_cast<float2 *>(dst + 8) = make_float2(X1[0] + Y1[0] + yt[8 * 17], X1[1] + Y1[1] + yt[9 * 17]);
+      *reinterpret_cast<float2 *>(dst + 8 * LOCKS_B) = make_float2(X0[2] + Y0[2] + yt[8], X0[3] + Y0[3] + yt[17 + 8]);
+      *reinterpret_cast<float2 *>(dst + 8 * LOCKS_B + 8) = make_float2(X1[2] + Y1[2] + yt[8 * 17 + 8], X1[3] + Y1[3] + yt[9 * 17 + 8]);
+      __syncwarp();
+    }
+  }
+
+  // ---- 2. eigenvectors and eigenvalues of all the warp's items at once
+  jacobi_phase<true>(mat, mat, lam_s, live, r, lane);
+
+  // ---- 3. basis, coefficients, centroid
+#pragma unroll 1
+  for (int s = 0; s < kBuildItems; ++s) {
+    if (!((live >> s) & 1u)) continue;
+    const float *U = mat + s * kMat, *lam = lam_s + s * LOCKS_B;   // U[mode][token] as pairs
+    // lane l < r: mode l
+    const float lam0 = lam[0], lx = lam[lane & 15];
+    const uint32_t above = __ballot_sync(0xffffffffu, lam0 > 0.f && lx > 1e-6f * lam0 && lx > 1e-10f * kn_s[s]);
+    const int r_eff = min(r, __ffs(~above) - 1);   // modes above the zero-mode thresholds (eigenvalues descend; never 16 of them)
+    const float isig = lane < r_eff ? rsqrtf(lx) : 0.f;
+    float2 v[8][2], mu[2];   // basis vectors of this lane's 4 dims
+    {
+      float2 dv[LOCKS_B][2];
+      float unused;
+      load_centred(s, dv, mu, false, unused);
+#pragma unroll
+      for (int l = 0; l < 8; ++l) {
+        v[l][0] = v[l][1] = make_float2(0.f, 0.f);
+        if (l < r_eff) {
+          const float4 *u4 = reinterpret_cast<const float4 *>(U + l * 2 * LOCKS_B);
+#pragma unroll
+          for (int i = 0; i < LOCKS_B; i += 2) {
+            const float4 u = u4[i / 2];
+            v[l][0] = fma2(dv[i][0], make_float2(u.x, u.y), v[l][0]);
+            v[l][1] = fma2(dv[i][1], make_float2(u.x, u.y), v[l][1]);
+            v[l][0] = fma2(dv[i + 1][0], make_float2(u.z, u.w), v[l][0]);
+            v[l][1] = fma2(dv[i + 1][1], make_float2(u.z, u.w), v[l][1]);
+          }
+        }
+      }
+    }
+    uint8_t *gout = sbase + ((int64_t)__shfl_sync(0xffffffffu, it_block, s) * p.Hkv + h) * p.S;
+    // sign: the entry of largest magnitude (lowest dim on ties) is positive.  Magnitudes order like their bit patterns; the
+    // lowest lane that holds the maximum owns the lowest such dim.
+    float best_mode = 0.f;         // lane l: largest magnitude of mode l
+    uint32_t neg = 0u;             // bit l: mode l is flipped
+#pragma unroll
+    for (int l = 0; l < 8; ++l) {
+      if (l >= r_eff) break;
+      const float is = __shfl_sync(0xffffffffu, isig, l);
+      const float2 is2 = make_float2(is, is);
+      v[l][0] = mul2(v[l][0], is2);
+      v[l][1] = mul2(v[l][1], is2);
+      float best = fabsf(v[l][0].x), bv = v[l][0].x;
+      if (fabsf(v[l][0].y) > best) { best = fabsf(v[l][0].y); bv = v[l][0].y; }
+      if (fabsf(v[l][1].x) > best) { best = fabsf(v[l][1].x); bv = v[l][1].x; }
+      if (fabsf(v[l][1].y) > best) { best = fabsf(v[l][1].y); bv = v[l][1].y; }
+      const uint32_t mxb = __reduce_max_sync(0xffffffffu, __float_as_uint(best));
+      const uint32_t who = __ballot_sync(0xffffffffu, __float_as_uint(best) == mxb), minus = __ballot_sync(0xffffffffu, bv < 0.f);
+      if (minus & who & -who) neg |= 1u << l;
+      if (lane == l) best_mode = __uint_as_float(mxb);
+    }
+    const __half sv = __float2half_rn(best_mode / 7.f);
+    const float sc_mode = inv_scale(__half2float(sv)) * ((neg >> (lane & 7)) & 1u ? -1.f : 1.f);
+    if (lane < r) *reinterpret_cast<__half *>(gout + i4_off_sv(r) + 2 * lane) = sv;
+    // codes: lane = 8 t + s8 owns dims 32 t + 4 s8 + {0,1,2,3} = (half, e) in {0,1}^2 of k-step s8; dim offset c = 2 half + e ->
+    // nibble 2 (s8 & 1) + half + 4 e.  x + 1.5 2^23 + 8 rounds half to even and leaves code + 8 in the low bits (a unit vector's
+    // largest entry is at least 0.088: no scale is subnormal, no code leaves -7 .. 7)
+#pragma unroll
+    for (int l = 0; l < 8; ++l) {
+      if (l >= r) break;
+      const float sc = __shfl_sync(0xffffffffu, sc_mode, l);
+      const float2 sc2 = make_float2(sc, sc), magic = make_float2(12582920.f, 12582920.f);
+      const float2 a = add2(mul2(v[l][0], sc2), magic), b = add2(mul2(v[l][1], sc2), magic);
+      uint32_t pw = (__float_as_uint(a.x) & 15u) | (__float_as_uint(a.y) & 15u) << 16 | (__float_as_uint(b.x) & 15u) << 4 |
+                    (__float_as_uint(b.y) & 15u) << 20;
+      pw <<= 8 * (lane & 1);
+      pw |= __shfl_xor_sync(0xffffffffu, pw, 1);
+      if ((lane & 1) == 0) *reinterpret_cast<uint32_t *>(gout + l * 64 + lane * 2) = pw;
+    }
+    // coefficients C = U Sigma: lane (x, t) has tokens x and x + 8, modes 2t and 2t + 1
+    {
+      const int x = lane >> 2, t = lane & 3;
+      const float sg = lane < r_eff ? ((neg >> lane) & 1u ? -sqrtf(lx) : sqrtf(lx)) : 0.f;
+      const float g0 = __shfl_sync(0xffffffffu, sg, 2 * t), g1 = __shfl_sync(0xffffffffu, sg, 2 * t + 1);
+      const float *u0 = U + 2 * t * 2 * LOCKS_B + 2 * x, *u1 = u0 + 2 * LOCKS_B;
+      const float ca = 2 * t < r_eff ? g0 * u0[0] : 0.f, cb = 2 * t + 1 < r_eff ? g1 * u1[0] : 0.f;
+      const float cc = 2 * t < r_eff ? g0 * u0[16] : 0.f, cd = 2 * t + 1 < r_eff ? g1 * u1[16] : 0.f;
+      float ma = fmaxf(fabsf(ca), fabsf(cb)), mb = fmaxf(fabsf(cc), fabsf(cd));
+#pragma unroll
+      for (int o = 1; o < 4; o <<= 1) {
+        ma = fmaxf(ma, __shfl_xor_sync(0xffffffffu, ma, o));
+        mb = fmaxf(mb, __shfl_xor_sync(0xffffffffu, mb, o));
+      }
+      const __half sa = __float2half_rn(ma / 127.f), sb = __float2half_rn(mb / 127.f);
+      const float ia = inv_scale(__half2float(sa)), ib = inv_scale(__half2float(sb));
+      auto code = [&](float v, float inv) { return (uint32_t)((int)round_code(v, inv, 127.f) + 128); };
+      if (t < r / 2)
+        *reinterpret_cast<uint32_t *>(gout + i4_off_coef(r) + (x * (r / 2) + t) * 4) =
+            code(ca, ia) | (code(cb, ia) << 8) | (code(cc, ib) << 16) | (code(cd, ib) << 24);
+      if (t == 0) {
+        __half *dst = reinterpret_cast<__half *>(gout + i4_off_sc(r)) + (x >> 1) * 4 + (x & 1);
+        dst[0] = sa;
+        dst[2] = sb;
+      }
+    }
+    // centroid: dim offset c = 2*half + e -> byte e*2 + half
+    {
+      const float mx = fmaxf(fmaxf(fabsf(mu[0].x), fabsf(mu[0].y)), fmaxf(fabsf(mu[1].x), fabsf(mu[1].y)));
+      const __half sh = __float2half_rn(__uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(mx))) / 127.f);
+      const float sc = inv_scale(__half2float(sh));
+      auto code = [&](float v) { return (uint32_t)((int)round_code(v, sc, 127.f) + 128); };
+      *reinterpret_cast<uint32_t *>(gout + i4_off_mu(r) + lane * 4) = code(mu[0].x) | (code(mu[1].x) << 8) | (code(mu[0].y) << 16) | (code(mu[1].y) << 24);
+      if (lane == 0) *reinterpret_cast<__half *>(gout + i4_off_smu(r)) = sh;
+      if (lane < 16 && i4_off_smu(r) + 2 + lane < p.S) gout[i4_off_smu(r) + 2 + lane] = 0;   // bytes between the payload and the stride
+    }
+  }
+}
+
 template <typename T, int FMT>
 __global__ void __launch_bounds__(kBuildWarps * 32, kBuildCtasPerSm) build_kernel(BuildParams p) {
   extern __shared__ __align__(16) uint8_t smem_raw[];
@@ -837,7 +1074,10 @@ int locks_launch_build(locks_ctx *c, const locks_kv *kv, int batch, const int32_
     else build_kernel<float, F_><<<grid, kBuildWarps * 32, smem, st>>>(p);                                                 \
   } while (0)
   switch (c->cfg.summary_fmt) {
-    case LOCKS_FMT_I4: LOCKS_BUILD_CASE(LOCKS_FMT_I4); break;
+    case LOCKS_FMT_I4:
+      if (bf) build_i4_kernel<<<grid, kBuildWarps * 32, kBuildWarps * kBuildI4SmemPerWarp, st>>>(p);
+      else build_kernel<float, LOCKS_FMT_I4><<<grid, kBuildWarps * 32, smem, st>>>(p);
+      break;
     case LOCKS_FMT_I8: LOCKS_BUILD_CASE(LOCKS_FMT_I8); break;
     case LOCKS_FMT_BF16: LOCKS_BUILD_CASE(LOCKS_FMT_BF16); break;
     default: LOCKS_BUILD_CASE(LOCKS_FMT_F32); break;
