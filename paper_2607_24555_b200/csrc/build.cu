@@ -17,6 +17,9 @@
 // The bytes of a summary decide near-ties between pages, so what is computed and in which order is kept exactly: a
 // preconditioned solver (build_page.cu's; 5 sweeps for 8) builds 131 008 page-heads in 870 us and is as accurate, but one
 // byte in ten thousand comes out differently, and one request in a few hundred then keeps another page.
+// Bound by instruction issue, fetch and latency, not by bytes (an eigenproblem per 4 KB page).  131 008 page-heads: 1348 us
+// with the pair that straddles two lanes rotated by both and all formats in one kernel (6 960 warp instructions each), 1281
+// us with every pair rotated once and build_i4_kernel's phases (5 370), 1095 us with the body of a sweep kept to two steps.
 #include <type_traits>
 #include "build_common.cuh"
 
@@ -122,7 +125,7 @@ __device__ __forceinline__ void jacobi_phase(const float *mat, float *us, float 
   // columns whose norm is rounding noise beside the largest (null directions) do not hold up convergence
   // One pair: a is the column that it kept from the step before, b the one that it has been passed; in even steps b is the
   // lower position (p), in odd ones a.  The lower position receives q' = s p + c q, the upper one p' = c p - s q.  What is
-  // passed on ends in a, what is kept in b.  `there` = false: the two ends of the row, which do not meet: they change places.
+  // kept ends in a, what is passed on in b.  `there` = false: the two ends of the row, which do not meet: a stays, b moves on.
   auto rotate = [&](auto odd, float2 (&a)[8], float2 (&b)[8], float &na, float &nb, bool there) {
     constexpr bool kOdd = decltype(odd)::value;
     const float g = dot(a, b), np = kOdd ? na : nb, nq = kOdd ? nb : na;
@@ -136,13 +139,13 @@ __device__ __forceinline__ void jacobi_phase(const float *mat, float *us, float 
     for (int i = 0; i < 8; ++i) {
       const float2 p = kOdd ? a[i] : b[i], q = kOdd ? b[i] : a[i];
       const float2 pp = fma2(C2, p, mul2(nS2, q)), qq = fma2(S2, p, mul2(C2, q));
-      a[i] = kOdd ? pp : qq;
-      b[i] = kOdd ? qq : pp;
+      a[i] = kOdd ? qq : pp;
+      b[i] = kOdd ? pp : qq;
     }
     const float cc = c * c, ss = sn * sn;
     const float n_p = fmaxf(fmaf(cc, np, fmaf(ss, nq, -x2)), 0.f), n_q = fmaxf(fmaf(ss, np, fmaf(cc, nq, x2)), 0.f);
-    na = kOdd ? n_p : n_q;
-    nb = kOdd ? n_q : n_p;
+    na = kOdd ? n_q : n_p;
+    nb = kOdd ? n_p : n_q;
   };
   const int up = (lane & ~(LPI - 1)) | ((j + 1) & (LPI - 1)), down = (lane & ~(LPI - 1)) | ((j - 1) & (LPI - 1));
   auto fetch = [&](float2 (&col)[8], float &norm, int from) {
@@ -164,23 +167,14 @@ __device__ __forceinline__ void jacobi_phase(const float *mat, float *us, float 
       floor_n = 1e-11f * seg_max(nm);   // squared norm = squared eigenvalue: modes below 3e-6 of the largest
     }
     bad = 0;
-#pragma unroll 2
-    for (int st2 = 0; st2 < 8; ++st2) {
+#pragma unroll 1
+    for (int st2 = 0; st2 < 8; ++st2) {   // (a body of this size: twice unrolled, a quarter of the warps wait for instructions)
       rotate(even, w[1], w[0], n[1], n[0], true);
       rotate(even, w[3], w[2], n[3], n[2], true);
-      fetch(w[1], n[1], up);   // a pair passes to the one before it: w[3] to the lane's first, w[1] to the lane below
-      rotate(odd, w[0], w[3], n[0], n[3], true);
-      rotate(odd, w[2], w[1], n[2], n[1], j != LPI - 1);
-      fetch(w[2], n[2], down);   // ... and then to the one after it: w[0] to the lane's second, w[2] to the lane above
-      // the lane's pairs are now (w[3], w[2]) and (w[1], w[0]), in this order: exchange the names
-#pragma unroll
-      for (int c = 0; c < 2; ++c) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) { const float2 y = w[c][i]; w[c][i] = w[c + 2][i]; w[c + 2][i] = y; }
-        const float y = n[c];
-        n[c] = n[c + 2];
-        n[c + 2] = y;
-      }
+      fetch(w[0], n[0], up);     // a pair passes to the one before it: w[2] to the lane's first, w[0] to the lane below
+      rotate(odd, w[1], w[2], n[1], n[2], true);
+      rotate(odd, w[3], w[0], n[3], n[0], j != LPI - 1);
+      fetch(w[0], n[0], down);   // ... and then to the one after it: w[2] to the lane's second, w[0] to the lane above
     }
     if (!__any_sync(0xffffffffu, bad != 0)) break;
   }
