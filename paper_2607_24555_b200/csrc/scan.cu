@@ -566,8 +566,8 @@ __global__ void __launch_bounds__(kScanWarps * 32, kScanCtasPerSm) scan_i4_kerne
 
   // query of the current problem: qb0/qb2 = this lane's dims of head x (tile 0) / head x + 8 (tile 1)
   uint32_t qb0[NH][8], qb2[NH][8];
-  float inv_s[NH], ksum[2 * NH];   // c2 / scale of head x (+8); 8 * sum_c q'[c] of heads 2t, 2t+1 (+8)
-  float inv2[2 * NH];              // c2 / scale of heads 2t, 2t+1 (+8)
+  float inv_s[NH], ksum[2];        // c2 / scale of head x (+8); 8 * sum_c q'[c] of heads 2t, 2t+1 (NH = 2: of heads x, x+8)
+  float inv2[2] = {0.f, 0.f};      // c2 / scale of heads 2t, 2t+1 (NH = 1)
   int cur_prob = -1;
   const __nv_bfloat16 *q = reinterpret_cast<const __nv_bfloat16 *>(p.q);
   const float c2 = p.sm_scale * kLog2e;
@@ -628,12 +628,15 @@ __global__ void __launch_bounds__(kScanWarps * 32, kScanCtasPerSm) scan_i4_kerne
         float s8;
         const int gx = PK ? (x & 3) : x + 8 * hh;   // head held by this lane's column
         load_q_row(q + ((int64_t)b * p.Hq + h * p.G + gx) * LOCKS_D, t, gx < p.G, qb0[hh], qb2[hh], inv_s[hh], s8);
-        // lane (x, t) owns head gx; the column fragment needs the heads of columns 2t, 2t+1
-        ksum[2 * hh] = __shfl_sync(0xffffffffu, s8, (2 * t) * 4);
-        ksum[2 * hh + 1] = __shfl_sync(0xffffffffu, s8, (2 * t + 1) * 4);
         inv_s[hh] *= c2;   // from here on: the factor that turns a scaled dot product into a log2-domain logit
-        inv2[2 * hh] = __shfl_sync(0xffffffffu, inv_s[hh], (2 * t) * 4);
-        inv2[2 * hh + 1] = __shfl_sync(0xffffffffu, inv_s[hh], (2 * t + 1) * 4);
+        if (NH == 2) {
+          ksum[hh] = s8;
+        } else {   // lane (x, t) owns head gx; the column fragment needs the heads of columns 2t, 2t+1
+          ksum[0] = __shfl_sync(0xffffffffu, s8, (2 * t) * 4);
+          ksum[1] = __shfl_sync(0xffffffffu, s8, (2 * t + 1) * 4);
+          inv2[0] = __shfl_sync(0xffffffffu, inv_s[hh], (2 * t) * 4);
+          inv2[1] = __shfl_sync(0xffffffffu, inv_s[hh], (2 * t + 1) * 4);
+        }
       }
     }
     if (kScanBulk) {
@@ -649,11 +652,10 @@ __global__ void __launch_bounds__(kScanWarps * 32, kScanCtasPerSm) scan_i4_kerne
     --inflight;
 
     const uint8_t *sb = ring + stage * kStageBytes;
-    // ---- centroid dots of the 8 pages.  Pages are the MMA rows (rows 8-15 idle) and the query is the B operand,
-    // the same register pairs MMA #1 uses: cenT[hh][0..1] = sum_c code_mu[page x][c] q'[head 2t, 2t+1 (+8 hh)][c]
-    float cenT[NH][4];
-#pragma unroll
-    for (int hh = 0; hh < NH; ++hh) cenT[hh][0] = cenT[hh][1] = cenT[hh][2] = cenT[hh][3] = 0.f;
+    // ---- centroid dots of the 8 pages.  NH = 1: pages are the MMA rows (rows 8-15 idle) and the query is the B operand, the
+    // same register pairs MMA #1 uses: cen[0..1] = sum_c code_mu[page x][c] q'[head 2t, 2t+1][c].  NH = 2: the heads are the rows
+    float acen[2 * NH];  // log2-domain centroid term: packed, of this lane's (page, head); else of pages 2t, 2t + 1 for head x (+8)
+    float cen[4] = {0.f, 0.f, 0.f, 0.f};
     {
       const uint4 *mp = reinterpret_cast<const uint4 *>(sb + boff(x & (LOCKS_GROUP - 1)) + i4_off_mu(R) + t * 32);
       const uint4 m0 = mp[0], m1 = mp[1];
@@ -663,29 +665,32 @@ __global__ void __launch_bounds__(kScanWarps * 32, kScanCtasPerSm) scan_i4_kerne
         const uint32_t w = mw[s];
         const uint32_t b0 = f16x2_sub(and_or(w, kMB, kMagic), kSub128);              // code
         const uint32_t b1 = f16x2_fma(and_or(w >> 8, kMB, kMagic), kSixteen, kNeg16x);  // 16 * code
-#pragma unroll
-        for (int hh = 0; hh < NH; ++hh) mma_f16(cenT[hh], b0, 0u, b1, 0u, qb0[hh][s], qb2[hh][s]);
+        if (NH == 2) mma_f16(cen, qb0[0][s], qb0[NH - 1][s], qb2[0][s], qb2[NH - 1][s], b0, b1);
+        else mma_f16(cen, b0, 0u, b1, 0u, qb0[0][s], qb2[0][s]);
       }
     }
-    // scaled at the lane that holds them (page x, heads 2t, 2t+1), then moved to the lanes that finish the pages
-    float acen[2 * NH];  // log2-domain centroid term: packed, of this lane's (page, head); else of pages 2t, 2t+1 for head x (+8)
-    {
-      const float smu = __half2float(*reinterpret_cast<const __half *>(sb + boff(x & (LOCKS_GROUP - 1)) + i4_off_smu(R)));
+    if (NH == 2) {   // the heads were the MMA's rows: the lane that finishes a page holds its dots already
 #pragma unroll
-      for (int hh = 0; hh < NH; ++hh) {
-        const float v0 = smu * inv2[2 * hh] * cenT[hh][0], v1 = smu * inv2[2 * hh + 1] * cenT[hh][1];
-        if (PK) {   // lane (x, t) finishes page 2t + (x >> 2), head x & 3: held by lane (that page, (x & 3) >> 1)
-          const int src = (2 * t + (x >> 2)) * 4 + ((x & 3) >> 1);
-          const float a0 = __shfl_sync(0xffffffffu, v0, src), a1 = __shfl_sync(0xffffffffu, v1, src);
-          acen[0] = (x & 1) ? a1 : a0;
-          acen[1] = 0.f;
-        } else {    // lane (x, t) finishes pages 2t, 2t + 1 for head x (+8 hh): held by lanes (page, x >> 1)
-          const int srcA = (2 * t) * 4 + (x >> 1), srcB = srcA + 4;
-          const float a0 = __shfl_sync(0xffffffffu, v0, srcA), a1 = __shfl_sync(0xffffffffu, v1, srcA);
-          const float b0 = __shfl_sync(0xffffffffu, v0, srcB), b1 = __shfl_sync(0xffffffffu, v1, srcB);
-          acen[2 * hh] = (x & 1) ? a1 : a0;
-          acen[2 * hh + 1] = (x & 1) ? b1 : b0;
-        }
+      for (int e = 0; e < 2; ++e) {
+        const float smu = __half2float(*reinterpret_cast<const __half *>(sb + boff(2 * t + e) + i4_off_smu(R)));
+#pragma unroll
+        for (int hh = 0; hh < NH; ++hh) acen[2 * hh + e] = smu * inv_s[hh] * cen[2 * hh + e];
+      }
+    } else {
+      // scaled at the lane that holds them (page x, heads 2t, 2t+1), then moved to the lanes that finish the pages
+      const float smu = __half2float(*reinterpret_cast<const __half *>(sb + boff(x & (LOCKS_GROUP - 1)) + i4_off_smu(R)));
+      const float v0 = smu * inv2[0] * cen[0], v1 = smu * inv2[1] * cen[1];
+      if (PK) {   // lane (x, t) finishes page 2t + (x >> 2), head x & 3: held by lane (that page, (x & 3) >> 1)
+        const int src = (2 * t + (x >> 2)) * 4 + ((x & 3) >> 1);
+        const float a0 = __shfl_sync(0xffffffffu, v0, src), a1 = __shfl_sync(0xffffffffu, v1, src);
+        acen[0] = (x & 1) ? a1 : a0;
+        acen[1] = 0.f;
+      } else {    // lane (x, t) finishes pages 2t, 2t + 1 for head x: held by lanes (page, x >> 1)
+        const int srcA = (2 * t) * 4 + (x >> 1), srcB = srcA + 4;
+        const float a0 = __shfl_sync(0xffffffffu, v0, srcA), a1 = __shfl_sync(0xffffffffu, v1, srcA);
+        const float b0 = __shfl_sync(0xffffffffu, v0, srcB), b1 = __shfl_sync(0xffffffffu, v1, srcB);
+        acen[0] = (x & 1) ? a1 : a0;
+        acen[1] = (x & 1) ? b1 : b0;
       }
     }
     float res[2 * NH];
@@ -799,6 +804,57 @@ __global__ void __launch_bounds__(kScanWarps * 32, kScanCtasPerSm) scan_i4_kerne
           if (t == 2 * k4 + hrow) res[0] = m + fast_lg2(e) + acen[0];
         }
       }
+    } else if constexpr (NH == 2) {
+      // ---- more than 8 heads: the 16 heads are the rows and the codes the other operand, page by page, so that the projection
+      // comes out as the operand of the logits MMA (no transpose) and no head column is moved between lanes
+#pragma unroll
+      for (int pg = 0; pg < LOCKS_GROUP; ++pg) {
+        const uint8_t *pb = sb + boff(pg);
+        const uint4 w4 = (R == 8 || x < R) ? *reinterpret_cast<const uint4 *>(pb + lane * 16) : make_uint4(0u, 0u, 0u, 0u);
+        const uint32_t wd[4] = {w4.x, w4.y, w4.z, w4.w};
+        float c[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const uint32_t u = wd[j], u8 = u >> 8;
+          if (j == 0) mma_f16_z(c, qb0[0][0], qb0[1][0], qb2[0][0], qb2[1][0], u & kM0, u & kM1);
+          else mma_f16(c, qb0[0][2 * j], qb0[1][2 * j], qb2[0][2 * j], qb2[1][2 * j], u & kM0, u & kM1);
+          mma_f16(c, qb0[0][2 * j + 1], qb0[1][2 * j + 1], qb2[0][2 * j + 1], qb2[1][2 * j + 1], u8 & kM0, u8 & kM1);
+        }
+        // projection of ranks 2t, 2t + 1 for heads x, x + 8: undo 2^-24, remove the +8 offset, apply the column scale
+        const float2 sv = (t < R / 2) ? h2f2(*reinterpret_cast<const uint32_t *>(pb + i4_off_sv(R) + 4 * t)) : make_float2(0.f, 0.f);
+        uint32_t hi[2], lo[2];
+#pragma unroll
+        for (int hh = 0; hh < 2; ++hh) {
+          const float p0 = fmaf(c[2 * hh], 16777216.f, -ksum[hh]) * sv.x, p1 = fmaf(c[2 * hh + 1], 16777216.f, -ksum[hh]) * sv.y;
+          hi[hh] = pack_f16(p0, p1);
+          const float2 hf = h2f2(hi[hh]);
+          lo[hh] = pack_f16(p0 - hf.x, p1 - hf.y);
+        }
+        const uint32_t cw = (t < R / 2) ? *reinterpret_cast<const uint32_t *>(pb + i4_off_coef(R) + (x * (R / 2) + t) * 4) : 0x80808080u;
+        const uint32_t b0 = f16x2_sub(__byte_perm(cw, 0x64646464u, 0x4140), kSub128);
+        const uint32_t b1 = f16x2_sub(__byte_perm(cw, 0x64646464u, 0x4342), kSub128);
+        float ca[4], cb[4];
+        mma_f16_z(ca, hi[0], hi[1], lo[0], lo[1], b0, b0);
+        mma_f16_z(cb, hi[0], hi[1], lo[0], lo[1], b1, b1);
+        const uint2 scw = *reinterpret_cast<const uint2 *>(pb + i4_off_sc(R) + 8 * t);
+        const float2 s01 = h2f2(scw.x), s89 = h2f2(scw.y);
+#pragma unroll
+        for (int hh = 0; hh < 2; ++hh) {
+          const float iv = inv_s[hh];   // logits (log2 domain) are y * iv, iv > 0
+          const float y0 = ca[2 * hh] * s01.x, y1 = ca[2 * hh + 1] * s01.y;
+          const float y2 = cb[2 * hh] * s89.x, y3 = cb[2 * hh + 1] * s89.y;
+          float my = fmaxf(fmaxf(y0, y1), fmaxf(y2, y3));
+          my = fmaxf(my, __shfl_xor_sync(0xffffffffu, my, 1));
+          my = fmaxf(my, __shfl_xor_sync(0xffffffffu, my, 2));
+          const float m = my * iv;
+          float e = fast_ex2(fmaf(y0, iv, -m)) + fast_ex2(fmaf(y1, iv, -m)) + fast_ex2(fmaf(y2, iv, -m)) +
+                    fast_ex2(fmaf(y3, iv, -m));
+          e += __shfl_xor_sync(0xffffffffu, e, 1);
+          e += __shfl_xor_sync(0xffffffffu, e, 2);
+          const float v = m + fast_lg2(e);
+          if (t == (pg >> 1)) res[2 * hh + (pg & 1)] = v;
+        }
+      }
     } else {
 #pragma unroll
     for (int pp = 0; pp < LOCKS_GROUP / 2; ++pp) {
@@ -808,24 +864,21 @@ __global__ void __launch_bounds__(kScanWarps * 32, kScanCtasPerSm) scan_i4_kerne
       const uint4 wa4 = (R == 8 || x < R) ? *reinterpret_cast<const uint4 *>(pbA + lane * 16) : make_uint4(0u, 0u, 0u, 0u);
       const uint4 wb4 = (R == 8 || x < R) ? *reinterpret_cast<const uint4 *>(pbB + lane * 16) : make_uint4(0u, 0u, 0u, 0u);
       const uint32_t wa[4] = {wa4.x, wa4.y, wa4.z, wa4.w}, wb[4] = {wb4.x, wb4.y, wb4.z, wb4.w};
-      float c1[NH][4];
+      float c1[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const uint32_t ua = wa[j], ub = wb[j], ua8 = ua >> 8, ub8 = ub >> 8;
-#pragma unroll
-        for (int hh = 0; hh < NH; ++hh) {
-          if (j == 0) mma_f16_z(c1[hh], ua & kM0, ub & kM0, ua & kM1, ub & kM1, qb0[hh][0], qb2[hh][0]);
-          else mma_f16(c1[hh], ua & kM0, ub & kM0, ua & kM1, ub & kM1, qb0[hh][2 * j], qb2[hh][2 * j]);
-          mma_f16(c1[hh], ua8 & kM0, ub8 & kM0, ua8 & kM1, ub8 & kM1, qb0[hh][2 * j + 1], qb2[hh][2 * j + 1]);
-        }
+        if (j == 0) mma_f16_z(c1, ua & kM0, ub & kM0, ua & kM1, ub & kM1, qb0[0][0], qb2[0][0]);
+        else mma_f16(c1, ua & kM0, ub & kM0, ua & kM1, ub & kM1, qb0[0][2 * j], qb2[0][2 * j]);
+        mma_f16(c1, ua8 & kM0, ub8 & kM0, ua8 & kM1, ub8 & kM1, qb0[0][2 * j + 1], qb2[0][2 * j + 1]);
       }
       if (PK) {
         // lanes t < 2 carry page A (columns 0-3), lanes t >= 2 page B (columns 4-7)
         const bool pa = t < 2;
         const uint8_t *pbs = pa ? pbA : pbB;
         const float sv = (R == 8 || x < R) ? __half2float(*reinterpret_cast<const __half *>(pbs + i4_off_sv(R) + 2 * x)) : 0.f;
-        const float p0 = fmaf(pa ? c1[0][0] : c1[0][2], 16777216.f, -ksum[0]) * sv;
-        const float p1 = fmaf(pa ? c1[0][1] : c1[0][3], 16777216.f, -ksum[1]) * sv;
+        const float p0 = fmaf(pa ? c1[0] : c1[2], 16777216.f, -ksum[0]) * sv;
+        const float p1 = fmaf(pa ? c1[1] : c1[3], 16777216.f, -ksum[1]) * sv;
         const uint32_t hi = pack_f16(p0, p1);
         const float2 hf = h2f2(hi);
         const uint32_t lo = pack_f16(p0 - hf.x, p1 - hf.y);
@@ -866,42 +919,33 @@ __global__ void __launch_bounds__(kScanWarps * 32, kScanCtasPerSm) scan_i4_kerne
         const uint8_t *pb = pq ? pbB : pbA;
         // projection of rank x for heads 2t, 2t+1: undo 2^-24, remove the +8 offset, apply the column scale
         const float sv = (R == 8 || x < R) ? __half2float(*reinterpret_cast<const __half *>(pb + i4_off_sv(R) + 2 * x)) : 0.f;
-        uint32_t hiT[NH], loT[NH];
-#pragma unroll
-        for (int hh = 0; hh < NH; ++hh) {
-          const float p0 = fmaf(c1[hh][2 * pq], 16777216.f, -ksum[2 * hh]) * sv;
-          const float p1 = fmaf(c1[hh][2 * pq + 1], 16777216.f, -ksum[2 * hh + 1]) * sv;
-          const uint32_t hi = pack_f16(p0, p1);
-          const float2 hf = h2f2(hi);
-          const uint32_t lo = pack_f16(p0 - hf.x, p1 - hf.y);
-          hiT[hh] = movm_trans(hi);   // -> lane (x = head, t): ranks 2t, 2t+1
-          loT[hh] = movm_trans(lo);
-        }
+        const float p0 = fmaf(c1[2 * pq], 16777216.f, -ksum[0]) * sv;
+        const float p1 = fmaf(c1[2 * pq + 1], 16777216.f, -ksum[1]) * sv;
+        const uint32_t hi = pack_f16(p0, p1);
+        const float2 hf = h2f2(hi);
+        const uint32_t lo = pack_f16(p0 - hf.x, p1 - hf.y);
+        const uint32_t hiT = movm_trans(hi), loT = movm_trans(lo);   // -> lane (x = head, t): ranks 2t, 2t+1
         // ---- MMA #2: rows = heads, k = ranks (hi | lo), cols = tokens
         const uint32_t cw = (t < R / 2) ? *reinterpret_cast<const uint32_t *>(pb + i4_off_coef(R) + (x * (R / 2) + t) * 4) : 0x80808080u;
         const uint32_t b0 = f16x2_sub(__byte_perm(cw, 0x64646464u, 0x4140), kSub128);
         const uint32_t b1 = f16x2_sub(__byte_perm(cw, 0x64646464u, 0x4342), kSub128);
         float ca[4], cb[4];
-        mma_f16_z(ca, hiT[0], NH == 2 ? hiT[NH - 1] : 0u, loT[0], NH == 2 ? loT[NH - 1] : 0u, b0, b0);
-        mma_f16_z(cb, hiT[0], NH == 2 ? hiT[NH - 1] : 0u, loT[0], NH == 2 ? loT[NH - 1] : 0u, b1, b1);
+        mma_f16_z(ca, hiT, 0u, loT, 0u, b0, b0);
+        mma_f16_z(cb, hiT, 0u, loT, 0u, b1, b1);
         const uint2 scw = *reinterpret_cast<const uint2 *>(pb + i4_off_sc(R) + 8 * t);
         const float2 s01 = h2f2(scw.x), s89 = h2f2(scw.y);
-#pragma unroll
-        for (int hh = 0; hh < NH; ++hh) {
-          const float iv = inv_s[hh];   // logits (log2 domain) are y * iv, iv > 0
-          const float y0 = ca[2 * hh] * s01.x, y1 = ca[2 * hh + 1] * s01.y;
-          const float y2 = cb[2 * hh] * s89.x, y3 = cb[2 * hh + 1] * s89.y;
-          float my = fmaxf(fmaxf(y0, y1), fmaxf(y2, y3));
-          my = fmaxf(my, __shfl_xor_sync(0xffffffffu, my, 1));
-          my = fmaxf(my, __shfl_xor_sync(0xffffffffu, my, 2));
-          const float m = my * iv;
-          float e = fast_ex2(fmaf(y0, iv, -m)) + fast_ex2(fmaf(y1, iv, -m)) + fast_ex2(fmaf(y2, iv, -m)) +
-                    fast_ex2(fmaf(y3, iv, -m));
-          e += __shfl_xor_sync(0xffffffffu, e, 1);
-          e += __shfl_xor_sync(0xffffffffu, e, 2);
-          const float v = m + fast_lg2(e);
-          if (t == (pg >> 1)) res[2 * hh + (pg & 1)] = v;
-        }
+        const float iv = inv_s[0];   // logits (log2 domain) are y * iv, iv > 0
+        const float y0 = ca[0] * s01.x, y1 = ca[1] * s01.y, y2 = cb[0] * s89.x, y3 = cb[1] * s89.y;
+        float my = fmaxf(fmaxf(y0, y1), fmaxf(y2, y3));
+        my = fmaxf(my, __shfl_xor_sync(0xffffffffu, my, 1));
+        my = fmaxf(my, __shfl_xor_sync(0xffffffffu, my, 2));
+        const float m = my * iv;
+        float e = fast_ex2(fmaf(y0, iv, -m)) + fast_ex2(fmaf(y1, iv, -m)) + fast_ex2(fmaf(y2, iv, -m)) +
+                  fast_ex2(fmaf(y3, iv, -m));
+        e += __shfl_xor_sync(0xffffffffu, e, 1);
+        e += __shfl_xor_sync(0xffffffffu, e, 2);
+        const float v = m + fast_lg2(e);
+        if (t == (pg >> 1)) res[pg & 1] = v;
       }
     }
       }
