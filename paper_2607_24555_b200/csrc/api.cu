@@ -155,7 +155,7 @@ int locks_create(const locks_config *cfg, void *workspace, size_t ws_bytes, lock
   if (!c) return LOCKS_ERR_INVALID_ARG;
   c->cfg = *cfg;
   c->prof_ev = nullptr; c->prof_cap = c->prof_n = 0;
-  c->att_cluster_max = -1;
+  c->att_clusters[0] = -1;
   for (int i = 0; i < LOCKS_HOST_GRAPHS; ++i) c->hg[i] = locks_host_graph{};
   c->hg_next = 0;
   c->part_slots = L.max_groups;

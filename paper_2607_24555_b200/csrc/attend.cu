@@ -644,32 +644,34 @@ int locks_launch_attend(locks_ctx *c, const void *q, const locks_kv *kv, int bat
   // Preferred: the splits of a problem as one thread-block cluster (2, 4, 8 or 16 CTAs) that merges through
   // distributed shared memory, as long as a CTA then has at most 8 tiles per warp to stream.
   p.cluster = 0;
-  if (c->att_cluster_max < 0) {   // largest cluster of this kernel the device can place (probed once)
-    c->att_cluster_max = 0;
+  if (c->att_clusters[0] < 0) {   // clusters of 2, 4, 8, 16 CTAs of this kernel that fit the device at once (probed once)
     cudaFuncSetAttribute(attend_bf16_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmem);
     cudaFuncSetAttribute(attend_bf16_kernel<1, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    for (int cs = 16; cs >= 2 && c->att_cluster_max == 0; cs /= 2) {
+    for (int i = 0; i < 4; ++i) {
       cudaLaunchConfig_t lc = {};
-      lc.gridDim = dim3(cs, 1, 1);
+      lc.gridDim = dim3(2 << i, 1, 1);
       lc.blockDim = dim3(LOCKS_ATT_WARPS * 32);
       lc.dynamicSmemBytes = kAttSmem;
       cudaLaunchAttribute at[1];
       at[0].id = cudaLaunchAttributeClusterDimension;
-      at[0].val.clusterDim.x = cs; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+      at[0].val.clusterDim.x = 2 << i; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
       lc.attrs = at;
       lc.numAttrs = 1;
       int nclusters = 0;
-      if (cudaOccupancyMaxActiveClusters(&nclusters, attend_bf16_kernel<1, true>, &lc) == cudaSuccess && nclusters > 0)
-        c->att_cluster_max = cs;
+      if (cudaOccupancyMaxActiveClusters(&nclusters, attend_bf16_kernel<1, true>, &lc) != cudaSuccess) nclusters = 0;
+      c->att_clusters[i] = nclusters;
     }
     (void)cudaGetLastError();   // a refused probe is not an error of this call
   }
-  if (bf && splits >= 2 && c->att_cluster_max >= 2) {
-    int cs = 2;
-    while (cs * 2 <= splits && cs * 2 <= c->att_cluster_max) cs *= 2;
-    if ((ntiles + cs - 1) / cs <= 8 * LOCKS_ATT_WARPS) {
+  if (bf && splits >= 2) {
+    // The largest size of which every problem's cluster is resident in one wave.  A cluster's CTAs have to share a GPC, so
+    // fewer large clusters fit than CTAs do: 32 problems as clusters of 16 (512 CTAs in 592 slots) take two waves, 36.7 us a
+    // step (4 x 8K tokens, budget 128 pages) against 30.8 as clusters of 8; 24 problems fit, 29.2 against 30.0.
+    int i = 3;
+    while (i >= 0 && ((2 << i) > splits || c->att_clusters[i] < batch * p.Hkv)) --i;
+    if (i >= 0 && (ntiles + (2 << i) - 1) / (2 << i) <= 8 * LOCKS_ATT_WARPS) {
       p.cluster = 1;
-      p.splits = cs;
+      p.splits = 2 << i;
       p.fused_merge = 1;   // no merge launch follows
     }
   }

@@ -90,7 +90,7 @@ struct locks_ctx {
   int last_launches;
   locks_host_graph hg[LOCKS_HOST_GRAPHS];
   int hg_next;
-  int att_cluster_max;     // largest thread-block cluster the attention kernel may use (-1: not probed yet)
+  int att_clusters[4];     // clusters of 2, 4, 8, 16 CTAs of the attention kernel that are resident at once (-1: not probed yet)
   // optional per-stage timing of eager decode steps (see locks_profile_begin)
   cudaEvent_t *prof_ev;    // [prof_cap][LOCKS_PROF_MARKS]
   int prof_cap, prof_n;
