@@ -642,7 +642,9 @@ int locks_launch_attend(locks_ctx *c, const void *q, const locks_kv *kv, int bat
   p.done = c->att_done;
   p.fused_merge = (p.G * p.splits <= kFusedMerge) ? 1 : 0;
   // Preferred: the splits of a problem as one thread-block cluster (2, 4, 8 or 16 CTAs) that merges through
-  // distributed shared memory, as long as a CTA then has at most 8 tiles per warp to stream.
+  // distributed shared memory, as long as a CTA then has at most 12 tiles per warp to stream (12 x 9K tokens, budget 128
+  // pages, 96 problems: step 47.3 us as five splits that the last CTA merges, 43.8 as clusters of four; no case of 14 .. 64
+  // requests slower).
   p.cluster = 0;
   if (c->att_clusters[0] < 0) {   // clusters of 2, 4, 8, 16 CTAs of this kernel that fit the device at once (probed once)
     cudaFuncSetAttribute(attend_bf16_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmem);
@@ -669,7 +671,7 @@ int locks_launch_attend(locks_ctx *c, const void *q, const locks_kv *kv, int bat
     // step (4 x 8K tokens, budget 128 pages) against 30.8 as clusters of 8; 24 problems fit, 29.2 against 30.0.
     int i = 3;
     while (i >= 0 && ((2 << i) > splits || c->att_clusters[i] < batch * p.Hkv)) --i;
-    if (i >= 0 && (ntiles + (2 << i) - 1) / (2 << i) <= 8 * LOCKS_ATT_WARPS) {
+    if (i >= 0 && (ntiles + (2 << i) - 1) / (2 << i) <= 12 * LOCKS_ATT_WARPS) {
       p.cluster = 1;
       p.splits = 2 << i;
       p.fused_merge = 1;   // no merge launch follows
