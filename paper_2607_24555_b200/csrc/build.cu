@@ -20,6 +20,10 @@
 // Bound by instruction issue, fetch and latency, not by bytes (an eigenproblem per 4 KB page).  131 008 page-heads: 1348 us
 // with the pair that straddles two lanes rotated by both and all formats in one kernel (6 960 warp instructions each), 1281
 // us with every pair rotated once and build_i4_kernel's phases (5 370), 1095 us with the body of a sweep kept to two steps.
+// Smaller builds are one or two waves long and bound by the latency of a group (8 pages of a KV head) and by how the groups
+// lie on the SMs; see build_i4_kernel: 16 .. 384 groups 99 -> 79 .. 93 us, 1024: 197 -> 131, 4096 (a prompt chunk of 2048
+// tokens in 32 layers): 385 -> 345, and chunks of 9 .. 40 pages in 32 layers, 130 .. 205 us before, 76 .. 131.
+#include <algorithm>
 #include <type_traits>
 #include "build_common.cuh"
 
@@ -57,10 +61,11 @@ __device__ __forceinline__ void plane_rotation(float a, float b, float g, float 
 // Result: the columns ranked by norm (descending, ties to the lower position), the 16 eigenvalues to lam_s[item][mode],
 // unit eigenvectors of the leading min(r, 8) modes to us as pairs (u, u): BY_MODE [item][mode][token], else
 // [item][token][mode] (r > 8: all 16, plain entries, [token][16]).
-template <bool BY_MODE>
-__device__ __forceinline__ void jacobi_phase(const float *mat, float *us, float *lam_s, uint32_t live, int r, int lane) {
-  constexpr int CPL = 4, LPI = LOCKS_B / CPL;
-  const int item = lane / LPI, j = lane % LPI;
+template <bool BY_MODE, int CPL, typename Vote>
+__device__ __forceinline__ void jacobi_phase(const float *mat, float *us, float *lam_s, uint32_t live, int r, int lane, int item0,
+                                             Vote vote) {
+  constexpr int LPI = LOCKS_B / CPL;
+  const int item = item0 + lane / LPI, j = lane % LPI;
   const bool item_live = (live >> item) & 1u;   // lanes of an absent item compute on zeros
   float2 w[CPL][8];
   {
@@ -170,13 +175,13 @@ __device__ __forceinline__ void jacobi_phase(const float *mat, float *us, float 
 #pragma unroll 1
     for (int st2 = 0; st2 < 8; ++st2) {   // (a body of this size: twice unrolled, a quarter of the warps wait for instructions)
       rotate(even, w[1], w[0], n[1], n[0], true);
-      rotate(even, w[3], w[2], n[3], n[2], true);
+      if constexpr (CPL == 4) rotate(even, w[3], w[2], n[3], n[2], true);
       fetch(w[0], n[0], up);     // a pair passes to the one before it: w[2] to the lane's first, w[0] to the lane below
-      rotate(odd, w[1], w[2], n[1], n[2], true);
-      rotate(odd, w[3], w[0], n[3], n[0], j != LPI - 1);
+      if constexpr (CPL == 4) rotate(odd, w[1], w[2], n[1], n[2], true);
+      rotate(odd, w[CPL - 1], w[0], n[CPL - 1], n[0], j != LPI - 1);
       fetch(w[0], n[0], down);   // ... and then to the one after it: w[2] to the lane's second, w[0] to the lane above
     }
-    if (!__any_sync(0xffffffffu, bad != 0)) break;
+    if (!vote(bad != 0)) break;
   }
   norms();
   int rank[CPL];
@@ -247,24 +252,36 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b) {
 // pairs; M leaves the MMA accumulators through one transposed array instead of two; all modes' basis vectors are formed
 // before any is quantised, so that their scales (a division, an fp16 rounding and a reciprocal each) are worked out by a
 // lane per mode, once; codes go straight to global memory.
-constexpr int kBuildI4SmemPerWarp = kBuildScratch + kBuildMat + 64 + kBuildItems * LOCKS_B * 4;
-__global__ void __launch_bounds__(kBuildWarps * 32, kBuildCtasPerSm) build_i4_kernel(BuildParams p) {
-  extern __shared__ __align__(16) uint8_t smem_raw[];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int h = blockIdx.y, r = p.r;
-  const int it_block = item_block(p, warp, lane);   // the warp's items: lane s < 8 works out item s
-  const uint32_t live = __ballot_sync(0xffffffffu, it_block >= 0);
-  if (!live) return;
-  const int layer = blockIdx.z / p.batch;
-  const __nv_bfloat16 *kbase = reinterpret_cast<const __nv_bfloat16 *>(p.k_layers ? p.k_layers[layer] : p.k);
-  uint8_t *sbase = p.summ_layers ? reinterpret_cast<uint8_t *>(p.summ_layers[layer]) : p.summ;
-  uint8_t *scratch = smem_raw + warp * kBuildI4SmemPerWarp;          // D half-tiles, then Y
-  float *mat = reinterpret_cast<float *>(scratch + kBuildScratch);   // [8][16][16] Gram; then [8][8][16] pairs (u, u) of U_r by mode
-  float *kn_s = mat + kBuildItems * kMat;                            // [8] squared norm of the page's keys
-  float *lam_s = kn_s + 16;                                          // [8][16] eigenvalues, descending
+//
+// A group is 8 pages of one (layer, request, KV head); W warps of a CTA work on it.  One keeps every lane busy all the time.
+// Of two, each takes 4 of the items in phases 1 and 3, and 8 lanes hold a matrix in phase 2: a group is done in 79 us on an
+// idle chip where one warp takes 99.  Whether a group's sweeps go on is one decision of all its warps, so that the bytes are
+// the same either way.
+constexpr int kI4Warps = 2, kI4CtasPerSm = 8, kI4Waves = 16;
+constexpr int kI4Group = kBuildMat + 64 + kBuildItems * LOCKS_B * 4;   // bytes: matrices, key norms, eigenvalues
+constexpr int kI4Smem = kI4Warps * (kBuildScratch + kI4Group);
+constexpr int kI4SmemCount = kI4Smem + 64;   // + the number of groups, a group's blocks and KV head
+
+__device__ __forceinline__ int build_pages(const BuildParams &p, int b, int &p0) {   // pages of request b to build, from p0 on
+  const int complete = p.seq_lens[b] / LOCKS_B;
+  p0 = p.page_begin ? p.page_begin[b] : 0;
+  const int p1 = min(min(p.page_end ? p.page_end[b] : complete, complete), p.Pmax);
+  return (int)max((int64_t)0, min((int64_t)p1 - p0, (int64_t)p.Pmax + LOCKS_B));
+}
+
+// kbase, sbase: the layer's keys and summaries at the group's KV head
+template <int W>
+__device__ __forceinline__ void build_i4_group(const BuildParams &p, uint8_t *smem_raw, int tid, int it_block, uint32_t live,
+                                               const __nv_bfloat16 *kbase, uint8_t *sbase) {
+  constexpr int kItems = kBuildItems / W;   // items of this warp
+  const int lane = tid & 31, warp = tid >> 5, wg = warp % W, r = p.r;
+  uint8_t *scratch = smem_raw + warp * kBuildScratch;   // D half-tiles, then Y
+  float *mat = reinterpret_cast<float *>(smem_raw + kI4Warps * kBuildScratch + warp / W * kI4Group);   // [8][16][16] Gram; then [8][8][16] pairs (u, u) of U_r by mode
+  float *kn_s = mat + kBuildItems * kMat;   // [8] squared norm of the page's keys
+  float *lam_s = kn_s + 16;                 // [8][16] eigenvalues, descending
   // deviations of item s: v[i][e] = key i minus the centroid, dims 4 lane + 2 e, + 1; knorm2: this lane's share
   auto load_centred = [&](int s, float2 (&v)[LOCKS_B][2], float2 (&mu)[2], bool want_norm, float &knorm2) {
-    const __nv_bfloat16 *K = kbase + (int64_t)__shfl_sync(0xffffffffu, it_block, s) * p.sb + (int64_t)h * p.sh + 4 * lane;
+    const __nv_bfloat16 *K = kbase + (int64_t)__shfl_sync(0xffffffffu, it_block, s) * p.sb + 4 * lane;
 #pragma unroll
     for (int i = 0; i < LOCKS_B; ++i) {
       const uint2 w = *reinterpret_cast<const uint2 *>(K + (int64_t)i * p.st);
@@ -291,7 +308,7 @@ __global__ void __launch_bounds__(kBuildWarps * 32, kBuildCtasPerSm) build_i4_ke
 
   // ---- 1. Gram matrices (see build_kernel)
 #pragma unroll 1
-  for (int s = 0; s < kBuildItems; ++s) {
+  for (int s = wg * kItems; s < (wg + 1) * kItems; ++s) {
     if (!((live >> s) & 1u)) continue;
     uint32_t hl[LOCKS_B][4];   // h01, h23, l01, l23 of this lane's 4 dims, per key
     {
@@ -361,11 +378,22 @@ __global__ void __launch_bounds__(kBuildWarps * 32, kBuildCtasPerSm) build_i4_ke
   }
 
   // ---- 2. eigenvectors and eigenvalues of all the warp's items at once
-  jacobi_phase<true>(mat, mat, lam_s, live, r, lane);
+  if constexpr (W == 1) {
+    jacobi_phase<true, 4>(mat, mat, lam_s, live, r, lane, 0, [](bool bad) { return __any_sync(0xffffffffu, bad) != 0; });
+  } else {
+    // the two warps' votes meet at a barrier of theirs
+    auto vote = [](bool bad) {
+      int any;
+      asm volatile("{\n .reg .pred a, b;\n setp.ne.s32 a, %1, 0;\n bar.red.or.pred b, 1, 64, a;\n selp.s32 %0, 1, 0, b;\n}\n"
+                   : "=r"(any) : "r"((int)bad) : "memory");
+      return any != 0;
+    };
+    jacobi_phase<true, 2>(mat, mat, lam_s, live, r, lane, wg * 4, vote);
+  }
 
   // ---- 3. basis, coefficients, centroid
 #pragma unroll 1
-  for (int s = 0; s < kBuildItems; ++s) {
+  for (int s = wg * kItems; s < (wg + 1) * kItems; ++s) {
     if (!((live >> s) & 1u)) continue;
     const float *U = mat + s * kMat, *lam = lam_s + s * LOCKS_B;   // U[mode][token] as pairs
     // lane l < r: mode l
@@ -394,7 +422,7 @@ __global__ void __launch_bounds__(kBuildWarps * 32, kBuildCtasPerSm) build_i4_ke
         }
       }
     }
-    uint8_t *gout = sbase + ((int64_t)__shfl_sync(0xffffffffu, it_block, s) * p.Hkv + h) * p.S;
+    uint8_t *gout = sbase + (int64_t)__shfl_sync(0xffffffffu, it_block, s) * p.Hkv * p.S;
     // sign: the entry of largest magnitude (lowest dim on ties) is positive.  Magnitudes order like their bit patterns; the
     // lowest lane that holds the maximum owns the lowest such dim.
     float best_mode = 0.f;         // lane l: largest magnitude of mode l
@@ -469,7 +497,94 @@ __global__ void __launch_bounds__(kBuildWarps * 32, kBuildCtasPerSm) build_i4_ke
       if (lane == 0) *reinterpret_cast<__half *>(gout + i4_off_smu(r)) = sh;
       if (lane < 16 && i4_off_smu(r) + 2 + lane < p.S) gout[i4_off_smu(r) + 2 + lane] = 0;   // bytes between the payload and the stride
     }
+  }}
+
+// The groups by the table's rows: of 16 pages of a row, 8 a warp.  For tables that are about full.
+__global__ void __launch_bounds__(kI4Warps * 32, kI4CtasPerSm) build_i4_table_kernel(BuildParams p) {
+  extern __shared__ __align__(16) uint8_t smem_raw[];
+  const int lane = threadIdx.x & 31, h = blockIdx.y, layer = blockIdx.z / p.batch;
+  const int it_block = item_block(p, threadIdx.x >> 5, lane);   // lane s < 8: item s
+  const uint32_t live = __ballot_sync(0xffffffffu, it_block >= 0);
+  if (!live) return;
+  build_i4_group<1>(p, smem_raw, threadIdx.x, it_block, live,
+                    reinterpret_cast<const __nv_bfloat16 *>(p.k_layers ? p.k_layers[layer] : p.k) + (int64_t)h * p.sh,
+                    (p.summ_layers ? reinterpret_cast<uint8_t *>(p.summ_layers[layer]) : p.summ) + (int64_t)h * p.S);
+}
+
+// The groups that there are, counted from the lengths and page ranges and dealt to the CTAs without gaps.
+template <int W>
+__device__ __forceinline__ void build_i4_groups(const BuildParams &p, uint8_t *smem_raw, const volatile int *count, int layers) {
+#pragma unroll 1
+  for (int round = 0;; ++round) {
+    int tid = threadIdx.x;
+    asm volatile("" : "+r"(tid));   // nothing that follows from it is worth a register across groups
+    const int lane = tid & 31, warp = tid >> 5;
+    int *blk_s = reinterpret_cast<int *>(smem_raw + kI4Warps * (kBuildScratch + kI4Group)) + 4;   // W > 1: blocks of the 8 items, KV head
+    const int groups = *count;   // of a layer
+    const int64_t g = ((int64_t)round * gridDim.x + blockIdx.x) * (kI4Warps / W) + warp / W;
+    const int layer = (int)(g / groups);
+    if (layer >= layers) break;
+    int it_block = -1, h = 0;   // lane s < 8: item s
+    if (W == 1 || warp == 0) {
+      int n = (int)(g - (int64_t)layer * groups);   // the group's place in its layer: by request, KV head, page
+      for (int b0 = 0; b0 < p.batch; b0 += 32) {
+        int p0 = 0;
+        const int have = b0 + lane < p.batch ? build_pages(p, b0 + lane, p0) : 0, mine = (have + kBuildItems - 1) / kBuildItems * p.Hkv;
+        int upto = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int v = __shfl_up_sync(0xffffffffu, upto, o);
+          if (lane >= o) upto += v;
+        }
+        const uint32_t past = __ballot_sync(0xffffffffu, n < upto);
+        if (past) {
+          const int src = __ffs(past) - 1;
+          const int end = __shfl_sync(0xffffffffu, have, src), per_head = (end + kBuildItems - 1) / kBuildItems;
+          n -= __shfl_sync(0xffffffffu, upto - mine, src);
+          h = n / per_head;
+          const int first = (n - h * per_head) * kBuildItems + lane, page = __shfl_sync(0xffffffffu, p0, src) + first;
+          if (lane < kBuildItems && first < end && page >= 0) {
+            it_block = p.block_table[(int64_t)(b0 + src) * p.Pmax + page];
+            if (it_block < 0 || it_block >= p.num_blocks) { it_block = -1; set_status(p.status, LOCKS_ERR_BAD_BLOCK); }
+          }
+          break;
+        }
+        n -= __shfl_sync(0xffffffffu, upto, 31);
+      }
+    }
+    if (W > 1) {   // one warp looks the items up: the warps of a group agree on them, whatever happens to the table meanwhile
+      if (warp == 0 && lane < kBuildItems) blk_s[lane] = it_block;
+      if (warp == 0 && lane == 0) blk_s[kBuildItems] = h;
+      __syncthreads();
+      it_block = lane < kBuildItems ? blk_s[lane] : -1;
+      h = blk_s[kBuildItems];
+    }
+    const uint32_t live = __ballot_sync(0xffffffffu, it_block >= 0);
+    if (live)
+      build_i4_group<W>(p, smem_raw, tid, it_block, live,
+                        reinterpret_cast<const __nv_bfloat16 *>(p.k_layers ? p.k_layers[layer] : p.k) + (int64_t)h * p.sh,
+                        (p.summ_layers ? reinterpret_cast<uint8_t *>(p.summ_layers[layer]) : p.summ) + (int64_t)h * p.S);
+    if (W > 1) __syncthreads();   // the group's shared memory is free
+    else __syncwarp();
   }
+}
+
+__global__ void __launch_bounds__(kI4Warps * 32, kI4CtasPerSm) build_i4_kernel(BuildParams p, int layers, int sms) {
+  extern __shared__ __align__(16) uint8_t smem_raw[];
+  int *count = reinterpret_cast<int *>(smem_raw + kI4Warps * (kBuildScratch + kI4Group));
+  if (threadIdx.x < 32) {
+    int n = 0, p0;
+    for (int b = threadIdx.x; b < p.batch; b += 32) n += (build_pages(p, b, p0) + kBuildItems - 1) / kBuildItems * p.Hkv;
+    n = __reduce_add_sync(0xffffffffu, n);
+    if (threadIdx.x == 0) *count = n;
+  }
+  __syncthreads();
+  const int groups = *count;
+  if (groups == 0) return;
+  // Two warps a group up to three waves of single ones: us with one / two at 128 groups 104 / 80, 1024: 168 / 131, 2048: 216 /
+  // 201, 3072: 294 / 284, 4096: 348 / 349, 16 376: 1126 / 1153.
+  if ((int64_t)groups * layers <= (int64_t)22 * sms) build_i4_groups<2>(p, smem_raw, count, layers);
+  else build_i4_groups<1>(p, smem_raw, count, layers);
 }
 
 template <typename T, int FMT>
@@ -606,7 +721,7 @@ __global__ void __launch_bounds__(kBuildWarps * 32, kBuildCtasPerSm) build_kerne
   }
 
   // ---- 2. eigenvectors and eigenvalues of all the warp's items at once
-  jacobi_phase<false>(mat, mat, lam_s, live, r, lane);
+  jacobi_phase<false, 4>(mat, mat, lam_s, live, r, lane, 0, [](bool bad) { return __any_sync(0xffffffffu, bad) != 0; });
 
   // ---- 3. per item: modes, basis, coefficients, quantisation
   uint8_t *blob = scratch;
@@ -1069,7 +1184,18 @@ int locks_launch_build(locks_ctx *c, const locks_kv *kv, int batch, const int32_
   } while (0)
   switch (c->cfg.summary_fmt) {
     case LOCKS_FMT_I4:
-      if (bf) build_i4_kernel<<<grid, kBuildWarps * 32, kBuildWarps * kBuildI4SmemPerWarp, st>>>(p);
+      if (bf) {
+        // Rows that can all be full (no page ranges, and a pool that holds them) and are many waves long are taken as they
+        // are: finding a group's place costs 3 % (8 x 32K tokens, 8 KV heads: 1094 us against 1126).  Otherwise the CTAs of
+        // empty rows cost more, in launches and in how the others are spread: a chunk of 128 of 512 pages in 32 layers, 386
+        // us by rows against 343.
+        const int layers = k_layers ? num_layers : 1;
+        const int64_t rows = (int64_t)batch * c->Pmax, most = (int64_t)((c->Pmax + kBuildItems - 1) / kBuildItems) * p.Hkv * batch * layers;
+        if (!pb && 4 * rows <= 5 * (int64_t)kv->num_blocks && most > 64 * (int64_t)c->num_sms)
+          build_i4_table_kernel<<<grid, kI4Warps * 32, kI4Smem, st>>>(p);
+        else
+          build_i4_kernel<<<(int)std::min<int64_t>(most, (int64_t)kI4Waves * kI4CtasPerSm * c->num_sms), kI4Warps * 32, kI4SmemCount, st>>>(p, layers, c->num_sms);
+      }
       else build_kernel<float, LOCKS_FMT_I4><<<grid, kBuildWarps * 32, smem, st>>>(p);
       break;
     case LOCKS_FMT_I8: LOCKS_BUILD_CASE(LOCKS_FMT_I8); break;

@@ -135,6 +135,43 @@ def test_bulk_build_partial_warps_and_degenerate_pages(rank, layout):
     assert differ <= 2e-3 * total, (differ, total)
 
 
+# The bulk build's ways to deal the pages out: by the table's rows (long rows in a pool that can fill them), one warp to a
+# group of eight pages (many), two warps (few), and rounds of a resident grid (four layers).  Groups are the same eight pages
+# each time, and the arithmetic does not depend on who works on them: the bytes are equal.
+def test_bulk_build_is_dealt_out_in_several_ways():
+    import paper_2607_24555_b200 as locks
+    from paper_2607_24555_b200.binding import KVView, make_config
+    dev, batch, hkv, rows = torch.device("cuda:0"), 40, 8, 264
+    lens = [rows * 16 - 17 * (i % 3) for i in range(batch)]
+    lens[3], lens[4], lens[33], lens[39] = 0, 15, 16 * 9 + 1, 16 * 8
+    pages = [-(-t // 16) for t in lens]
+    nb = 9000
+    ctx = locks.Context(make_config(16, hkv, 8, "i4", "bf16", batch, rows, 256), device=dev)
+    gen = torch.Generator(device=dev).manual_seed(5)
+    k = torch.randn(nb, hkv, 16, 128, generator=gen, device=dev).to(torch.bfloat16)
+    table = torch.randint(nb, (batch, rows), generator=gen, device=dev, dtype=torch.int32)   # pages may share a block
+    seq = torch.tensor(lens, dtype=torch.int32, device=dev)
+    kv = KVView(k, k, (hkv * 2048, 2048, 128), nb, table, seq)
+    ones = torch.ones(batch, dtype=torch.int32, device=dev)
+    builds = [ctx.new_summaries(nb) for _ in range(3)]
+    ctx.locks_build_summaries(kv, batch, builds[0])
+    ctx.locks_build_summaries(kv, batch, builds[1], 0 * ones, rows * ones)
+    for at in range(0, rows, 64):
+        ctx.locks_build_summaries(kv, batch, builds[2], at * ones, (at + 64) * ones)
+    layers = [ctx.new_summaries(nb) for _ in range(4)]
+    keep = ctx.locks_build_summaries_layers(kv, [k] * 4, layers, batch, 0 * ones, rows * ones)
+    assert ctx.locks_poll_status() == 0 and keep
+    host = table.cpu()
+    built = torch.zeros(nb, dtype=torch.bool)
+    for b, t in enumerate(lens):
+        built[host[b, :t // 16].long()] = True
+    assert torch.equal((builds[0].view(nb, -1) != 0).any(1).cpu(), built)
+    once = np.bincount(np.concatenate([host[b, :t // 16].numpy() for b, t in enumerate(lens)]), minlength=nb) == 1
+    once = torch.from_numpy(once).to(dev)   # a block in several pages is built beside other pages each time
+    for other in builds[1:] + layers:
+        assert torch.equal(builds[0][once], other[once])
+
+
 # The scan of int4 summaries at 32- and 64-token pages: every rank, one and two tiles of query heads, group sizes that fill
 # neither, sequences that end inside a group of eight pages, more groups than warps (strides), extreme logits.
 @pytest.mark.parametrize("B", [32, 64])
