@@ -9,7 +9,7 @@
 
 #define LOCKS_D 128          // head dimension the kernels are written for
 #define LOCKS_B 16           // tokens per page of the main (tensor-core) paths; pages of 32 and 64 tokens
-                             // (cfg.page_size) go through the plain fp32 kernels, which take the size at run time
+                             // (cfg.page_size) are taken as tiles of 16 by attention and have kernels of their own for the scan and the builds
 #define LOCKS_GROUP 8        // pages scored together by one warp in the scan (one ring stage, one partial)
 #define LOCKS_SEL_THREADS 512
 #define LOCKS_SEL_MAX_EPT 16 // pages per thread a selector CTA ranks at most (512 threads: 8192 pages or list entries)
@@ -56,7 +56,7 @@ struct locks_host_graph {
 struct locks_ctx {
   locks_config cfg;
   int G, k, S, Pmax, max_groups;
-  int B;                   // tokens per page (cfg.page_size): 16, or 32 / 64 on the plain kernels
+  int B;                   // tokens per page (cfg.page_size): 16, or 32 / 64
   int num_sms;
   int part_slots;          // partial slots per (request, head) the last scan launch may have filled
   int part_balanced;       // the last scan launch wrote per-problem partial counts to part_cnt instead
