@@ -457,14 +457,22 @@ __global__ void __launch_bounds__(LOCKS_ATT_WARPS * 32, LOCKS_ATT_CTAS_PER_SM) a
   if (threadIdx.x == 0) p.done[prob] = 0;   // ready for the next launch
 }
 
-// Plain fp32-arithmetic path for any element type (the fp32 parity configuration).
-template <typename T>
-__global__ void __launch_bounds__(128) attend_generic_kernel(AttParams p) {
-  __shared__ float so[4][LOCKS_D];
-  __shared__ float sm[4], sl[4];
+// fp32 caches, in fp32 arithmetic: a CTA of four warps takes a split's pages for NH query heads of a KV head at a time, a warp
+// every fourth page in tiles of 8 tokens.  A lane owns 4 dims of every row; the 8 NH partial dot products of a tile are summed
+// by halves (each step a lane passes on the half that is not its own: 31 shuffles for 32 sums), after which a lane holds the
+// score of one (head, token).  Bound by the latency of a tile's chain (16 rows in flight a warp) and by its shuffles.
+// Steps with fp32 caches, before (a warp per head, token after token, each with a warp reduction of its own) and after this
+// kernel and scan_f32_kernel: 30 requests x 32 pages, 4 heads, 226 -> 70 us; 25 x 169..666 tokens, all pages, 122 -> 41; 48 x
+// 237..968, 5 heads, 377 -> 114; 3 x 31K, 8 heads, 357 -> 99.
+template <int NH>
+__global__ void __launch_bounds__(128, 3) attend_f32_kernel(AttParams p) {
+  constexpr int kTok = 8, NV = kTok * NH, kDup = 32 / NV;   // kDup lanes hold the same score
+  static_assert(NH == 1 || NH == 4, "scores have to fill or divide a warp");
+  __shared__ float so[4][NH][LOCKS_D];
+  __shared__ float sm[4][NH], sl[4][NH];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int split = blockIdx.x, hq = blockIdx.y, b = blockIdx.z;
-  const int h = hq / p.G;
+  const int parts = (p.G + NH - 1) / NH;
+  const int split = blockIdx.x, h = blockIdx.y / parts, g0 = blockIdx.y % parts * NH, b = blockIdx.z;
   pdl_wait();
   const int64_t prob = (int64_t)b * p.Hkv + h;
   const int Tn = p.seq_lens[b];
@@ -476,52 +484,97 @@ __global__ void __launch_bounds__(128) attend_generic_kernel(AttParams p) {
   }
   int lo, hi;
   slice_of(npages, split, p.splits, lo, hi);
-  const T *K = reinterpret_cast<const T *>(p.k), *V = reinterpret_cast<const T *>(p.v), *Q = reinterpret_cast<const T *>(p.q);
-  float qv[4], o[4] = {0.f, 0.f, 0.f, 0.f};
+  const float *K = reinterpret_cast<const float *>(p.k), *V = reinterpret_cast<const float *>(p.v);
+  const int64_t row0 = (int64_t)b * p.Hq + h * p.G + g0;   // first of the CTA's query heads
+  float4 q[NH], o[NH];
 #pragma unroll
-  for (int u = 0; u < 4; ++u) qv[u] = ldf<T>(Q, ((int64_t)b * p.Hq + hq) * LOCKS_D + lane * 4 + u);
-  float m = -INFINITY, l = 0.f;
+  for (int g = 0; g < NH; ++g) {
+    q[g] = o[g] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (g0 + g < p.G) q[g] = reinterpret_cast<const float4 *>(p.q)[(row0 + g) * (LOCKS_D / 4) + lane];
+  }
+  const int tok = lane / kDup % kTok;   // this lane's score: head lane / (kDup kTok), token tok of the tile
+  float m = -INFINITY, l = 0.f;         // of the lane's head; l: its tokens' share
   const float c2 = p.sm_scale * kLog2e;
+  int block = 0, ntok = 0;
+  bool good = lo + warp < hi && resolve_page(p, b, prob, lo + warp, Tn, block, ntok);
   for (int idx = lo + warp; idx < hi; idx += 4) {
-    int block, ntok;
-    if (!resolve_page(p, b, prob, idx, Tn, block, ntok)) continue;
-    const int64_t base = (int64_t)block * p.sb + (int64_t)(h / p.kvdiv) * p.sh;
-    for (int i = 0; i < ntok; ++i) {
-      float s = 0.f;
+    int next_block = 0, next_ntok = 0;   // resolved one page ahead
+    const bool next_good = idx + 4 < hi && resolve_page(p, b, prob, idx + 4, Tn, next_block, next_ntok);
+    if (good) {
+      const int64_t base = (int64_t)block * p.sb + (int64_t)(h / p.kvdiv) * p.sh + 4 * lane;
+      for (int t0 = 0; t0 < ntok; t0 += kTok) {
+        float4 k[kTok], v[kTok];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) s += qv[u] * ldf<T>(K, base + (int64_t)i * p.st + lane * 4 + u);
-      s = warp_sum(s) * c2;
-      const float mn = fmaxf(m, s);
-      const float alpha = exp2f(m - mn), pw = exp2f(s - mn);
-      l = l * alpha + pw;
+        for (int t = 0; t < kTok; ++t) {   // rows past the end: the last row again, with a weight of zero
+          const int64_t at = base + (int64_t)min(t0 + t, ntok - 1) * p.st;
+          k[t] = *reinterpret_cast<const float4 *>(K + at);
+          v[t] = *reinterpret_cast<const float4 *>(V + at);
+        }
+        float s[NV];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) o[u] = o[u] * alpha + pw * ldf<T>(V, base + (int64_t)i * p.st + lane * 4 + u);
-      m = mn;
+        for (int g = 0; g < NH; ++g)
+#pragma unroll
+          for (int t = 0; t < kTok; ++t)
+            s[g * kTok + t] = fmaf(q[g].w, k[t].w, fmaf(q[g].z, k[t].z, fmaf(q[g].y, k[t].y, q[g].x * k[t].x)));
+        halving_sum<NV>(s, lane);
+        const float sc = t0 + tok < ntok ? s[0] * c2 : -INFINITY;
+        float mn = sc;
+#pragma unroll
+        for (int x = kDup; x < kDup * kTok; x <<= 1) mn = fmaxf(mn, __shfl_xor_sync(0xffffffffu, mn, x));
+        mn = fmaxf(mn, m);
+        if (__any_sync(0xffffffffu, mn > m)) {
+          const float alpha = exp2f(m - mn);
+          l *= alpha;
+          m = mn;
+#pragma unroll
+          for (int g = 0; g < NH; ++g) {
+            const float a = __shfl_sync(0xffffffffu, alpha, g * kTok * kDup);
+            o[g].x *= a; o[g].y *= a; o[g].z *= a; o[g].w *= a;
+          }
+        }
+        const float pw = exp2f(sc - mn);
+        l += pw;
+#pragma unroll
+        for (int t = 0; t < kTok; ++t)
+#pragma unroll
+          for (int g = 0; g < NH; ++g) {
+            const float w = __shfl_sync(0xffffffffu, pw, (g * kTok + t) * kDup);
+            o[g].x = fmaf(w, v[t].x, o[g].x); o[g].y = fmaf(w, v[t].y, o[g].y);
+            o[g].z = fmaf(w, v[t].z, o[g].z); o[g].w = fmaf(w, v[t].w, o[g].w);
+          }
+      }
     }
+    good = next_good; block = next_block; ntok = next_ntok;
   }
 #pragma unroll
-  for (int u = 0; u < 4; ++u) so[warp][lane * 4 + u] = o[u];
-  if (lane == 0) { sm[warp] = m; sl[warp] = l; }
+  for (int x = kDup; x < kDup * kTok; x <<= 1) l += __shfl_xor_sync(0xffffffffu, l, x);
+#pragma unroll
+  for (int g = 0; g < NH; ++g) *reinterpret_cast<float4 *>(&so[warp][g][4 * lane]) = o[g];
+  if (lane % (kDup * kTok) == 0) { sm[warp][lane / (kDup * kTok)] = m; sl[warp][lane / (kDup * kTok)] = l; }
   __syncthreads();
   const int dim = threadIdx.x;
-  float M = fmaxf(fmaxf(sm[0], sm[1]), fmaxf(sm[2], sm[3]));
-  float L = 0.f, acc = 0.f;
-  if (M > -INFINITY) {
-    for (int w = 0; w < 4; ++w) {
-      const float sc = exp2f(sm[w] - M);
-      L += sl[w] * sc;
-      acc += so[w][dim] * sc;
+#pragma unroll
+  for (int g = 0; g < NH; ++g) {
+    if (g0 + g >= p.G) break;
+    const float M = fmaxf(fmaxf(sm[0][g], sm[1][g]), fmaxf(sm[2][g], sm[3][g]));
+    float L = 0.f, acc = 0.f;
+    if (M > -INFINITY) {
+      for (int w = 0; w < 4; ++w) {
+        const float sc = exp2f(sm[w][g] - M);
+        L += sl[w][g] * sc;
+        acc += so[w][g][dim] * sc;
+      }
+      acc /= L;
     }
-    acc /= L;
-  }
-  const float lse2 = (M > -INFINITY) ? M + log2f(L) : -INFINITY;
-  if (p.splits == 1) {
-    stf<T>(reinterpret_cast<T *>(p.out), ((int64_t)b * p.Hq + hq) * LOCKS_D + dim, acc);
-    if (p.lse && dim == 0) p.lse[(int64_t)b * p.Hq + hq] = lse2 * kLn2;
-  } else {
-    const int64_t slot = ((int64_t)b * p.Hq + hq) * p.splits + split;
-    p.part_o[slot * LOCKS_D + dim] = acc;
-    if (dim == 0) p.part_lse[slot] = lse2;
+    const float lse2 = (M > -INFINITY) ? M + log2f(L) : -INFINITY;
+    if (p.splits == 1) {
+      reinterpret_cast<float *>(p.out)[(row0 + g) * LOCKS_D + dim] = acc;
+      if (p.lse && dim == 0) p.lse[row0 + g] = lse2 * kLn2;
+    } else {
+      const int64_t slot = (row0 + g) * p.splits + split;
+      p.part_o[slot * LOCKS_D + dim] = acc;
+      if (dim == 0) p.part_lse[slot] = lse2;
+    }
   }
 }
 
@@ -626,7 +679,7 @@ int locks_launch_attend(locks_ctx *c, const void *q, const locks_kv *kv, int bat
   const bool dense = ids == nullptr;
   const bool bf = c->cfg.kv_dtype == LOCKS_BF16;   // tensor-core kernel
   p.sub_shift = !bf ? 0 : (c->B == 64 ? 2 : (c->B == 32 ? 1 : 0));
-  // one wave: as many splits per problem as resident CTA slots allow, at least one tile (generic kernel: page) per warp
+  // one wave: as many splits per problem as resident CTA slots allow, at least one tile (fp32 kernel: page) per warp
   const int ntiles = (dense ? c->Pmax : c->k) << p.sub_shift;
   int slots = c->num_sms * LOCKS_ATT_CTAS_PER_SM;
   if (slots > LOCKS_ATT_SLOT_BOUND) slots = LOCKS_ATT_SLOT_BOUND;
@@ -637,7 +690,7 @@ int locks_launch_attend(locks_ctx *c, const void *q, const locks_kv *kv, int bat
   if (splits < 1) splits = 1;
   // With clearly more problems than SMs every SM streams for several CTAs already: splitting a problem in
   // two only adds the merge (config 2, 256 problems: -1.5 to -2 us per step with one CTA per problem)
-  if (!dense && 2 * batch * p.Hkv >= 3 * c->num_sms) splits = 1;
+  if (bf && !dense && 2 * batch * p.Hkv >= 3 * c->num_sms) splits = 1;
   p.splits = splits;
   p.done = c->att_done;
   p.fused_merge = (p.G * p.splits <= kFusedMerge) ? 1 : 0;
@@ -697,7 +750,8 @@ int locks_launch_attend(locks_ctx *c, const void *q, const locks_kv *kv, int bat
     LOCKS_ATT_CASE(2, false);
 #undef LOCKS_ATT_CASE
   } else {
-    locks_launch_pdl(attend_generic_kernel<float>, dim3(p.splits, p.Hq, batch), dim3(128), 0, st, p);
+    if (p.G == 1) locks_launch_pdl(attend_f32_kernel<1>, dim3(p.splits, p.Hkv, batch), dim3(128), 0, st, p);
+    else locks_launch_pdl(attend_f32_kernel<4>, dim3(p.splits, p.Hkv * ((p.G + 3) / 4), batch), dim3(128), 0, st, p);
   }
   int rc = locks_check_launch(c);
   if (rc != LOCKS_OK || p.splits == 1 || (bf && p.fused_merge)) return rc;

@@ -260,6 +260,22 @@ __device__ __forceinline__ float warp_sum(float v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
+// N sums over the lanes of a warp, N a power of two up to 32: s[0] of lane i becomes the sum over all lanes of s[i / (32 / N)],
+// added in warp_sum's order.  In the first log2(N) steps a lane passes on the half of its sums that are not its own.
+template <int N>
+__device__ __forceinline__ void halving_sum(float (&s)[N], int lane) {
+#pragma unroll
+  for (int o = 16, n = N; o > 0; o >>= 1, n = n > 1 ? n / 2 : 1) {
+    if (n == 1) { s[0] += __shfl_xor_sync(0xffffffffu, s[0], o); continue; }
+    const bool up = lane & o;
+#pragma unroll
+    for (int i = 0; i < N / 2; ++i) {
+      if (i >= n / 2) break;
+      const float give = up ? s[i] : s[i + n / 2], keep = up ? s[i + n / 2] : s[i];
+      s[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+    }
+  }
+}
 __device__ __forceinline__ float warp_max(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));

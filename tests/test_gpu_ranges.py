@@ -184,6 +184,24 @@ def test_wide_page_scan(B, lens, Hq, Hkv, rank, qs):
     check_select_and_attend(gc, gc.oracle_summaries(), out_tol=2e-2)
 
 
+# fp32 caches and summaries: one query head per KV head, fewer than four, more than four and not a multiple, sixteen; every
+# rank of the fast scan and one beside them; last pages of 1, 8, 9 and 15 tokens, groups of eight pages that end early, splits
+# without pages.  fp32 sums of 128 products: 1e-5 of outputs of a few units, scores 2e-7 of at most a hundred.
+@pytest.mark.parametrize("rank", [2, 4, 8, 3])
+@pytest.mark.parametrize("lens,Hq,Hkv,layout", [([16 * 40 + 1, 16 * 9 + 8], 2, 2, "HND"), ([16 * 77 + 9, 5, 16 * 17], 6, 2, "NHD"),
+                                                ([16 * 30 + 15] * 3, 5, 1, "HND"), ([16 * 300, 16 * 8 + 1], 32, 2, "HND"),
+                                                ([16 * 25 - 1] * 70, 8, 4, "HND")])
+def test_fp32_scan_and_attention(lens, Hq, Hkv, layout, rank):
+    from gpu_util import GpuCase, check_select_and_attend
+    w = locks_synth.Workload("f32", lens, Hq=Hq, Hkv=Hkv, rank=rank, budget=16 * 7, dtype="f32", fmt="f32", seed=rank + Hq, layout=layout,
+                             tail_fill=float("nan"))
+    gc = GpuCase(w)
+    check_select_and_attend(gc, gc.oracle_summaries(), out_tol=2e-5, mass_tol=1e-4)
+    out, lse = gc.gpu_attend()
+    oout, olse = oracle.attend(gc.cache, t2np(gc.case.q), gc.sm)
+    assert np.abs(out - oout).max() <= 2e-5 and np.abs(lse - olse).max() <= 1e-4 * max(1.0, np.abs(olse).max() / 10)
+
+
 # The K largest of up to 8192 keys in list order, ties to the earlier entry (exact: whole numbers against a sort).  Keys that
 # leave the first histogram's threshold bin empty, full or crowded: all equal, two values, a crowd beside far outliers (a
 # range of 32 bits), equal keys across the threshold, a smooth spread; as few as one winner, as many as there are entries.
