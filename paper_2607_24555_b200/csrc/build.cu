@@ -257,7 +257,7 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b) {
 // Of two, each takes 4 of the items in phases 1 and 3, and 8 lanes hold a matrix in phase 2: a group is done in 79 us on an
 // idle chip where one warp takes 99.  Whether a group's sweeps go on is one decision of all its warps, so that the bytes are
 // the same either way.
-constexpr int kI4Warps = 2, kI4CtasPerSm = 8, kI4Waves = 16;
+constexpr int kI4Warps = 2, kI4CtasPerSm = 8, kI4Waves = 32, kI4Pairs = 22;
 constexpr int kI4Group = kBuildMat + 64 + kBuildItems * LOCKS_B * 4;   // bytes: matrices, key norms, eigenvalues
 constexpr int kI4Smem = kI4Warps * (kBuildScratch + kI4Group);
 constexpr int kI4SmemCount = kI4Smem + 64;   // + the number of groups, a group's blocks and KV head
@@ -583,7 +583,7 @@ __global__ void __launch_bounds__(kI4Warps * 32, kI4CtasPerSm) build_i4_kernel(B
   if (groups == 0) return;
   // Two warps a group up to three waves of single ones: us with one / two at 128 groups 104 / 80, 1024: 168 / 131, 2048: 216 /
   // 201, 3072: 294 / 284, 4096: 348 / 349, 16 376: 1126 / 1153.
-  if ((int64_t)groups * layers <= (int64_t)22 * sms) build_i4_groups<2>(p, smem_raw, count, layers);
+  if ((int64_t)groups * layers <= (int64_t)kI4Pairs * sms) build_i4_groups<2>(p, smem_raw, count, layers);
   else build_i4_groups<1>(p, smem_raw, count, layers);
 }
 
@@ -1194,7 +1194,15 @@ int locks_launch_build(locks_ctx *c, const locks_kv *kv, int batch, const int32_
         if (!pb && 4 * rows <= 5 * (int64_t)kv->num_blocks && most > 64 * (int64_t)c->num_sms)
           build_i4_table_kernel<<<grid, kI4Warps * 32, kI4Smem, st>>>(p);
         else
-          build_i4_kernel<<<(int)std::min<int64_t>(most, (int64_t)kI4Waves * kI4CtasPerSm * c->num_sms), kI4Warps * 32, kI4SmemCount, st>>>(p, layers, c->num_sms);
+        {
+          // A CTA per two groups, as many as the pool's blocks can make up: rounds of a smaller grid let the warps drift apart
+          // (163 840 groups in 16 waves of CTAs 14.9 ms, in one round 13.4).  With page ranges few of the rows' groups may
+          // be there: at most 32 waves, so that the empty ones cost no more than some 30 us.
+          const int64_t groups = std::min(most, (kv->num_blocks / kBuildItems + (int64_t)batch) * p.Hkv * layers);
+          int64_t ctas = std::max((groups + 1) / 2, std::min<int64_t>(groups, (int64_t)kI4Pairs * c->num_sms));
+          if (pb) ctas = std::min<int64_t>(ctas, (int64_t)kI4Waves * kI4CtasPerSm * c->num_sms);
+          build_i4_kernel<<<(unsigned)std::min<int64_t>(ctas, INT32_MAX), kI4Warps * 32, kI4SmemCount, st>>>(p, layers, c->num_sms);
+        }
       }
       else build_kernel<float, LOCKS_FMT_I4><<<grid, kBuildWarps * 32, smem, st>>>(p);
       break;

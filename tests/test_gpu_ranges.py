@@ -136,7 +136,7 @@ def test_bulk_build_partial_warps_and_degenerate_pages(rank, layout):
 
 
 # The bulk build's ways to deal the pages out: by the table's rows (long rows in a pool that can fill them), one warp to a
-# group of eight pages (many), two warps (few), and rounds of a resident grid (four layers).  Groups are the same eight pages
+# group of eight pages (many), two warps (few), and rounds of a grid that the pool bounds (eight layers, pages that share blocks).  Groups are the same eight pages
 # each time, and the arithmetic does not depend on who works on them: the bytes are equal.
 def test_bulk_build_is_dealt_out_in_several_ways():
     import paper_2607_24555_b200 as locks
@@ -158,8 +158,8 @@ def test_bulk_build_is_dealt_out_in_several_ways():
     ctx.locks_build_summaries(kv, batch, builds[1], 0 * ones, rows * ones)
     for at in range(0, rows, 64):
         ctx.locks_build_summaries(kv, batch, builds[2], at * ones, (at + 64) * ones)
-    layers = [ctx.new_summaries(nb) for _ in range(4)]
-    keep = ctx.locks_build_summaries_layers(kv, [k] * 4, layers, batch, 0 * ones, rows * ones)
+    layers = [ctx.new_summaries(nb) for _ in range(8)]
+    keep = ctx.locks_build_summaries_layers(kv, [k] * 8, layers, batch, 0 * ones, rows * ones)
     assert ctx.locks_poll_status() == 0 and keep
     host = table.cpu()
     built = torch.zeros(nb, dtype=torch.bool)
