@@ -398,8 +398,10 @@ __device__ __forceinline__ void build_i4_group(const BuildParams &p, uint8_t *sm
     const float *U = mat + s * kMat, *lam = lam_s + s * LOCKS_B;   // U[mode][token] as pairs
     // lane l < r: mode l
     const float lam0 = lam[0], lx = lam[lane & 15];
-    const uint32_t above = __ballot_sync(0xffffffffu, lam0 > 0.f && lx > 1e-6f * lam0 && lx > 1e-10f * kn_s[s]);
-    const int r_eff = min(r, __ffs(~above) - 1);   // modes above the zero-mode thresholds (eigenvalues descend; never 16 of them)
+    // modes above the zero-mode thresholds (eigenvalues descend).  The 16th is nothing but rounding (D sums to zero), but not always
+    // below them: where the diagonal of M swallows many small products (one large entry per key) it reads 3e-6 of the first.
+    const uint32_t above = __ballot_sync(0xffffffffu, lam0 > 0.f && lx > 1e-6f * lam0 && lx > 1e-10f * kn_s[s]) & 0x7fffu;
+    const int r_eff = min(r, __ffs(~above) - 1);
     const float isig = lane < r_eff ? rsqrtf(lx) : 0.f;
     float2 v[8][2], mu[2];   // basis vectors of this lane's 4 dims
     {

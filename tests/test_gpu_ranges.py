@@ -135,6 +135,42 @@ def test_bulk_build_partial_warps_and_degenerate_pages(rank, layout):
     assert differ <= 2e-3 * total, (differ, total)
 
 
+def _bulk_bytes_by_key_type(keys, rank):
+    """int4 summaries of pages [n, 16, 128] in one head: from bf16 keys (build_i4_group) and from the same values in fp32
+    (build_kernel), which computes in the same order."""
+    import paper_2607_24555_b200 as locks
+    from paper_2607_24555_b200.binding import KVView, make_config
+    n, got = len(keys), []
+    for dt in (torch.bfloat16, torch.float32):
+        ctx = locks.Context(make_config(2, 1, rank, "i4", "bf16" if dt == torch.bfloat16 else "f32", 1, n, 256))
+        k = keys.to(dt).contiguous()
+        kv = KVView(k, k, (2048, 2048, 128), n, torch.arange(n, dtype=torch.int32, device="cuda:0")[None].contiguous(),
+                    torch.tensor([16 * n], dtype=torch.int32, device="cuda:0"))
+        summ = ctx.new_summaries(n)
+        ctx.locks_build_summaries(kv, 1, summ)
+        assert ctx.locks_poll_status() == 0
+        got.append(summ.view(n, -1))
+    return got
+
+
+# Sixteen keys with one large entry each and small ones beside it: 15 equal modes, and a 16th that is nothing but what the Gram
+# matrix's diagonal lost in the sums, up to 3e-6 of the others.  It must not cost the page its basis.
+@pytest.mark.parametrize("rank", [2, 4, 8])
+def test_bulk_build_of_pages_with_equal_modes(rank):
+    gen = torch.Generator().manual_seed(rank)
+    pages = []
+    for m in range(0, 128, 4):
+        for e in range(-36, -16):
+            big = 1.0 + m / 128.0
+            k = 2.0 ** (e / 2) * big * (torch.randint(0, 2, (16, 128), generator=gen) * 2.0 - 1.0)
+            k[torch.arange(16), torch.arange(16)] = big
+            pages.append(k)
+    bf, f32 = _bulk_bytes_by_key_type(torch.stack(pages).to(torch.bfloat16).cuda(), rank)
+    at = 64 * rank + 16 * rank + 128 + 32   # the basis scales: fp16, one per mode
+    assert bool((bf[:, at:at + 2 * rank].contiguous().view(torch.float16) > 0).all())
+    assert torch.equal(bf, f32)
+
+
 # The bulk build's ways to deal the pages out: by the table's rows (long rows in a pool that can fill them), one warp to a
 # group of eight pages (many), two warps (few), and rounds of a grid that the pool bounds (eight layers, pages that share blocks).  Groups are the same eight pages
 # each time, and the arithmetic does not depend on who works on them: the bytes are equal.
