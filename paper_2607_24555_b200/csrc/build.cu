@@ -449,14 +449,15 @@ __device__ __forceinline__ void build_i4_group(const BuildParams &p, uint8_t *sm
     const float sc_mode = inv_scale(__half2float(sv)) * ((neg >> (lane & 7)) & 1u ? -1.f : 1.f);
     if (lane < r) *reinterpret_cast<__half *>(gout + i4_off_sv(r) + 2 * lane) = sv;
     // codes: lane = 8 t + s8 owns dims 32 t + 4 s8 + {0,1,2,3} = (half, e) in {0,1}^2 of k-step s8; dim offset c = 2 half + e ->
-    // nibble 2 (s8 & 1) + half + 4 e.  x + 1.5 2^23 + 8 rounds half to even and leaves code + 8 in the low bits (a unit vector's
-    // largest entry is at least 0.088: no scale is subnormal, no code leaves -7 .. 7)
+    // nibble 2 (s8 & 1) + half + 4 e.  x + 1.5 2^23 + 8 rounds half to even and leaves code + 8 in the low bits (a scale would have
+    // to be below 7 steps of fp16 for a code to leave -7 .. 7; the smallest that pages of noise modes gave is 13).  The product is
+    // rounded by itself: packed, the two become one fma, and what rounds to a tie first gets another code (a byte in 8 million).
 #pragma unroll
     for (int l = 0; l < 8; ++l) {
       if (l >= r) break;
       const float sc = __shfl_sync(0xffffffffu, sc_mode, l);
-      const float2 sc2 = make_float2(sc, sc), magic = make_float2(12582920.f, 12582920.f);
-      const float2 a = add2(mul2(v[l][0], sc2), magic), b = add2(mul2(v[l][1], sc2), magic);
+      auto magic = [&](float x) { return __fadd_rn(__fmul_rn(x, sc), 12582920.f); };
+      const float2 a = make_float2(magic(v[l][0].x), magic(v[l][0].y)), b = make_float2(magic(v[l][1].x), magic(v[l][1].y));
       uint32_t pw = (__float_as_uint(a.x) & 15u) | (__float_as_uint(a.y) & 15u) << 16 | (__float_as_uint(b.x) & 15u) << 4 |
                     (__float_as_uint(b.y) & 15u) << 20;
       pw <<= 8 * (lane & 1);

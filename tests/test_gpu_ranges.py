@@ -171,6 +171,16 @@ def test_bulk_build_of_pages_with_equal_modes(rank):
     assert torch.equal(bf, f32)
 
 
+# Random pages, enough of them for values whose product with the inverse scale rounds to a tie (one in ten million): the bytes
+# do not depend on the type that holds the keys.
+@pytest.mark.parametrize("rank", [2, 4, 8])
+def test_bulk_build_rounds_codes_alike(rank):
+    gen = torch.Generator(device="cuda:0").manual_seed(rank)
+    keys = 3.0 * torch.randn(100_000, 16, 128, generator=gen, device="cuda:0")
+    bf, f32 = _bulk_bytes_by_key_type((keys + 2.0 * torch.randn(len(keys), 1, 128, generator=gen, device="cuda:0")).to(torch.bfloat16), rank)
+    assert torch.equal(bf, f32), int((bf != f32).sum())
+
+
 # The bulk build's ways to deal the pages out: by the table's rows (long rows in a pool that can fill them), one warp to a
 # group of eight pages (many), two warps (few), and rounds of a grid that the pool bounds (eight layers, pages that share blocks).  Groups are the same eight pages
 # each time, and the arithmetic does not depend on who works on them: the bytes are equal.
