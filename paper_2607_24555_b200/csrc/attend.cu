@@ -29,7 +29,7 @@ struct AttParams {
   int32_t *done;   // [batch*Hkv] split-arrival counters (zero between launches)
   int batch, Hq, Hkv, G, Pmax, kbud, num_blocks, splits;
   int B;             // tokens per page
-  int sub_shift;     // bf16 kernel: a page is 2^sub_shift tiles of 16 tokens (0, 1, 2 for pages of 16, 32, 64 tokens)
+  int sub_shift;     // bf16 kernel, wide pages: a page is 2^sub_shift tiles of 16 tokens (1, 2 for pages of 32, 64 tokens)
   int kvdiv;         // the KV head of problem h is h / kvdiv (1; per-head page tables: G, with G = 1 and Hkv = Hq here)
   int fused_merge;   // 1: the last CTA of a problem merges its splits; 0: a separate merge kernel follows
   int cluster;       // 1: the splits of a problem form one thread-block cluster and merge through its shared memory
@@ -83,10 +83,13 @@ __device__ __forceinline__ uint32_t movm_trans_b16(uint32_t v) {
 //                                                                   B = P^T after an 8x8 movmatrix transpose)
 // so both products use all 16 rows of the tile and the accumulator is 32 registers per 8 heads.
 //
-// Pages of 32 and 64 tokens are two and four such tiles; the list of pages is walked tile by tile.
-// Pages of 32 and 64 tokens are two and four such tiles: the page list is walked tile by tile (32-token pages, 4 requests
-// x 128 pages of 32 tokens: 71 + 6 us on the fp32 kernel that reads the pages once per query head, 15 us here).
-template <int NH, bool CONTIG>
+// WIDE: pages of 32 and 64 tokens are two and four such tiles, and the page list is walked tile by tile.  Their weights and sums
+// are those of fp32 arithmetic: P goes in as three bf16 parts (24 bits), and since the tensor core truncates what it adds to an
+// accumulator, every product starts from zero and is added to the running sum by a rounding fp32 addition.  Against fp64, over 18
+// batches at both sizes: outputs 1.648e-3 .. 1.680e-3, all of it the rounding of the result (P in bf16: up to 2.29e-3), log-sum-exp
+// 3.3e-7 on average, as an fp32 kernel has it (3.4e-7).  4 x 128 pages of 32 tokens: 12.6 us; P in bf16 11.1, plain fp32 arithmetic
+// 18.9 (sums by halves) and 40.6 (a warp reduction per token).
+template <int NH, bool CONTIG, bool WIDE>
 __global__ void __launch_bounds__(LOCKS_ATT_WARPS * 32, LOCKS_ATT_CTAS_PER_SM) attend_bf16_kernel(AttParams p) {
   extern __shared__ __align__(128) uint8_t smem[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -117,13 +120,14 @@ __global__ void __launch_bounds__(LOCKS_ATT_WARPS * 32, LOCKS_ATT_CTAS_PER_SM) a
   const float c2 = p.sm_scale * kLog2e;
   pdl_wait();   // page table from the selector, appended K/V rows, sequence lengths
   const int T = p.seq_lens[b];
-  int npages = p.ids ? p.cnt[prob] : (T + p.B - 1) / p.B;
+  const int B = WIDE ? p.B : LOCKS_B;
+  int npages = p.ids ? p.cnt[prob] : (T + B - 1) / B;
   if (p.ids && (npages < 0 || npages > p.kbud)) {   // a count beyond the table's row: use the row, report it
     if (threadIdx.x == 0) set_status(p.status, LOCKS_ERR_BAD_BLOCK);
     npages = npages < 0 ? 0 : p.kbud;
   }
   int lo, hi;
-  slice_of(npages << p.sub_shift, split, p.splits, lo, hi);
+  slice_of(npages << (WIDE ? p.sub_shift : 0), split, p.splits, lo, hi);
 
   float oacc[8][NH][4];
 #pragma unroll
@@ -144,16 +148,14 @@ __global__ void __launch_bounds__(LOCKS_ATT_WARPS * 32, LOCKS_ATT_CTAS_PER_SM) a
 
   // page ids and physical blocks of this warp's pages are resolved 32 at a time, one lane each, so the
   // two dependent global loads are paid once per batch instead of once per page
-  const int first = lo + warp, sub_mask = (1 << p.sub_shift) - 1;
+  const int first = lo + warp, sub_shift = WIDE ? p.sub_shift : 0, sub_mask = (1 << sub_shift) - 1;
   auto resolve_batch = [&](int jb, int &blk, int &nt) {
     const int idx = first + (jb + lane) * LOCKS_ATT_WARPS;
     blk = 0;
     nt = 0;
     if (idx < hi) {
-      if (resolve_page(p, b, prob, idx >> p.sub_shift, T, blk, nt))
-        nt = min(LOCKS_B, nt - (idx & sub_mask) * LOCKS_B);   // tokens of this tile (none past the sequence's end)
-      else
-        blk = nt = 0;
+      if (!resolve_page(p, b, prob, idx >> sub_shift, T, blk, nt)) blk = nt = 0;
+      else if (WIDE) nt = min(LOCKS_B, nt - (idx & sub_mask) * LOCKS_B);   // tokens of this tile (none past the sequence's end)
     }
   };
   int blk_cur, nt_cur, blk_nxt = 0, nt_nxt = 0;
@@ -164,7 +166,7 @@ __global__ void __launch_bounds__(LOCKS_ATT_WARPS * 32, LOCKS_ATT_CTAS_PER_SM) a
     const int block = __shfl_sync(0xffffffffu, blk_cur, j & 31);
     const int ntok = __shfl_sync(0xffffffffu, nt_cur, j & 31);
     uint8_t *kt = ring + stage * kAttStage, *vt = kt + kTile;
-    const int sub = (first + j * LOCKS_ATT_WARPS) & sub_mask;   // tile within its page
+    const int sub = WIDE ? (first + j * LOCKS_ATT_WARPS) & sub_mask : 0;   // tile within its page
     const int64_t base = ((int64_t)block * p.sb + (int64_t)hkv * p.sh + (int64_t)(sub * LOCKS_B) * p.st) * 2 + goff0;
     const uint8_t *kp = Kb + base, *vp = Vb + base;
 #pragma unroll
@@ -232,11 +234,21 @@ __global__ void __launch_bounds__(LOCKS_ATT_WARPS * 32, LOCKS_ATT_CTAS_PER_SM) a
         uint32_t r[4];
         ldsm_x4(r, kt + tok * 256 + ((ch ^ (tok & 7)) << 4));
 #pragma unroll
-        for (int hh = 0; hh < NH; ++hh) mma_bf16(sacc[hh], r[0], r[1], r[2], r[3], qb[hh][s][0], qb[hh][s][1]);
+        for (int hh = 0; hh < NH; ++hh) {
+          if (WIDE && s > 0) {
+            float c[4];
+            mma_bf16_z(c, r[0], r[1], r[2], r[3], qb[hh][s][0], qb[hh][s][1]);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) sacc[hh][e] += c[e];
+          } else {
+            mma_bf16(sacc[hh], r[0], r[1], r[2], r[3], qb[hh][s][0], qb[hh][s][1]);
+          }
+        }
       }
     }
     // ---- online softmax down the token rows; this lane: tokens x, x + 8, heads 2t, 2t+1 (+8)
-    uint32_t pb0[NH], pb1[NH];
+    constexpr int kParts = WIDE ? 3 : 1;
+    uint32_t pb0[NH][kParts], pb1[NH][kParts];
     const bool v0ok = x < ntok, v1ok = x + 8 < ntok;
 #pragma unroll
     for (int hh = 0; hh < NH; ++hh) {
@@ -270,8 +282,20 @@ __global__ void __launch_bounds__(LOCKS_ATT_WARPS * 32, LOCKS_ATT_CTAS_PER_SM) a
       lrun[hh][0] += p00 + p10;
       lrun[hh][1] += p01 + p11;
       // P^T rows (tokens) -> B fragment (k = tokens 2t, 2t+1 | 8 + 2t.., n = head x)
-      pb0[hh] = movm_trans_b16(pack_bf16(p00, p01));
-      pb1[hh] = movm_trans_b16(pack_bf16(p10, p11));
+      float w[4] = {p00, p01, p10, p11};
+#pragma unroll
+      for (int u = 0; u < kParts; ++u) {
+        if (!WIDE) {
+          pb0[hh][u] = movm_trans_b16(pack_bf16(w[0], w[1]));
+          pb1[hh][u] = movm_trans_b16(pack_bf16(w[2], w[3]));
+          continue;
+        }
+        // truncated, so that no part is negative; and none but the first is zero: an infinite value stays infinite
+        pb0[hh][u] = movm_trans_b16(__byte_perm(__float_as_uint(w[0]), __float_as_uint(w[1]), 0x7632));
+        pb1[hh][u] = movm_trans_b16(__byte_perm(__float_as_uint(w[2]), __float_as_uint(w[3]), 0x7632));
+#pragma unroll
+        for (int e = 0; e < 4; ++e) w[e] = fmaxf(w[e] - __uint_as_float(__float_as_uint(w[e]) & 0xFFFF0000u), 1.17549435e-38f);
+      }
     }
     // ---- O^T += V^T P^T
     {
@@ -282,7 +306,18 @@ __global__ void __launch_bounds__(LOCKS_ATT_WARPS * 32, LOCKS_ATT_CTAS_PER_SM) a
         uint32_t r[4];
         ldsm_x4_trans(r, vt + tok * 256 + ((ch ^ (tok & 7)) << 4));
 #pragma unroll
-        for (int hh = 0; hh < NH; ++hh) mma_bf16(oacc[mt][hh], r[0], r[1], r[2], r[3], pb0[hh], pb1[hh]);
+        for (int hh = 0; hh < NH; ++hh) {
+          if (WIDE) {   // the smallest part first
+            float c[4];
+            mma_bf16_z(c, r[0], r[1], r[2], r[3], pb0[hh][kParts - 1], pb1[hh][kParts - 1]);
+#pragma unroll
+            for (int u = kParts - 2; u >= 0; --u) mma_bf16(c, r[0], r[1], r[2], r[3], pb0[hh][u], pb1[hh][u]);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) oacc[mt][hh][e] += c[e];
+          } else {
+            mma_bf16(oacc[mt][hh], r[0], r[1], r[2], r[3], pb0[hh][0], pb1[hh][0]);
+          }
+        }
       }
     }
     __syncwarp();
@@ -678,6 +713,7 @@ int locks_launch_attend(locks_ctx *c, const void *q, const locks_kv *kv, int bat
   }
   const bool dense = ids == nullptr;
   const bool bf = c->cfg.kv_dtype == LOCKS_BF16;   // tensor-core kernel
+  const bool wide = c->B != LOCKS_B;
   p.sub_shift = !bf ? 0 : (c->B == 64 ? 2 : (c->B == 32 ? 1 : 0));
   // one wave: as many splits per problem as resident CTA slots allow, at least one tile (fp32 kernel: page) per warp
   const int ntiles = (dense ? c->Pmax : c->k) << p.sub_shift;
@@ -700,8 +736,8 @@ int locks_launch_attend(locks_ctx *c, const void *q, const locks_kv *kv, int bat
   // requests slower).
   p.cluster = 0;
   if (c->att_clusters[0] < 0) {   // clusters of 2, 4, 8, 16 CTAs of this kernel that fit the device at once (probed once)
-    cudaFuncSetAttribute(attend_bf16_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmem);
-    cudaFuncSetAttribute(attend_bf16_kernel<1, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cudaFuncSetAttribute(attend_bf16_kernel<1, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmem);
+    cudaFuncSetAttribute(attend_bf16_kernel<1, true, false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     for (int i = 0; i < 4; ++i) {
       cudaLaunchConfig_t lc = {};
       lc.gridDim = dim3(2 << i, 1, 1);
@@ -713,7 +749,7 @@ int locks_launch_attend(locks_ctx *c, const void *q, const locks_kv *kv, int bat
       lc.attrs = at;
       lc.numAttrs = 1;
       int nclusters = 0;
-      if (cudaOccupancyMaxActiveClusters(&nclusters, attend_bf16_kernel<1, true>, &lc) != cudaSuccess) nclusters = 0;
+      if (cudaOccupancyMaxActiveClusters(&nclusters, attend_bf16_kernel<1, true, false>, &lc) != cudaSuccess) nclusters = 0;
       c->att_clusters[i] = nclusters;
     }
     (void)cudaGetLastError();   // a refused probe is not an error of this call
@@ -734,20 +770,24 @@ int locks_launch_attend(locks_ctx *c, const void *q, const locks_kv *kv, int bat
     const bool contig = kv->stride_token == LOCKS_D;
     const dim3 grid(p.splits, p.Hkv, batch), blk(LOCKS_ATT_WARPS * 32);
     const bool attrs = locks_attrs_needed(LOCKS_ATTR_ATTEND);
-#define LOCKS_ATT_CASE(NH_, CONTIG_)                                                                                  \
-  do {                                                                                                               \
-    if (attrs) {                                                                                                     \
-      cudaFuncSetAttribute(attend_bf16_kernel<NH_, CONTIG_>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmem); \
-      cudaFuncSetAttribute(attend_bf16_kernel<NH_, CONTIG_>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);     \
-    }                                                                                                                \
-    if ((p.G > 8) != (NH_ == 2) || contig != CONTIG_) break;                                                         \
-    if (p.cluster) locks_launch_pdl_cluster(attend_bf16_kernel<NH_, CONTIG_>, grid, blk, kAttSmem, p.splits, st, p); \
-    else locks_launch_pdl(attend_bf16_kernel<NH_, CONTIG_>, grid, blk, kAttSmem, st, p);                             \
+#define LOCKS_ATT_CASE(NH_, CONTIG_, WIDE_)                                                                                  \
+  do {                                                                                                                      \
+    if (attrs) {                                                                                                            \
+      cudaFuncSetAttribute(attend_bf16_kernel<NH_, CONTIG_, WIDE_>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmem); \
+      cudaFuncSetAttribute(attend_bf16_kernel<NH_, CONTIG_, WIDE_>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);     \
+    }                                                                                                                       \
+    if ((p.G > 8) != (NH_ == 2) || contig != CONTIG_ || wide != WIDE_) break;                                               \
+    if (p.cluster) locks_launch_pdl_cluster(attend_bf16_kernel<NH_, CONTIG_, WIDE_>, grid, blk, kAttSmem, p.splits, st, p); \
+    else locks_launch_pdl(attend_bf16_kernel<NH_, CONTIG_, WIDE_>, grid, blk, kAttSmem, st, p);                             \
   } while (0)
-    LOCKS_ATT_CASE(1, true);
-    LOCKS_ATT_CASE(1, false);
-    LOCKS_ATT_CASE(2, true);
-    LOCKS_ATT_CASE(2, false);
+    LOCKS_ATT_CASE(1, true, false);
+    LOCKS_ATT_CASE(1, false, false);
+    LOCKS_ATT_CASE(2, true, false);
+    LOCKS_ATT_CASE(2, false, false);
+    LOCKS_ATT_CASE(1, true, true);
+    LOCKS_ATT_CASE(1, false, true);
+    LOCKS_ATT_CASE(2, true, true);
+    LOCKS_ATT_CASE(2, false, true);
 #undef LOCKS_ATT_CASE
   } else {
     if (p.G == 1) locks_launch_pdl(attend_f32_kernel<1>, dim3(p.splits, p.Hkv, batch), dim3(128), 0, st, p);
@@ -818,10 +858,10 @@ extern "C" int locks_sparse_attend_noalloc(const locks_config *cfg, const void *
     void *ptr = nullptr;
     if (cudaGetSymbolAddress(&ptr, g_noalloc_scratch) != cudaSuccess || ptr == nullptr) return LOCKS_ERR_CUDA;
     if (cudaDeviceGetAttribute(&nd.num_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return LOCKS_ERR_CUDA;
-    cudaFuncSetAttribute(attend_bf16_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmem);
-    cudaFuncSetAttribute(attend_bf16_kernel<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmem);
-    cudaFuncSetAttribute(attend_bf16_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmem);
-    cudaFuncSetAttribute(attend_bf16_kernel<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmem);
+    cudaFuncSetAttribute(attend_bf16_kernel<1, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmem);
+    cudaFuncSetAttribute(attend_bf16_kernel<2, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmem);
+    cudaFuncSetAttribute(attend_bf16_kernel<1, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmem);
+    cudaFuncSetAttribute(attend_bf16_kernel<2, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmem);
     nd.scratch = reinterpret_cast<unsigned char *>(ptr);
     nd.ready = true;
   }
@@ -852,11 +892,11 @@ extern "C" int locks_sparse_attend_noalloc(const locks_config *cfg, const void *
   dim3 grid(p.splits, p.Hkv, batch);
   const bool contig = kv->stride_token == LOCKS_D;
   if (G <= 8) {
-    if (contig) attend_bf16_kernel<1, true><<<grid, LOCKS_ATT_WARPS * 32, kAttSmem, st>>>(p);
-    else attend_bf16_kernel<1, false><<<grid, LOCKS_ATT_WARPS * 32, kAttSmem, st>>>(p);
+    if (contig) attend_bf16_kernel<1, true, false><<<grid, LOCKS_ATT_WARPS * 32, kAttSmem, st>>>(p);
+    else attend_bf16_kernel<1, false, false><<<grid, LOCKS_ATT_WARPS * 32, kAttSmem, st>>>(p);
   } else {
-    if (contig) attend_bf16_kernel<2, true><<<grid, LOCKS_ATT_WARPS * 32, kAttSmem, st>>>(p);
-    else attend_bf16_kernel<2, false><<<grid, LOCKS_ATT_WARPS * 32, kAttSmem, st>>>(p);
+    if (contig) attend_bf16_kernel<2, true, false><<<grid, LOCKS_ATT_WARPS * 32, kAttSmem, st>>>(p);
+    else attend_bf16_kernel<2, false, false><<<grid, LOCKS_ATT_WARPS * 32, kAttSmem, st>>>(p);
   }
   return cudaPeekAtLastError() == cudaSuccess ? LOCKS_OK : LOCKS_ERR_CUDA;
 }

@@ -27,6 +27,28 @@ def test_dense_attention_ragged_rows(lens, Hq, Hkv, B, layout):
     assert gc.status() == 0
 
 
+# Pages of 32 and 64 tokens: weights and sums in fp32.  Sums of 128 products and of a few thousand weighted values are off by
+# 1e-6 of the result at most, a bf16 result's rounding boundary is that near to one value in a thousand; weights rounded to
+# bf16 move a third of the results.
+@pytest.mark.parametrize("B", [32, 64])
+@pytest.mark.parametrize("lens,Hq,Hkv,qs,layout", [([40, 9.1], 8, 2, 1.0, "HND"), ([75.3], 32, 2, 2.0, "NHD"), ([30] * 6, 12, 4, 0.5, "HND"),
+                                                   ([2.9, 21.4, 11.55], 5, 1, 1.0, "NHD"), ([8, 33.02] * 3, 3, 3, 1.0, "HND"), ([6] * 40, 8, 8, 1.0, "HND")])
+def test_wide_page_attention_rounds_once(B, lens, Hq, Hkv, qs, layout):
+    from gpu_util import GpuCase
+    gc = GpuCase(locks_synth.Workload("wide", [int(n * B) for n in lens], Hq=Hq, Hkv=Hkv, B=B, budget=6 * B, seed=B + Hq, q_scale=qs,
+                                      layout=layout, tail_fill=float("nan")))
+    P = [-(-t // B) for t in gc.w.seq_lens]
+    ids = np.stack([np.stack([np.pad(np.unique(np.linspace(0, p - 1, min(p, 6)).astype(np.int32)), (0, 6), constant_values=-1)[:6]] * Hkv) for p in P])
+    cnt = (ids >= 0).sum(-1).astype(np.int32)
+    for table in ((None, None), (ids, cnt)):
+        out, lse = gc.gpu_attend(*table)
+        oout, olse = oracle.attend(gc.cache, t2np(gc.case.q), gc.sm, *table)
+        want = torch.from_numpy(oout).to(torch.bfloat16).double().numpy()
+        assert (out != want).mean() <= 5e-3
+        assert np.abs(lse - olse).max() <= 3e-6 * max(1.0, np.abs(olse).max() / 10)
+    assert gc.status() == 0
+
+
 def _page_keys(kind, B, rng):
     """[B, 128] keys: the workloads' structure, and pages whose Gram matrix has close, equal, few or no eigenvalues."""
     d = 128
