@@ -32,6 +32,7 @@ struct AttParams {
   int sub_shift;     // bf16 kernel, wide pages: a page is 2^sub_shift tiles of 16 tokens (1, 2 for pages of 32, 64 tokens)
   int kvdiv;         // the KV head of problem h is h / kvdiv (1; per-head page tables: G, with G = 1 and Hkv = Hq here)
   int fused_merge;   // 1: the last CTA of a problem merges its splits; 0: a separate merge kernel follows
+  uint64_t per_split;   // 2^32 / splits + 1
   int cluster;       // 1: the splits of a problem form one thread-block cluster and merge through its shared memory
   float sm_scale;
 };
@@ -50,14 +51,12 @@ constexpr int kAttSmem = LOCKS_ATT_WARPS * kAttStages * kAttStage;
 // go to the parallel merge kernel.
 constexpr int kFusedMerge = 64;
 
-// Slice `part` of `parts` nearly equal slices of n list entries.  Taken from the length the device sees: the table's
-// row (what the host could slice) is usually longer than the sequence, and equal slices of the row leave the last CTAs
-// of a problem idle: dense attention over 16 requests of 3K .. 12K tokens in rows of 32K 144.5 us, 3.6 TB/s; sliced by
-// length 94.2 us, 5.55 TB/s (0.86 of the copy bandwidth).
-__device__ __forceinline__ void slice_of(int n, int part, int parts, int &lo, int &hi) {
-  const int per = (n + parts - 1) / parts;
-  lo = min(part * per, n);
-  hi = min(lo + per, n);
+// Length of a slice when n list entries are cut into p.splits: ceil(n / p.splits), n below 2^25, without a division (the kernel for
+// more than 8 heads takes 8.4 us for 4 x 32 pages and 37.4 for 131K tokens with this; with a division, which costs it registers in
+// the loop, 8.7 and 39.1).  Taken from the lengths that the device sees: the table's row (what the host could slice) is
+// usually longer than the sequence, and equal slices of the row leave the last CTAs of a problem idle.
+__device__ __forceinline__ int slice_length(const AttParams &p, int n) {
+  return (int)(((uint64_t)(uint32_t)(n + p.splits - 1) * p.per_split) >> 32);
 }
 
 // Resolve the idx-th page of this problem's list: logical page, physical block, valid tokens.
@@ -86,7 +85,7 @@ __device__ __forceinline__ uint32_t movm_trans_b16(uint32_t v) {
 // WIDE: pages of 32 and 64 tokens are two and four such tiles, and the page list is walked tile by tile.  Their weights and sums
 // are those of fp32 arithmetic: P goes in as three bf16 parts (24 bits), and since the tensor core truncates what it adds to an
 // accumulator, every product starts from zero and is added to the running sum by a rounding fp32 addition.  Against fp64, over 18
-// batches at both sizes: outputs 1.648e-3 .. 1.680e-3, all of it the rounding of the result (P in bf16: up to 2.29e-3), log-sum-exp
+// batches at both sizes: outputs 1.38e-3 .. 1.70e-3, all of it the rounding of the result (P in bf16: up to 2.29e-3), log-sum-exp
 // 3.3e-7 on average, as an fp32 kernel has it (3.4e-7).  4 x 128 pages of 32 tokens: 12.6 us; P in bf16 11.1, plain fp32 arithmetic
 // 18.9 (sums by halves) and 40.6 (a warp reduction per token).
 template <int NH, bool CONTIG, bool WIDE>
@@ -126,8 +125,8 @@ __global__ void __launch_bounds__(LOCKS_ATT_WARPS * 32, LOCKS_ATT_CTAS_PER_SM) a
     if (threadIdx.x == 0) set_status(p.status, LOCKS_ERR_BAD_BLOCK);
     npages = npages < 0 ? 0 : p.kbud;
   }
-  int lo, hi;
-  slice_of(npages << (WIDE ? p.sub_shift : 0), split, p.splits, lo, hi);
+  const int per = slice_length(p, npages << (WIDE ? p.sub_shift : 0));
+  const int lo = split * per, hi = min(lo + per, npages << (WIDE ? p.sub_shift : 0));
 
   float oacc[8][NH][4];
 #pragma unroll
@@ -153,10 +152,8 @@ __global__ void __launch_bounds__(LOCKS_ATT_WARPS * 32, LOCKS_ATT_CTAS_PER_SM) a
     const int idx = first + (jb + lane) * LOCKS_ATT_WARPS;
     blk = 0;
     nt = 0;
-    if (idx < hi) {
-      if (!resolve_page(p, b, prob, idx >> sub_shift, T, blk, nt)) blk = nt = 0;
-      else if (WIDE) nt = min(LOCKS_B, nt - (idx & sub_mask) * LOCKS_B);   // tokens of this tile (none past the sequence's end)
-    }
+    if (idx < hi && !resolve_page(p, b, prob, idx >> sub_shift, T, blk, nt)) nt = 0;
+    if constexpr (WIDE) nt = min(LOCKS_B, nt - (idx & sub_mask) * LOCKS_B);   // tokens of this tile (none past the sequence's end)
   };
   int blk_cur, nt_cur, blk_nxt = 0, nt_nxt = 0;
   resolve_batch(0, blk_cur, nt_cur);
@@ -235,11 +232,11 @@ __global__ void __launch_bounds__(LOCKS_ATT_WARPS * 32, LOCKS_ATT_CTAS_PER_SM) a
         ldsm_x4(r, kt + tok * 256 + ((ch ^ (tok & 7)) << 4));
 #pragma unroll
         for (int hh = 0; hh < NH; ++hh) {
-          if (WIDE && s > 0) {
+          if constexpr (WIDE) {
             float c[4];
             mma_bf16_z(c, r[0], r[1], r[2], r[3], qb[hh][s][0], qb[hh][s][1]);
 #pragma unroll
-            for (int e = 0; e < 4; ++e) sacc[hh][e] += c[e];
+            for (int e = 0; e < 4; ++e) sacc[hh][e] = s > 0 ? sacc[hh][e] + c[e] : c[e];
           } else {
             mma_bf16(sacc[hh], r[0], r[1], r[2], r[3], qb[hh][s][0], qb[hh][s][1]);
           }
@@ -247,8 +244,7 @@ __global__ void __launch_bounds__(LOCKS_ATT_WARPS * 32, LOCKS_ATT_CTAS_PER_SM) a
       }
     }
     // ---- online softmax down the token rows; this lane: tokens x, x + 8, heads 2t, 2t+1 (+8)
-    constexpr int kParts = WIDE ? 3 : 1;
-    uint32_t pb0[NH][kParts], pb1[NH][kParts];
+    uint32_t pb0[NH], pb1[NH], rest0[NH][2], rest1[NH][2];   // P^T; wide pages: its leading and its further parts
     const bool v0ok = x < ntok, v1ok = x + 8 < ntok;
 #pragma unroll
     for (int hh = 0; hh < NH; ++hh) {
@@ -282,19 +278,21 @@ __global__ void __launch_bounds__(LOCKS_ATT_WARPS * 32, LOCKS_ATT_CTAS_PER_SM) a
       lrun[hh][0] += p00 + p10;
       lrun[hh][1] += p01 + p11;
       // P^T rows (tokens) -> B fragment (k = tokens 2t, 2t+1 | 8 + 2t.., n = head x)
-      float w[4] = {p00, p01, p10, p11};
-#pragma unroll
-      for (int u = 0; u < kParts; ++u) {
-        if (!WIDE) {
-          pb0[hh][u] = movm_trans_b16(pack_bf16(w[0], w[1]));
-          pb1[hh][u] = movm_trans_b16(pack_bf16(w[2], w[3]));
-          continue;
-        }
+      if constexpr (!WIDE) {
+        pb0[hh] = movm_trans_b16(pack_bf16(p00, p01));
+        pb1[hh] = movm_trans_b16(pack_bf16(p10, p11));
+      } else {
         // truncated, so that no part is negative; and none but the first is zero: an infinite value stays infinite
-        pb0[hh][u] = movm_trans_b16(__byte_perm(__float_as_uint(w[0]), __float_as_uint(w[1]), 0x7632));
-        pb1[hh][u] = movm_trans_b16(__byte_perm(__float_as_uint(w[2]), __float_as_uint(w[3]), 0x7632));
+        float w[4] = {p00, p01, p10, p11};
 #pragma unroll
-        for (int e = 0; e < 4; ++e) w[e] = fmaxf(w[e] - __uint_as_float(__float_as_uint(w[e]) & 0xFFFF0000u), 1.17549435e-38f);
+        for (int u = 0; u < 3; ++u) {
+          const uint32_t a = movm_trans_b16(__byte_perm(__float_as_uint(w[0]), __float_as_uint(w[1]), 0x7632));
+          const uint32_t c = movm_trans_b16(__byte_perm(__float_as_uint(w[2]), __float_as_uint(w[3]), 0x7632));
+          if (u == 0) { pb0[hh] = a; pb1[hh] = c; }
+          else { rest0[hh][u - 1] = a; rest1[hh][u - 1] = c; }
+#pragma unroll
+          for (int e = 0; e < 4; ++e) w[e] = fmaxf(w[e] - __uint_as_float(__float_as_uint(w[e]) & 0xFFFF0000u), 1.17549435e-38f);
+        }
       }
     }
     // ---- O^T += V^T P^T
@@ -307,15 +305,15 @@ __global__ void __launch_bounds__(LOCKS_ATT_WARPS * 32, LOCKS_ATT_CTAS_PER_SM) a
         ldsm_x4_trans(r, vt + tok * 256 + ((ch ^ (tok & 7)) << 4));
 #pragma unroll
         for (int hh = 0; hh < NH; ++hh) {
-          if (WIDE) {   // the smallest part first
+          if constexpr (WIDE) {   // the smallest part first
             float c[4];
-            mma_bf16_z(c, r[0], r[1], r[2], r[3], pb0[hh][kParts - 1], pb1[hh][kParts - 1]);
-#pragma unroll
-            for (int u = kParts - 2; u >= 0; --u) mma_bf16(c, r[0], r[1], r[2], r[3], pb0[hh][u], pb1[hh][u]);
+            mma_bf16_z(c, r[0], r[1], r[2], r[3], rest0[hh][1], rest1[hh][1]);
+            mma_bf16(c, r[0], r[1], r[2], r[3], rest0[hh][0], rest1[hh][0]);
+            mma_bf16(c, r[0], r[1], r[2], r[3], pb0[hh], pb1[hh]);
 #pragma unroll
             for (int e = 0; e < 4; ++e) oacc[mt][hh][e] += c[e];
           } else {
-            mma_bf16(oacc[mt][hh], r[0], r[1], r[2], r[3], pb0[hh][0], pb1[hh][0]);
+            mma_bf16(oacc[mt][hh], r[0], r[1], r[2], r[3], pb0[hh], pb1[hh]);
           }
         }
       }
@@ -517,8 +515,7 @@ __global__ void __launch_bounds__(128, 3) attend_f32_kernel(AttParams p) {
     if (threadIdx.x == 0) set_status(p.status, LOCKS_ERR_BAD_BLOCK);
     npages = npages < 0 ? 0 : p.kbud;
   }
-  int lo, hi;
-  slice_of(npages, split, p.splits, lo, hi);
+  const int per = slice_length(p, npages), lo = split * per, hi = min(lo + per, npages);
   const float *K = reinterpret_cast<const float *>(p.k), *V = reinterpret_cast<const float *>(p.v);
   const int64_t row0 = (int64_t)b * p.Hq + h * p.G + g0;   // first of the CTA's query heads
   float4 q[NH], o[NH];
@@ -729,7 +726,6 @@ int locks_launch_attend(locks_ctx *c, const void *q, const locks_kv *kv, int bat
   if (bf && !dense && 2 * batch * p.Hkv >= 3 * c->num_sms) splits = 1;
   p.splits = splits;
   p.done = c->att_done;
-  p.fused_merge = (p.G * p.splits <= kFusedMerge) ? 1 : 0;
   // Preferred: the splits of a problem as one thread-block cluster (2, 4, 8 or 16 CTAs) that merges through
   // distributed shared memory, as long as a CTA then has at most 12 tiles per warp to stream (12 x 9K tokens, budget 128
   // pages, 96 problems: step 47.3 us as five splits that the last CTA merges, 43.8 as clusters of four; no case of 14 .. 64
@@ -766,6 +762,12 @@ int locks_launch_attend(locks_ctx *c, const void *q, const locks_kv *kv, int bat
       p.fused_merge = 1;   // no merge launch follows
     }
   }
+  if (!p.cluster) {   // as many slices as the longest list has: 8 problems of 901 pages 24.2 us as 70 splits, 26.7 as 74
+    const int per = (ntiles + splits - 1) / splits;
+    p.splits = (ntiles + per - 1) / per;
+    p.fused_merge = (p.G * p.splits <= kFusedMerge) ? 1 : 0;
+  }
+  p.per_split = (1ull << 32) / p.splits + 1;
   if (bf) {
     const bool contig = kv->stride_token == LOCKS_D;
     const dim3 grid(p.splits, p.Hkv, batch), blk(LOCKS_ATT_WARPS * 32);
@@ -883,7 +885,9 @@ extern "C" int locks_sparse_attend_noalloc(const locks_config *cfg, const void *
   if (splits > most) splits = most;
   if (splits > kNoAllocMaxSplits) splits = kNoAllocMaxSplits;
   if (splits < 1) splits = 1;
-  p.splits = splits;
+  const int per = (npages + splits - 1) / splits;
+  p.splits = (npages + per - 1) / per;
+  p.per_split = (1ull << 32) / p.splits + 1;
   p.sub_shift = 0;
   p.fused_merge = 1;
   p.cluster = 0;

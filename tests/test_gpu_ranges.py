@@ -27,6 +27,27 @@ def test_dense_attention_ragged_rows(lens, Hq, Hkv, B, layout):
     assert gc.status() == 0
 
 
+# The slices of a page list cover it once whatever their number: 128 of one long list, one page to a warp and fewer, lists that
+# end one page into a slice or one before its end, and a row much longer than its requests.  The bound is that of P in bf16.
+@pytest.mark.parametrize("lens,row,Hq,Hkv", [([16 * 8188 + 5], 0, 16, 1), ([16 * 901] * 4, 0, 32, 2), ([16 * 7], 0, 4, 4), ([16 * 297 + 1, 16 * 296], 0, 12, 1),
+                                             ([16 * 149, 16 * 3, 16 * 148 + 1, 9] * 4, 3000, 8, 2), ([16 * 501], 0, 32, 8), ([16 * 60, 16 * 59 + 1] * 20, 500, 28, 4)])
+def test_slices_of_dense_attention(lens, row, Hq, Hkv):
+    import paper_2607_24555_b200 as locks
+    from gpu_util import GpuCase
+    from paper_2607_24555_b200.binding import KVView, make_config
+    gc = GpuCase(locks_synth.Workload("slices", lens, Hq=Hq, Hkv=Hkv, budget=256, seed=Hq + len(lens), tail_fill=float("nan")))
+    want, want_lse = oracle.attend(gc.cache, t2np(gc.case.q), gc.sm)
+    if row:
+        table = torch.zeros(len(lens), row, dtype=torch.int32, device="cuda:0")
+        table[:, :gc.max_pages] = gc.case.block_table
+        gc.ctx = locks.Context(make_config(Hq, Hkv, 8, "i4", "bf16", len(lens), row, 256))
+        gc.kv = KVView(gc.case.k, gc.case.v, gc.case.strides, gc.case.num_blocks, table, gc.case.seq_lens)
+    out, lse = gc.gpu_attend()
+    assert np.abs(out - want).max() <= 2e-2
+    assert np.abs(lse - want_lse).max() <= 1e-3 * max(1.0, np.abs(want_lse).max() / 10)
+    assert gc.status() == 0
+
+
 # Pages of 32 and 64 tokens: weights and sums in fp32.  Sums of 128 products and of a few thousand weighted values are off by
 # 1e-6 of the result at most, a bf16 result's rounding boundary is that near to one value in a thousand; weights rounded to
 # bf16 move a third of the results.
