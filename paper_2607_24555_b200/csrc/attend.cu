@@ -125,7 +125,16 @@ __global__ void __launch_bounds__(LOCKS_ATT_WARPS * 32, LOCKS_ATT_CTAS_PER_SM) a
     if (threadIdx.x == 0) set_status(p.status, LOCKS_ERR_BAD_BLOCK);
     npages = npages < 0 ? 0 : p.kbud;
   }
-  const int per = slice_length(p, npages << (WIDE ? p.sub_shift : 0));
+  // Dense attention slices all requests by the longest of them, so that the CTAs have equally much to do (16 requests of 3K .. 12K
+  // tokens: 82 us in rows of 12K and of 32K tokens; each by its own length 87, by rows of 32K 144).  Not with more than 8 heads:
+  // there the loop over the lengths costs the other loop more (131K tokens 37.3 -> 39.7).
+  int longest = npages;
+  if (NH == 1 && !p.ids) {
+#pragma unroll 1
+    for (int i = lane; i < p.batch; i += 32) longest = max(longest, (p.seq_lens[i] + B - 1) / B);
+    longest = __reduce_max_sync(0xffffffffu, longest);
+  }
+  const int per = slice_length(p, longest << (WIDE ? p.sub_shift : 0));
   const int lo = split * per, hi = min(lo + per, npages << (WIDE ? p.sub_shift : 0));
 
   float oacc[8][NH][4];
