@@ -738,7 +738,8 @@ int locks_launch_attend(locks_ctx *c, const void *q, const locks_kv *kv, int bat
   // Preferred: the splits of a problem as one thread-block cluster (2, 4, 8 or 16 CTAs) that merges through
   // distributed shared memory, as long as a CTA then has at most 12 tiles per warp to stream (12 x 9K tokens, budget 128
   // pages, 96 problems: step 47.3 us as five splits that the last CTA merges, 43.8 as clusters of four; no case of 14 .. 64
-  // requests slower).
+  // requests slower), or 8 where the cluster leaves more than half of the CTAs that there is room for unused (dense, 1 x 8K
+  // tokens: 13.2 us as clusters of 16, 12.4 as 72 splits; with 16 heads, whose splits cost more to merge, 20.5 and 21.4).
   p.cluster = 0;
   if (c->att_clusters[0] < 0) {   // clusters of 2, 4, 8, 16 CTAs of this kernel that fit the device at once (probed once)
     cudaFuncSetAttribute(attend_bf16_kernel<1, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmem);
@@ -765,7 +766,8 @@ int locks_launch_attend(locks_ctx *c, const void *q, const locks_kv *kv, int bat
     // step (4 x 8K tokens, budget 128 pages) against 30.8 as clusters of 8; 24 problems fit, 29.2 against 30.0.
     int i = 3;
     while (i >= 0 && ((2 << i) > splits || c->att_clusters[i] < batch * p.Hkv)) --i;
-    if (i >= 0 && (ntiles + (2 << i) - 1) / (2 << i) <= 12 * LOCKS_ATT_WARPS) {
+    const int most_tiles = i >= 0 && ((4 << i) >= splits || p.G > 8) ? 12 : 8;
+    if (i >= 0 && (ntiles + (2 << i) - 1) / (2 << i) <= most_tiles * LOCKS_ATT_WARPS) {
       p.cluster = 1;
       p.splits = 2 << i;
       p.fused_merge = 1;   // no merge launch follows
