@@ -551,6 +551,11 @@ __global__ void __launch_bounds__(128, 3) attend_f32_kernel(AttParams p) {
           k[t] = *reinterpret_cast<const float4 *>(K + at);
           v[t] = *reinterpret_cast<const float4 *>(V + at);
         }
+        if (t0 + kTok > ntok) {   // ... and values of zero: an infinite one times zero is not zero
+#pragma unroll
+          for (int t = 1; t < kTok; ++t)
+            if (t0 + t >= ntok) v[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
         float s[NV];
 #pragma unroll
         for (int g = 0; g < NH; ++g)

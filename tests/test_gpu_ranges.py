@@ -291,6 +291,23 @@ def test_fp32_scan_and_attention(lens, Hq, Hkv, layout, rank):
     assert np.abs(out - oout).max() <= 2e-5 and np.abs(lse - olse).max() <= 1e-4 * max(1.0, np.abs(olse).max() / 10)
 
 
+# An infinite value makes an output infinite, not undefined, wherever in its tile the token sits: the last token of a page that is
+# not full, of one that is, and one in the middle (bf16 caches of wide pages carry their weights in several parts).
+@pytest.mark.parametrize("dtype,B", [("f32", 16), ("f32", 32), ("bf16", 32), ("bf16", 64)])
+@pytest.mark.parametrize("Hq", [1, 4])
+def test_infinite_values_stay_infinite(dtype, B, Hq):
+    from gpu_util import GpuCase
+    w = locks_synth.Workload("inf", [5 * B + 3, 4 * B - 1, 3 * B], Hq=Hq, Hkv=1, B=B, dtype=dtype, fmt="f32" if dtype == "f32" else "i4", budget=2 * B, seed=B)
+    gc = GpuCase(w)
+    want = torch.from_numpy(oracle.attend(gc.cache, t2np(gc.case.q), gc.sm)[0]).cuda()
+    for b, (page, slot, dim, v) in enumerate([(5, 2, 5, "inf"), (3, B - 2, 70, "-inf"), (1, 9, 127, "inf")]):
+        gc.case.v[int(gc.case.block_table[b, page]), 0, slot, dim] = float(v)
+        want[b, :, dim] = float(v)
+    out, _ = gc.gpu_attend()
+    assert np.array_equal(np.isinf(out), torch.isinf(want).cpu().numpy()) and not np.isnan(out).any()
+    assert np.array_equal(np.sign(out[np.isinf(out)]), torch.sign(want[torch.isinf(want)]).cpu().numpy())
+
+
 # The K largest of up to 8192 keys in list order, ties to the earlier entry (exact: whole numbers against a sort).  Keys that
 # leave the first histogram's threshold bin empty, full or crowded: all equal, two values, a crowd beside far outliers (a
 # range of 32 bits), equal keys across the threshold, a smooth spread; as few as one winner, as many as there are entries.
