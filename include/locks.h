@@ -249,7 +249,8 @@ int locks_selection_quality(locks_ctx *ctx, const float *exact_logmass, const lo
 /* Stage B, sparse paged attention (Sec. 3 "Decode-time attention"; App. E): for every query head,
  * softmax(q.k_i/sqrt(d))-weighted mean of v_i over the tokens i < T_b of the listed pages
  * (split over CTAs, partial results merged by log-sum-exp).  page_ids == NULL: every page, i.e.
- * dense flash-decode over the whole cache (the dense baseline).
+ * dense flash-decode over the whole cache (the dense baseline).  A length or a page count beyond the table's row is
+ * reported (LOCKS_ERR_BAD_BLOCK in the status word); the row is attended.
  *   out [batch][Hq][d] (q_dtype), lse optional [batch][Hq] fp32 (natural log). */
 int locks_sparse_attend(locks_ctx *ctx, const void *q, const locks_kv *kv, int batch,
                         const int32_t *page_ids, const int32_t *page_count, void *out, float *lse,

@@ -121,9 +121,10 @@ __global__ void __launch_bounds__(LOCKS_ATT_WARPS * 32, LOCKS_ATT_CTAS_PER_SM) a
   const int T = p.seq_lens[b];
   const int B = WIDE ? p.B : LOCKS_B;
   int npages = p.ids ? p.cnt[prob] : (T + B - 1) / B;
-  if (p.ids && (npages < 0 || npages > p.kbud)) {   // a count beyond the table's row: use the row, report it
+  const int row = p.ids ? p.kbud : p.Pmax;
+  if ((p.ids && npages < 0) || npages > row) {   // a count or a length beyond the table's row: use the row, report it
     if (threadIdx.x == 0) set_status(p.status, LOCKS_ERR_BAD_BLOCK);
-    npages = npages < 0 ? 0 : p.kbud;
+    npages = npages < 0 ? 0 : row;
   }
   // Dense attention slices all requests by the longest of them, so that the CTAs have equally much to do (16 requests of 3K .. 12K
   // tokens: 82 us in rows of 12K and of 32K tokens; each by its own length 87, by rows of 32K 144).  Not with more than 8 heads:
@@ -132,7 +133,7 @@ __global__ void __launch_bounds__(LOCKS_ATT_WARPS * 32, LOCKS_ATT_CTAS_PER_SM) a
   if (NH == 1 && !p.ids) {
 #pragma unroll 1
     for (int i = lane; i < p.batch; i += 32) longest = max(longest, (p.seq_lens[i] + B - 1) / B);
-    longest = __reduce_max_sync(0xffffffffu, longest);
+    longest = min(__reduce_max_sync(0xffffffffu, longest), p.Pmax);
   }
   const int per = slice_length(p, longest << (WIDE ? p.sub_shift : 0));
   const int lo = split * per, hi = min(lo + per, npages << (WIDE ? p.sub_shift : 0));
@@ -520,9 +521,10 @@ __global__ void __launch_bounds__(128, 3) attend_f32_kernel(AttParams p) {
   const int Tn = p.seq_lens[b];
   const int P = (Tn + p.B - 1) / p.B;
   int npages = p.ids ? p.cnt[prob] : P;
-  if (p.ids && (npages < 0 || npages > p.kbud)) {
+  const int row = p.ids ? p.kbud : p.Pmax;
+  if ((p.ids && npages < 0) || npages > row) {
     if (threadIdx.x == 0) set_status(p.status, LOCKS_ERR_BAD_BLOCK);
-    npages = npages < 0 ? 0 : p.kbud;
+    npages = npages < 0 ? 0 : row;
   }
   const int per = slice_length(p, npages), lo = split * per, hi = min(lo + per, npages);
   const float *K = reinterpret_cast<const float *>(p.k), *V = reinterpret_cast<const float *>(p.v);

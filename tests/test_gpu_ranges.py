@@ -48,6 +48,21 @@ def test_slices_of_dense_attention(lens, row, Hq, Hkv):
     assert gc.status() == 0
 
 
+# A length beyond the table's row is reported, and the row is attended as if the length ended with it: the slices do not depend on
+# pages that do not exist (and no loop walks them).
+@pytest.mark.parametrize("dtype,B,rows,Hq,Hkv", [("bf16", 16, 64, 8, 2), ("bf16", 16, 61, 32, 2), ("bf16", 32, 40, 8, 2), ("f32", 16, 64, 8, 2), ("f32", 16, 500, 32, 8)])
+def test_length_beyond_the_row(dtype, B, rows, Hq, Hkv):
+    from gpu_util import GpuCase
+    gc = GpuCase(locks_synth.Workload("long", [B * rows, B * 30], Hq=Hq, Hkv=Hkv, B=B, dtype=dtype, fmt="f32" if dtype == "f32" else "i4", budget=4 * B, seed=4))
+    want, want_lse = gc.gpu_attend()
+    assert gc.status() == 0
+    for extra in (1, 5 * B, 10_000 * B):
+        gc.case.seq_lens[0] = B * rows + extra
+        out, lse = gc.gpu_attend()
+        assert gc.status() == -6   # LOCKS_ERR_BAD_BLOCK
+        assert np.array_equal(out, want) and np.array_equal(lse, want_lse)
+
+
 # Pages of 32 and 64 tokens: weights and sums in fp32.  Sums of 128 products and of a few thousand weighted values are off by
 # 1e-6 of the result at most, a bf16 result's rounding boundary is that near to one value in a thousand; weights rounded to
 # bf16 move a third of the results.
