@@ -1102,15 +1102,51 @@ __global__ void __launch_bounds__(kScanWarps * 32, kScanCtasPerSm) scan_i4_kerne
 }
 
 // ------------------------------------------------------------------------------------------------
-// int4 summaries of 32- and 64-token pages (B = 8 NT), bf16 queries.  The arithmetic of scan_i4_kernel with the query heads
-// as MMA rows and the codes as the other operand: the projection then comes out as the operand of the logits MMA, with no
-// transpose, and the centroid dots come out in the lanes that finish the pages.  With 8 heads or fewer half of the rows are
-// idle, which these page sizes can afford: half or a quarter as many summaries for the same context.  A warp takes groups
-// of 8 pages in strides; no staging, the loads of a summary (1 .. 1.3 KB) go straight to fragments and other warps cover
-// their latency.  4 x 16K tokens, 32-token pages, 4 heads per KV head (floor 2.4 us): 137 us in the plain kernel, which passes
-// over a summary once per head; the whole step 176 -> 65 us.
+// int4 summaries of 32- and 64-token pages (B = 8 NT), bf16 queries.  The query heads are MMA rows and the codes the other
+// operand: the projection then comes out as the operand of the logits MMA, with no transpose, and the centroid dots come out in
+// the lanes that finish the pages.  With 8 heads or fewer half of the rows are idle, which these page sizes can afford: half or
+// a quarter as many summaries for the same context.  A warp takes groups of 8 pages in strides; no staging, the loads of a
+// summary (1 .. 1.3 KB) go straight to fragments and other warps cover their latency.
+//
+// The scores are as near to fp64 as scan_generic_kernel's, whose work this is (they decide which pages are kept): codes enter
+// as signed whole numbers and the query as its bf16 bits, scaled by a power of two; the projection in three fp16 parts; and since
+// the tensor core truncates what it adds to an accumulator, every product of 16 terms starts from zero and is added in fp32 with
+// rounding.  Logits, exponentials and logarithms are those of the plain kernel.  Mean error of a score over 22 batches: 2.1e-7, the
+// plain kernel 2.9e-7, and 4.3e-7 with scan_i4_kernel's numerics.  Scan and selection of 4 x 400 pages of 32 tokens, 8 KV heads
+// of 4: 20.2 us, of 1 x 1000 pages, 2 of 16: 16.2; with scan_i4_kernel's numerics 18.0 and 14.4, in fp32 arithmetic by halves as
+// scan_f32_kernel does it 23.3 and 22.8, in the plain kernel 132 and 344.
 // ------------------------------------------------------------------------------------------------
 constexpr int kWideWarps = 4;
+
+// A query head as MMA operand registers, as load_q_row has them, but exact: lane (.., t) holds dims 32 t .. 32 t + 31 of `row`, a0[s]
+// dims 4 s, 4 s + 1, a2[s] dims 4 s + 2, 4 s + 3, scaled to 2^13 <= max |q| < 2^14 (elements below 2^-30 of it round).  inv undoes it.
+__device__ __forceinline__ void load_q_row_exact(const __nv_bfloat16 *row, int t, bool valid, uint32_t (&a0)[8], uint32_t (&a2)[8], float &inv) {
+  uint4 v[4] = {};
+  if (valid) {
+    const uint4 *qp = reinterpret_cast<const uint4 *>(row + 32 * t);
+#pragma unroll
+    for (int m = 0; m < 4; ++m) v[m] = __ldg(qp + m);
+  }
+  const uint32_t *w = reinterpret_cast<const uint32_t *>(v);
+  uint32_t mx = 0u;  // largest |q| of the row as a bf16 bit pattern (orders like the value)
+#pragma unroll
+  for (int i = 0; i < 16; ++i) mx = __vmaxu2(mx, w[i] & 0x7FFF7FFFu);
+  mx = max(mx & 0xFFFFu, mx >> 16);
+  mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+  mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+  const float fm = __uint_as_float(mx << 16);
+  int e = 14;
+  if (fm > 0.f && fm < INFINITY) (void)frexpf(fm, &e);   // fm = f 2^e, f in [0.5, 1)
+  e = max(e, -100);
+  const float s = ldexpf(1.f, 14 - e);
+  inv = ldexpf(1.f, e - 14);
+#pragma unroll
+  for (int ks = 0; ks < 8; ++ks) {
+    const uint32_t u0 = w[2 * ks], u1 = w[2 * ks + 1];
+    a0[ks] = pack_f16(__uint_as_float(u0 << 16) * s, __uint_as_float(u0 & 0xFFFF0000u) * s);
+    a2[ks] = pack_f16(__uint_as_float(u1 << 16) * s, __uint_as_float(u1 & 0xFFFF0000u) * s);
+  }
+}
 
 template <int R, int NT, int NH>
 __global__ void __launch_bounds__(kWideWarps * 32) scan_wide_kernel(ScanParams p) {
@@ -1126,19 +1162,25 @@ __global__ void __launch_bounds__(kWideWarps * 32) scan_wide_kernel(ScanParams p
   if (grp * LOCKS_GROUP >= nsc) return;
 
   uint32_t qb0[2][8], qb2[2][8];
-  float inv_s[NH], ksum[NH];
+  float inv[NH];
 #pragma unroll
   for (int hh = 0; hh < 2; ++hh) {
     if (hh < NH) {
       const int g = x + 8 * hh;
-      load_q_row(reinterpret_cast<const __nv_bfloat16 *>(p.q) + ((int64_t)b * p.Hq + h * p.G + g) * LOCKS_D, t, g < p.G, qb0[hh],
-                 qb2[hh], inv_s[hh], ksum[hh]);
-      inv_s[hh] *= p.sm_scale * kLog2e;   // turns a scaled dot product into a log2-domain logit
+      load_q_row_exact(reinterpret_cast<const __nv_bfloat16 *>(p.q) + ((int64_t)b * p.Hq + h * p.G + g) * LOCKS_D, t, g < p.G, qb0[hh],
+                       qb2[hh], inv[hh]);
     } else {
 #pragma unroll
       for (int s = 0; s < 8; ++s) qb0[hh][s] = qb2[hh][s] = 0u;
     }
   }
+  // sum[2 hh], sum[2 hh + 1] (heads x, x + 8) += the products of one k-step
+  auto add_product = [&](float (&sum)[4], int s, uint32_t b0, uint32_t b1) {
+    float c[4];
+    mma_f16_z(c, qb0[0][s], qb0[1][s], qb2[0][s], qb2[1][s], b0, b1);
+#pragma unroll
+    for (int i = 0; i < 2 * NH; ++i) sum[i] = s > 0 ? sum[i] + c[i] : c[i];
+  };
   const int32_t *bt = p.block_table + (int64_t)b * p.Pmax;
   const uint8_t *summ = p.summ + (int64_t)h * S;
   const int64_t page_stride = (int64_t)p.Hkv * S;
@@ -1153,7 +1195,7 @@ __global__ void __launch_bounds__(kWideWarps * 32) scan_wide_kernel(ScanParams p
     const uint32_t valid = __ballot_sync(0xffffffffu, have) & 0xffu;   // pages of the group that are scored
     if (!have) block = 0;
     // ---- centroid dots: columns = pages.  cen: heads x (+ 8), pages 2t, 2t + 1
-    float cen[4] = {0.f, 0.f, 0.f, 0.f};
+    float cen[4];
     float smu;
     {
       const uint8_t *pb = summ + (int64_t)__shfl_sync(0xffffffffu, block, x) * page_stride;
@@ -1162,24 +1204,22 @@ __global__ void __launch_bounds__(kWideWarps * 32) scan_wide_kernel(ScanParams p
       smu = __half2float(*reinterpret_cast<const __half *>(pb + i4_off_smu(R, B)));
       const uint32_t mw[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
 #pragma unroll
-      for (int s = 0; s < 8; ++s) {
-        const uint32_t b0 = f16x2_sub(and_or(mw[s], 0x00FF00FFu, 0x64006400u), 0x64806480u);                    // code
-        const uint32_t b1 = f16x2_fma(and_or(mw[s] >> 8, 0x00FF00FFu, 0x64006400u), 0x4C004C00u, 0xF480F480u);   // 16 * code
-        mma_f16(cen, qb0[0][s], qb0[1][s], qb2[0][s], qb2[1][s], b0, b1);
-      }
+      for (int s = 0; s < 8; ++s)
+        add_product(cen, s, f16x2_sub(and_or(mw[s], 0x00FF00FFu, 0x64006400u), 0x64806480u),
+                    f16x2_sub(and_or(mw[s] >> 8, 0x00FF00FFu, 0x64006400u), 0x64806480u));
     }
-    float res[NH][2];
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
       const float sm = __shfl_sync(0xffffffffu, smu, (2 * t + e) * 4);
 #pragma unroll
-      for (int hh = 0; hh < NH; ++hh) res[hh][e] = cen[2 * hh + e] * sm * inv_s[hh];
+      for (int hh = 0; hh < NH; ++hh) cen[2 * hh + e] *= inv[hh] * sm;
     }
+    float res[NH][2];   // scores of this lane's heads for pages 2t, 2t + 1
 #pragma unroll 2
     for (int pg = 0; pg < LOCKS_GROUP; ++pg) {
       const uint8_t *pb = summ + (int64_t)__shfl_sync(0xffffffffu, block, pg) * page_stride;
       // lane (x, t): basis of rank x, quarter t; coefficients of tokens 8 n + x, ranks 2t, 2t + 1; scales of tokens 8 n + 2t, + 1
-      const uint4 w4 = (R == 8 || x < R) ? *reinterpret_cast<const uint4 *>(pb + lane * 16) : make_uint4(0u, 0u, 0u, 0u);
+      const uint4 w4 = (R == 8 || x < R) ? *reinterpret_cast<const uint4 *>(pb + lane * 16) : make_uint4(0x88888888u, 0x88888888u, 0x88888888u, 0x88888888u);
       uint32_t cw[NT], sc[NT];
 #pragma unroll
       for (int n = 0; n < NT; ++n) {
@@ -1187,52 +1227,63 @@ __global__ void __launch_bounds__(kWideWarps * 32) scan_wide_kernel(ScanParams p
         sc[n] = *reinterpret_cast<const uint32_t *>(pb + i4_off_sc(R, B) + 2 * (8 * n + 2 * t));
       }
       const float2 sv = (t < R / 2) ? h2f2(*reinterpret_cast<const uint32_t *>(pb + i4_off_sv(R, B) + 4 * t)) : make_float2(0.f, 0.f);
-      // ---- projection: rows = heads, columns = ranks
+      // ---- projection: rows = heads, columns = ranks.  A nibble n in the mantissa of 1024 is 1024 + n (less 1032) or 1024 + 16 n
+      // (a sixteenth, less 72): n - 8, exactly
       float c[4];
       const uint32_t wd[4] = {w4.x, w4.y, w4.z, w4.w};
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const uint32_t u = wd[j], u8 = u >> 8;
-        if (j == 0) mma_f16_z(c, qb0[0][0], qb0[1][0], qb2[0][0], qb2[1][0], u & 0x000F000Fu, u & 0x00F000F0u);
-        else mma_f16(c, qb0[0][2 * j], qb0[1][2 * j], qb2[0][2 * j], qb2[1][2 * j], u & 0x000F000Fu, u & 0x00F000F0u);
-        mma_f16(c, qb0[0][2 * j + 1], qb0[1][2 * j + 1], qb2[0][2 * j + 1], qb2[1][2 * j + 1], u8 & 0x000F000Fu, u8 & 0x00F000F0u);
+      for (int s = 0; s < 8; ++s) {
+        const uint32_t u = s & 1 ? wd[s / 2] >> 8 : wd[s / 2];
+        add_product(c, s, f16x2_sub(and_or(u, 0x000F000Fu, 0x64006400u), 0x64086408u),
+                    f16x2_fma(and_or(u, 0x00F000F0u, 0x64006400u), 0x2C002C00u, 0xD480D480u));
       }
-      uint32_t hi[2] = {0u, 0u}, lo[2] = {0u, 0u};
+      // scaled by 2^-6: |c| <= 2^24 and a scale of a unit vector's codes at most 1 / 7, so nothing leaves fp16
+      uint32_t hi[2] = {0u, 0u}, mid[2] = {0u, 0u}, lo[2] = {0u, 0u};
 #pragma unroll
-      for (int hh = 0; hh < NH; ++hh) {   // undo 2^-24, remove the + 8 offset, apply the column scale
-        const float p0 = fmaf(c[2 * hh], 16777216.f, -ksum[hh]) * sv.x, p1 = fmaf(c[2 * hh + 1], 16777216.f, -ksum[hh]) * sv.y;
+      for (int hh = 0; hh < NH; ++hh) {
+        float p0 = c[2 * hh] * (sv.x * 0.015625f), p1 = c[2 * hh + 1] * (sv.y * 0.015625f);
         hi[hh] = pack_f16(p0, p1);
-        const float2 hf = h2f2(hi[hh]);
-        lo[hh] = pack_f16(p0 - hf.x, p1 - hf.y);
+        const float2 f = h2f2(hi[hh]);
+        p0 -= f.x; p1 -= f.y;
+        mid[hh] = pack_f16(p0, p1);
+        const float2 g = h2f2(mid[hh]);
+        lo[hh] = pack_f16(p0 - g.x, p1 - g.y);
       }
-      // ---- logits: rows = heads, k = ranks (hi | lo), columns = tokens
-      float y[NT][4];
+      // ---- logits: rows = heads, k = ranks (hi | mid, then lo), columns = tokens
+      float y[NT][2 * NH], a[NH], mx[NH];
+#pragma unroll
+      for (int hh = 0; hh < NH; ++hh) {
+        const float a0 = __shfl_sync(0xffffffffu, cen[2 * hh], (lane & ~3) + (pg >> 1)), a1 = __shfl_sync(0xffffffffu, cen[2 * hh + 1], (lane & ~3) + (pg >> 1));
+        a[hh] = pg & 1 ? a1 : a0;
+        mx[hh] = -INFINITY;
+      }
 #pragma unroll
       for (int n = 0; n < NT; ++n) {
         const uint32_t cf = f16x2_sub(__byte_perm(cw[n], 0x64646464u, 0x4140), 0x64806480u);
-        mma_f16_z(y[n], hi[0], hi[1], lo[0], lo[1], cf, cf);
+        float z[4], zl[4];
+        mma_f16_z(z, hi[0], hi[1], mid[0], mid[1], cf, cf);
+        mma_f16_z(zl, lo[0], lo[1], 0u, 0u, cf, cf);
+        const float2 s2 = h2f2(sc[n]);
+#pragma unroll
+        for (int hh = 0; hh < NH; ++hh) {
+          const float un = inv[hh] * 64.f;
+          y[n][2 * hh] = p.sm_scale * fmaf((z[2 * hh] + zl[2 * hh]) * un, s2.x, a[hh]);
+          y[n][2 * hh + 1] = p.sm_scale * fmaf((z[2 * hh + 1] + zl[2 * hh + 1]) * un, s2.y, a[hh]);
+          mx[hh] = fmaxf(mx[hh], fmaxf(y[n][2 * hh], y[n][2 * hh + 1]));
+        }
       }
 #pragma unroll
       for (int hh = 0; hh < NH; ++hh) {
-        float my = -INFINITY;
-#pragma unroll
-        for (int n = 0; n < NT; ++n) {
-          const float2 s2 = h2f2(sc[n]);
-          y[n][2 * hh] *= s2.x;
-          y[n][2 * hh + 1] *= s2.y;
-          my = fmaxf(my, fmaxf(y[n][2 * hh], y[n][2 * hh + 1]));
-        }
-        my = fmaxf(my, __shfl_xor_sync(0xffffffffu, my, 1));
-        my = fmaxf(my, __shfl_xor_sync(0xffffffffu, my, 2));
-        const float iv = inv_s[hh], m = my * iv;
+        mx[hh] = fmaxf(mx[hh], __shfl_xor_sync(0xffffffffu, mx[hh], 1));
+        mx[hh] = fmaxf(mx[hh], __shfl_xor_sync(0xffffffffu, mx[hh], 2));
         float e = 0.f;
 #pragma unroll
-        for (int n = 0; n < NT; ++n) e += fast_ex2(fmaf(y[n][2 * hh], iv, -m)) + fast_ex2(fmaf(y[n][2 * hh + 1], iv, -m));
+        for (int n = 0; n < NT; ++n) e += expf(y[n][2 * hh] - mx[hh]) + expf(y[n][2 * hh + 1] - mx[hh]);
         e += __shfl_xor_sync(0xffffffffu, e, 1);
         e += __shfl_xor_sync(0xffffffffu, e, 2);
-        const float v = m + fast_lg2(e);
+        const float v = mx[hh] + logf(e);
         if (t == (pg >> 1)) {
-          if (pg & 1) res[hh][1] += v; else res[hh][0] += v;
+          if (pg & 1) res[hh][1] = v; else res[hh][0] = v;
         }
       }
     }
@@ -1243,16 +1294,19 @@ __global__ void __launch_bounds__(kWideWarps * 32) scan_wide_kernel(ScanParams p
       float pm = -INFINITY, ps = 0.f;
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
-        const float v = res[hh][e] * kLn2;
         const bool in = (valid >> (2 * t + e)) & 1u;
-        if (g < p.G && in) p.shat[((int64_t)b * p.Hq + h * p.G + g) * p.Pmax + page0 + e] = v;
-        lse_accumulate(pm, ps, in && page0 + e >= 1 ? v : -INFINITY);
+        if (g < p.G && in) p.shat[((int64_t)b * p.Hq + h * p.G + g) * p.Pmax + page0 + e] = res[hh][e];
+        if (in && page0 + e >= 1) {
+          const float nm = fmaxf(pm, res[hh][e]);
+          ps = ps * expf(pm - nm) + expf(res[hh][e] - nm);
+          pm = nm;
+        }
       }
 #pragma unroll
       for (int o = 1; o < 4; o <<= 1) {
         const float om = __shfl_xor_sync(0xffffffffu, pm, o), os = __shfl_xor_sync(0xffffffffu, ps, o);
         const float nm = fmaxf(pm, om);
-        if (nm > -INFINITY) { ps = ps * __expf(pm - nm) + os * __expf(om - nm); pm = nm; }
+        if (nm > -INFINITY) { ps = ps * expf(pm - nm) + os * expf(om - nm); pm = nm; }
       }
       if (t == 0 && g < p.G) p.part[((int64_t)b * p.Hq + h * p.G + g) * p.max_groups + grp] = make_float2(pm, ps);
     }

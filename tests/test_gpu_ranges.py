@@ -288,6 +288,29 @@ def test_wide_page_scan(B, lens, Hq, Hkv, rank, qs):
     check_select_and_attend(gc, gc.oracle_summaries(), out_tol=2e-2)
 
 
+# ... and its scores are no further from fp64 than those of the plain kernel in fp32 arithmetic, which scans the same summaries for
+# fp32 queries of the same values.
+@pytest.mark.parametrize("B", [32, 64])
+@pytest.mark.parametrize("lens,Hq,Hkv,rank,qs", [([40, 30], 8, 2, 8, 1.0), ([200], 32, 2, 8, 2.0), ([60], 6, 3, 2, 1.0), ([60], 12, 1, 4, 1.0),
+                                                 ([60], 8, 1, 8, 6.0), ([100], 28, 4, 4, 2.0)])
+def test_wide_page_scan_is_as_accurate_as_fp32(B, lens, Hq, Hkv, rank, qs):
+    import paper_2607_24555_b200 as locks
+    from gpu_util import GpuCase, upload
+    from paper_2607_24555_b200.binding import KVView, make_config
+    w = locks_synth.Workload("wide", [n * B + 3 for n in lens], Hq=Hq, Hkv=Hkv, B=B, rank=rank, budget=6 * B, seed=B + rank, q_scale=qs)
+    gc = GpuCase(w)
+    summ = gc.oracle_summaries()
+    want = oracle.page_logmass(gc.cache, t2np(gc.case.q), rank, gc.fmt, summ, float(np.float32(gc.sm)))
+    fast = gc.gpu_select(upload(summ))[2]
+    plain = GpuCase(w)
+    plain.ctx = locks.Context(make_config(Hq, Hkv, rank, "i4", "f32", w.n, gc.max_pages, w.budget, B=B))
+    k32 = gc.case.k.float()
+    plain.kv = KVView(k32, k32, gc.case.strides, gc.case.num_blocks, gc.case.block_table, gc.case.seq_lens)
+    slow = plain.gpu_select(upload(summ), gc.case.q.float())[2]
+    off = [np.concatenate([np.abs(x[b, :, :n] - want[b, :, :n]).ravel() for b, n in enumerate(lens)]).mean() for x in (fast, slow)]
+    assert off[0] <= off[1], off
+
+
 # fp32 caches and summaries: one query head per KV head, fewer than four, more than four and not a multiple, sixteen; every
 # rank of the fast scan and one beside them; last pages of 1, 8, 9 and 15 tokens, groups of eight pages that end early, splits
 # without pages.  fp32 sums of 128 products: 1e-5 of outputs of a few units, scores 2e-7 of at most a hundred.
