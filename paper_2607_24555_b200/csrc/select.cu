@@ -120,8 +120,8 @@ __device__ __forceinline__ void publish_range(SelShared &sh, uint32_t kmin, uint
 // sh.red), in element order and with ties to the lower element.  Winner number pos of element e is written as
 //   kEmitIds:   ids[1 + pos] = c0 + e                         (final table of a single-chunk problem)
 //   kEmitList:  list_key[pos] = key, list_idx[pos] = c0 + e   (a chunk's candidate list)
-//   kEmitFinal: ids[1 + pos] = page of entry e                (final table from the problem's lists; pages at sh.key[4096 + e]
-//                                                              if there are at most 4096 entries, else in list_idx)
+//   kEmitFinal: ids[1 + pos] = page of entry e                (final table from the problem's lists; pages at sh.key[4096 + e])
+//   kEmitEntry: sh.key[pos] = e                               (the same from more than 4096 entries: see select_finish)
 // The keys' offsets from the smallest one need far fewer than 32 bits (page masses lie within a few units of each other),
 // and one pass over their leading 8 bits usually leaves a few dozen keys in the bin of the K-th largest: these are ranked
 // pair by pair.  A fuller bin is divided again; a bin of equal keys, or one that wins whole, needs no ranking.
@@ -131,7 +131,7 @@ __device__ __forceinline__ void publish_range(SelShared &sh, uint32_t kmin, uint
 // 62.0 -> 58.1, 24 chat requests 59.4 -> 57.1, 1 x 128K (lists of 9 chunks, ranked twice) 42.4 -> 41.2.  Running this code
 // once on made-up keys before the wait for the scan, to have it in the instruction caches, costs 1 .. 6 us: the selector's
 // CTAs become resident only when the scan is nearly over.
-enum { kEmitIds = 0, kEmitList = 1, kEmitFinal = 2 };
+enum { kEmitIds = 0, kEmitList = 1, kEmitFinal = 2, kEmitEntry = 3 };
 constexpr int kFinalPages = kMaxKeys / 2;
 
 __device__ __noinline__ void select_emit(int nslab, int K, int mode, int c0, int32_t *ids, uint32_t *list_key, int32_t *list_idx) {
@@ -247,7 +247,8 @@ __device__ __noinline__ void select_emit(int nslab, int K, int mode, int c0, int
       const int e = w * 32 + __ffs(won) - 1;
       if (mode == kEmitIds) ids[1 + pos] = c0 + e;
       else if (mode == kEmitList) { list_key[pos] = sh.key[e]; list_idx[pos] = c0 + e; }
-      else ids[1 + pos] = list_key ? (int32_t)sh.key[kFinalPages + e] : __ldcg(list_idx + e);
+      else if (mode == kEmitFinal) ids[1 + pos] = (int32_t)sh.key[kFinalPages + e];
+      else sh.key[pos] = (uint32_t)e;   // (the keys are bits of sh.gt and sh.eq by now)
     }
     return;
   }
@@ -289,7 +290,8 @@ __device__ __noinline__ void select_emit(int nslab, int K, int mode, int c0, int
       const int e = i * LOCKS_SEL_THREADS + tid, pos = (pre & 0xffff) + __popc(gw & lt) + min(eq_before, remaining);
       if (mode == kEmitIds) ids[1 + pos] = c0 + e;
       else if (mode == kEmitList) { list_key[pos] = sh.key[e]; list_idx[pos] = c0 + e; }
-      else ids[1 + pos] = list_key ? (int32_t)sh.key[kFinalPages + e] : __ldcg(list_idx + e);
+      else if (mode == kEmitFinal) ids[1 + pos] = (int32_t)sh.key[kFinalPages + e];
+      else sh.key[pos] = (uint32_t)e;   // (the keys are bits of sh.gt and sh.eq by now)
     }
   }
 }
@@ -470,8 +472,19 @@ __device__ __noinline__ void select_finish(int32_t *done, int chunks, int kc, in
     if (key) { kmin = min(kmin, key); kmax = max(kmax, key); }
   }
   publish_range(sh, kmin, kmax);
-  if (K2 > 0)
-    select_emit(nslab, K2, kEmitFinal, 0, ids, pages_too ? sh.key : nullptr, const_cast<int32_t *>(ci));
+  if (K2 > 0) {
+    select_emit(nslab, K2, pages_too ? kEmitFinal : kEmitEntry, 0, ids, nullptr, nullptr);
+    if (!pages_too) {   // the winners' pages, four loads in flight a thread
+      __syncthreads();
+      for (int j0 = tid; j0 < K2; j0 += 4 * LOCKS_SEL_THREADS) {
+        int page[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) page[u] = j0 + u * LOCKS_SEL_THREADS < K2 ? __ldcg(ci + sh.key[j0 + u * LOCKS_SEL_THREADS]) : 0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) if (j0 + u * LOCKS_SEL_THREADS < K2) ids[1 + j0 + u * LOCKS_SEL_THREADS] = page[u];
+      }
+    }
+  }
   if (tid == 0) {
     ids[0] = 0;
     ids[k - 1] = P - 1;

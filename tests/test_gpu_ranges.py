@@ -378,3 +378,29 @@ def test_ranking_of_candidate_lists(parts, kc, kind):
             assert cnt[b, h] == len(best)
             assert np.array_equal(ids[b, h, :len(best)], p[best])
             assert np.all(ids[b, h, len(best):] == -1)
+
+
+# Selection in chunks whose lists together have fewer and more than 4096 entries (where the winners' pages are kept differs), with few
+# and many winners.  All heads score a page alike, in steps that fp32 separates: the table is that of a stable sort.
+@pytest.mark.parametrize("pages,Hq,Hkv,k", [(8448, 32, 2, 128), (20000, 16, 1, 300), (20000, 16, 1, 2000), (40000, 8, 1, 1000), (65792, 32, 2, 128), (65792, 32, 2, 3)])
+def test_selection_from_chunk_lists(pages, Hq, Hkv, k):
+    import paper_2607_24555_b200 as locks
+    from paper_2607_24555_b200.binding import KVView, make_config
+    rng = np.random.default_rng(pages + k)
+    lens = [pages * 16 - 3, (pages - 777) * 16]
+    ctx = locks.Context(make_config(Hq, Hkv, 8, "i4", "bf16", 2, pages, k * 16))
+    dummy = torch.zeros(1, Hkv, 16, 128, dtype=torch.bfloat16, device="cuda:0")
+    kv = KVView(dummy, dummy, (Hkv * 2048, 2048, 128), 1, torch.zeros(2, pages, dtype=torch.int32, device="cuda:0"),
+                torch.tensor(lens, dtype=torch.int32, device="cuda:0"))
+    score = (np.round(3.0 * rng.standard_normal((2, Hkv, 1, pages)) * 64) / 64).astype(np.float32)
+    mass = torch.from_numpy(np.tile(score, (1, 1, Hq // Hkv, 1)).reshape(2, Hq, pages)).cuda()
+    ids = torch.full((2, Hkv, k), -7, dtype=torch.int32, device="cuda:0")
+    cnt = torch.full((2, Hkv), -7, dtype=torch.int32, device="cuda:0")
+    for _ in range(2):
+        ctx.locks_select_scored(torch.full((1, 2, Hq), -2.0, device="cuda:0"), kv, 2, ids, cnt, None, mass)
+    assert ctx.locks_poll_status() == 0 and bool((cnt == k).all())
+    for b, t in enumerate(lens):
+        P = -(-t // 16)
+        for h in range(Hkv):
+            best = 1 + np.sort(np.argsort(-score[b, h, 0, 1:P - 1], kind="stable")[:k - 2])
+            assert np.array_equal(ids[b, h].cpu().numpy(), np.concatenate([[0], best, [P - 1]]))
