@@ -225,14 +225,14 @@ __device__ __forceinline__ void jacobi_phase(const float *mat, float *us, float 
   __syncwarp();
 }
 
-// Physical block of item `lane` (< 8) of this warp, -1 if there is none; page ranges as locks_build_summaries has them.
-__device__ __forceinline__ int item_block(const BuildParams &p, int warp, int lane) {
+// Physical block of item `lane` (< 8) of warp `warp` among those of request b, -1 if there is none; page ranges as
+// locks_build_summaries has them.
+__device__ __forceinline__ int item_block(const BuildParams &p, int b, int warp, int lane) {
   if (lane >= kBuildItems) return -1;
-  const int b = blockIdx.z % p.batch;
   const int complete = p.seq_lens[b] / LOCKS_B;
   const int p0 = p.page_begin ? p.page_begin[b] : 0;
   const int p1 = min(p.page_end ? p.page_end[b] : complete, complete);
-  const int page = p0 + (blockIdx.x * kBuildWarps + warp) * kBuildItems + lane;
+  const int page = p0 + warp * kBuildItems + lane;
   if (page < 0 || page >= p1 || page >= p.Pmax) return -1;
   const int block = p.block_table[(int64_t)b * p.Pmax + page];
   if (block >= 0 && block < p.num_blocks) return block;
@@ -502,11 +502,14 @@ __device__ __forceinline__ void build_i4_group(const BuildParams &p, uint8_t *sm
     }
   }}
 
-// The groups by the table's rows: of 16 pages of a row, 8 a warp.  For tables that are about full.
+// The groups by the table's rows: of 16 pages of a row, 8 a warp.  For tables that are about full, but nothing says that they are:
+// the first pages of all rows come first in the grid, so that the CTAs of pages that are not there start, and end, while the
+// others work (8 requests of 2K tokens in rows of 34 816, us: 119, row after row 146, dealt out 88; 32 of 4K in rows of 32K: 500, 573
+// and 518; rows of 32K that are full: 967, 956 and 991).
 __global__ void __launch_bounds__(kI4Warps * 32, kI4CtasPerSm) build_i4_table_kernel(BuildParams p) {
   extern __shared__ __align__(16) uint8_t smem_raw[];
-  const int lane = threadIdx.x & 31, h = blockIdx.y, layer = blockIdx.z / p.batch;
-  const int it_block = item_block(p, threadIdx.x >> 5, lane);   // lane s < 8: item s
+  const int lane = threadIdx.x & 31, h = blockIdx.x, layer = blockIdx.y / p.batch;
+  const int it_block = item_block(p, blockIdx.y % p.batch, blockIdx.z * kI4Warps + (threadIdx.x >> 5), lane);   // lane s < 8: item s
   const uint32_t live = __ballot_sync(0xffffffffu, it_block >= 0);
   if (!live) return;
   build_i4_group<1>(p, smem_raw, threadIdx.x, it_block, live,
@@ -595,7 +598,7 @@ __global__ void __launch_bounds__(kBuildWarps * 32, kBuildCtasPerSm) build_kerne
   extern __shared__ __align__(16) uint8_t smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int h = blockIdx.y;
-  const int it_block = item_block(p, warp, lane);   // the warp's items: lane s < 8 works out item s
+  const int it_block = item_block(p, blockIdx.z % p.batch, blockIdx.x * kBuildWarps + warp, lane);   // the warp's items: lane s < 8 works out item s
   const uint32_t live = __ballot_sync(0xffffffffu, it_block >= 0);
   if (!live) return;
 
@@ -1189,13 +1192,14 @@ int locks_launch_build(locks_ctx *c, const locks_kv *kv, int batch, const int32_
     case LOCKS_FMT_I4:
       if (bf) {
         // Rows that can all be full (no page ranges, and a pool that holds them) and are many waves long are taken as they
-        // are: finding a group's place costs 3 % (8 x 32K tokens, 8 KV heads: 1094 us against 1126).  Otherwise the CTAs of
-        // empty rows cost more, in launches and in how the others are spread: a chunk of 128 of 512 pages in 32 layers, 386
-        // us by rows against 343.
+        // are: finding a group's place costs 3 % (8 x 32K tokens, 8 KV heads: 1094 us against 1126).  A pool can hold more than
+        // the batch uses; the grid's order then keeps most of what dealing out would save (build_i4_table_kernel).  Otherwise the
+        // CTAs of empty rows cost more, in launches and in how the others are spread: a chunk of 128 of 512 pages in 32
+        // layers, 386 us by rows against 343.
         const int layers = k_layers ? num_layers : 1;
         const int64_t rows = (int64_t)batch * c->Pmax, most = (int64_t)((c->Pmax + kBuildItems - 1) / kBuildItems) * p.Hkv * batch * layers;
-        if (!pb && 4 * rows <= 5 * (int64_t)kv->num_blocks && most > 64 * (int64_t)c->num_sms)
-          build_i4_table_kernel<<<grid, kI4Warps * 32, kI4Smem, st>>>(p);
+        if (!pb && 4 * rows <= 5 * (int64_t)kv->num_blocks && most > 64 * (int64_t)c->num_sms && grid.x <= 65535)
+          build_i4_table_kernel<<<dim3(p.Hkv, batch * layers, grid.x), kI4Warps * 32, kI4Smem, st>>>(p);
         else
         {
           // A CTA per two groups, as many as the pool's blocks can make up: rounds of a smaller grid let the warps drift apart

@@ -276,6 +276,31 @@ def test_bulk_build_is_dealt_out_in_several_ways():
         assert torch.equal(builds[0][once], other[once])
 
 
+# Short requests in long rows and a pool that could fill them: the same bytes as by page ranges, nothing outside, whatever takes them.
+def test_bulk_build_of_short_requests_in_a_large_pool():
+    import paper_2607_24555_b200 as locks
+    from paper_2607_24555_b200.binding import KVView, make_config
+    dev, hkv, row, nb = torch.device("cuda:0"), 8, 2176, 14_000
+    lens = [2048, 16 * 7 + 15, 0, 16 * 8, 2100, 16 * 9, 1, 16 * 129]
+    ctx = locks.Context(make_config(16, hkv, 8, "i4", "bf16", 8, row, 256), device=dev)
+    gen = torch.Generator(device=dev).manual_seed(8)
+    table = torch.full((8, row), -1, dtype=torch.int32, device=dev)   # slots past a request's pages are not looked at
+    used = torch.randperm(nb, generator=gen, device=dev)[:sum(-(-t // 16) for t in lens)].to(torch.int32)
+    at = 0
+    for b, t in enumerate(lens):
+        table[b, :-(-t // 16)] = used[at:at - (-t // 16)]
+        at += -(-t // 16)
+    k = torch.zeros(nb, hkv, 16, 128, dtype=torch.bfloat16, device=dev)
+    k[used.long()] = torch.randn(len(used), hkv, 16, 128, generator=gen, device=dev).to(torch.bfloat16)
+    kv = KVView(k, k, (hkv * 2048, 2048, 128), nb, table, torch.tensor(lens, dtype=torch.int32, device=dev))
+    whole, ranges = ctx.new_summaries(nb), ctx.new_summaries(nb)
+    ctx.locks_build_summaries(kv, 8, whole)
+    ctx.locks_build_summaries(kv, 8, ranges, torch.zeros(8, dtype=torch.int32, device=dev), torch.full((8,), row, dtype=torch.int32, device=dev))
+    assert ctx.locks_poll_status() == 0
+    assert torch.equal(whole, ranges)
+    assert int((whole.view(nb, -1) != 0).any(1).sum()) == sum(t // 16 for t in lens)
+
+
 # The scan of int4 summaries at 32- and 64-token pages: every rank, one and two tiles of query heads, group sizes that fill
 # neither, sequences that end inside a group of eight pages, more groups than warps (strides), extreme logits.
 @pytest.mark.parametrize("B", [32, 64])
