@@ -134,11 +134,12 @@ template <int B> __device__ __forceinline__ void solve_modes(PageShared<B> &sh, 
 #pragma unroll 1
   for (int sweep = 0; sweep < (B == LOCKS_B ? 1 : 2) * LOCKS_BUILD_SWEEPS; ++sweep) {
     ranks();
-    // pairs count for the stop test if one of them is among the r largest columns and neither is rounding noise beside
-    // the largest (squared norm = squared eigenvalue: modes below 3e-6 of the largest)
+    // pairs count for the stop test if one of them is among the r largest columns and neither is below the modes that are
+    // kept (squared norm = squared eigenvalue: those above 1e-6 of the largest are).  A mode that is kept before its column has met
+    // the largest one leans on it, and its basis vector, divided by its own small singular value, grows up to 300 times too long.
     const uint32_t b0 = __float_as_uint(n[0]), b1 = __float_as_uint(n[1]);
     const float top = __uint_as_float(__reduce_min_sync(0xffffffffu, min(rank[0] < r ? b0 : 0x7F7FFFFFu, rank[1] < r ? b1 : 0x7F7FFFFFu))) * 0.999f;
-    const float floor_n = 1e-11f * __uint_as_float(__reduce_max_sync(0xffffffffu, max(b0, b1)));
+    const float floor_n = 5e-13f * __uint_as_float(__reduce_max_sync(0xffffffffu, max(b0, b1)));
     // Odd-even transposition: a rotated pair swaps places, which lets every two columns meet once in B steps.  w[0] is the
     // column that a pair keeps from the step before, w[1] the one that it has been passed; which of the two is the lower
     // position alternates, and so do the signs of the rotation and of the swap, which leaves one formula for every step.

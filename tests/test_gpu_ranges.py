@@ -193,6 +193,30 @@ def test_bulk_build_partial_warps_and_degenerate_pages(rank, layout):
     assert differ <= 2e-3 * total, (differ, total)
 
 
+# Modes just above the threshold below which they are dropped (an eigenvalue of 1e-6 of the largest): they are kept, so they have to
+# have converged.  Their eigenvalues are known to 3 % in fp32, and the lengths of their basis vectors to half of that.
+@pytest.mark.parametrize("B", [16, 32, 64])
+@pytest.mark.parametrize("r", [2, 4, 8])
+def test_step_build_of_weak_modes(B, r):
+    import paper_2607_24555_b200 as locks
+    from paper_2607_24555_b200.binding import KVView, make_config
+    n, gen = 512, torch.Generator().manual_seed(B + r)
+    U = torch.linalg.qr(torch.cat([torch.ones(n, B, 1), torch.randn(n, B, 7, generator=gen)], 2).double())[0][:, :, 1:]   # centred
+    V = torch.linalg.qr(torch.randn(n, 128, 7, generator=gen).double())[0]
+    sv = (torch.rand(n, 7, generator=gen) * 1.5e-6 + 1.3e-6).sqrt()
+    sv[:, 0] = 1.0
+    keys = ((U * sv[:, None]) @ V.transpose(1, 2)).float().cuda()[:, None].contiguous()
+    ctx = locks.Context(make_config(2, 1, r, "f32", "f32", n, 3, 2 * B, B=B))
+    kv = KVView(keys, keys, (B * 128, B * 128, 128), n, torch.arange(n, dtype=torch.int32, device="cuda:0")[:, None].repeat(1, 3).contiguous(),
+                torch.full((n,), B, dtype=torch.int32, device="cuda:0"))
+    summ, q = ctx.new_summaries(n), torch.zeros(n, 2, 128, device="cuda:0")
+    ctx.locks_decode_step(q, None, None, kv, summ, n, torch.empty_like(q))
+    assert ctx.locks_poll_status() == 0
+    basis = summ.view(n, -1).view(torch.float32)[:, 128:128 + 128 * r].reshape(n, r, 128).norm(dim=2)
+    assert bool((basis[:, 0] - 1).abs().max() < 5e-5)   # the fp32 Gram matrix: 2^-24 x sqrt(128 B) x 4 deviations at B = 64
+    assert bool(((basis == 0) | ((basis - 1).abs() < 0.1)).all()), basis.max()
+
+
 def _bulk_bytes_by_key_type(keys, rank):
     """int4 summaries of pages [n, 16, 128] in one head: from bf16 keys (build_i4_group) and from the same values in fp32
     (build_kernel), which computes in the same order."""
