@@ -217,6 +217,60 @@ def test_step_build_of_weak_modes(B, r):
     assert bool(((basis == 0) | ((basis - 1).abs() < 0.1)).all()), basis.max()
 
 
+# The quantised formats of the page that a decode step fills, the last row being the step's own token.  The buffer is full of ones
+# before: a byte that is not written shows.  Ordinary pages against the oracle's fp64 build: everything within one code of it once a
+# mode's sign is settled, and one byte in a thousand different (bf16 entries: one in 200).  Pages whose bases are arbitrary inside an
+# eigenspace: the reconstruction, as good as the oracle's but for half an int4 step (1/14 of an entry).
+@pytest.mark.parametrize("B", [16, 32, 64])
+@pytest.mark.parametrize("fmt", ["i4", "i8", "bf16"])
+def test_step_build_of_a_filled_page_in_every_format(fmt, B):
+    from common import oracle_cache
+    from gpu_util import GpuCase
+    kinds = [None] * 8 + ["identical", "rank1", "orthogonal", "two_keys", "blocks"]
+    for r in (2, 4, 8):
+        w = locks_synth.Workload("fill", [B * (2 + i % 3) for i in range(len(kinds))] + [2 * B + 5], Hq=4, Hkv=2, B=B, fmt=fmt, rank=r, budget=2 * B, seed=B + r)
+        gc = GpuCase(w)
+        rng = np.random.default_rng(B * 10 + r)
+        kn, vn, qn = locks_synth.new_token(w, 0, device="cuda:0")
+        blocks = [int(gc.case.block_table[b, -(-t // B) - 1]) for b, t in enumerate(w.seq_lens)]
+        for b, kind in enumerate(kinds):
+            page = None if kind is None else torch.from_numpy(np.stack([_page_keys(kind, B, rng) for _ in range(2)])).to(gc.case.k)
+            if kind is not None:
+                gc.case.k[blocks[b]] = page
+            kn[b] = gc.case.k[blocks[b], :, B - 1] if page is None else page[:, B - 1]
+            gc.case.k[blocks[b], :, B - 1] = 100.0   # the step writes this row
+        gc.case.seq_lens -= 1
+        summ = torch.full_like(gc.ctx.new_summaries(gc.case.num_blocks), 255)
+        out = torch.empty(w.n, w.Hq, w.d, dtype=torch.bfloat16, device="cuda:0")
+        gc.ctx.locks_decode_step(qn, kn, vn, gc.kv, summ, w.n, out)
+        assert gc.status() == 0
+        gc.cache = oracle_cache(gc.case)
+        want, got = gc.oracle_summaries(), summ.cpu().numpy()
+        assert np.array_equal(np.flatnonzero((got != 255).reshape(len(got), -1).any(1)), np.sort(blocks[:len(kinds)]))
+        payload = oracle.summary_payload_bytes(gc.fmt, r, B, w.d)
+        total = differ = 0
+        for b, kind in enumerate(kinds):
+            for h in range(2):
+                g_blob, o_blob = got[blocks[b], h], want[blocks[b], h]
+                assert not g_blob[payload:].any()
+                g, o = oracle.unpack(gc.fmt, r, g_blob, B, w.d), oracle.unpack(gc.fmt, r, o_blob, B, w.d)
+                step = {"i4": 1 / 7, "i8": 1 / 127, "bf16": 1 / 128}[fmt] * 1.01
+                assert np.abs(g[0] - o[0]).max() <= np.abs(o[0]).max() / 126
+                if kind is not None:
+                    k = gc.case.k[blocks[b], h].double().cpu().numpy()
+                    D = k - k.mean(0)
+                    worse = np.linalg.norm(D - g[2] @ g[1]) - np.linalg.norm(D - o[2] @ o[1])
+                    assert worse <= 0.1 * max(np.linalg.norm(D), 1e-6), (kind, worse)
+                    continue
+                flip = np.where((g[1] * o[1]).sum(1) < 0, -1.0, 1.0)
+                assert (np.abs(g[1] * flip[:, None] - o[1]).max(1) <= step * np.abs(o[1]).max(1)).all()
+                assert (np.abs(g[2] * flip - o[2]).max(1) <= 1.01 / 127 * np.abs(o[2]).max(1)).all()
+                if (flip > 0).all():
+                    total += payload
+                    differ += int((g_blob[:payload] != o_blob[:payload]).sum())
+        assert total > 0 and differ <= (5e-3 if fmt == "bf16" else 1e-3) * total, (differ, total)
+
+
 def _bulk_bytes_by_key_type(keys, rank):
     """int4 summaries of pages [n, 16, 128] in one head: from bf16 keys (build_i4_group) and from the same values in fp32
     (build_kernel), which computes in the same order."""
