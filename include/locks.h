@@ -119,7 +119,8 @@ size_t locks_workspace_bytes(const locks_config *cfg);
  * host object; *out must be released with locks_destroy().  Errors: INVALID_ARG (bad field, NULL),
  * UNSUPPORTED (shape the kernels do not cover: d != 128, B not in {16, 32, 64}, G > 16, mixed dtypes, I4 rank not
  * in {2,4,8}), WORKSPACE (ws_bytes too small or misaligned).  Pages of 32 and 64 tokens: build, select, attend and
- * the decode step (bf16 attention and scans of I4 summaries on the tensor cores, the rest plain fp32 kernels); the
+ * the decode step (bf16 attention and scans of I4 summaries on the tensor cores, with the accuracy of fp32
+ * arithmetic: attention weights are not rounded to bf16 as at 16 tokens; the rest plain fp32 kernels); the
  * diagnostics, the KV fake quantiser, the page-sharded calls, the multi-layer build and the allocation-free
  * attention entry point return UNSUPPORTED for them. */
 int locks_create(const locks_config *cfg, void *workspace, size_t ws_bytes, locks_ctx **out);
@@ -262,7 +263,9 @@ int locks_sparse_attend(locks_ctx *ctx, const void *q, const locks_kv *kv, int b
  *      if k_new == NULL the cache and seq_lens already include the token being decoded;
  *   2. locks_select on the resident summaries;  3. locks_sparse_attend on the selected pages;
  *   4. if a page became complete at this step (T_b % B == 0) build its summary, so that it is a
- *      candidate from the next step on (the newly written token is never scored, App. E(i)).
+ *      candidate from the next step on (the newly written token is never scored, App. E(i)).  Its bytes may differ
+ *      from those that locks_build_summaries gives for the same page, in about one of ten thousand (another solver,
+ *      as accurate).
  * These are the results; inside, the token is counted from the first kernel on, its rows are written by
  * the selector's kernel (no page summary depends on them) and seq_lens is stored back there, so the
  * append costs no launch of its own.  k_new / v_new: device, 16-byte aligned.  A sequence whose

@@ -49,7 +49,7 @@ Layout make_layout(const locks_config *c) {
   // KV head) problems and a context of up to 8192 pages, one CTA ranks a whole problem.  Otherwise a problem is
   // cut into chunks whose top-(k-2) lists are ranked by the chunk that arrives last, and the chunk size is the
   // one a small cost model likes best (microseconds, fitted to measurements on B200 at 2 .. 256 problems,
-  // G = 4 .. 16, 8K .. 64K pages): a CTA's chain of round trips costs about 6 plus 1.2 per batch of 16 score
+  // G = 4 .. 16, 8K .. 64K pages, of a selector that ranked by three radix passes; not fitted again since): a CTA's chain of round trips costs about 6 plus 1.2 per batch of 16 score
   // loads per thread beyond the first one and a half, plus 0.15 per 512 pages; the CTAs of a launch run in
   // waves of one per SM; the final ranking costs 3.3 plus 0.43 per 512 candidates.
   const int per_thread = (c->max_pages_per_seq + LOCKS_SEL_THREADS - 1) / LOCKS_SEL_THREADS;

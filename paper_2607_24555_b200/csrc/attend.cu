@@ -1,11 +1,12 @@
 // Stage B: sparse paged attention over the selected pages (Sec. 3 "Decode-time attention", App. E):
 //   o_g = sum_i softmax_i(q_g . k_i / sqrt(d)) v_i   over tokens i < T of the pages in the table,
-// computed split-K: every CTA takes a slice of the page list, every warp streams whole pages
-// (K tile 16x128 + V tile 16x128) through its own two-stage shared-memory ring with 16-byte async
-// copies into an XOR-swizzled layout, scores them with m16n8k16 bf16 MMAs (the G query heads of the
-// KV head are the M rows), keeps a running (max, sum, O) per head, and the CTA merges its warps by
-// log-sum-exp.  Partial (o, lse) per split are merged by a second small kernel.
-// A NULL page table means "all pages": the same kernel is the dense flash-decode baseline.
+// computed split-K: every CTA takes a slice of the page list, every warp streams tiles of 16 tokens
+// (K 16x128 + V 16x128) through its own two-stage shared-memory ring with 16-byte async
+// copies into an XOR-swizzled layout, scores them with m16n8k16 bf16 MMAs (tokens are the rows, the G query heads
+// of the KV head the columns), keeps a running (max, sum, O) per head, and the CTA merges its warps by
+// log-sum-exp.  The splits of a problem are merged by the thread-block cluster that they form, by the CTA that
+// arrives last, or by a second small kernel.  fp32 caches: attend_f32_kernel.
+// A NULL page table means "all pages": the same kernels are the dense flash-decode baseline.
 #include <cooperative_groups.h>
 #include <mutex>
 #include "locks_internal.cuh"

@@ -16,7 +16,10 @@
 //
 // The bytes of a summary decide near-ties between pages, so what is computed and in which order is kept exactly: a
 // preconditioned solver (build_page.cu's; 5 sweeps for 8) builds 131 008 page-heads in 870 us and is as accurate, but one
-// byte in ten thousand comes out differently, and one request in a few hundred then keeps another page.
+// byte in ten thousand comes out differently, and one request in a few hundred then keeps another page.  The page that a step
+// fills is built with that solver: a bulk build of the same page gives other bytes at that rate.
+// A mode between 1e-6 and 3e-6 of the largest is kept, but does not hold up the sweeps (floor_n), so its basis vector may be too
+// long; on such pages the step build is the more accurate one.
 // Bound by instruction issue, fetch and latency, not by bytes (an eigenproblem per 4 KB page).  131 008 page-heads: 1348 us
 // with the pair that straddles two lanes rotated by both and all formats in one kernel (6 960 warp instructions each), 1281
 // us with every pair rotated once and build_i4_kernel's phases (5 370), 1095 us with the body of a sweep kept to two steps.
@@ -587,8 +590,8 @@ __global__ void __launch_bounds__(kI4Warps * 32, kI4CtasPerSm) build_i4_kernel(B
   __syncthreads();
   const int groups = *count;
   if (groups == 0) return;
-  // Two warps a group up to three waves of single ones: us with one / two at 128 groups 104 / 80, 1024: 168 / 131, 2048: 216 /
-  // 201, 3072: 294 / 284, 4096: 348 / 349, 16 376: 1126 / 1153.
+  // Two warps a group up to 22 groups per SM (1.4 waves of single ones, 2.8 of pairs): us with one / two at 128 groups 104 / 80,
+  // 1024: 168 / 131, 2048: 216 / 201, 3072: 294 / 284, 4096: 348 / 349, 16 376: 1126 / 1153.
   if ((int64_t)groups * layers <= (int64_t)kI4Pairs * sms) build_i4_groups<2>(p, smem_raw, count, layers);
   else build_i4_groups<1>(p, smem_raw, count, layers);
 }
@@ -1155,7 +1158,7 @@ int locks_launch_build(locks_ctx *c, const locks_kv *kv, int batch, const int32_
     const locks_scan_geom geo = locks_scan_geometry(c, batch);
     p.hint = c->hint_dev; p.hint_wpp = geo.wpp; p.hint_rounds = geo.rounds; p.hint_W = geo.W;
   }
-  if (just_filled) return locks_launch_build_pages(c, p, st);   // a step's few pages: latency counts, one CTA per page
+  if (just_filled) return locks_launch_build_pages(c, p, st);   // a step's few pages: latency counts
   if (c->B != LOCKS_B) {   // pages of 32 / 64 tokens: the plain kernel (row-major formats; one layer per launch)
     if (k_layers) return LOCKS_ERR_UNSUPPORTED;
     const int B = c->B, smem = build_wide_smem(B);

@@ -1,5 +1,7 @@
 // Summary build of the pages that a decode step has just filled (any page size).  The method is that of build.cu (Sec. 4
-// "Build"); here the latency of one page counts, because the step that filled it ends with its summary.
+// "Build"); here the latency of one page counts, because the step that filled it ends with its summary.  The solver is another
+// one, so a bulk build of the same page differs in about one byte in ten thousand (this one is the nearer to fp64: 7e-5 of the
+// bytes differ from such a build, of the bulk build's 1.2e-4).
 //
 // What bounds it is one dependent chain, the eigenproblem of the B x B Gram matrix M.  One warp solves it by one-sided
 // Jacobi in registers: a pair of columns belongs to L lanes that hold B / L rows of both, so a step (B / 2 pairs at once)

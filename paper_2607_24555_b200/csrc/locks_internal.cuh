@@ -222,7 +222,7 @@ static inline int locks_check_launch(locks_ctx *c) {
 // Function attributes (dynamic shared-memory limit, non-portable cluster size) belong to a device, not to the
 // process: true exactly once per (current device, kernel family), so that a process that drives several GPUs
 // sets them on each.  Thread-safe.
-enum { LOCKS_ATTR_SELECT = 0, LOCKS_ATTR_ATTEND = 1, LOCKS_ATTR_EXACT = 3, LOCKS_ATTR_BUILD = 4 /* + format */, LOCKS_ATTR_SCAN = 8,
+enum { LOCKS_ATTR_SELECT = 0, LOCKS_ATTR_ATTEND = 1, LOCKS_ATTR_EXACT = 3, LOCKS_ATTR_SCAN = 8,
        LOCKS_ATTR_BUILD_PAGE = 20 /* + page size / 32 */, LOCKS_ATTR_BUILD_WIDE = 24 /* + format */ };
 bool locks_attrs_needed(int family);
 

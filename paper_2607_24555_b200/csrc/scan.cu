@@ -3,13 +3,17 @@
 // for every page j <= P-2 of every request and every query head g, plus a per-(head, 8-page group)
 // partial (max, sum exp) over the candidate pages 1..P-2 that the selector turns into log Z_g.
 //
-// Two kernels:
-//   scan_generic_kernel   any format / rank / dtype, plain fp32 ALU arithmetic (parity config, fallback
-//                         shapes).  One warp per group of 8 pages.
-//   scan_i4_kernel<R>     the bytes-bound path for int4/int8 blobs of rank R = 2, 4, 8 with bf16 queries (ranks
-//                         below 8 run the rank-8 tile with the missing ranks fed as zeros).  Persistent warps,
-//                         each streaming groups of 8 blobs through its own shared-memory ring with bulk
-//                         async copies (TMA engine) and mbarriers, no CTA-wide synchronisation.  Per page pair:
+// Four kernels:
+//   scan_generic_kernel   any format / rank / dtype / page size, plain fp32 ALU arithmetic: int8 and bf16 bases, other
+//                         ranks, fp32 queries on int4 summaries, the rival scorers.  One warp per group of 8 pages.
+//   scan_f32_kernel       fp32 summaries of rank 2, 4, 8 at 16-token pages: the same arithmetic, four heads at a time.
+//   scan_wide_kernel      int4 summaries of rank 2, 4, 8 at 32- and 64-token pages with bf16 queries, on the tensor cores:
+//                         query heads as MMA rows.
+//   scan_i4_kernel<R>     the bytes-bound path: int4 summaries of rank R = 2, 4, 8 at 16-token pages with bf16 queries.
+//                         Persistent warps, each streaming groups of 8 blobs through its own shared-memory ring with bulk
+//                         async copies (TMA engine) and mbarriers, no CTA-wide synchronisation.  More than 8 heads per KV
+//                         head are MMA rows, page by page.  Up to 8 are columns; ranks below 8 run the rank-8 tile with the
+//                         missing ranks fed as zeros (ranks 2 and 4 with up to 4 heads: several pages to a tile).  Per page pair:
 //                           MMA#1  P[2 pages x 8 ranks, heads] = codesV[16 x d] . q^T[d x heads]   (8 x m16n8k16 fp16)
 //                         per page, after an 8x8 movmatrix transpose of the fp16 hi/lo projection:
 //                           MMA#2  L[heads, tokens] = (P_hi | P_lo)[heads x 16] . codesC^T          (2 x m16n8k16 fp16)

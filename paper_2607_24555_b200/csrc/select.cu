@@ -78,7 +78,7 @@ constexpr int kElemBits = 13;    // kMaxKeys = 2^13 elements
 
 struct SelShared {
   uint32_t key[kMaxKeys];             // order-preserving keys, element i of thread t at i*512 + t; 0 = not a candidate
-  int hist[3 * 256];                  // radix histograms, rotating
+  int hist[3 * 256];                  // histograms of the key offsets' leading bits, rotating
   __align__(16) uint32_t gt[256];     // winners, one bit per element in element order
   __align__(16) uint32_t eq[256];     // elements of the threshold bin, where it holds equal keys or wins whole
   __align__(16) uint32_t list[kListMax];
