@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(LOCKS_ATT_WARPS * 32, LOCKS_ATT_CTAS_PER_SM) a
   pdl_wait();   // page table from the selector, appended K/V rows, sequence lengths
   const int T = p.seq_lens[b];
   const int B = WIDE ? p.B : LOCKS_B;
-  int npages = p.ids ? p.cnt[prob] : (T + B - 1) / B;
+  int npages = p.ids ? p.cnt[prob] : max((T + B - 1) / B, 0);
   const int row = p.ids ? p.kbud : p.Pmax;
   if ((p.ids && npages < 0) || npages > row) {   // a count or a length beyond the table's row: use the row, report it
     if (threadIdx.x == 0) set_status(p.status, LOCKS_ERR_BAD_BLOCK);
@@ -520,8 +520,7 @@ __global__ void __launch_bounds__(128, 3) attend_f32_kernel(AttParams p) {
   pdl_wait();
   const int64_t prob = (int64_t)b * p.Hkv + h;
   const int Tn = p.seq_lens[b];
-  const int P = (Tn + p.B - 1) / p.B;
-  int npages = p.ids ? p.cnt[prob] : P;
+  int npages = p.ids ? p.cnt[prob] : max((Tn + p.B - 1) / p.B, 0);
   const int row = p.ids ? p.kbud : p.Pmax;
   if ((p.ids && npages < 0) || npages > row) {
     if (threadIdx.x == 0) set_status(p.status, LOCKS_ERR_BAD_BLOCK);

@@ -63,6 +63,19 @@ def test_length_beyond_the_row(dtype, B, rows, Hq, Hkv):
         assert np.array_equal(out, want) and np.array_equal(lse, want_lse)
 
 
+# A length of zero or less attends nothing: zeros, and a log-sum-exp of minus infinity.
+@pytest.mark.parametrize("dtype,B,Hq", [("bf16", 16, 8), ("bf16", 16, 32), ("bf16", 64, 8), ("f32", 16, 8)])
+def test_length_of_nothing(dtype, B, Hq):
+    from gpu_util import GpuCase
+    gc = GpuCase(locks_synth.Workload("none", [B * 40, B * 30, B * 20], Hq=Hq, Hkv=2, B=B, dtype=dtype, fmt="f32" if dtype == "f32" else "i4", budget=4 * B, seed=4))
+    want, want_lse = gc.gpu_attend()
+    gc.case.seq_lens[0], gc.case.seq_lens[2] = 0, -1000 * B
+    out, lse = gc.gpu_attend()
+    assert not out[[0, 2]].any() and np.isneginf(lse[[0, 2]]).all()
+    assert np.abs(out[1] - want[1]).max() <= 2e-2 and np.abs(lse[1] - want_lse[1]).max() <= 1e-5 * np.abs(want_lse[1]).max()
+    assert gc.status() == 0
+
+
 # Pages of 32 and 64 tokens: weights and sums in fp32.  Sums of 128 products and of a few thousand weighted values are off by
 # 1e-6 of the result at most, a bf16 result's rounding boundary is that near to one value in a thousand; weights rounded to
 # bf16 move a third of the results.
