@@ -483,7 +483,8 @@ int locks_decode_step(locks_ctx *ctx, const void *q, const void *k_new, const vo
                                k_new ? ctx->seq_eff + batch : nullptr, ctx->side)) != LOCKS_OK)
     return rc;
   if (cudaEventRecord(ctx->ev_join, ctx->side) != cudaSuccess) return LOCKS_ERR_CUDA;
-  if ((rc = locks_launch_select(ctx, ctx->shat, &kv_step, batch, ids, cnt, nullptr, k_new ? &app : nullptr, st)) != LOCKS_OK)
+  if ((rc = locks_launch_select(ctx, ctx->shat, &kv_step, batch, ids, cnt, nullptr, k_new ? &app : nullptr, st,
+                                locks_attend_fills(ctx, batch))) != LOCKS_OK)
     return rc;
   mark(2);
   if ((rc = locks_launch_attend(ctx, q, &kv_step, batch, ids, cnt, out, nullptr, st)) != LOCKS_OK) return rc;

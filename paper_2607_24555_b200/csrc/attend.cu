@@ -713,41 +713,32 @@ int locks_launch_merge_shards(locks_ctx *c, const void *part_out, const float *p
   return locks_check_launch(c);
 }
 
-int locks_launch_attend(locks_ctx *c, const void *q, const locks_kv *kv, int batch, const int32_t *ids,
-                        const int32_t *cnt, void *out, float *lse, cudaStream_t st) {
-  AttParams p;
-  p.q = q; p.k = kv->k; p.v = kv->v; p.sb = kv->stride_block; p.sh = kv->stride_head; p.st = kv->stride_token;
-  p.block_table = kv->block_table; p.seq_lens = kv->seq_lens; p.ids = ids; p.cnt = cnt;
-  p.part_o = c->att_o; p.part_lse = c->att_lse; p.out = out; p.lse = lse; p.status = c->status;
-  p.batch = batch; p.Hq = c->cfg.num_q_heads; p.Hkv = c->cfg.num_kv_heads; p.G = c->G; p.Pmax = c->Pmax;
-  p.kbud = c->k; p.num_blocks = kv->num_blocks; p.sm_scale = c->cfg.sm_scale; p.B = c->B; p.kvdiv = 1;
-  if (c->cfg.combine == LOCKS_COMBINE_PER_HEAD && ids) {   // one page table per query head: groups of one
-    p.kvdiv = p.G; p.Hkv = p.Hq; p.G = 1;
-  }
-  const bool dense = ids == nullptr;
+namespace {
+
+// How the problems of a launch are cut: splits per problem, and how these are merged.
+struct AttGeom { int splits, cluster, fused_merge; };
+
+AttGeom attend_geometry(locks_ctx *c, int batch, int Hkv, int G, bool dense) {
   const bool bf = c->cfg.kv_dtype == LOCKS_BF16;   // tensor-core kernel
-  const bool wide = c->B != LOCKS_B;
-  p.sub_shift = !bf ? 0 : (c->B == 64 ? 2 : (c->B == 32 ? 1 : 0));
+  const int sub_shift = !bf ? 0 : (c->B == 64 ? 2 : (c->B == 32 ? 1 : 0));
   // one wave: as many splits per problem as resident CTA slots allow, at least one tile (fp32 kernel: page) per warp
-  const int ntiles = (dense ? c->Pmax : c->k) << p.sub_shift;
+  const int ntiles = (dense ? c->Pmax : c->k) << sub_shift;
   int slots = c->num_sms * LOCKS_ATT_CTAS_PER_SM;
   if (slots > LOCKS_ATT_SLOT_BOUND) slots = LOCKS_ATT_SLOT_BOUND;
-  int splits = slots / (batch * p.Hkv);
+  int splits = slots / (batch * Hkv);
   const int most = (ntiles + LOCKS_ATT_WARPS - 1) / LOCKS_ATT_WARPS;
   if (splits > most) splits = most;
   if (splits > LOCKS_ATT_MAX_SPLITS) splits = LOCKS_ATT_MAX_SPLITS;
   if (splits < 1) splits = 1;
   // With clearly more problems than SMs every SM streams for several CTAs already: splitting a problem in
   // two only adds the merge (config 2, 256 problems: -1.5 to -2 us per step with one CTA per problem)
-  if (bf && !dense && 2 * batch * p.Hkv >= 3 * c->num_sms) splits = 1;
-  p.splits = splits;
-  p.done = c->att_done;
+  if (bf && !dense && 2 * batch * Hkv >= 3 * c->num_sms) splits = 1;
+  AttGeom g = {splits, 0, 0};
   // Preferred: the splits of a problem as one thread-block cluster (2, 4, 8 or 16 CTAs) that merges through
   // distributed shared memory, as long as a CTA then has at most 12 tiles per warp to stream (12 x 9K tokens, budget 128
   // pages, 96 problems: step 47.3 us as five splits that the last CTA merges, 43.8 as clusters of four; no case of 14 .. 64
   // requests slower), or 8 where the cluster leaves more than half of the CTAs that there is room for unused (dense, 1 x 8K
   // tokens: 13.2 us as clusters of 16, 12.4 as 72 splits; with 16 heads, whose splits cost more to merge, 20.5 and 21.4).
-  p.cluster = 0;
   if (c->att_clusters[0] < 0) {   // clusters of 2, 4, 8, 16 CTAs of this kernel that fit the device at once (probed once)
     cudaFuncSetAttribute(attend_bf16_kernel<1, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmem);
     cudaFuncSetAttribute(attend_bf16_kernel<1, true, false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -772,19 +763,46 @@ int locks_launch_attend(locks_ctx *c, const void *q, const locks_kv *kv, int bat
     // fewer large clusters fit than CTAs do: 32 problems as clusters of 16 (512 CTAs in 592 slots) take two waves, 36.7 us a
     // step (4 x 8K tokens, budget 128 pages) against 30.8 as clusters of 8; 24 problems fit, 29.2 against 30.0.
     int i = 3;
-    while (i >= 0 && ((2 << i) > splits || c->att_clusters[i] < batch * p.Hkv)) --i;
-    const int most_tiles = i >= 0 && ((4 << i) >= splits || p.G > 8) ? 12 : 8;
+    while (i >= 0 && ((2 << i) > splits || c->att_clusters[i] < batch * Hkv)) --i;
+    const int most_tiles = i >= 0 && ((4 << i) >= splits || G > 8) ? 12 : 8;
     if (i >= 0 && (ntiles + (2 << i) - 1) / (2 << i) <= most_tiles * LOCKS_ATT_WARPS) {
-      p.cluster = 1;
-      p.splits = 2 << i;
-      p.fused_merge = 1;   // no merge launch follows
+      g.cluster = 1;
+      g.splits = 2 << i;
+      g.fused_merge = 1;   // no merge launch follows
     }
   }
-  if (!p.cluster) {   // as many slices as the longest list has: 8 problems of 901 pages 24.2 us as 70 splits, 26.7 as 74
+  if (!g.cluster) {   // as many slices as the longest list has: 8 problems of 901 pages 24.2 us as 70 splits, 26.7 as 74
     const int per = (ntiles + splits - 1) / splits;
-    p.splits = (ntiles + per - 1) / per;
-    p.fused_merge = (p.G * p.splits <= kFusedMerge) ? 1 : 0;
+    g.splits = (ntiles + per - 1) / per;
+    g.fused_merge = (G * g.splits <= kFusedMerge) ? 1 : 0;
   }
+  return g;
+}
+
+}  // namespace
+
+bool locks_attend_fills(locks_ctx *c, int batch) {
+  const int Hkv = c->cfg.num_kv_heads;
+  return 8 * attend_geometry(c, batch, Hkv, c->G, false).splits * Hkv * batch > 7 * c->num_sms * LOCKS_ATT_CTAS_PER_SM;
+}
+
+int locks_launch_attend(locks_ctx *c, const void *q, const locks_kv *kv, int batch, const int32_t *ids,
+                        const int32_t *cnt, void *out, float *lse, cudaStream_t st) {
+  AttParams p;
+  p.q = q; p.k = kv->k; p.v = kv->v; p.sb = kv->stride_block; p.sh = kv->stride_head; p.st = kv->stride_token;
+  p.block_table = kv->block_table; p.seq_lens = kv->seq_lens; p.ids = ids; p.cnt = cnt;
+  p.part_o = c->att_o; p.part_lse = c->att_lse; p.out = out; p.lse = lse; p.status = c->status;
+  p.batch = batch; p.Hq = c->cfg.num_q_heads; p.Hkv = c->cfg.num_kv_heads; p.G = c->G; p.Pmax = c->Pmax;
+  p.kbud = c->k; p.num_blocks = kv->num_blocks; p.sm_scale = c->cfg.sm_scale; p.B = c->B; p.kvdiv = 1;
+  if (c->cfg.combine == LOCKS_COMBINE_PER_HEAD && ids) {   // one page table per query head: groups of one
+    p.kvdiv = p.G; p.Hkv = p.Hq; p.G = 1;
+  }
+  const bool bf = c->cfg.kv_dtype == LOCKS_BF16;   // tensor-core kernel
+  const bool wide = c->B != LOCKS_B;
+  p.sub_shift = !bf ? 0 : (c->B == 64 ? 2 : (c->B == 32 ? 1 : 0));
+  p.done = c->att_done;
+  const AttGeom geo = attend_geometry(c, batch, p.Hkv, p.G, ids == nullptr);
+  p.splits = geo.splits; p.cluster = geo.cluster; p.fused_merge = geo.fused_merge;
   p.per_split = (1ull << 32) / p.splits + 1;
   if (bf) {
     const bool contig = kv->stride_token == LOCKS_D;

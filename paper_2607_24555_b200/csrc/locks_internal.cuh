@@ -144,8 +144,11 @@ __device__ __forceinline__ void locks_update_partition_hint(int32_t *hint, const
 // seq_inc = 1: lengths are taken one token longer than kv->seq_lens says and published in ctx->seq_eff
 int locks_launch_scan(locks_ctx *c, const void *q, const void *summaries, const locks_kv *kv, int batch,
                       float *shat, int seq_inc, cudaStream_t st);
+// attend_first: the kernel that follows may take its slots at once (see select_kernel)
 int locks_launch_select(locks_ctx *c, const float *shat, const locks_kv *kv, int batch, int32_t *ids,
-                        int32_t *cnt, float *logshare, const locks_append *app, cudaStream_t st);
+                        int32_t *cnt, float *logshare, const locks_append *app, cudaStream_t st, bool attend_first = false);
+// Whether a step's attention needs almost every slot there is
+bool locks_attend_fills(locks_ctx *c, int batch);
 int locks_launch_attend(locks_ctx *c, const void *q, const locks_kv *kv, int batch, const int32_t *ids,
                         const int32_t *cnt, void *out, float *lse, cudaStream_t st);
 int locks_launch_build(locks_ctx *c, const locks_kv *kv, int batch, const int32_t *pb, const int32_t *pe,

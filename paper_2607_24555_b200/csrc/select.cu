@@ -38,6 +38,7 @@ struct SelParams {
   int32_t *status;
   int batch, Hq, Hkv, G, Pmax, max_groups, k, chunks, kc, chunk_pages, part_slots;
   int combine;       // LOCKS_COMBINE_*
+  int attend_first;  // let the next kernel be scheduled at once
   int Bshift;        // log2 of the page size (4, 5 or 6)
   locks_append app;  // decode step only: the new token's K/V rows, written here beside the ranking
 };
@@ -84,7 +85,6 @@ struct SelShared {
   __align__(16) uint32_t list[kListMax];
   int nlist;
   int misc[16];                       // arrival flag
-  float lz2[16];                      // log2-domain log Z_g
   float lzm[kNW], lzs[kNW];           // per-warp (max, sum) of the log Z reduction
   uint32_t red[2 * kNW];              // per-warp smallest and largest valid key
 };
@@ -296,35 +296,79 @@ __device__ __noinline__ void select_emit(int nslab, int K, int mode, int c0, int
   }
 }
 
-// log Z_g of every head of the group from the scan's partials (max_i, sum_i), part0 = head 0's row,
-// -> sh.lz2[g] (log2 domain):
-// log2 Z = M + log2 sum_i sum_i 2^(max_i - M), M = max_i max_i.  The block's warps are dealt to (head, slice)
-// pairs; a lane keeps eight loads in flight.  Ends with the block synchronised.
-__device__ __noinline__ void group_logz(const float2 *part0, int G, int max_groups, int nparts) {
+// What a launch's rankings have in common before the length is known: a CTA's scores and partials sit at addresses that do not
+// depend on it, so one round trip fetches them together with it.
+struct KeyInputs {
+  const float *shat0;      // scores of the group's head 0, page 0
+  const float2 *part0;     // partials of head 0
+  const int32_t *seq_len, *part_cnt;   // part_cnt: this problem's, or nullptr
+  int G, Pmax, max_groups, part_slots, c0, chunk_pages, Bshift, combine;
+};
+
+// Keys of a chunk: log m_bar of page c0 + i*512 + t as an order-preserving integer in sh.key[i*512 + t] (0 for pages that are not
+// candidates), and their range in sh.red.  A thread takes the scores of all HB >= G heads of SB = 16 / HB slabs at once, 16 loads in
+// flight, the next batch while the current one is reduced.  log Z_g comes from the scan's partials (max_i, sum_i):
+// log2 Z = M + log2 sum_i sum_i 2^(max_i - M), M = max_i max_i; the block's warps are dealt to (head, slice) pairs.
+// combine: share-average (the paper's rule) subtracts log Z_g per head and averages; group-mass sums the raw masses (log Z_g = 0,
+// no 1/G); group-max keeps the largest raw score.
+// `begin(T, P)` is called once the length is there; false: nothing to rank (returns 0 slabs).
+// Bound by a chain of round trips: the length, the first batch of scores and the first partials travel together (before, the length
+// alone came first, then 2000 cycles of address arithmetic with a 64-bit division, then the rest).
+template <int HB, typename Begin>
+__device__ __forceinline__ int chunk_keys(const KeyInputs &in, Begin begin, float *logshare_row) {
+  constexpr int SB = 16 / HB, NP = HB == 16 ? 8 : 4;   // NP: partials in flight per lane
   SelShared &sh = shared_state();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int gw = min(G, kNW);            // heads handled per round
-  const int nslice = max(1, kNW / G);    // warps per head
-#pragma unroll 1
-  for (int g0 = 0; g0 < G; g0 += kNW) {  // one round unless G > 16
-    const int slice = warp / gw, g = g0 + warp - slice * gw;
-    float m = -INFINITY, s = 0.f;
-    if (g < G && slice < nslice) {
-      const float2 *pp = part0 + (int64_t)g * max_groups;
-#pragma unroll 1
-      for (int i0 = slice * 32 + lane; i0 < nparts; i0 += 256 * nslice) {
-        float2 v[8];   // eight loads in flight: up to 256 partials of a head in one round trip
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, G = in.G;
+  const float *row0 = in.shat0 + in.c0 + tid;
+  float cur[HB][SB], nxt[HB][SB];
+  auto load = [&](int i0, int last, float (&x)[HB][SB]) {   // pages 1 .. last
+    const float *r = row0 + i0 * LOCKS_SEL_THREADS;   // offsets within one request fit 32 bits
 #pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = (i0 + 32 * nslice * u < nparts) ? pp[i0 + 32 * nslice * u] : make_float2(-INFINITY, 0.f);
+    for (int sl = 0; sl < SB; ++sl) {
+      const int page = in.c0 + (i0 + sl) * LOCKS_SEL_THREADS + tid;
+      const bool ok = page >= 1 && page <= last && (i0 + sl) * LOCKS_SEL_THREADS < in.chunk_pages;
+#pragma unroll
+      for (int u = 0; u < HB; ++u) x[u][sl] = (ok && u < G) ? r[u * in.Pmax + sl * LOCKS_SEL_THREADS] : -INFINITY;
+    }
+  };
+  const int T = *in.seq_len;
+  const int counted = in.part_cnt ? *in.part_cnt : in.part_slots;
+  load(0, in.Pmax - 1, cur);
+  const int nslice = max(1, kNW / G), slice = warp / min(G, kNW), g = warp - slice * min(G, kNW);   // (G <= 16)
+  const bool has_head = slice < nslice && in.combine == LOCKS_COMBINE_SHARE_AVG;
+  const float2 *pp = in.part0 + (int64_t)g * in.max_groups;
+  const int pstep = 32 * nslice, p0 = slice * 32 + lane;
+  const int most = in.part_cnt ? in.max_groups : in.part_slots;   // what may be read before the count is known
+  float2 v[NP];
+#pragma unroll
+  for (int u = 0; u < NP; ++u) v[u] = (has_head && p0 + pstep * u < most) ? pp[p0 + pstep * u] : make_float2(-INFINITY, 0.f);
+  // ---- the length is there
+  const int P = (T + (1 << in.Bshift) - 1) >> in.Bshift;
+  if (!begin(T, P)) return 0;
+  // slabs of 512 pages that hold at least one candidate of this chunk (the configured maximum context is usually longer)
+  const int nslab = (min(P - 1, in.c0 + in.chunk_pages) - in.c0 + LOCKS_SEL_THREADS - 1) / LOCKS_SEL_THREADS;
+  const int nparts = in.part_cnt ? min(max(counted, 0), in.max_groups) : min(counted, (P - 1 + LOCKS_GROUP - 1) / LOCKS_GROUP);
+  if (in.combine == LOCKS_COMBINE_SHARE_AVG) {
+    float m = -INFINITY, s = 0.f;
+    if (has_head) {
+#pragma unroll 1
+      for (int i0 = p0;;) {
         float nm = m;
 #pragma unroll
-        for (int u = 0; u < 8; ++u) nm = fmaxf(nm, v[u].x);
+        for (int u = 0; u < NP; ++u) {
+          if (i0 + pstep * u >= nparts) v[u] = make_float2(-INFINITY, 0.f);
+          nm = fmaxf(nm, v[u].x);
+        }
         if (nm > -INFINITY) {
           s *= ex2f((m - nm) * kLog2e);
 #pragma unroll
-          for (int u = 0; u < 8; ++u) s = fmaf(v[u].y, ex2f((v[u].x - nm) * kLog2e), s);
+          for (int u = 0; u < NP; ++u) s = fmaf(v[u].y, ex2f((v[u].x - nm) * kLog2e), s);
           m = nm;
         }
+        i0 += NP * pstep;
+        if (i0 - lane >= nparts) break;   // (the whole warp leaves together)
+#pragma unroll
+        for (int u = 0; u < NP; ++u) v[u] = i0 + pstep * u < nparts ? pp[i0 + pstep * u] : make_float2(-INFINITY, 0.f);
       }
       const uint32_t top = __reduce_max_sync(0xffffffffu, order_key(m));
       const float M = __uint_as_float((top & 0x80000000u) ? top & 0x7FFFFFFFu : ~top);
@@ -334,111 +378,62 @@ __device__ __noinline__ void group_logz(const float2 *part0, int G, int max_grou
       m = M;
     }
     if (lane == 0) { sh.lzm[warp] = m; sh.lzs[warp] = s; }
-    __syncthreads();
-    if (threadIdx.x < min(G - g0, kNW)) {
+  }
+  __syncthreads();
+  // every warp for itself: lane g < G merges the slices of head g
+  float lz[HB];
+  {
+    float l2 = 0.f;
+    if (in.combine == LOCKS_COMBINE_SHARE_AVG && lane < G) {
       float M = -INFINITY, S = 0.f;
 #pragma unroll 1
-      for (int sl = 0; sl < nslice; ++sl) M = fmaxf(M, sh.lzm[sl * gw + threadIdx.x]);
+      for (int sl = 0; sl < nslice; ++sl) M = fmaxf(M, sh.lzm[sl * G + lane]);
 #pragma unroll 1
       for (int sl = 0; sl < nslice; ++sl) {
-        const float wm = sh.lzm[sl * gw + threadIdx.x];
-        if (wm > -INFINITY) S = fmaf(sh.lzs[sl * gw + threadIdx.x], ex2f((wm - M) * kLog2e), S);
+        const float wm = sh.lzm[sl * G + lane];
+        if (wm > -INFINITY) S = fmaf(sh.lzs[sl * G + lane], ex2f((wm - M) * kLog2e), S);
       }
-      sh.lz2[g0 + threadIdx.x] = M * kLog2e + lg2f(S);
+      l2 = M * kLog2e + lg2f(S);
     }
-    __syncthreads();
+    __syncwarp();
+#pragma unroll
+    for (int u = 0; u < HB; ++u) lz[u] = __shfl_sync(0xffffffffu, l2, u);
   }
-}
-
-// Keys of a chunk: log m_bar of page c0 + i*512 + t as an order-preserving integer in sh.key[i*512 + t]
-// (0 for pages that are not candidates).  Scores are fetched in batches of (16 / SB) heads x SB slabs, 16
-// loads in flight per thread, the next batch while the current one is reduced; the first batch is in
-// flight during the log Z reduction.  Per page a running (max, sum) over the heads, log2 domain.
-// combine: share-average (the paper's rule) subtracts log Z_g per head and averages; group-mass sums the raw
-// masses (log Z_g = 0, no 1/G); group-max keeps the largest raw score.
-template <int SB>
-__device__ __noinline__ void chunk_keys(const float *shat0, const float2 *part0, float *logshare0, int G, int Pmax,
-                                        int max_groups, int nparts, int c0, int nslab, int P, int combine) {
-  constexpr int HB = 16 / SB;
-  SelShared &sh = shared_state();
-  const int tid = threadIdx.x;
-  const float *row0 = shat0 + c0 + tid;   // shat0: scores of the group's head 0, page 0
-  const int nG = (G + HB - 1) / HB, nb = ((nslab + SB - 1) / SB) * nG;
-  float cur[HB][SB], nxt[HB][SB];
-  auto load = [&](int i0, int g0, float (&x)[HB][SB]) {
-    bool ok[SB];
-#pragma unroll
-    for (int sl = 0; sl < SB; ++sl) {
-      const int page = c0 + (i0 + sl) * LOCKS_SEL_THREADS + tid;
-      ok[sl] = i0 + sl < nslab && page >= 1 && page <= P - 2;
-    }
-    const float *r = row0 + g0 * Pmax + i0 * LOCKS_SEL_THREADS;   // offsets within one request fit 32 bits
-#pragma unroll
-    for (int u = 0; u < HB; ++u)
-#pragma unroll
-      for (int sl = 0; sl < SB; ++sl)
-        x[u][sl] = (ok[sl] && g0 + u < G) ? r[u * Pmax + sl * LOCKS_SEL_THREADS] : -INFINITY;
-  };
-  load(0, 0, cur);
-  if (combine == LOCKS_COMBINE_SHARE_AVG) {
-    group_logz(part0, G, max_groups, nparts);
-  } else {
-    if (tid < 16) sh.lz2[tid] = 0.f;
-    __syncthreads();
-  }
-  const float logG = combine == LOCKS_COMBINE_SHARE_AVG ? __logf((float)G) : 0.f;
+  const float logG = in.combine == LOCKS_COMBINE_SHARE_AVG ? __logf((float)G) : 0.f;
   uint32_t kmin = 0xFFFFFFFFu, kmax = 0u;
-  float m[SB], s[SB];
-#pragma unroll
-  for (int sl = 0; sl < SB; ++sl) { m[sl] = -INFINITY; s[sl] = 0.f; }
-  int i0 = 0, g0 = 0;
 #pragma unroll 1
-  for (int bi = 0; bi < nb; ++bi) {
-    int i1 = i0, g1 = g0 + HB;   // the batch after this one
-    if (g1 >= G) { g1 = 0; i1 += SB; }
-    if (bi + 1 < nb) load(i1, g1, nxt);
+  for (int i0 = 0; i0 < nslab; i0 += SB) {
+    if (i0 + SB < nslab) load(i0 + SB, P - 2, nxt);
 #pragma unroll
     for (int sl = 0; sl < SB; ++sl) {
-      float bm = -INFINITY;
+      const int i = i0 + sl, page = in.c0 + i * LOCKS_SEL_THREADS + tid;
+      if (i >= nslab) break;
+      float m = -INFINITY;
 #pragma unroll
       for (int u = 0; u < HB; ++u) {
-        cur[u][sl] = fmaf(cur[u][sl], kLog2e, g0 + u < G ? -sh.lz2[g0 + u] : 0.f);   // heads past the group stay -inf
-        bm = fmaxf(bm, cur[u][sl]);
+        cur[u][sl] = fmaf(cur[u][sl], kLog2e, -lz[u]);   // heads past the group stay -inf
+        m = fmaxf(m, cur[u][sl]);
       }
-      const float nm = fmaxf(m[sl], bm);
-      float acc = s[sl] * ex2f(m[sl] - nm);
+      float acc = 0.f;
 #pragma unroll
-      for (int u = 0; u < HB; ++u) acc += ex2f(cur[u][sl] - nm);
-      s[sl] = acc;
-      m[sl] = nm;
-    }
-    if (g0 + HB >= G) {   // all heads seen: keys of these slabs
-#pragma unroll
-      for (int sl = 0; sl < SB; ++sl) {
-        const int i = i0 + sl, page = c0 + i * LOCKS_SEL_THREADS + tid;
-        if (i < nslab) {
-          const bool valid = page >= 1 && page <= P - 2;
-          const float val = (combine == LOCKS_COMBINE_GROUP_MAX ? m[sl] : m[sl] + lg2f(s[sl])) * kLn2 - logG;
-          const uint32_t key = order_key(val);
-          sh.key[i * LOCKS_SEL_THREADS + tid] = valid ? key : 0u;
-          if (valid) {
-            kmin = min(kmin, key);
-            kmax = max(kmax, key);
-            if (logshare0) logshare0[page] = val;
-          }
-        }
-        m[sl] = -INFINITY;
-        s[sl] = 0.f;
+      for (int u = 0; u < HB; ++u) acc += ex2f(cur[u][sl] - m);
+      const bool valid = page >= 1 && page <= P - 2;
+      const float val = (in.combine == LOCKS_COMBINE_GROUP_MAX ? m : m + lg2f(acc)) * kLn2 - logG;
+      const uint32_t key = order_key(val);
+      sh.key[i * LOCKS_SEL_THREADS + tid] = valid ? key : 0u;
+      if (valid) {
+        kmin = min(kmin, key);
+        kmax = max(kmax, key);
+        if (logshare_row) logshare_row[page] = val;
       }
     }
 #pragma unroll
     for (int u = 0; u < HB; ++u)
 #pragma unroll
       for (int sl = 0; sl < SB; ++sl) cur[u][sl] = nxt[u][sl];
-    i0 = i1;
-    g0 = g1;
   }
   publish_range(sh, kmin, kmax);
+  return nslab;
 }
 
 // Several chunks per problem: the chunk that arrives last ranks the problem's candidate lists.
@@ -492,45 +487,46 @@ __device__ __noinline__ void select_finish(int32_t *done, int chunks, int kc, in
   }
 }
 
+template <int HB>
 __global__ void __launch_bounds__(LOCKS_SEL_THREADS, 2) select_kernel(SelParams p) {
-  SelShared &sh = shared_state();
   const int chunk = blockIdx.x, h = blockIdx.y, b = blockIdx.z, tid = threadIdx.x;
-  pdl_trigger();
+  const int prob = b * p.Hkv + h, c0 = chunk * p.chunk_pages;   // first page of this chunk
+  int32_t *ids = p.ids + (int64_t)prob * p.k;
+  const int64_t list0 = (int64_t)prob * p.chunks * p.kc;
+  KeyInputs in;
+  in.shat0 = p.shat + ((int64_t)b * p.Hq + h * p.G) * p.Pmax;
+  in.part0 = p.part + ((int64_t)b * p.Hq + h * p.G) * p.max_groups;
+  in.seq_len = p.seq_lens + b;
+  in.part_cnt = p.part_cnt ? p.part_cnt + (p.pc_div == 1 ? prob : prob / p.pc_div) : nullptr;
+  in.G = p.G; in.Pmax = p.Pmax; in.max_groups = p.max_groups; in.part_slots = p.part_slots; in.c0 = c0;
+  in.chunk_pages = p.chunk_pages; in.Bshift = p.Bshift; in.combine = p.combine;
+  if (p.attend_first) pdl_trigger();
   pdl_wait();   // the scan's scores and partials
-  const int T = p.seq_lens[b];
-  if (p.app.k_new && chunk == 0 && tid >= LOCKS_SEL_THREADS - 32)
-    append_token(p.app, p.batch, p.Hkv, p.Pmax, b, h, tid & 31, T, p.status, p.Bshift);
-  const int P = (T + (1 << p.Bshift) - 1) >> p.Bshift;
-  const int64_t prob = (int64_t)b * p.Hkv + h;
-  int32_t *ids = p.ids + prob * p.k;
-  if (P <= p.k) {  // every page is kept
-    if (chunk == 0) {
-      for (int j = tid; j < p.k; j += LOCKS_SEL_THREADS) ids[j] = j < P ? j : -1;
-      if (tid == 0) p.cnt[prob] = P;
+  int P = 0;
+  const int nslab = chunk_keys<HB>(in, [&](int T, int np) {
+    P = np;
+    if (p.app.k_new && chunk == 0 && tid >= LOCKS_SEL_THREADS - 32)
+      append_token(p.app, p.batch, p.Hkv, p.Pmax, b, h, tid & 31, T, p.status, p.Bshift);
+    if (P <= p.k) {  // every page is kept
+      if (chunk == 0) {
+        for (int j = tid; j < p.k; j += LOCKS_SEL_THREADS) ids[j] = j < P ? j : -1;
+        if (tid == 0) p.cnt[prob] = P;
+      }
+      return false;
     }
-    return;
-  }
-  const int c0 = chunk * p.chunk_pages;  // first page of this chunk
-  if (c0 > P - 2) {  // chunk past the candidates: an empty list
+    return c0 <= P - 2;
+  }, p.logshare ? p.logshare + (int64_t)prob * p.Pmax : nullptr);
+  // Attention's CTAs are called when the keys are there, not at once: waiting, they would hold the slots in which the step's build
+  // starts when the scan ends (32 x 16K tokens, budget 16 pages: 59.4 -> 53.3 us a step, 8 x 24K 59.2 -> 52.9).  Where attention
+  // itself needs more than 7/8 of the slots it comes first (17 x 8K tokens, 544 of 592: 55.7 us; the build first 61.6).
+  pdl_trigger();
+  if (P <= p.k) return;
+  if (nslab == 0) {  // chunk past the candidates: an empty list
     if (p.chunks > 1) {
-      for (int j = tid; j < p.kc; j += LOCKS_SEL_THREADS) p.cand_key[(prob * p.chunks + chunk) * p.kc + j] = 0u;
-      select_finish(p.sel_done + prob, p.chunks, p.kc, p.k, ids, p.cnt + prob, p.cand_key + prob * p.chunks * p.kc,
-                    p.cand_idx + prob * p.chunks * p.kc, P);
+      for (int j = tid; j < p.kc; j += LOCKS_SEL_THREADS) p.cand_key[list0 + (int64_t)chunk * p.kc + j] = 0u;
+      select_finish(p.sel_done + prob, p.chunks, p.kc, p.k, ids, p.cnt + prob, p.cand_key + list0, p.cand_idx + list0, P);
     }
     return;
-  }
-  // slabs of 512 pages that hold at least one candidate of this chunk (the configured maximum context
-  // is usually longer than the sequence)
-  const int nslab = (min(P - 1, c0 + p.chunk_pages) - c0 + LOCKS_SEL_THREADS - 1) / LOCKS_SEL_THREADS;
-  {
-    const float *shat0 = p.shat + ((int64_t)b * p.Hq + h * p.G) * p.Pmax;
-    const float2 *part0 = p.part + ((int64_t)b * p.Hq + h * p.G) * p.max_groups;
-    float *ls0 = p.logshare ? p.logshare + prob * p.Pmax : nullptr;
-    const int nparts = p.part_cnt ? min(max(p.part_cnt[prob / p.pc_div], 0), p.max_groups)
-                                  : min(p.part_slots, (P - 1 + LOCKS_GROUP - 1) / LOCKS_GROUP);
-    if (nslab >= 3) chunk_keys<4>(shat0, part0, ls0, p.G, p.Pmax, p.max_groups, nparts, c0, nslab, P, p.combine);
-    else if (nslab == 2) chunk_keys<2>(shat0, part0, ls0, p.G, p.Pmax, p.max_groups, nparts, c0, nslab, P, p.combine);
-    else chunk_keys<1>(shat0, part0, ls0, p.G, p.Pmax, p.max_groups, nparts, c0, nslab, P, p.combine);
   }
   const int cand_in_chunk = min(P - 2, c0 + p.chunk_pages - 1) - max(1, c0) + 1;
   const int K = min(p.k - 2, cand_in_chunk);
@@ -542,11 +538,10 @@ __global__ void __launch_bounds__(LOCKS_SEL_THREADS, 2) select_kernel(SelParams 
       p.cnt[prob] = p.k;
     }
   } else {
-    uint32_t *lk = p.cand_key + (prob * p.chunks + chunk) * p.kc;
+    uint32_t *lk = p.cand_key + list0 + (int64_t)chunk * p.kc;
     for (int j = K + tid; j < p.kc; j += LOCKS_SEL_THREADS) lk[j] = 0u;   // fewer candidates than list slots
-    if (K > 0) select_emit(nslab, K, kEmitList, c0, nullptr, lk, p.cand_idx + (prob * p.chunks + chunk) * p.kc);
-    select_finish(p.sel_done + prob, p.chunks, p.kc, p.k, ids, p.cnt + prob, p.cand_key + prob * p.chunks * p.kc,
-                  p.cand_idx + prob * p.chunks * p.kc, P);
+    if (K > 0) select_emit(nslab, K, kEmitList, c0, nullptr, lk, p.cand_idx + list0 + (int64_t)chunk * p.kc);
+    select_finish(p.sel_done + prob, p.chunks, p.kc, p.k, ids, p.cnt + prob, p.cand_key + list0, p.cand_idx + list0, P);
   }
 }
 
@@ -661,16 +656,15 @@ int locks_launch_ext_partials(locks_ctx *c, const float *logz_parts, int nparts,
 int locks_launch_merge_selection(locks_ctx *c, const float *cand_key, const int32_t *cand_page, int nparts, int batch,
                                  int32_t *ids, int32_t *cnt, cudaStream_t st) {
   if (nparts < 1 || (int64_t)nparts * c->sel_kc > kMaxKeys) return LOCKS_ERR_UNSUPPORTED;
-  if (locks_attrs_needed(LOCKS_ATTR_SELECT))
-    cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 116 * 1024);
   merge_selection_kernel<<<dim3(c->cfg.num_kv_heads, batch), LOCKS_SEL_THREADS, sizeof(SelShared), st>>>(
       cand_key, cand_page, nparts, batch, c->cfg.num_kv_heads, c->sel_kc, ids, cnt);
   return locks_check_launch(c);
 }
 
 int locks_launch_select(locks_ctx *c, const float *shat, const locks_kv *kv, int batch, int32_t *ids,
-                        int32_t *cnt, float *logshare, const locks_append *app, cudaStream_t st) {
+                        int32_t *cnt, float *logshare, const locks_append *app, cudaStream_t st, bool attend_first) {
   SelParams p;
+  p.attend_first = attend_first;
   if (app) p.app = *app;
   else p.app.k_new = nullptr;
   p.status = c->status;
@@ -694,10 +688,16 @@ int locks_launch_select(locks_ctx *c, const float *shat, const locks_kv *kv, int
   // while others idle (measured: +15 us at 192 CTAs); such launches ask for enough shared memory to keep one
   // CTA per SM.
   constexpr int kSmemAlone = 116 * 1024;
-  if (locks_attrs_needed(LOCKS_ATTR_SELECT))
-    cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemAlone);
   const int64_t nctas = (int64_t)c->sel_chunks * p.Hkv * batch;
   const size_t smem = 2 * nctas <= 3 * (int64_t)c->num_sms ? (size_t)kSmemAlone : sizeof(SelShared);
-  locks_launch_pdl(select_kernel, dim3(c->sel_chunks, p.Hkv, batch), dim3(LOCKS_SEL_THREADS), smem, st, p);
+  const dim3 grid(c->sel_chunks, p.Hkv, batch), blk(LOCKS_SEL_THREADS);
+  if (locks_attrs_needed(LOCKS_ATTR_SELECT)) {
+    cudaFuncSetAttribute(select_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemAlone);
+    cudaFuncSetAttribute(select_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemAlone);
+    cudaFuncSetAttribute(select_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemAlone);
+  }
+  if (p.G <= 4) locks_launch_pdl(select_kernel<4>, grid, blk, smem, st, p);
+  else if (p.G <= 8) locks_launch_pdl(select_kernel<8>, grid, blk, smem, st, p);
+  else locks_launch_pdl(select_kernel<16>, grid, blk, smem, st, p);
   return locks_check_launch(c);
 }
