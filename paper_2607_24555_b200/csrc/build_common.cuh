@@ -20,6 +20,10 @@ struct BuildParams {
   // (the append runs in another kernel at the same time); append_pos[b] = its position or -1
   const void *k_new;
   const int32_t *append_pos;
+  // decode step whose build starts beside the scan, before any length is published: the token is counted here (seq_inc = 1),
+  // and the caller's length is stored by whoever comes last of the request's page-heads, which have read it by then, and the
+  // selector (arrivals[b] counts them; zero between steps).  seq_commit == nullptr: seq_lens are the step's.
+  int32_t *seq_commit, *arrivals;
   // bulk build of several layers in one launch: per-layer key caches and summary buffers (device arrays), or null
   const void *const *k_layers;
   void *const *summ_layers;

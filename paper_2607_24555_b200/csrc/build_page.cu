@@ -196,10 +196,21 @@ __global__ void __launch_bounds__(page_threads(B) * page_ctas(B)) build_page_ker
     locks_update_partition_hint(p.hint, p.seq_lens, p.batch, p.Hkv, p.kpages, p.hint_wpp, p.hint_rounds, p.hint_W, lane);
   const int prob = blockIdx.x * PPC + sub;
   if (prob >= p.batch * p.Hkv) return;
-  const int b = prob / p.Hkv, h = prob - b * p.Hkv, Tb = p.seq_lens[b];
+  const int b = prob / p.Hkv, h = prob - b * p.Hkv;
+  int Tb = p.seq_lens[b], at_new = p.append_pos ? p.append_pos[b] : -1;
+  if (p.seq_commit) {
+    sync();   // every thread of the page has read the length
+    const bool room = Tb < p.Pmax * B;   // a sequence that has no room for the token keeps its length
+    at_new = room ? Tb : -1;
+    Tb += room;
+    if (tid == 0) {
+      __threadfence();
+      if (atomicAdd(p.arrivals + b, 1) == p.Hkv) { p.arrivals[b] = 0; p.seq_commit[b] = Tb; }
+    }
+  }
   if (Tb <= 0 || (Tb & (B - 1)) != 0) return;
   const int page = Tb / B - 1;
-  const bool last_from_new = p.k_new && p.append_pos && p.append_pos[b] == Tb - 1;   // the last row is this step's token
+  const bool last_from_new = p.k_new && at_new == Tb - 1;   // the last row is this step's token
   if (page >= p.Pmax) return;
   const int block = p.block_table[(int64_t)b * p.Pmax + page];
   if (block < 0 || block >= p.num_blocks) {

@@ -85,6 +85,7 @@ struct locks_ctx {
   int32_t *cnt_int;        // [max_batch][Hkv]
   char *stage_q, *stage_kn, *stage_vn, *stage_out;
   int32_t *seq_eff;        // [2][max_batch] decode step in flight: effective lengths, append positions
+  int32_t *arrivals;       // [max_batch] readers of a request's length that are done (zero between steps; see BuildParams)
   cudaStream_t side;       // build of freshly filled pages runs beside attend
   cudaEvent_t ev_fork, ev_join;
   int last_launches;
@@ -105,6 +106,7 @@ struct locks_append {
   const int32_t *block_table;
   const int32_t *seq_eff;      // published by the scan: [batch] lengths, [batch] append positions
   int32_t *seq_commit;         // the caller's sequence lengths
+  int32_t *arrivals;           // [batch] when the step's build may still read them (see BuildParams), or nullptr
   int num_blocks, esz;
 };
 
@@ -115,6 +117,8 @@ struct locks_scan_geom {
   int cta_reduce;            // all warps of a CTA share one problem for the whole launch
 };
 locks_scan_geom locks_scan_geometry(const locks_ctx *c, int batch);
+// Whether the CTAs of a step's build fit beside this step's scan
+bool locks_scan_leaves_room(const locks_ctx *c, int batch);
 
 // Which partition suits these lengths: iterations of the longest warp, strided = rounds * ceil(max groups / wpp)
 // against balanced = ceil(units / warps); the balanced one has to win by more than its set-up costs.
@@ -153,8 +157,8 @@ int locks_launch_attend(locks_ctx *c, const void *q, const locks_kv *kv, int bat
                         const int32_t *cnt, void *out, float *lse, cudaStream_t st);
 int locks_launch_build(locks_ctx *c, const locks_kv *kv, int batch, const int32_t *pb, const int32_t *pe,
                        int just_filled, void *summaries, const void *k_new, const int32_t *append_pos,
-                       cudaStream_t st, const void *const *k_layers = nullptr, void *const *summ_layers = nullptr,
-                       int num_layers = 1);
+                       cudaStream_t st, int32_t *seq_commit = nullptr, const void *const *k_layers = nullptr,
+                       void *const *summ_layers = nullptr, int num_layers = 1);
 
 // envelope = 0: exact page log-mass; 1: the min/max envelope bound of the page's largest logit
 int locks_launch_exact_scan(locks_ctx *c, const void *q, const locks_kv *kv, int batch, float *shat, int envelope,
@@ -226,7 +230,7 @@ static inline int locks_check_launch(locks_ctx *c) {
 // process: true exactly once per (current device, kernel family), so that a process that drives several GPUs
 // sets them on each.  Thread-safe.
 enum { LOCKS_ATTR_SELECT = 0, LOCKS_ATTR_ATTEND = 1, LOCKS_ATTR_EXACT = 3, LOCKS_ATTR_SCAN = 8,
-       LOCKS_ATTR_BUILD_PAGE = 20 /* + page size / 32 */, LOCKS_ATTR_BUILD_WIDE = 24 /* + format */ };
+       LOCKS_ATTR_BUILD_PAGE = 20 /* + page size / 32 */, LOCKS_ATTR_BUILD_WIDE = 24 /* + format */, LOCKS_ATTR_SCAN_WIDE = 28 /* + rank / 4 */ };
 bool locks_attrs_needed(int family);
 
 // ---------------------------------------------------------------- I4 blob geometry (d = 128; B = 16 unless given)

@@ -1337,6 +1337,12 @@ locks_scan_geom locks_scan_geometry(const locks_ctx *c, int batch) {
   return g;
 }
 
+// Only the tensor scan fills every SM for as long as it lasts; of two slots on an SM a build CTA (four page-heads) takes one.
+bool locks_scan_leaves_room(const locks_ctx *c, int batch) {
+  if (!(c->cfg.summary_fmt == LOCKS_FMT_I4 && c->cfg.q_dtype == LOCKS_BF16 && c->B == LOCKS_B)) return true;
+  return locks_scan_geometry(c, batch).grid + (batch * c->cfg.num_kv_heads + 3) / 4 <= kScanCtasPerSm * c->num_sms;
+}
+
 int locks_launch_scan(locks_ctx *c, const void *q, const void *summaries, const locks_kv *kv, int batch,
                       float *shat, int seq_inc, cudaStream_t st) {
   ScanParams p;
@@ -1433,8 +1439,16 @@ int locks_launch_scan(locks_ctx *c, const void *q, const void *summaries, const 
     // 32- and 64-token pages: about four CTAs of four warps per SM, each warp striding a problem's groups
     const int most = (c->max_groups + kWideWarps - 1) / kWideWarps, want = (4 * c->num_sms + batch * p.Hkv - 1) / (batch * p.Hkv);
     const dim3 grid(most < want ? most : want, p.Hkv, batch), blk(kWideWarps * 32);
+    // The kernel itself uses no shared memory.  With the runtime's choice of the split between L1 and shared memory the step's
+    // build (61 KB a CTA), launched beside it, finds no SM until the scan drains (4 x 16K tokens, 32-token pages, a page filled:
+    // 73 us a step, 55 with the split all on shared memory; no page filled 32.8 either way).
+#define LOCKS_WIDE_SPLIT(R_, NT_, NH_) cudaFuncSetAttribute(scan_wide_kernel<R_, NT_, NH_>, cudaFuncAttributePreferredSharedMemoryCarveout, 100)
 #define LOCKS_WIDE_LAUNCH(R_)                                                                                \
   do {                                                                                                      \
+    if (locks_attrs_needed(LOCKS_ATTR_SCAN_WIDE + R_ / 4)) {                                                \
+      LOCKS_WIDE_SPLIT(R_, 4, 1); LOCKS_WIDE_SPLIT(R_, 4, 2);                                               \
+      LOCKS_WIDE_SPLIT(R_, 8, 1); LOCKS_WIDE_SPLIT(R_, 8, 2);                                               \
+    }                                                                                                       \
     if (c->B == 32 && c->G <= 8) locks_launch_pdl(scan_wide_kernel<R_, 4, 1>, grid, blk, 0, st, p);         \
     else if (c->B == 32) locks_launch_pdl(scan_wide_kernel<R_, 4, 2>, grid, blk, 0, st, p);                 \
     else if (c->G <= 8) locks_launch_pdl(scan_wide_kernel<R_, 8, 1>, grid, blk, 0, st, p);                  \
@@ -1444,6 +1458,7 @@ int locks_launch_scan(locks_ctx *c, const void *q, const void *summaries, const 
     else if (p.r == 4) LOCKS_WIDE_LAUNCH(4);
     else LOCKS_WIDE_LAUNCH(2);
 #undef LOCKS_WIDE_LAUNCH
+#undef LOCKS_WIDE_SPLIT
   } else {
     dim3 grid((c->max_groups + 3) / 4, p.Hkv, batch);
     const bool qbf = c->cfg.q_dtype == LOCKS_BF16;

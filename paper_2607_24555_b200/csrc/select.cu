@@ -46,11 +46,16 @@ struct SelParams {
 // Decode step: the CTA of (request b, KV head h) writes the new token's K and V rows of that head into the
 // cache (one warp, a few independent loads and stores beside the ranking's own loads), and the CTA of
 // head 0 stores the step's length back to the caller's array.  Nothing reads the caller's array between
-// the scan (complete before this kernel passes its wait) and the end of the step: the step's other
-// kernels take lengths from the published copy.
+// the scan (complete before this kernel passes its wait) and the end of the step, except a build that started
+// beside the scan (a.arrivals): the step's other kernels take lengths from the published copy.
 __device__ __forceinline__ void append_token(const locks_append &a, int batch, int Hkv, int Pmax, int b, int h,
                                              int lane, int T, int32_t *status, int Bshift) {
-  if (h == 0 && lane == 0) a.seq_commit[b] = T;
+  if (h == 0 && lane == 0) {
+    if (!a.arrivals || atomicAdd(a.arrivals + b, 1) == Hkv) {   // the last to arrive stores (BuildParams::seq_commit)
+      if (a.arrivals) a.arrivals[b] = 0;
+      a.seq_commit[b] = T;
+    }
+  }
   const int at = a.seq_eff[batch + b];
   if (at < 0) return;
   const int page = at >> Bshift, slot = at & ((1 << Bshift) - 1);

@@ -520,3 +520,31 @@ def test_selection_from_chunk_lists(pages, Hq, Hkv, k):
         for h in range(Hkv):
             best = 1 + np.sort(np.argsort(-score[b, h, 0, 1:P - 1], kind="stable")[:k - 2])
             assert np.array_equal(ids[b, h].cpu().numpy(), np.concatenate([[0], best, [P - 1]]))
+
+
+# A step whose build runs beside the scan counts the step's token itself, and the last of the request's page-heads and the selector
+# stores the length.  Requests before, at and after a page boundary, and one without room for the token; KV heads that fill the
+# build's CTAs (4, 2 or 1 page-heads) and that do not; three steps, so that what one step leaves behind shows in the next.
+@pytest.mark.parametrize("Hkv", [1, 3, 4])
+@pytest.mark.parametrize("B,dtype", [(16, "bf16"), (32, "bf16"), (64, "bf16"), (16, "f32")])
+def test_lengths_of_steps_whose_build_starts_at_once(B, dtype, Hkv):
+    from gpu_util import GpuCase
+    rows = 24
+    w = locks_synth.Workload("lengths", [B * rows, B * 9 - 1, B * 9 - 2, B * 9, 1, B * 20 - 3], Hq=4 * Hkv, Hkv=Hkv, B=B, dtype=dtype,
+                             fmt="i4" if dtype == "bf16" else "f32", rank=8, budget=4 * B, seed=B + Hkv)
+    gc = GpuCase(w)
+    want = gc.case.seq_lens.clone()
+    summ = gc.gpu_build()
+    before = summ.clone()
+    out = torch.empty(w.n, w.Hq, w.d, dtype=gc.case.k.dtype, device="cuda:0")
+    width = gc.case.block_table.shape[1] * B
+    for step in range(3):
+        kn, vn, qn = locks_synth.new_token(w, step, device="cuda:0")
+        gc.ctx.locks_decode_step(qn, kn, vn, gc.kv, summ, w.n, out)
+        torch.cuda.synchronize()
+        want = torch.minimum(want + 1, torch.full_like(want, width))
+        assert torch.equal(gc.case.seq_lens, want), step
+        changed = (summ != before).reshape(len(summ), -1).any(1).nonzero().flatten().tolist()
+        before = summ.clone()
+        filled = [int(gc.case.block_table[b, int(t) // B - 1]) for b, t in enumerate(want.tolist()) if t % B == 0 and t > 0 and b > 0]
+        assert set(filled) <= set(changed) <= set(filled) | {int(gc.case.block_table[0, rows - 1])}, step
