@@ -7,7 +7,6 @@
 // log-sum-exp.  The splits of a problem are merged by the thread-block cluster that they form, by the CTA that
 // arrives last, or by a second small kernel.  fp32 caches: attend_f32_kernel.
 // A NULL page table means "all pages": the same kernels are the dense flash-decode baseline.
-#include <cooperative_groups.h>
 #include <mutex>
 #include "locks_internal.cuh"
 
@@ -48,6 +47,16 @@ constexpr int kTile = LOCKS_B * LOCKS_D * 2;                 // 4096 B: one K or
 constexpr int kAttStage = 2 * kTile;                         // K + V
 constexpr int kAttStages = LOCKS_ATT_STAGES;                  // ring depth per warp
 constexpr int kAttSmem = LOCKS_ATT_WARPS * kAttStages * kAttStage;
+// Clusters: behind the rings a CTA keeps room for its slice of the other CTAs' partials (see attend_bf16_kernel).  At most 8 KB, so
+// that four CTAs still fit on an SM: 16 heads in slices of at most 15 / 16 of 8 KB, and the (max, sum) of the slice's heads.
+constexpr int kAttSmemMost = kAttSmem + 8192;
+constexpr int kWarpRow = LOCKS_D + 4;   // floats per head of a warp's partial: the four lanes of a quad on different banks
+__host__ __device__ constexpr int slice_heads(int slice) { return (slice + LOCKS_D - 1) / LOCKS_D + 1; }
+constexpr int cluster_smem(int G, int splits) {
+  const int slice = G * LOCKS_D / splits;   // (at most 16 splits, so a multiple of 8)
+  return kAttSmem + ((splits - 1) * slice * 4 + splits * slice_heads(slice) * 8 + 127) / 128 * 128;
+}
+static_assert(cluster_smem(16, 16) <= kAttSmemMost && cluster_smem(16, 8) <= kAttSmemMost && cluster_smem(15, 16) <= kAttSmemMost, "");
 // A single CTA merging many splits of many heads is a serial tail: beyond 64 (head, split) pairs the splits of a problem
 // go to the parallel merge kernel.
 constexpr int kFusedMerge = 64;
@@ -60,16 +69,30 @@ __device__ __forceinline__ int slice_length(const AttParams &p, int n) {
   return (int)(((uint64_t)(uint32_t)(n + p.splits - 1) * p.per_split) >> 32);
 }
 
-// Resolve the idx-th page of this problem's list: logical page, physical block, valid tokens.
-__device__ __forceinline__ bool resolve_page(const AttParams &p, int b, int64_t prob, int idx, int T, int &block,
-                                             int &ntok) {
-  const int page = p.ids ? p.ids[prob * p.kbud + idx] : idx;
+// Resolve a logical page of request b: physical block, valid tokens.
+__device__ __forceinline__ bool resolve_page(const AttParams &p, int b, int page, int T, int &block, int &ntok) {
   if (page < 0 || page >= p.Pmax) { set_status(p.status, LOCKS_ERR_BAD_BLOCK); return false; }
   block = p.block_table[(int64_t)b * p.Pmax + page];
   if (block < 0 || block >= p.num_blocks) { set_status(p.status, LOCKS_ERR_BAD_BLOCK); return false; }
   ntok = min(p.B, T - page * p.B);
   return ntok > 0;
 }
+
+// ---- thread-block clusters: an address of this CTA's shared memory in CTA `rank` of the cluster, stores to it, the barrier
+__device__ __forceinline__ uint32_t cluster_addr(const void *p, int rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ void cluster_st4(uint32_t a, float4 v) {
+  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+}
+__device__ __forceinline__ void cluster_st2(uint32_t a, float2 v) {
+  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
+}
+__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 __device__ __forceinline__ uint32_t movm_trans_b16(uint32_t v) {
   uint32_t d;
@@ -101,6 +124,7 @@ __global__ void __launch_bounds__(LOCKS_ATT_WARPS * 32, LOCKS_ATT_CTAS_PER_SM) a
   const uint8_t *Kb = reinterpret_cast<const uint8_t *>(p.k);
   const uint8_t *Vb = reinterpret_cast<const uint8_t *>(p.v);
   pdl_trigger();
+  if (p.cluster) cluster_arrive_relaxed();   // "this CTA has started": its shared memory may be written to from here on
 
   // query as the B operand: lane (x, t) holds head x (+8), dims 16 s + 2t.. and 16 s + 8 + 2t..
   uint32_t qb[NH][8][2];
@@ -121,8 +145,17 @@ __global__ void __launch_bounds__(LOCKS_ATT_WARPS * 32, LOCKS_ATT_CTAS_PER_SM) a
   pdl_wait();   // page table from the selector, appended K/V rows, sequence lengths
   const int T = p.seq_lens[b];
   const int B = WIDE ? p.B : LOCKS_B;
-  int npages = p.ids ? p.cnt[prob] : max((T + B - 1) / B, 0);
-  const int row = p.ids ? p.kbud : p.Pmax;
+  int npages = p.ids ? p.cnt[prob] : 0;
+  const int row = p.ids ? p.kbud : p.Pmax, sub_shift = WIDE ? p.sub_shift : 0;
+  // A sparse list is nearly always as long as its row: the page ids that this warp starts with are then fetched together with
+  // length and count instead of after them.
+  int id_ahead = 0;
+  if (p.ids) {
+    const int idx = (split * slice_length(p, row << sub_shift) + warp + lane * LOCKS_ATT_WARPS) >> sub_shift;
+    if (idx < row) id_ahead = p.ids[prob * p.kbud + idx];
+  } else {
+    npages = max((T + B - 1) / B, 0);
+  }
   if ((p.ids && npages < 0) || npages > row) {   // a count or a length beyond the table's row: use the row, report it
     if (threadIdx.x == 0) set_status(p.status, LOCKS_ERR_BAD_BLOCK);
     npages = npages < 0 ? 0 : row;
@@ -136,8 +169,8 @@ __global__ void __launch_bounds__(LOCKS_ATT_WARPS * 32, LOCKS_ATT_CTAS_PER_SM) a
     for (int i = lane; i < p.batch; i += 32) longest = max(longest, (p.seq_lens[i] + B - 1) / B);
     longest = min(__reduce_max_sync(0xffffffffu, longest), p.Pmax);
   }
-  const int per = slice_length(p, longest << (WIDE ? p.sub_shift : 0));
-  const int lo = split * per, hi = min(lo + per, npages << (WIDE ? p.sub_shift : 0));
+  const int per = slice_length(p, longest << sub_shift);
+  const int lo = split * per, hi = min(lo + per, npages << sub_shift);
 
   float oacc[8][NH][4];
 #pragma unroll
@@ -158,12 +191,15 @@ __global__ void __launch_bounds__(LOCKS_ATT_WARPS * 32, LOCKS_ATT_CTAS_PER_SM) a
 
   // page ids and physical blocks of this warp's pages are resolved 32 at a time, one lane each, so the
   // two dependent global loads are paid once per batch instead of once per page
-  const int first = lo + warp, sub_shift = WIDE ? p.sub_shift : 0, sub_mask = (1 << sub_shift) - 1;
+  const int first = lo + warp, sub_mask = (1 << sub_shift) - 1;
   auto resolve_batch = [&](int jb, int &blk, int &nt) {
     const int idx = first + (jb + lane) * LOCKS_ATT_WARPS;
     blk = 0;
     nt = 0;
-    if (idx < hi && !resolve_page(p, b, prob, idx >> sub_shift, T, blk, nt)) nt = 0;
+    if (idx < hi) {
+      const int page = !p.ids ? idx >> sub_shift : (jb == 0 && npages == row ? id_ahead : p.ids[prob * p.kbud + (idx >> sub_shift)]);
+      if (!resolve_page(p, b, page, T, blk, nt)) nt = 0;
+    }
     if constexpr (WIDE) nt = min(LOCKS_B, nt - (idx & sub_mask) * LOCKS_B);   // tokens of this tile (none past the sequence's end)
   };
   int blk_cur, nt_cur, blk_nxt = 0, nt_nxt = 0;
@@ -339,8 +375,10 @@ __global__ void __launch_bounds__(LOCKS_ATT_WARPS * 32, LOCKS_ATT_CTAS_PER_SM) a
 #pragma unroll
       for (int o = 4; o < 32; o <<= 1) lrun[hh][c] += __shfl_xor_sync(0xffffffffu, lrun[hh][c], o);
   __syncthreads();  // every warp is done with its ring: reuse it for the merge
-  float *wo = reinterpret_cast<float *>(ring);          // [16 heads][128] fp32
-  float *wm = wo + 16 * LOCKS_D, *wl = wm + 16;          // [16], [16]
+  // a warp's partial: [16 heads][kWarpRow] fp32, then (max, sum) of the 16 heads
+  constexpr int NT = LOCKS_ATT_WARPS * 32, kWarpBytes = kAttStages * kAttStage;
+  float *wo = reinterpret_cast<float *>(ring);
+  float2 *ws = reinterpret_cast<float2 *>(wo + 16 * kWarpRow);
 #pragma unroll
   for (int hh = 0; hh < NH; ++hh) {
 #pragma unroll
@@ -348,110 +386,118 @@ __global__ void __launch_bounds__(LOCKS_ATT_WARPS * 32, LOCKS_ATT_CTAS_PER_SM) a
       const int row = 8 * hh + 2 * t + c;
 #pragma unroll
       for (int mt = 0; mt < 8; ++mt) {
-        wo[row * LOCKS_D + 16 * mt + x] = oacc[mt][hh][c];
-        wo[row * LOCKS_D + 16 * mt + 8 + x] = oacc[mt][hh][2 + c];
+        wo[row * kWarpRow + 16 * mt + x] = oacc[mt][hh][c];
+        wo[row * kWarpRow + 16 * mt + 8 + x] = oacc[mt][hh][2 + c];
       }
-      if (x == 0) { wm[row] = mrun[hh][c]; wl[row] = lrun[hh][c]; }
+      if (x == 0) ws[row] = make_float2(mrun[hh][c], lrun[hh][c]);
     }
   }
   __syncthreads();
-  if (p.cluster) {
-    // The splits of this (request, KV head) are the CTAs of one cluster.  Each CTA first folds its warps into
-    // one unnormalised partial in its own shared memory; after a cluster barrier CTA r produces a slice of the
-    // problem's G x 128 outputs by reading every CTA's partial through distributed shared memory; a second
-    // barrier keeps every CTA's memory alive until its peers are done.  No partial leaves the SMs.
-    namespace cg = cooperative_groups;
-    cg::cluster_group cluster = cg::this_cluster();
-    constexpr int NT = LOCKS_ATT_WARPS * 32;
-    // the CTA's partial replaces warp 0's in place (element e is read and written by one thread only); its
-    // (max, sum) go to the idle tail of warp 1's ring, because other threads still read warp 0's
-    float *co = reinterpret_cast<float *>(smem);
-    float *cm = reinterpret_cast<float *>(smem + kAttStages * kAttStage) + 16 * LOCKS_D + 32, *cl = cm + 16;
-    for (int e = threadIdx.x; e < p.G * LOCKS_D; e += NT) {
-      const int g = e / LOCKS_D, dim = e - g * LOCKS_D;
-      float M = -INFINITY;
+  // the CTA's (max, sum) of head g, and the factors of its warps' partials
+  auto fold_head = [&](int g, float (&sc)[LOCKS_ATT_WARPS]) -> float2 {
+    float2 v[LOCKS_ATT_WARPS];
+    float M = -INFINITY, L = 0.f;
 #pragma unroll
-      for (int w = 0; w < LOCKS_ATT_WARPS; ++w)
-        M = fmaxf(M, reinterpret_cast<const float *>(smem + w * kAttStages * kAttStage)[16 * LOCKS_D + g]);
-      float L = 0.f, o = 0.f;
-      if (M > -INFINITY) {
-#pragma unroll
-        for (int w = 0; w < LOCKS_ATT_WARPS; ++w) {
-          const float *ww = reinterpret_cast<const float *>(smem + w * kAttStages * kAttStage);
-          const float sc = ex2f(ww[16 * LOCKS_D + g] - M);
-          L += ww[16 * LOCKS_D + 16 + g] * sc;
-          o += ww[g * LOCKS_D + dim] * sc;
-        }
-      }
-      co[e] = o;
-      if (dim == 0) { cm[g] = M; cl[g] = L; }
+    for (int w = 0; w < LOCKS_ATT_WARPS; ++w) {
+      v[w] = reinterpret_cast<const float2 *>(smem + w * kWarpBytes + 16 * kWarpRow * 4)[g];
+      M = fmaxf(M, v[w].x);
     }
-    cluster.sync();
-    const int nout = p.G * LOCKS_D, per = (nout + p.splits - 1) / p.splits;
-    const int e1 = min(nout, (split + 1) * per);
-    for (int e = split * per + threadIdx.x; e < e1; e += NT) {
-      const int g = e / LOCKS_D;
-      float mv[16], lv[16], ov[16];
 #pragma unroll
-      for (int c = 0; c < 16; ++c) {
-        mv[c] = -INFINITY; lv[c] = 0.f; ov[c] = 0.f;
-        if (c < p.splits) {
-          mv[c] = cluster.map_shared_rank(cm, c)[g];
-          lv[c] = cluster.map_shared_rank(cl, c)[g];
-          ov[c] = cluster.map_shared_rank(co, c)[e];
-        }
+    for (int w = 0; w < LOCKS_ATT_WARPS; ++w) {
+      sc[w] = M > -INFINITY ? ex2f(v[w].x - M) : 0.f;
+      L += v[w].y * sc[w];
+    }
+    return make_float2(M, L);
+  };
+  auto fold_dims = [&](int g, int d4, const float (&sc)[LOCKS_ATT_WARPS]) -> float4 {   // dims d4 .. d4 + 3, unnormalised
+    float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int w = 0; w < LOCKS_ATT_WARPS; ++w) {
+      const float4 v = *reinterpret_cast<const float4 *>(smem + w * kWarpBytes + (g * kWarpRow + d4) * 4);
+      o.x += v.x * sc[w]; o.y += v.y * sc[w]; o.z += v.z * sc[w]; o.w += v.w * sc[w];
+    }
+    return o;
+  };
+  if (p.cluster) {
+    // The splits of this (request, KV head) are the CTAs of one cluster, and CTA r finishes a slice of the problem's G x 128
+    // outputs.  Every CTA folds its warps and stores the folded partial, slice by slice, straight into the shared memory of the
+    // CTA that finishes it; after one cluster barrier every CTA reads its slice's partials from its own memory, and nobody's
+    // memory is touched from outside any more.  Bound by the latency of one chain: stores to peers, barrier, local loads.  Steps, with
+    // the peers' partials read remotely after a barrier, and a second barrier to keep the peers alive, and now: 8 x 32K tokens 56.8
+    // -> 54.7 us, 24 chat requests 53.0 -> 51.4, 1 x 1M (16 heads) 73.3 -> 72.0, 11 x 14K 49.4 -> 47.8.
+    const int slice = p.G * LOCKS_D / p.splits, nh = slice_heads(slice);
+    float *rx = reinterpret_cast<float *>(smem + kAttSmem);                    // [splits - 1][slice]: the peers' partials
+    float2 *rms = reinterpret_cast<float2 *>(rx + (p.splits - 1) * slice);     // [splits][nh]: (max, sum) of the slice's heads
+    float *own = reinterpret_cast<float *>(smem + (LOCKS_ATT_WARPS - 1) * kWarpBytes) + 16 * kWarpRow + 32;   // idle tail of a ring
+    cluster_wait();   // the peers have started
+    for (int i = threadIdx.x; i < p.G * (LOCKS_D / 4); i += NT) {
+      const int g = i / (LOCKS_D / 4), d4 = 4 * (i % (LOCKS_D / 4)), e = g * LOCKS_D + d4, r = e / slice;
+      float sc[LOCKS_ATT_WARPS];
+      (void)fold_head(g, sc);
+      const float4 o = fold_dims(g, d4, sc);
+      if (r == split) *reinterpret_cast<float4 *>(own + e - r * slice) = o;
+      else cluster_st4(cluster_addr(rx + (split - (split > r)) * slice + e - r * slice, r), o);
+    }
+    for (int i = threadIdx.x; i < p.splits * nh; i += NT) {
+      const int r = i / nh, j = i - r * nh, g = r * slice / LOCKS_D + j;
+      if (g * LOCKS_D < (r + 1) * slice) {
+        float sc[LOCKS_ATT_WARPS];
+        cluster_st2(cluster_addr(rms + split * nh + j, r), fold_head(g, sc));
       }
+    }
+    cluster_arrive();
+    cluster_wait();
+    const int g0 = split * slice / LOCKS_D;
+    for (int e = threadIdx.x; e < slice; e += NT) {
+      const int g = (split * slice + e) / LOCKS_D, dim = split * slice + e - g * LOCKS_D;
+      const float2 *ms = rms + g - g0;
       float M = -INFINITY;
-#pragma unroll
-      for (int c = 0; c < 16; ++c) M = fmaxf(M, mv[c]);
+#pragma unroll 4
+      for (int c = 0; c < p.splits; ++c) M = fmaxf(M, ms[c * nh].x);
       float L = 0.f, o = 0.f;
       if (M > -INFINITY) {
-#pragma unroll
-        for (int c = 0; c < 16; ++c) {
-          const float sc = ex2f(mv[c] - M);
-          L = fmaf(lv[c], sc, L);
-          o = fmaf(ov[c], sc, o);
+#pragma unroll 4
+        for (int c = 0; c < p.splits; ++c) {
+          const float2 v = ms[c * nh];
+          const float sc = ex2f(v.x - M);
+          L = fmaf(v.y, sc, L);
+          o = fmaf(c == split ? own[e] : rx[(c - (c > split)) * slice + e], sc, o);
         }
         o /= L;
       }
       const int64_t row = (int64_t)b * p.Hq + h * p.G + g;
-      reinterpret_cast<__nv_bfloat16 *>(p.out)[row * LOCKS_D + (e - g * LOCKS_D)] = __float2bfloat16_rn(o);
-      if (p.lse && e == g * LOCKS_D) p.lse[row] = (M > -INFINITY) ? (M + log2f(L)) * kLn2 : -INFINITY;
+      reinterpret_cast<__nv_bfloat16 *>(p.out)[row * LOCKS_D + dim] = __float2bfloat16_rn(o);
+      if (p.lse && dim == 0) p.lse[row] = (M > -INFINITY) ? (M + log2f(L)) * kLn2 : -INFINITY;
     }
-    cluster.sync();
     return;
   }
-  for (int e = threadIdx.x; e < p.G * LOCKS_D; e += LOCKS_ATT_WARPS * 32) {
-    const int g = e / LOCKS_D, dim = e - g * LOCKS_D;
-    float M = -INFINITY;
-#pragma unroll
-    for (int w = 0; w < LOCKS_ATT_WARPS; ++w)
-      M = fmaxf(M, reinterpret_cast<const float *>(smem + w * kAttStages * kAttStage)[16 * LOCKS_D + g]);
-    float L = 0.f, o = 0.f;
-    if (M > -INFINITY) {
-#pragma unroll
-      for (int w = 0; w < LOCKS_ATT_WARPS; ++w) {
-        const float *ww = reinterpret_cast<const float *>(smem + w * kAttStages * kAttStage);
-        const float sc = ex2f(ww[16 * LOCKS_D + g] - M);
-        L += ww[16 * LOCKS_D + 16 + g] * sc;
-        o += ww[g * LOCKS_D + dim] * sc;
-      }
-      o /= L;
-    }
+  for (int i = threadIdx.x; i < p.G * (LOCKS_D / 4); i += NT) {
+    const int g = i / (LOCKS_D / 4), d4 = 4 * (i % (LOCKS_D / 4));
+    float sc[LOCKS_ATT_WARPS];
+    const float2 ML = fold_head(g, sc);
+    float4 o = fold_dims(g, d4, sc);
+    if (ML.x > -INFINITY) { o.x /= ML.y; o.y /= ML.y; o.z /= ML.y; o.w /= ML.y; }
     const int hq = h * p.G + g;
-    const float lse2 = (M > -INFINITY) ? M + log2f(L) : -INFINITY;
+    const float lse2 = (ML.x > -INFINITY) ? ML.x + log2f(ML.y) : -INFINITY;
     if (p.splits == 1) {
-      reinterpret_cast<__nv_bfloat16 *>(p.out)[((int64_t)b * p.Hq + hq) * LOCKS_D + dim] = __float2bfloat16_rn(o);
-      if (p.lse && dim == 0) p.lse[(int64_t)b * p.Hq + hq] = lse2 * kLn2;
+      const int64_t row = (int64_t)b * p.Hq + hq;
+      __nv_bfloat16 *dst = reinterpret_cast<__nv_bfloat16 *>(p.out) + row * LOCKS_D + d4;
+      if ((uintptr_t)p.out % 8 == 0) {   // (the caller's buffer need not be aligned)
+        *reinterpret_cast<uint2 *>(dst) = make_uint2(pack_bf16(o.x, o.y), pack_bf16(o.z, o.w));
+      } else {
+        dst[0] = __float2bfloat16_rn(o.x); dst[1] = __float2bfloat16_rn(o.y);
+        dst[2] = __float2bfloat16_rn(o.z); dst[3] = __float2bfloat16_rn(o.w);
+      }
+      if (p.lse && d4 == 0) p.lse[row] = lse2 * kLn2;
     } else {
       const int64_t slot = ((int64_t)b * p.Hq + hq) * p.splits + split;
-      p.part_o[slot * LOCKS_D + dim] = o;
-      if (dim == 0) p.part_lse[slot] = lse2;
+      *reinterpret_cast<float4 *>(p.part_o + slot * LOCKS_D + d4) = o;
+      if (d4 == 0) p.part_lse[slot] = lse2;
     }
   }
   if (p.splits == 1 || !p.fused_merge) return;
   // the last CTA of this (request, KV head) to arrive merges the splits' partials by log-sum-exp
-  __shared__ int sh_last;
+  int &sh_last = *reinterpret_cast<int *>(smem + kWarpBytes - 16);   // idle tail of a ring
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) sh_last = (atomicAdd(&p.done[prob], 1) == p.splits - 1);
@@ -460,7 +506,6 @@ __global__ void __launch_bounds__(LOCKS_ATT_WARPS * 32, LOCKS_ATT_CTAS_PER_SM) a
   __threadfence();
   // weights of the splits: sh_w[g][s] = 2^(lse_s - max), then normalised by their sum
   float *sh_w = reinterpret_cast<float *>(smem);   // [G][splits] <= 16 x 64 floats, the rings are idle now
-  constexpr int NT = LOCKS_ATT_WARPS * 32;
   for (int e = threadIdx.x; e < p.G * p.splits; e += NT) {
     const int g = e / p.splits, s2 = e - g * p.splits;
     sh_w[e] = __ldcg(p.part_lse + ((int64_t)b * p.Hq + h * p.G + g) * p.splits + s2);
@@ -539,10 +584,11 @@ __global__ void __launch_bounds__(128, 3) attend_f32_kernel(AttParams p) {
   float m = -INFINITY, l = 0.f;         // of the lane's head; l: its tokens' share
   const float c2 = p.sm_scale * kLog2e;
   int block = 0, ntok = 0;
-  bool good = lo + warp < hi && resolve_page(p, b, prob, lo + warp, Tn, block, ntok);
+  auto page_at = [&](int idx) { return p.ids ? p.ids[prob * p.kbud + idx] : idx; };
+  bool good = lo + warp < hi && resolve_page(p, b, page_at(lo + warp), Tn, block, ntok);
   for (int idx = lo + warp; idx < hi; idx += 4) {
     int next_block = 0, next_ntok = 0;   // resolved one page ahead
-    const bool next_good = idx + 4 < hi && resolve_page(p, b, prob, idx + 4, Tn, next_block, next_ntok);
+    const bool next_good = idx + 4 < hi && resolve_page(p, b, page_at(idx + 4), Tn, next_block, next_ntok);
     if (good) {
       const int64_t base = (int64_t)block * p.sb + (int64_t)(h / p.kvdiv) * p.sh + 4 * lane;
       for (int t0 = 0; t0 < ntok; t0 += kTok) {
@@ -740,13 +786,13 @@ AttGeom attend_geometry(locks_ctx *c, int batch, int Hkv, int G, bool dense) {
   // requests slower), or 8 where the cluster leaves more than half of the CTAs that there is room for unused (dense, 1 x 8K
   // tokens: 13.2 us as clusters of 16, 12.4 as 72 splits; with 16 heads, whose splits cost more to merge, 20.5 and 21.4).
   if (c->att_clusters[0] < 0) {   // clusters of 2, 4, 8, 16 CTAs of this kernel that fit the device at once (probed once)
-    cudaFuncSetAttribute(attend_bf16_kernel<1, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmem);
+    cudaFuncSetAttribute(attend_bf16_kernel<1, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmemMost);
     cudaFuncSetAttribute(attend_bf16_kernel<1, true, false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     for (int i = 0; i < 4; ++i) {
       cudaLaunchConfig_t lc = {};
       lc.gridDim = dim3(2 << i, 1, 1);
       lc.blockDim = dim3(LOCKS_ATT_WARPS * 32);
-      lc.dynamicSmemBytes = kAttSmem;
+      lc.dynamicSmemBytes = kAttSmemMost;
       cudaLaunchAttribute at[1];
       at[0].id = cudaLaunchAttributeClusterDimension;
       at[0].val.clusterDim.x = 2 << i; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
@@ -811,11 +857,11 @@ int locks_launch_attend(locks_ctx *c, const void *q, const locks_kv *kv, int bat
 #define LOCKS_ATT_CASE(NH_, CONTIG_, WIDE_)                                                                                  \
   do {                                                                                                                      \
     if (attrs) {                                                                                                            \
-      cudaFuncSetAttribute(attend_bf16_kernel<NH_, CONTIG_, WIDE_>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmem); \
+      cudaFuncSetAttribute(attend_bf16_kernel<NH_, CONTIG_, WIDE_>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmemMost); \
       cudaFuncSetAttribute(attend_bf16_kernel<NH_, CONTIG_, WIDE_>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);     \
     }                                                                                                                       \
     if ((p.G > 8) != (NH_ == 2) || contig != CONTIG_ || wide != WIDE_) break;                                               \
-    if (p.cluster) locks_launch_pdl_cluster(attend_bf16_kernel<NH_, CONTIG_, WIDE_>, grid, blk, kAttSmem, p.splits, st, p); \
+    if (p.cluster) locks_launch_pdl_cluster(attend_bf16_kernel<NH_, CONTIG_, WIDE_>, grid, blk, cluster_smem(p.G, p.splits), p.splits, st, p); \
     else locks_launch_pdl(attend_bf16_kernel<NH_, CONTIG_, WIDE_>, grid, blk, kAttSmem, st, p);                             \
   } while (0)
     LOCKS_ATT_CASE(1, true, false);
@@ -896,10 +942,10 @@ extern "C" int locks_sparse_attend_noalloc(const locks_config *cfg, const void *
     void *ptr = nullptr;
     if (cudaGetSymbolAddress(&ptr, g_noalloc_scratch) != cudaSuccess || ptr == nullptr) return LOCKS_ERR_CUDA;
     if (cudaDeviceGetAttribute(&nd.num_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return LOCKS_ERR_CUDA;
-    cudaFuncSetAttribute(attend_bf16_kernel<1, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmem);
-    cudaFuncSetAttribute(attend_bf16_kernel<2, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmem);
-    cudaFuncSetAttribute(attend_bf16_kernel<1, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmem);
-    cudaFuncSetAttribute(attend_bf16_kernel<2, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmem);
+    cudaFuncSetAttribute(attend_bf16_kernel<1, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmemMost);
+    cudaFuncSetAttribute(attend_bf16_kernel<2, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmemMost);
+    cudaFuncSetAttribute(attend_bf16_kernel<1, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmemMost);
+    cudaFuncSetAttribute(attend_bf16_kernel<2, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmemMost);
     nd.scratch = reinterpret_cast<unsigned char *>(ptr);
     nd.ready = true;
   }

@@ -321,7 +321,7 @@ struct KeyInputs {
 // alone came first, then 2000 cycles of address arithmetic with a 64-bit division, then the rest).
 template <int HB, typename Begin>
 __device__ __forceinline__ int chunk_keys(const KeyInputs &in, Begin begin, float *logshare_row) {
-  constexpr int SB = 16 / HB, NP = HB == 16 ? 8 : 4;   // NP: partials in flight per lane
+  constexpr int SB = 16 / HB, NP = HB == 16 ? 5 : 4;   // NP: partials in flight per lane
   SelShared &sh = shared_state();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, G = in.G;
   const float *row0 = in.shat0 + in.c0 + tid;

@@ -548,3 +548,23 @@ def test_lengths_of_steps_whose_build_starts_at_once(B, dtype, Hkv):
         before = summ.clone()
         filled = [int(gc.case.block_table[b, int(t) // B - 1]) for b, t in enumerate(want.tolist()) if t % B == 0 and t > 0 and b > 0]
         assert set(filled) <= set(changed) <= set(filled) | {int(gc.case.block_table[0, rows - 1])}, step
+
+
+# The splits of a problem merge through the shared memory of their cluster (16, 8, 4 or 2 CTAs, by the number of problems; the last
+# case has one CTA each): slices of whole heads, of parts of heads and across heads, lists shorter than their row, an output buffer
+# that is aligned to its elements only.  Tolerance: P and the result in bf16 (see test_gpu_parity.py).
+@pytest.mark.parametrize("n,Hkv,G", [(1, 3, 5), (1, 2, 16), (3, 4, 1), (2, 4, 12), (5, 8, 7), (10, 4, 9), (5, 8, 16), (25, 4, 4), (25, 4, 3), (50, 4, 5), (64, 4, 8)])
+def test_splits_merge_in_their_cluster(n, Hkv, G):
+    from gpu_util import GpuCase
+    w = locks_synth.Workload("merge", [900 + 7 * i % 60 if i % 5 else 100 + i for i in range(n)], Hq=G * Hkv, Hkv=Hkv, budget=768, seed=n + G)
+    gc = GpuCase(w)
+    ids, cnt, _, _ = gc.gpu_select(gc.gpu_build())
+    want, want_lse = oracle.attend(gc.cache, t2np(gc.case.q), gc.sm, ids, cnt)
+    d_ids, d_cnt = torch.from_numpy(ids).cuda(), torch.from_numpy(cnt).cuda()
+    for shift in (0, 1):
+        out = torch.empty(w.n * w.Hq * w.d + 1, dtype=torch.bfloat16, device="cuda:0")[shift:][:w.n * w.Hq * w.d].view(w.n, w.Hq, w.d)
+        lse = torch.empty(w.n, w.Hq, dtype=torch.float32, device="cuda:0")
+        gc.ctx.locks_sparse_attend(gc.case.q, gc.kv, w.n, d_ids, d_cnt, out, lse)
+        torch.cuda.synchronize()
+        assert np.abs(out.float().cpu().numpy() - want).max() <= 2e-2 and np.abs(lse.cpu().numpy() - want_lse).max() <= 1e-3
+    assert gc.status() == 0
