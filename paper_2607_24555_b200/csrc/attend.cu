@@ -428,10 +428,13 @@ __global__ void __launch_bounds__(LOCKS_ATT_WARPS * 32, LOCKS_ATT_CTAS_PER_SM) a
     const int slice = p.G * LOCKS_D / p.splits, nh = slice_heads(slice);
     float *rx = reinterpret_cast<float *>(smem + kAttSmem);                    // [splits - 1][slice]: the peers' partials
     float2 *rms = reinterpret_cast<float2 *>(rx + (p.splits - 1) * slice);     // [splits][nh]: (max, sum) of the slice's heads
-    float *own = reinterpret_cast<float *>(smem + (LOCKS_ATT_WARPS - 1) * kWarpBytes) + 16 * kWarpRow + 32;   // idle tail of a ring
+    // idle tails of two rings: this CTA's own slice; [nh][splits] the CTAs' factors, and their share of the denominator
+    float *own = reinterpret_cast<float *>(smem + (LOCKS_ATT_WARPS - 1) * kWarpBytes) + 16 * kWarpRow + 32;
+    float2 *factor = reinterpret_cast<float2 *>(smem + 16 * kWarpRow * 4 + 128);
+    const float inv_slice = 1.f / (float)slice;   // e / slice for e < 2048: (e + 1/2) / slice is at least 1 / 2048 from a whole number
     cluster_wait();   // the peers have started
     for (int i = threadIdx.x; i < p.G * (LOCKS_D / 4); i += NT) {
-      const int g = i / (LOCKS_D / 4), d4 = 4 * (i % (LOCKS_D / 4)), e = g * LOCKS_D + d4, r = e / slice;
+      const int g = i / (LOCKS_D / 4), d4 = 4 * (i % (LOCKS_D / 4)), e = g * LOCKS_D + d4, r = (int)(((float)e + 0.5f) * inv_slice);
       float sc[LOCKS_ATT_WARPS];
       (void)fold_head(g, sc);
       const float4 o = fold_dims(g, d4, sc);
@@ -447,27 +450,37 @@ __global__ void __launch_bounds__(LOCKS_ATT_WARPS * 32, LOCKS_ATT_CTAS_PER_SM) a
     }
     cluster_arrive();
     cluster_wait();
+    const int lg = __ffs(p.splits) - 1;   // splits is a power of two
+    for (int i = threadIdx.x; i < p.splits * nh; i += NT) {
+      const int j = i >> lg, c = i & (p.splits - 1);
+      if ((split * slice / LOCKS_D + j) * LOCKS_D >= (split + 1) * slice) continue;
+      float M = -INFINITY;
+#pragma unroll 8
+      for (int u = 0; u < p.splits; ++u) M = fmaxf(M, rms[u * nh + j].x);
+      const float2 v = rms[c * nh + j];
+      const float sc = M > -INFINITY ? ex2f(v.x - M) : 0.f;
+      factor[i] = make_float2(sc, v.y * sc);
+    }
+    __syncthreads();
     const int g0 = split * slice / LOCKS_D;
     for (int e = threadIdx.x; e < slice; e += NT) {
       const int g = (split * slice + e) / LOCKS_D, dim = split * slice + e - g * LOCKS_D;
-      const float2 *ms = rms + g - g0;
-      float M = -INFINITY;
-#pragma unroll 4
-      for (int c = 0; c < p.splits; ++c) M = fmaxf(M, ms[c * nh].x);
+      const float2 *fc = factor + (g - g0) * p.splits;
       float L = 0.f, o = 0.f;
-      if (M > -INFINITY) {
 #pragma unroll 4
-        for (int c = 0; c < p.splits; ++c) {
-          const float2 v = ms[c * nh];
-          const float sc = ex2f(v.x - M);
-          L = fmaf(v.y, sc, L);
-          o = fmaf(c == split ? own[e] : rx[(c - (c > split)) * slice + e], sc, o);
-        }
-        o /= L;
+      for (int c = 0; c < p.splits; ++c) {
+        const float2 f = fc[c];
+        L += f.y;
+        o = fmaf(c == split ? own[e] : rx[(c - (c > split)) * slice + e], f.x, o);
       }
+      if (L != 0.f) o /= L;   // (0: no tokens)
       const int64_t row = (int64_t)b * p.Hq + h * p.G + g;
       reinterpret_cast<__nv_bfloat16 *>(p.out)[row * LOCKS_D + dim] = __float2bfloat16_rn(o);
-      if (p.lse && dim == 0) p.lse[row] = (M > -INFINITY) ? (M + log2f(L)) * kLn2 : -INFINITY;
+      if (p.lse && dim == 0) {
+        float M = -INFINITY;
+        for (int c = 0; c < p.splits; ++c) M = fmaxf(M, rms[c * nh + g - g0].x);
+        p.lse[row] = (M > -INFINITY) ? (M + log2f(L)) * kLn2 : -INFINITY;
+      }
     }
     return;
   }
