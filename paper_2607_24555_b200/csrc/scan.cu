@@ -352,14 +352,12 @@ __device__ __forceinline__ void mma_f16_z(float (&d)[4], uint32_t a0, uint32_t a
 // A query head as MMA operand registers: lane (.., t) holds dims 32 t .. 32 t + 31 of `row`; a0[s] dims 4 s, 4 s + 1, a2[s]
 // dims 4 s + 2, 4 s + 3 divided by 16 (see "Numerics").  inv = 1 / the power of two that the row was scaled by, sum8 = 8 times
 // the sum of the scaled row.  All four lanes of a row take part.
-__device__ __forceinline__ void load_q_row(const __nv_bfloat16 *row, int t, bool valid, uint32_t (&a0)[8], uint32_t (&a2)[8],
-                                           float &inv, float &sum8) {
-  uint4 v[4] = {};
-  if (valid) {
-    const uint4 *qp = reinterpret_cast<const uint4 *>(row + 32 * t);
+__device__ __forceinline__ void fetch_q_row(const __nv_bfloat16 *row, int t, bool valid, uint4 (&v)[4]) {
+  const uint4 *qp = reinterpret_cast<const uint4 *>(row + 32 * t);
 #pragma unroll
-    for (int m = 0; m < 4; ++m) v[m] = __ldg(qp + m);
-  }
+  for (int m = 0; m < 4; ++m) v[m] = valid ? __ldg(qp + m) : make_uint4(0u, 0u, 0u, 0u);
+}
+__device__ __forceinline__ void load_q_row(const uint4 (&v)[4], uint32_t (&a0)[8], uint32_t (&a2)[8], float &inv, float &sum8) {
   const uint32_t *w = reinterpret_cast<const uint32_t *>(v);
   uint32_t mx = 0u;  // largest |q| of the row as a bf16 bit pattern (orders like the value)
 #pragma unroll
@@ -482,6 +480,19 @@ __global__ void __launch_bounds__(kScanWarps * 32, kScanCtasPerSm) scan_i4_kerne
   if (!BAL && slot >= nslots) return;
   const int gstep = BAL ? 1 : wpp, pstep = BAL ? 1 : nslots, g0 = BAL ? 0 : sub;   // cursor stepping
 
+  // a problem's query heads (head held by this lane's column), as stored
+  auto fetch_query = [&](int prob, uint4 (&raw)[NH][4]) {
+#pragma unroll
+    for (int hh = 0; hh < NH; ++hh) {
+      const int gx = PK ? (x & 3) : x + 8 * hh;
+      fetch_q_row(reinterpret_cast<const __nv_bfloat16 *>(p.q) + ((int64_t)prob * p.G + gx) * LOCKS_D, t, gx < p.G, raw[hh]);
+    }
+  };
+  // The query that a warp starts with is under way while lengths and block ids are fetched and the first copies are issued.
+  uint4 q_first[NH][4];
+  int q_prob = -1;
+  if (!BAL && slot < nprob) { q_prob = slot; fetch_query(slot, q_first); }
+
   auto groups_of = [&](int b) {   // 8-page groups of scored pages of request b
     const int P = (step_len(p, b) + LOCKS_B - 1) / LOCKS_B;
     return P <= p.k ? 0 : (P - 1 + LOCKS_GROUP - 1) / LOCKS_GROUP;
@@ -533,6 +544,8 @@ __global__ void __launch_bounds__(kScanWarps * 32, kScanCtasPerSm) scan_i4_kerne
     const int r = u0 - fstart, hh0 = r / fng;
     cp.prob = fb * p.Hkv + hh0;
     cp.grp = r - hh0 * fng;
+    q_prob = cp.prob;
+    fetch_query(q_prob, q_first);
     // partials of a problem sit at (warp - first warp that owns one of its units): 0 for every problem this
     // warp enters at its first group; for the first one, count the warps between its first unit and u0
     if (cp.grp > 0) {
@@ -661,7 +674,6 @@ __global__ void __launch_bounds__(kScanWarps * 32, kScanCtasPerSm) scan_i4_kerne
   float inv_s[NH], ksum[2];        // c2 / scale of head x (+8); 8 * sum_c q'[c] of heads 2t, 2t+1 (NH = 2: of heads x, x+8)
   float inv2[2] = {0.f, 0.f};      // c2 / scale of heads 2t, 2t+1 (NH = 1)
   int cur_prob = -1;
-  const __nv_bfloat16 *q = reinterpret_cast<const __nv_bfloat16 *>(p.q);
   const float c2 = p.sm_scale * kLog2e;
 
   // candidate partial (max, sum exp) of the current problem, kept per lane and reduced across the warp
@@ -680,14 +692,14 @@ __global__ void __launch_bounds__(kScanWarps * 32, kScanCtasPerSm) scan_i4_kerne
     if (BAL && finished && lane == 0) p.part_cnt[cur_prob] = pslot + 1;
 #pragma unroll
     for (int hh = 0; hh < NH; ++hh) {
-      float m = pm[hh], sacc = ps[hh];
+      float m = pm[hh];   // lanes sharing a head: t (1, 2) and, packed, x bit 2
 #pragma unroll
-      for (int o = 1; o <= 16; o <<= 1) {
-        if (o == 4 || o == 8 || (o == 16 && !PK)) continue;   // lanes sharing a head: t (1, 2) and, packed, x bit 2
-        const float om = __shfl_xor_sync(0xffffffffu, m, o), os = __shfl_xor_sync(0xffffffffu, sacc, o);
-        const float nm = fmaxf(m, om);
-        if (nm > -INFINITY) { sacc = sacc * __expf(m - nm) + os * __expf(om - nm); m = nm; }
-      }
+      for (int o = 1; o <= 16; o <<= 1)
+        if (o < 4 || (o == 16 && PK)) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+      float sacc = m > -INFINITY ? ps[hh] * __expf(pm[hh] - m) : 0.f;
+#pragma unroll
+      for (int o = 1; o <= 16; o <<= 1)
+        if (o < 4 || (o == 16 && PK)) sacc += __shfl_xor_sync(0xffffffffu, sacc, o);
       const int g = PK ? (x & 3) : x + 8 * hh;
       if (t == 0 && (!PK || x < 4) && g < p.G) {
         if (CR && to_smem) red[warp * 16 + g] = make_float2(m, sacc);
@@ -698,38 +710,44 @@ __global__ void __launch_bounds__(kScanWarps * 32, kScanCtasPerSm) scan_i4_kerne
     }
   };
 
+  auto start_problem = [&](const uint4 (&raw)[NH][4], int pslot) {
+    cur_prob = cc.prob;
+    cur_b = cc.b;
+    cur_h = cc.h;
+    cur_pslot = pslot;
+#pragma unroll
+    for (int hh = 0; hh < NH; ++hh)
+      srow[hh] = p.shat + ((int64_t)cur_b * p.Hq + cur_h * p.G + (PK ? (x & 3) : x + 8 * hh)) * p.Pmax;
+#pragma unroll
+    for (int hh = 0; hh < NH; ++hh) {
+      float s8;
+      load_q_row(raw[hh], qb0[hh], qb2[hh], inv_s[hh], s8);
+      inv_s[hh] *= c2;   // from here on: the factor that turns a scaled dot product into a log2-domain logit
+      if (NH == 2) {
+        ksum[hh] = s8;
+      } else {   // lane (x, t) owns head gx; the column fragment needs the heads of columns 2t, 2t+1
+        ksum[0] = __shfl_sync(0xffffffffu, s8, (2 * t) * 4);
+        ksum[1] = __shfl_sync(0xffffffffu, s8, (2 * t + 1) * 4);
+        inv2[0] = __shfl_sync(0xffffffffu, inv_s[hh], (2 * t) * 4);
+        inv2[1] = __shfl_sync(0xffffffffu, inv_s[hh], (2 * t + 1) * 4);
+      }
+    }
+  };
+  if (cc.prob < nprob) {   // the first problem's query, fetched at the start
+    if (cc.prob != q_prob) fetch_query(cc.prob, q_first);
+    start_problem(q_first, BAL ? pslot_first : sub);
+  }
+
   int it = 0;
   bool ok = true;
   while (cc.prob < nprob) {
     const int stage = it % kScanStages;
     const uint32_t parity = (it / kScanStages) & 1;
-    const int b = cc.b, h = cc.h;
-    // a new problem's query is fetched and normalised BEFORE waiting for the group's summaries, so that the
-    // round trip of the query load runs beside the copy instead of after it
-    if (cc.prob != cur_prob) {
-      if (cur_prob >= 0) flush(false, true);
-      cur_prob = cc.prob;
-      cur_b = b;
-      cur_h = h;
-      cur_pslot = BAL ? (it == 0 ? pslot_first : 0) : sub;
-#pragma unroll
-      for (int hh = 0; hh < NH; ++hh)
-        srow[hh] = p.shat + ((int64_t)b * p.Hq + h * p.G + (PK ? (x & 3) : x + 8 * hh)) * p.Pmax;
-#pragma unroll
-      for (int hh = 0; hh < NH; ++hh) {
-        float s8;
-        const int gx = PK ? (x & 3) : x + 8 * hh;   // head held by this lane's column
-        load_q_row(q + ((int64_t)b * p.Hq + h * p.G + gx) * LOCKS_D, t, gx < p.G, qb0[hh], qb2[hh], inv_s[hh], s8);
-        inv_s[hh] *= c2;   // from here on: the factor that turns a scaled dot product into a log2-domain logit
-        if (NH == 2) {
-          ksum[hh] = s8;
-        } else {   // lane (x, t) owns head gx; the column fragment needs the heads of columns 2t, 2t+1
-          ksum[0] = __shfl_sync(0xffffffffu, s8, (2 * t) * 4);
-          ksum[1] = __shfl_sync(0xffffffffu, s8, (2 * t + 1) * 4);
-          inv2[0] = __shfl_sync(0xffffffffu, inv_s[hh], (2 * t) * 4);
-          inv2[1] = __shfl_sync(0xffffffffu, inv_s[hh], (2 * t + 1) * 4);
-        }
-      }
+    if (cc.prob != cur_prob) {   // (fetched before the wait for the group's summaries: the round trip runs beside the copy)
+      flush(false, true);
+      uint4 raw[NH][4];
+      fetch_query(cc.prob, raw);
+      start_problem(raw, BAL ? 0 : sub);
     }
     if (kScanBulk) {
       if (!mbar_wait(&full[stage], parity)) {
@@ -1083,12 +1101,11 @@ __global__ void __launch_bounds__(kScanWarps * 32, kScanCtasPerSm) scan_i4_kerne
     __syncthreads();
     if (warp == 0 && lane < p.G) {
       float m = -INFINITY, sacc = 0.f;
+      float2 v[kScanWarps];
 #pragma unroll
-      for (int w = 0; w < kScanWarps; ++w) {
-        const float2 v = red[w * 16 + lane];
-        const float nm = fmaxf(m, v.x);
-        if (nm > -INFINITY) { sacc = sacc * __expf(m - nm) + v.y * __expf(v.x - nm); m = nm; }
-      }
+      for (int w = 0; w < kScanWarps; ++w) { v[w] = red[w * 16 + lane]; m = fmaxf(m, v[w].x); }
+#pragma unroll
+      for (int w = 0; w < kScanWarps; ++w) sacc += m > -INFINITY ? v[w].y * __expf(v[w].x - m) : 0.f;
       const int pb = slot / p.Hkv, ph = slot - pb * p.Hkv;
       p.part[((int64_t)pb * p.Hq + ph * p.G + lane) * p.max_groups + sub / kScanWarps] = make_float2(m, sacc);
     }
