@@ -688,13 +688,13 @@ int locks_launch_select(locks_ctx *c, const float *shat, const locks_kv *kv, int
   p.Bshift = c->B == 64 ? 6 : (c->B == 32 ? 5 : 4);
   p.part_cnt = c->part_balanced ? c->part_cnt : nullptr;
   if (p.chunk_pages > kMaxKeys || (int64_t)c->sel_chunks * c->sel_kc > kMaxKeys || p.G > 16) return LOCKS_ERR_UNSUPPORTED;
-  // Two CTAs fit on an SM (64 registers per thread).  That halves the waves of a launch with many more CTAs
-  // than SMs, but with up to about 1.5 CTAs per SM the block scheduler stacks pairs on the SMs that drain first
-  // while others idle (measured: +15 us at 192 CTAs); such launches ask for enough shared memory to keep one
-  // CTA per SM.
+  // Two CTAs fit on an SM (64 registers per thread).  As long as every CTA can have an SM of its own it asks for enough shared memory
+  // to get one: the block scheduler otherwise stacks pairs on the SMs that drain first (8 x 32K tokens 56.9 us a step, in pairs
+  // 58.1).  More CTAs than SMs run in pairs, in one wave (192 CTAs of 24 chat requests 52.4 -> 48.3 us, 216 of 27 requests 81.2 ->
+  // 77.5; 144 CTAs 60.2 alone, 60.7 in pairs).
   constexpr int kSmemAlone = 116 * 1024;
   const int64_t nctas = (int64_t)c->sel_chunks * p.Hkv * batch;
-  const size_t smem = 2 * nctas <= 3 * (int64_t)c->num_sms ? (size_t)kSmemAlone : sizeof(SelShared);
+  const size_t smem = nctas <= c->num_sms ? (size_t)kSmemAlone : sizeof(SelShared);
   const dim3 grid(c->sel_chunks, p.Hkv, batch), blk(LOCKS_SEL_THREADS);
   if (locks_attrs_needed(LOCKS_ATTR_SELECT)) {
     cudaFuncSetAttribute(select_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemAlone);
