@@ -48,8 +48,10 @@ struct SelParams {
 // head 0 stores the step's length back to the caller's array.  Nothing reads the caller's array between
 // the scan (complete before this kernel passes its wait) and the end of the step, except a build that started
 // beside the scan (a.arrivals): the step's other kernels take lengths from the published copy.
-__device__ __forceinline__ void append_token(const locks_append &a, int batch, int Hkv, int Pmax, int b, int h,
-                                             int lane, int T, int32_t *status, int Bshift) {
+__device__ __noinline__ void append_token(const SelParams &p, int b, int h, int lane, int T) {
+  const locks_append &a = p.app;
+  const int batch = p.batch, Hkv = p.Hkv, Pmax = p.Pmax, Bshift = p.Bshift;
+  int32_t *status = p.status;
   if (h == 0 && lane == 0) {
     if (!a.arrivals || atomicAdd(a.arrivals + b, 1) == Hkv) {   // the last to arrive stores (BuildParams::seq_commit)
       if (a.arrivals) a.arrivals[b] = 0;
@@ -139,7 +141,7 @@ __device__ __forceinline__ void publish_range(SelShared &sh, uint32_t kmin, uint
 enum { kEmitIds = 0, kEmitList = 1, kEmitFinal = 2, kEmitEntry = 3 };
 constexpr int kFinalPages = kMaxKeys / 2;
 
-__device__ __noinline__ void select_emit(int nslab, int K, int mode, int c0, int32_t *ids, uint32_t *list_key, int32_t *list_idx) {
+__device__ __forceinline__ void emit_winners(int nslab, int K, int mode, int c0, int32_t *ids, uint32_t *list_key, int32_t *list_idx) {
   SelShared &sh = shared_state();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (tid < 256) sh.hist[tid] = 0;
@@ -164,7 +166,8 @@ __device__ __noinline__ void select_emit(int nslab, int K, int mode, int c0, int
       if (k && (left < 32 ? d >> left : 0u) == above) atomicAdd(&hc[(d >> shift) & ((1u << width) - 1u)], 1);
     }
     __syncthreads();
-    // every warp: lane l owns bins 8 (31 - l) .. + 7, so lane order is descending digit order
+    // every warp for itself (one warp alone, and a barrier, take 2300 cycles where this takes 1100): lane l owns bins 8 (31 - l) .. + 7,
+    // so lane order is descending digit order
     const int base = 8 * (31 - lane);
     const int4 lo = *reinterpret_cast<const int4 *>(hc + base), hi = *reinterpret_cast<const int4 *>(hc + base + 4);
     const int c[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
@@ -301,6 +304,11 @@ __device__ __noinline__ void select_emit(int nslab, int K, int mode, int c0, int
   }
 }
 
+// The same as a real call, where a kernel needs it twice
+__device__ __noinline__ void select_emit(int nslab, int K, int mode, int c0, int32_t *ids, uint32_t *list_key, int32_t *list_idx) {
+  emit_winners(nslab, K, mode, c0, ids, list_key, list_idx);
+}
+
 // What a launch's rankings have in common before the length is known: a CTA's scores and partials sit at addresses that do not
 // depend on it, so one round trip fetches them together with it.
 struct KeyInputs {
@@ -322,6 +330,7 @@ struct KeyInputs {
 template <int HB, typename Begin>
 __device__ __forceinline__ int chunk_keys(const KeyInputs &in, Begin begin, float *logshare_row) {
   constexpr int SB = 16 / HB, NP = HB == 16 ? 5 : 4;   // NP: partials in flight per lane
+  constexpr int NSLICE = kNW / HB;                     // warps per head
   SelShared &sh = shared_state();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, G = in.G;
   const float *row0 = in.shat0 + in.c0 + tid;
@@ -339,10 +348,11 @@ __device__ __forceinline__ int chunk_keys(const KeyInputs &in, Begin begin, floa
   const int T = *in.seq_len;
   const int counted = in.part_cnt ? *in.part_cnt : in.part_slots;
   load(0, in.Pmax - 1, cur);
-  const int nslice = max(1, kNW / G), slice = warp / min(G, kNW), g = warp - slice * min(G, kNW);   // (G <= 16)
-  const bool has_head = slice < nslice && in.combine == LOCKS_COMBINE_SHARE_AVG;
+  const int slice = warp / HB, g = warp % HB;
+  const bool has_head = g < G && in.combine == LOCKS_COMBINE_SHARE_AVG;
   const float2 *pp = in.part0 + (int64_t)g * in.max_groups;
-  const int pstep = 32 * nslice, p0 = slice * 32 + lane;
+  constexpr int pstep = 32 * NSLICE;
+  const int p0 = slice * 32 + lane;
   const int most = in.part_cnt ? in.max_groups : in.part_slots;   // what may be read before the count is known
   float2 v[NP];
 #pragma unroll
@@ -385,22 +395,17 @@ __device__ __forceinline__ int chunk_keys(const KeyInputs &in, Begin begin, floa
     if (lane == 0) { sh.lzm[warp] = m; sh.lzs[warp] = s; }
   }
   __syncthreads();
-  // every warp for itself: lane g < G merges the slices of head g
+  // every warp for itself: lanes g, g + HB .. hold the slices of head g
   float lz[HB];
   {
-    float l2 = 0.f;
-    if (in.combine == LOCKS_COMBINE_SHARE_AVG && lane < G) {
-      float M = -INFINITY, S = 0.f;
-#pragma unroll 1
-      for (int sl = 0; sl < nslice; ++sl) M = fmaxf(M, sh.lzm[sl * G + lane]);
-#pragma unroll 1
-      for (int sl = 0; sl < nslice; ++sl) {
-        const float wm = sh.lzm[sl * G + lane];
-        if (wm > -INFINITY) S = fmaf(sh.lzs[sl * G + lane], ex2f((wm - M) * kLog2e), S);
-      }
-      l2 = M * kLog2e + lg2f(S);
-    }
-    __syncwarp();
+    const int w = lane % kNW;
+    float m = sh.lzm[w], s = sh.lzs[w], M = m;
+#pragma unroll
+    for (int o = HB; o < kNW; o <<= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+    if (NSLICE > 1) s = M > -INFINITY ? s * ex2f((m - M) * kLog2e) : 0.f;
+#pragma unroll
+    for (int o = HB; o < kNW; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    const float l2 = in.combine == LOCKS_COMBINE_SHARE_AVG && lane < G ? M * kLog2e + lg2f(s) : 0.f;
 #pragma unroll
     for (int u = 0; u < HB; ++u) lz[u] = __shfl_sync(0xffffffffu, l2, u);
   }
@@ -492,9 +497,10 @@ __device__ __noinline__ void select_finish(int32_t *done, int chunks, int kc, in
   }
 }
 
-template <int HB>
-__global__ void __launch_bounds__(LOCKS_SEL_THREADS, 2) select_kernel(SelParams p) {
-  const int chunk = blockIdx.x, h = blockIdx.y, b = blockIdx.z, tid = threadIdx.x;
+// HB: 4, 8 or 16 >= heads per KV head.  ONE: a CTA ranks its whole problem.
+template <int HB, bool ONE>
+__global__ void __launch_bounds__(LOCKS_SEL_THREADS, 2) select_kernel(const __grid_constant__ SelParams p) {
+  const int chunk = ONE ? 0 : blockIdx.x, h = blockIdx.y, b = blockIdx.z, tid = threadIdx.x;
   const int prob = b * p.Hkv + h, c0 = chunk * p.chunk_pages;   // first page of this chunk
   int32_t *ids = p.ids + (int64_t)prob * p.k;
   const int64_t list0 = (int64_t)prob * p.chunks * p.kc;
@@ -511,7 +517,7 @@ __global__ void __launch_bounds__(LOCKS_SEL_THREADS, 2) select_kernel(SelParams 
   const int nslab = chunk_keys<HB>(in, [&](int T, int np) {
     P = np;
     if (p.app.k_new && chunk == 0 && tid >= LOCKS_SEL_THREADS - 32)
-      append_token(p.app, p.batch, p.Hkv, p.Pmax, b, h, tid & 31, T, p.status, p.Bshift);
+      append_token(p, b, h, tid & 31, T);
     if (P <= p.k) {  // every page is kept
       if (chunk == 0) {
         for (int j = tid; j < p.k; j += LOCKS_SEL_THREADS) ids[j] = j < P ? j : -1;
@@ -527,7 +533,7 @@ __global__ void __launch_bounds__(LOCKS_SEL_THREADS, 2) select_kernel(SelParams 
   pdl_trigger();
   if (P <= p.k) return;
   if (nslab == 0) {  // chunk past the candidates: an empty list
-    if (p.chunks > 1) {
+    if constexpr (!ONE) {
       for (int j = tid; j < p.kc; j += LOCKS_SEL_THREADS) p.cand_key[list0 + (int64_t)chunk * p.kc + j] = 0u;
       select_finish(p.sel_done + prob, p.chunks, p.kc, p.k, ids, p.cnt + prob, p.cand_key + list0, p.cand_idx + list0, P);
     }
@@ -535,8 +541,8 @@ __global__ void __launch_bounds__(LOCKS_SEL_THREADS, 2) select_kernel(SelParams 
   }
   const int cand_in_chunk = min(P - 2, c0 + p.chunk_pages - 1) - max(1, c0) + 1;
   const int K = min(p.k - 2, cand_in_chunk);
-  if (p.chunks == 1) {
-    if (K > 0) select_emit(nslab, K, kEmitIds, c0, ids, nullptr, nullptr);
+  if constexpr (ONE) {
+    if (K > 0) emit_winners(nslab, K, kEmitIds, c0, ids, nullptr, nullptr);
     if (tid == 0) {
       ids[0] = 0;
       ids[p.k - 1] = P - 1;
@@ -696,13 +702,18 @@ int locks_launch_select(locks_ctx *c, const float *shat, const locks_kv *kv, int
   const int64_t nctas = (int64_t)c->sel_chunks * p.Hkv * batch;
   const size_t smem = nctas <= c->num_sms ? (size_t)kSmemAlone : sizeof(SelShared);
   const dim3 grid(c->sel_chunks, p.Hkv, batch), blk(LOCKS_SEL_THREADS);
-  if (locks_attrs_needed(LOCKS_ATTR_SELECT)) {
-    cudaFuncSetAttribute(select_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemAlone);
-    cudaFuncSetAttribute(select_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemAlone);
-    cudaFuncSetAttribute(select_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemAlone);
-  }
-  if (p.G <= 4) locks_launch_pdl(select_kernel<4>, grid, blk, smem, st, p);
-  else if (p.G <= 8) locks_launch_pdl(select_kernel<8>, grid, blk, smem, st, p);
-  else locks_launch_pdl(select_kernel<16>, grid, blk, smem, st, p);
+  const bool attrs = locks_attrs_needed(LOCKS_ATTR_SELECT), one = c->sel_chunks == 1;
+#define LOCKS_SELECT_CASE(HB_, ONE_, FITS_)                                                                                  \
+  do {                                                                                                                      \
+    if (attrs) cudaFuncSetAttribute(select_kernel<HB_, ONE_>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemAlone);     \
+    if ((FITS_) && one == ONE_) locks_launch_pdl(select_kernel<HB_, ONE_>, grid, blk, smem, st, p);                         \
+  } while (0)
+  LOCKS_SELECT_CASE(4, true, p.G <= 4);
+  LOCKS_SELECT_CASE(8, true, p.G > 4 && p.G <= 8);
+  LOCKS_SELECT_CASE(16, true, p.G > 8);
+  LOCKS_SELECT_CASE(4, false, p.G <= 4);
+  LOCKS_SELECT_CASE(8, false, p.G > 4 && p.G <= 8);
+  LOCKS_SELECT_CASE(16, false, p.G > 8);
+#undef LOCKS_SELECT_CASE
   return locks_check_launch(c);
 }
