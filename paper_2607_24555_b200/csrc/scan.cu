@@ -652,15 +652,15 @@ __global__ void __launch_bounds__(kScanWarps * 32, kScanCtasPerSm) scan_i4_kerne
     next_block = (lane < LOCKS_GROUP && sub * LOCKS_GROUP + lane < cp.nsc) ? spec_block : 0;
   else
     next_block = fetch_block(cp);
-#pragma unroll
-  for (int s = 0; s < kScanStages; ++s) {
+  auto produce = [&](int stage) {
     if (cp.prob < nprob) {
-      issue(s, cp, next_block);
+      issue(stage, cp, next_block);
       ++inflight;
       advance(cp, inflight < n_units);
       next_block = fetch_block(cp);
     }
-  }
+  };
+  produce(0);
 
   const uint32_t kM0 = 0x000F000Fu, kM1 = 0x00F000F0u;
   uint32_t kMB = 0x00FF00FFu, kMagic = 0x64006400u;
@@ -737,6 +737,10 @@ __global__ void __launch_bounds__(kScanWarps * 32, kScanCtasPerSm) scan_i4_kerne
     if (cc.prob != q_prob) fetch_query(cc.prob, q_first);
     start_problem(q_first, BAL ? pslot_first : sub);
   }
+  // The rest of the ring is filled after the query has been worked out: every warp's first group then goes ahead of everybody's
+  // second one, where two groups of every warp (31 MB) take 5 us to arrive.
+#pragma unroll
+  for (int s = 1; s < kScanStages; ++s) produce(s);
 
   int it = 0;
   bool ok = true;
