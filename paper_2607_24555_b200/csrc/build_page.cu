@@ -251,6 +251,8 @@ __global__ void __launch_bounds__(page_threads(B) * page_ctas(B)) build_page_ker
 #pragma unroll
   for (int w = 0; w < NW; ++w) knorm2 += sh.kn[w];
   // ---- Gram matrix: KS slices of the dimensions, a thread owns TI x TJ entries of its slice's sum
+  // (a dimension's entries in 8- and 16-byte loads, the additions in the same order: a step that fills a page of 16 tokens, 1 x 8016
+  // tokens, 27.6 -> 26.7 us; entry by entry before, bound by the latency of 64 short iterations)
   {
     constexpr int KS = PageShared<B>::KS, TN = NT / KS, TJ = B == 16 ? 4 : 8, TI = B * B / TN / TJ, NJ = B / TJ;
     const int ks = tid / TN, tt = tid % TN, i0 = (tt / NJ) * TI, j0 = (tt % NJ) * TJ;
@@ -260,13 +262,13 @@ __global__ void __launch_bounds__(page_threads(B) * page_ctas(B)) build_page_ker
 #pragma unroll
       for (int j = 0; j < TJ; ++j) acc[i][j] = 0.f;
     const float *d = sh.dt + ks * (LOCKS_D / KS) * DS;
-#pragma unroll 4
+#pragma unroll(B == 16 ? 8 : 4)
     for (int cc = 0; cc < LOCKS_D / KS; ++cc, d += DS) {
-      float x[TI], y[TJ];
+      __align__(16) float x[TI], y[TJ];
 #pragma unroll
-      for (int i = 0; i < TI; ++i) x[i] = d[i0 + i];
+      for (int i = 0; i < TI; i += 2) *reinterpret_cast<float2 *>(x + i) = *reinterpret_cast<const float2 *>(d + i0 + i);
 #pragma unroll
-      for (int j = 0; j < TJ; ++j) y[j] = d[j0 + j];
+      for (int j = 0; j < TJ; j += 4) *reinterpret_cast<float4 *>(y + j) = *reinterpret_cast<const float4 *>(d + j0 + j);
 #pragma unroll
       for (int i = 0; i < TI; ++i)
 #pragma unroll
