@@ -480,9 +480,11 @@ int locks_decode_step(locks_ctx *ctx, const void *q, const void *k_new, const vo
   // published the lengths, beside the selector and attention.
   const bool early = locks_scan_leaves_room(ctx, batch);
   app.arrivals = early ? ctx->arrivals : nullptr;
+  bool forked = false;
   auto build = [&]() -> int {
     if (cudaEventRecord(ctx->ev_fork, st) != cudaSuccess || cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0) != cudaSuccess)
       return LOCKS_ERR_CUDA;
+    forked = true;
     const int e = early ? locks_launch_build(ctx, kv, batch, nullptr, nullptr, 1, summaries, k_new, nullptr, ctx->side,
                                              k_new ? kv->seq_lens : nullptr)
                         : locks_launch_build(ctx, &kv_step, batch, nullptr, nullptr, 1, summaries, k_new,
@@ -490,25 +492,27 @@ int locks_decode_step(locks_ctx *ctx, const void *q, const void *k_new, const vo
     if (e == LOCKS_OK && cudaEventRecord(ctx->ev_join, ctx->side) != cudaSuccess) return LOCKS_ERR_CUDA;
     return e;
   };
-  // a step that is broken off leaves no half-counted arrivals behind
+  // A step that is broken off joins its streams like any other, so that whatever follows on `st` comes after all that it has
+  // launched (a launch can be reported as failed and run: locks_check_launch sees errors that others left pending), and then
+  // clears the arrivals, which may be half counted.
   auto fail = [&](int e) {
-    if (early && k_new) (void)cudaMemsetAsync(ctx->arrivals, 0, (size_t)batch * 4, ctx->side);
+    if (forked && cudaEventRecord(ctx->ev_join, ctx->side) == cudaSuccess) (void)cudaStreamWaitEvent(st, ctx->ev_join, 0);
+    if (early && k_new) (void)cudaMemsetAsync(ctx->arrivals, 0, (size_t)batch * 4, st);
     return e;
   };
   mark(0);
   if (early && (rc = build()) != LOCKS_OK) return fail(rc);
   if ((rc = locks_launch_scan(ctx, q, summaries, kv, batch, ctx->shat, k_new ? 1 : 0, st)) != LOCKS_OK) return fail(rc);
   mark(1);
-  if (!early && (rc = build()) != LOCKS_OK) return rc;
+  if (!early && (rc = build()) != LOCKS_OK) return fail(rc);
   if ((rc = locks_launch_select(ctx, ctx->shat, &kv_step, batch, ids, cnt, nullptr, k_new ? &app : nullptr, st,
                                 locks_attend_fills(ctx, batch))) != LOCKS_OK)
     return fail(rc);
   mark(2);
-  if ((rc = locks_launch_attend(ctx, q, &kv_step, batch, ids, cnt, out, nullptr, st)) != LOCKS_OK) return rc;
+  if ((rc = locks_launch_attend(ctx, q, &kv_step, batch, ids, cnt, out, nullptr, st)) != LOCKS_OK) return fail(rc);
   mark(3);
   if (pe && !capturing) ctx->prof_n++;
-  if (cudaStreamWaitEvent(st, ctx->ev_join, 0) != cudaSuccess) return LOCKS_ERR_CUDA;
-  return LOCKS_OK;
+  return cudaStreamWaitEvent(st, ctx->ev_join, 0) == cudaSuccess ? LOCKS_OK : fail(LOCKS_ERR_CUDA);
 }
 
 namespace {
