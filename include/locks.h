@@ -263,7 +263,8 @@ int locks_sparse_attend(locks_ctx *ctx, const void *q, const locks_kv *kv, int b
  *      if k_new == NULL the cache and seq_lens already include the token being decoded;
  *   2. locks_select on the resident summaries;  3. locks_sparse_attend on the selected pages;
  *   4. if a page became complete at this step (T_b % B == 0) build its summary, so that it is a
- *      candidate from the next step on (the newly written token is never scored, App. E(i)).  Its bytes may differ
+ *      candidate from the next step on (the newly written token is never scored, App. E(i)).  No score of this step
+ *      reads it, not even that of another request of the batch that holds the same block.  Its bytes may differ
  *      from those that locks_build_summaries gives for the same page, in about one of ten thousand (another solver,
  *      as accurate).
  * These are the results; inside, the token is counted from the first kernel on, its rows are written by

@@ -35,7 +35,7 @@ int validate(const locks_config *c) {
 }
 
 struct Layout {
-  size_t status, shat, part, part_cnt, sel_done, cand_val, cand_idx, att_o, att_lse, att_done, ids, cnt, sq, skn, svn, sout, seq_eff, arrivals, total;
+  size_t status, shat, part, part_cnt, sel_done, cand_val, cand_idx, att_o, att_lse, att_done, ids, cnt, sq, skn, svn, sout, seq_eff, arrivals, stage_summ, total;
   int G, k, S, max_groups, sel_ept, sel_chunks, sel_kc;
 };
 
@@ -103,7 +103,8 @@ Layout make_layout(const locks_config *c) {
   L.svn = take(nb * Hkv * LOCKS_D * esz);
   L.sout = take(nb * Hq * LOCKS_D * esz);
   L.seq_eff = take(2 * nb * 4);
-  L.arrivals = take(nb * 4);
+  L.arrivals = take(nb * (1 + Hkv) * 4);
+  L.stage_summ = take(nb * Hkv * L.S);
   L.total = o;
   return L;
 }
@@ -204,6 +205,8 @@ int locks_create(const locks_config *cfg, void *workspace, size_t ws_bytes, lock
   c->cnt_int = reinterpret_cast<int32_t *>(ws + L.cnt);
   c->seq_eff = reinterpret_cast<int32_t *>(ws + L.seq_eff);
   c->arrivals = reinterpret_cast<int32_t *>(ws + L.arrivals);
+  c->staged = c->arrivals + cfg->max_batch;
+  c->stage_summ = ws + L.stage_summ;
   c->stage_q = ws + L.sq; c->stage_kn = ws + L.skn; c->stage_vn = ws + L.svn; c->stage_out = ws + L.sout;
   if (cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) != cudaSuccess ||
       cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
@@ -212,7 +215,7 @@ int locks_create(const locks_config *cfg, void *workspace, size_t ws_bytes, lock
       cudaMemsetAsync(c->att_done, 0, (size_t)cfg->max_batch * cfg->num_q_heads * 4, 0) != cudaSuccess ||
       cudaMemsetAsync(c->sel_done, 0, (size_t)cfg->max_batch * cfg->num_q_heads * 4, 0) != cudaSuccess ||
       cudaMemsetAsync(c->part_cnt, 0, (size_t)cfg->max_batch * cfg->num_kv_heads * 4, 0) != cudaSuccess ||
-      cudaMemsetAsync(c->arrivals, 0, (size_t)cfg->max_batch * 4, 0) != cudaSuccess ||
+      cudaMemsetAsync(c->arrivals, 0, (size_t)cfg->max_batch * (1 + cfg->num_kv_heads) * 4, 0) != cudaSuccess ||
       cudaStreamSynchronize(0) != cudaSuccess) {
     if (c->hint_host) cudaFreeHost(c->hint_host);
     delete c;
@@ -299,7 +302,7 @@ int locks_build_summaries_layers(locks_ctx *ctx, const locks_kv *kv, const void 
   if ((int64_t)batch * num_layers > 65535 || ((page_begin == nullptr) != (page_end == nullptr))) return LOCKS_ERR_INVALID_ARG;
   ctx->last_launches = 0;
   return locks_launch_build(ctx, &kv0, batch, page_begin, page_end, 0, nullptr, nullptr, nullptr, (cudaStream_t)stream,
-                            nullptr, k_layers, summaries_layers, num_layers);
+                            false, nullptr, k_layers, summaries_layers, num_layers);
 }
 
 // ---- page-sharded decode: one long request whose pages are dealt to several GPUs (three small exchanges) ------
@@ -477,16 +480,17 @@ int locks_decode_step(locks_ctx *ctx, const void *q, const void *k_new, const vo
   // step's scan.  The token itself it takes from k_new, since the selector's kernel is writing it into the cache at the same
   // time.  Where the scan leaves room on the chip the build runs beside it, counting the token itself; where the scan takes every
   // SM (its warps have fixed shares, and a CTA that had to wait for a build would end last) the build starts when the scan has
-  // published the lengths, beside the selector and attention.
+  // published the lengths, beside the selector and attention.  Either way a summary is put in place when the scan is over (BuildParams::stage).
   const bool early = locks_scan_leaves_room(ctx, batch);
   app.arrivals = early ? ctx->arrivals : nullptr;
+  const locks_staged staged = {early ? ctx->stage_summ : nullptr, reinterpret_cast<char *>(summaries), ctx->staged, kv->block_table, kv->num_blocks, ctx->S};
   bool forked = false;
   auto build = [&]() -> int {
     if (cudaEventRecord(ctx->ev_fork, st) != cudaSuccess || cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0) != cudaSuccess)
       return LOCKS_ERR_CUDA;
     forked = true;
     const int e = early ? locks_launch_build(ctx, kv, batch, nullptr, nullptr, 1, summaries, k_new, nullptr, ctx->side,
-                                             k_new ? kv->seq_lens : nullptr)
+                                             true, k_new ? kv->seq_lens : nullptr)
                         : locks_launch_build(ctx, &kv_step, batch, nullptr, nullptr, 1, summaries, k_new,
                                              k_new ? ctx->seq_eff + batch : nullptr, ctx->side);
     if (e == LOCKS_OK && cudaEventRecord(ctx->ev_join, ctx->side) != cudaSuccess) return LOCKS_ERR_CUDA;
@@ -494,10 +498,10 @@ int locks_decode_step(locks_ctx *ctx, const void *q, const void *k_new, const vo
   };
   // A step that is broken off joins its streams like any other, so that whatever follows on `st` comes after all that it has
   // launched (a launch can be reported as failed and run: locks_check_launch sees errors that others left pending), and then
-  // clears the arrivals, which may be half counted.
+  // clears the arrivals (and those of staged summaries behind them), which may be half counted.
   auto fail = [&](int e) {
     if (forked && cudaEventRecord(ctx->ev_join, ctx->side) == cudaSuccess) (void)cudaStreamWaitEvent(st, ctx->ev_join, 0);
-    if (early && k_new) (void)cudaMemsetAsync(ctx->arrivals, 0, (size_t)batch * 4, st);
+    if (early) (void)cudaMemsetAsync(ctx->arrivals, 0, (size_t)ctx->cfg.max_batch * (1 + ctx->cfg.num_kv_heads) * 4, st);
     return e;
   };
   mark(0);
@@ -506,7 +510,7 @@ int locks_decode_step(locks_ctx *ctx, const void *q, const void *k_new, const vo
   mark(1);
   if (!early && (rc = build()) != LOCKS_OK) return fail(rc);
   if ((rc = locks_launch_select(ctx, ctx->shat, &kv_step, batch, ids, cnt, nullptr, k_new ? &app : nullptr, st,
-                                locks_attend_fills(ctx, batch))) != LOCKS_OK)
+                                locks_attend_fills(ctx, batch), &staged)) != LOCKS_OK)
     return fail(rc);
   mark(2);
   if ((rc = locks_launch_attend(ctx, q, &kv_step, batch, ids, cnt, out, nullptr, st)) != LOCKS_OK) return fail(rc);

@@ -1144,7 +1144,7 @@ __global__ void __launch_bounds__(32) build_wide_kernel(BuildParams p, int B) {
 
 int locks_launch_build(locks_ctx *c, const locks_kv *kv, int batch, const int32_t *pb, const int32_t *pe,
                        int just_filled, void *summaries, const void *k_new, const int32_t *append_pos,
-                       cudaStream_t st, int32_t *seq_commit, const void *const *k_layers, void *const *summ_layers, int num_layers) {
+                       cudaStream_t st, bool early, int32_t *seq_commit, const void *const *k_layers, void *const *summ_layers, int num_layers) {
   BuildParams p;
   p.k = kv->k; p.sb = kv->stride_block; p.sh = kv->stride_head; p.st = kv->stride_token;
   p.block_table = kv->block_table; p.seq_lens = kv->seq_lens; p.page_begin = pb; p.page_end = pe;
@@ -1153,7 +1153,8 @@ int locks_launch_build(locks_ctx *c, const locks_kv *kv, int batch, const int32_
   p.r = c->cfg.rank; p.S = c->S; p.fmt = c->cfg.summary_fmt; p.esz = c->cfg.kv_dtype == LOCKS_BF16 ? 2 : 4;
   p.k_layers = just_filled ? nullptr : k_layers; p.summ_layers = just_filled ? nullptr : summ_layers;
   p.k_new = just_filled ? k_new : nullptr; p.append_pos = just_filled ? append_pos : nullptr;
-  p.seq_commit = seq_commit; p.arrivals = c->arrivals;
+  p.seq_commit = early ? seq_commit : nullptr; p.arrivals = c->arrivals;
+  p.stage = early ? reinterpret_cast<uint8_t *>(c->stage_summ) : nullptr; p.staged = c->staged;
   p.hint = nullptr; p.kpages = c->k; p.hint_wpp = 1; p.hint_rounds = 1; p.hint_W = 1;
   if (just_filled && c->hint_dev && c->cfg.summary_fmt == LOCKS_FMT_I4 && c->cfg.q_dtype == LOCKS_BF16) {
     const locks_scan_geom geo = locks_scan_geometry(c, batch);

@@ -24,6 +24,11 @@ struct BuildParams {
   // and the caller's length is stored by whoever comes last of the request's page-heads, which have read it by then, and the
   // selector (arrivals[b] counts them; zero between steps).  seq_commit == nullptr: seq_lens are the step's.
   int32_t *seq_commit, *arrivals;
+  // the same build: a summary that is ready before the step's scores are waits in stage[page-head] (S bytes each), since another
+  // request may hold the page's block.  staged[page-head] counts the page-head and the selector, which comes when the scan is over;
+  // the second of them puts the summary in place and leaves a zero.  stage == nullptr: the scan is over, summaries go in place.
+  uint8_t *stage;
+  int32_t *staged;
   // bulk build of several layers in one launch: per-layer key caches and summary buffers (device arrays), or null
   const void *const *k_layers;
   void *const *summ_layers;

@@ -38,11 +38,16 @@ template <int B> struct PageShared {
   float sig[16];                      // singular values with the sign of their mode
   float mx[4], kn[4];
   uint8_t codes[16 * LOCKS_D];        // int4 codes before packing
+  int early, pad[3];                  // the summary has to wait (BuildParams::stage); a CTA's pages start on 16 bytes
 };
+
+static_assert(sizeof(PageShared<16>) % 16 == 0 && sizeof(PageShared<32>) % 16 == 0, "");
 
 // Eigenvectors and eigenvalues of the symmetric matrix m0 * 2^-ex (unit scale), by one warp: sh.us[mode][token] and
 // sh.lam[mode] of the modes in descending order (the first min(r, B) are accurate, the rest are not needed).
-template <int B> __device__ __forceinline__ void solve_modes(PageShared<B> &sh, float scale, float unscale, int r, int lane) {
+// sh.early: whether the selector has yet to come to `staged` (BuildParams::stage).  In the usual case it has long been there; asked for
+// here, the answer arrives while the modes are put in order.
+template <int B> __device__ __forceinline__ void solve_modes(PageShared<B> &sh, float scale, float unscale, int r, int lane, const int32_t *staged) {
   constexpr int L = 64 / B, R = B / L, R2 = R / 2;   // lanes per pair of columns; rows, and packed pairs of rows, per lane
   const int pair = lane / L, row0 = (lane % L) * R;
   const float *m0 = sh.m[0];
@@ -172,6 +177,8 @@ template <int B> __device__ __forceinline__ void solve_modes(PageShared<B> &sh, 
     }
     if (!__any_sync(0xffffffffu, bad != 0)) break;
   }
+  int come = 1;
+  if (staged && lane == 0) asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(come) : "l"(staged) : "memory");
   ranks();
 #pragma unroll
   for (int c = 0; c < 2; ++c) {
@@ -183,6 +190,7 @@ template <int B> __device__ __forceinline__ void solve_modes(PageShared<B> &sh, 
         *reinterpret_cast<float4 *>(sh.us + rank[c] * B + row0 + 2 * i) =
             make_float4(w[c][i].x * inv, w[c][i].y * inv, w[c][i + 1].x * inv, w[c][i + 1].y * inv);
   }
+  if (lane == 0) sh.early = come == 0;
 }
 
 template <int B>
@@ -303,7 +311,7 @@ __global__ void __launch_bounds__(page_threads(B) * page_ctas(B)) build_page_ker
       scale = __uint_as_float((uint32_t)(127 - ex) << 23);
       unscale = __uint_as_float((uint32_t)(127 + ex) << 23);
     }
-    solve_modes<B>(sh, scale, unscale, r, lane);
+    solve_modes<B>(sh, scale, unscale, r, lane, p.stage ? p.staged + prob : nullptr);
   }
   sync();
   // ---- modes kept
@@ -315,7 +323,7 @@ __global__ void __launch_bounds__(page_threads(B) * page_ctas(B)) build_page_ker
     if (lam0 > 0.f && ll > 1e-6f * lam0 && ll > 1e-10f * knorm2) r_eff = l + 1; else break;
   }
   const int fmt = p.fmt, wide = fmt == LOCKS_FMT_BF16 ? 2 : 1;
-  uint8_t *gout = p.summ + ((int64_t)block * p.Hkv + h) * p.S;
+  uint8_t *const place = p.summ + ((int64_t)block * p.Hkv + h) * p.S, *const gout = sh.early ? p.stage + (int64_t)prob * p.S : place;
   float *fout = reinterpret_cast<float *>(gout);
   // ---- basis V = D^T U Sigma^-1: a warp per mode, a lane owns dimensions lane, lane + 32 ..
 #pragma unroll 1
@@ -425,9 +433,23 @@ __global__ void __launch_bounds__(page_threads(B) * page_ctas(B)) build_page_ker
     else
       gout[wb_off_mu(r, wide, B) + c] = code;
   }
-  if (fmt == LOCKS_FMT_F32) return;
-  if (tid == 0) *reinterpret_cast<__half *>(gout + osmu) = s;
-  if (osmu + 2 + tid < p.S) gout[osmu + 2 + tid] = 0;   // bytes between the payload and the padded stride stay zero
+  if (fmt != LOCKS_FMT_F32) {
+    if (tid == 0) *reinterpret_cast<__half *>(gout + osmu) = s;
+    if (osmu + 2 + tid < p.S) gout[osmu + 2 + tid] = 0;   // bytes between the payload and the padded stride stay zero
+  }
+  if (!p.stage) return;
+  if (sh.early) {   // the scan may have ended meanwhile; if not, the selector will find the summary
+    sync();
+    if (tid == 0) {
+      __threadfence();
+      sh.early = atomicAdd(p.staged + prob, 1) == 0;
+      __threadfence();
+    }
+    sync();
+    if (sh.early) return;
+    for (int i = tid; i < p.S / 16; i += NT) reinterpret_cast<uint4 *>(place)[i] = reinterpret_cast<const uint4 *>(gout)[i];
+  }
+  if (tid == 0) p.staged[prob] = 0;
 }
 
 template <int B> int launch_pages(locks_ctx *c, const BuildParams &p, cudaStream_t st) {

@@ -86,6 +86,8 @@ struct locks_ctx {
   char *stage_q, *stage_kn, *stage_vn, *stage_out;
   int32_t *seq_eff;        // [2][max_batch] decode step in flight: effective lengths, append positions
   int32_t *arrivals;       // [max_batch] readers of a request's length that are done (zero between steps; see BuildParams)
+  int32_t *staged;         // [max_batch][Hkv], behind arrivals: which of a staged summary's two parties have come (zero between steps)
+  char *stage_summ;        // [max_batch][Hkv][S] summaries of a step that were ready before its scores
   cudaStream_t side;       // build of freshly filled pages runs beside attend
   cudaEvent_t ev_fork, ev_join;
   int last_launches;
@@ -108,6 +110,15 @@ struct locks_append {
   int32_t *seq_commit;         // the caller's sequence lengths
   int32_t *arrivals;           // [batch] when the step's build may still read them (see BuildParams), or nullptr
   int num_blocks, esz;
+};
+
+// Summaries that the step's build may leave for the selector to put in place (see BuildParams); stage == nullptr: none.
+struct locks_staged {
+  const char *stage;
+  char *summ;
+  int32_t *staged;
+  const int32_t *block_table;
+  int num_blocks, S;
 };
 
 // Geometry of a tensor-scan launch: known on the host, used by the launcher and by the partition hint
@@ -150,14 +161,16 @@ int locks_launch_scan(locks_ctx *c, const void *q, const void *summaries, const 
                       float *shat, int seq_inc, cudaStream_t st);
 // attend_first: the kernel that follows may take its slots at once (see select_kernel)
 int locks_launch_select(locks_ctx *c, const float *shat, const locks_kv *kv, int batch, int32_t *ids,
-                        int32_t *cnt, float *logshare, const locks_append *app, cudaStream_t st, bool attend_first = false);
+                        int32_t *cnt, float *logshare, const locks_append *app, cudaStream_t st, bool attend_first = false,
+                        const locks_staged *staged = nullptr);
 // Whether a step's attention needs almost every slot there is
 bool locks_attend_fills(locks_ctx *c, int batch);
 int locks_launch_attend(locks_ctx *c, const void *q, const locks_kv *kv, int batch, const int32_t *ids,
                         const int32_t *cnt, void *out, float *lse, cudaStream_t st);
+// early: the pages that a step fills, beside its scan (BuildParams::seq_commit, stage)
 int locks_launch_build(locks_ctx *c, const locks_kv *kv, int batch, const int32_t *pb, const int32_t *pe,
                        int just_filled, void *summaries, const void *k_new, const int32_t *append_pos,
-                       cudaStream_t st, int32_t *seq_commit = nullptr, const void *const *k_layers = nullptr,
+                       cudaStream_t st, bool early = false, int32_t *seq_commit = nullptr, const void *const *k_layers = nullptr,
                        void *const *summ_layers = nullptr, int num_layers = 1);
 
 // envelope = 0: exact page log-mass; 1: the min/max envelope bound of the page's largest logit

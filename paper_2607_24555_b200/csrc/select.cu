@@ -41,6 +41,7 @@ struct SelParams {
   int attend_first;  // let the next kernel be scheduled at once
   int Bshift;        // log2 of the page size (4, 5 or 6)
   locks_append app;  // decode step only: the new token's K/V rows, written here beside the ranking
+  locks_staged staged;  // decode step only: summaries that were ready before the scores
 };
 
 // Decode step: the CTA of (request b, KV head h) writes the new token's K and V rows of that head into the
@@ -79,6 +80,28 @@ __device__ __noinline__ void append_token(const SelParams &p, int b, int h, int 
     reinterpret_cast<uint4 *>(reinterpret_cast<uint32_t *>(a.k) + dst)[lane] = kk;
     reinterpret_cast<uint4 *>(reinterpret_cast<uint32_t *>(a.v) + dst)[lane] = vv;
   }
+}
+
+// The summary of the page that request b has filled in this step, if its build was done before the scan: put in place now that no
+// score reads it any more.  If the build is not done it will do so itself.
+__device__ __noinline__ void place_staged(const SelParams &p, int b, int h, int lane, int T) {
+  const locks_staged &s = p.staged;
+  const int page = (T >> p.Bshift) - 1, prob = b * p.Hkv + h;
+  if (T <= 0 || (T & ((1 << p.Bshift) - 1)) || page >= p.Pmax) return;   // as build_page_kernel has it
+  const int block = s.block_table[(int64_t)b * p.Pmax + page];
+  if (block < 0 || block >= s.num_blocks) return;
+  int done = 0;
+  if (lane == 0) {
+    __threadfence();
+    done = atomicAdd(s.staged + prob, 1);
+    if (done) s.staged[prob] = 0;
+    __threadfence();
+  }
+  __syncwarp();
+  if (!__shfl_sync(0xffffffffu, done, 0)) return;
+  const uint4 *src = reinterpret_cast<const uint4 *>(s.stage + (int64_t)prob * s.S);
+  uint4 *dst = reinterpret_cast<uint4 *>(s.summ + ((int64_t)block * p.Hkv + h) * s.S);
+  for (int i = lane; i < s.S / 16; i += 32) dst[i] = __ldcg(src + i);
 }
 
 constexpr int kListMax = 256;    // keys of the threshold bin that are ranked pair by pair
@@ -518,6 +541,7 @@ __global__ void __launch_bounds__(LOCKS_SEL_THREADS, 2) select_kernel(const __gr
     P = np;
     if (p.app.k_new && chunk == 0 && tid >= LOCKS_SEL_THREADS - 32)
       append_token(p, b, h, tid & 31, T);
+    if (p.staged.stage && chunk == 0 && tid >= LOCKS_SEL_THREADS - 32) place_staged(p, b, h, tid & 31, T);
     if (P <= p.k) {  // every page is kept
       if (chunk == 0) {
         for (int j = tid; j < p.k; j += LOCKS_SEL_THREADS) ids[j] = j < P ? j : -1;
@@ -673,11 +697,14 @@ int locks_launch_merge_selection(locks_ctx *c, const float *cand_key, const int3
 }
 
 int locks_launch_select(locks_ctx *c, const float *shat, const locks_kv *kv, int batch, int32_t *ids,
-                        int32_t *cnt, float *logshare, const locks_append *app, cudaStream_t st, bool attend_first) {
+                        int32_t *cnt, float *logshare, const locks_append *app, cudaStream_t st, bool attend_first,
+                        const locks_staged *staged) {
   SelParams p;
   p.attend_first = attend_first;
   if (app) p.app = *app;
   else p.app.k_new = nullptr;
+  if (staged) p.staged = *staged;
+  else p.staged.stage = nullptr;
   p.status = c->status;
   p.shat = shat; p.part = c->part; p.seq_lens = kv->seq_lens; p.ids = ids; p.cnt = cnt; p.logshare = logshare;
   p.cand_key = reinterpret_cast<uint32_t *>(c->cand_val); p.cand_idx = c->cand_idx; p.sel_done = c->sel_done;

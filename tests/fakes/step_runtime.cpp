@@ -11,6 +11,7 @@
 #include "locks.h"
 
 struct locks_append;
+struct locks_staged;
 
 static bool early_build = false;
 static std::string fail_call;
@@ -52,9 +53,9 @@ void __cudaRegisterFunction(void **, const char *, char *, const char *, int, ui
 bool locks_scan_leaves_room(const locks_ctx *, int) { return early_build; }
 bool locks_attend_fills(locks_ctx *, int) { return false; }
 int locks_launch_scan(locks_ctx *, const void *, const void *, const locks_kv *, int, float *, int, cudaStream_t st) { return launch("scan", st); }
-int locks_launch_select(locks_ctx *, const float *, const locks_kv *, int, int32_t *, int32_t *, float *, const locks_append *, cudaStream_t st, bool) { return launch("select", st); }
+int locks_launch_select(locks_ctx *, const float *, const locks_kv *, int, int32_t *, int32_t *, float *, const locks_append *, cudaStream_t st, bool, const locks_staged *) { return launch("select", st); }
 int locks_launch_attend(locks_ctx *, const void *, const locks_kv *, int, const int32_t *, const int32_t *, void *, float *, cudaStream_t st) { return launch("attend", st); }
-int locks_launch_build(locks_ctx *, const locks_kv *, int, const int32_t *, const int32_t *, int, void *, const void *, const int32_t *, cudaStream_t st, int32_t *,
+int locks_launch_build(locks_ctx *, const locks_kv *, int, const int32_t *, const int32_t *, int, void *, const void *, const int32_t *, cudaStream_t st, bool, int32_t *,
                        const void *const *, void *const *, int) { return launch("build", st); }
 
 int main(int argc, char **argv) {

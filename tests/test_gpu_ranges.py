@@ -550,6 +550,52 @@ def test_lengths_of_steps_whose_build_starts_at_once(B, dtype, Hkv):
         assert set(filled) <= set(changed) <= set(filled) | {int(gc.case.block_table[0, rows - 1])}, step
 
 
+# A request's last page may be an inner page of another one (a shared prompt of a whole number of pages).  The step writes its
+# summary anew, but every score of the step is that of the old one, whichever is done first: the build (the plain scan of int8 bases with
+# 16 heads takes ten times as long) or the scan.  The old summary here is another page's, so that the selections differ.
+@pytest.mark.parametrize("B,fmt,dtype,rank,Hq,Hkv", [(16, "i4", "bf16", 8, 8, 2), (16, "i4", "bf16", 2, 32, 2), (16, "i8", "bf16", 2, 16, 1), (16, "bf16", "bf16", 4, 32, 2),
+                                                     (16, "f32", "f32", 8, 8, 2), (32, "i4", "bf16", 8, 8, 2), (64, "i4", "bf16", 4, 12, 4), (32, "i8", "bf16", 8, 16, 1)])
+def test_summary_of_a_shared_page_changes_after_the_scores(B, fmt, dtype, rank, Hq, Hkv):
+    from gpu_util import GpuCase
+    w = locks_synth.Workload("shared", [B * 41 + 3, B * 30, B * 37, B * 30], Hq=Hq, Hkv=Hkv, B=B, fmt=fmt, dtype=dtype, rank=rank, budget=6 * B, seed=B + rank)
+    gc = GpuCase(w)
+    gc.ctx.locks_set_scan_partition(1)
+    table = gc.case.block_table
+    table[1, :30] = table[0, :30]
+    table[3, :30] = table[0, :30]
+    shared = int(table[0, 29])
+    own = [int(table[2, 36])]
+    summ = gc.gpu_build()
+    after = gc.gpu_select(summ)[0]
+    best = int(table[0, int(np.nanargmax(gc.gpu_select(summ)[3][0, 0, 1:40])) + 1])
+    assert best != shared
+    old = summ.clone().reshape(gc.case.num_blocks, -1)
+    old[shared] = old[best]
+    want = gc.gpu_select(old.reshape(summ.shape))[:2]
+    assert not np.array_equal(want[0][0], after[0])
+    out = torch.empty(w.n, w.Hq, w.d, dtype=gc.case.k.dtype, device="cuda:0")
+    results = []
+    for _ in range(3):
+        now = old.clone().reshape(summ.shape)
+        ids = torch.full((w.n, Hkv, gc.k), -7, dtype=torch.int32, device="cuda:0")
+        cnt = torch.full((w.n, Hkv), -7, dtype=torch.int32, device="cuda:0")
+        gc.ctx.locks_decode_step(gc.case.q, None, None, gc.kv, now, w.n, out, ids, cnt)
+        torch.cuda.synchronize()
+        assert np.array_equal(ids.cpu().numpy(), want[0]) and np.array_equal(cnt.cpu().numpy(), want[1])
+        results.append(now.reshape(old.shape))
+        changed = (results[-1] != old).any(1).nonzero().flatten().tolist()
+        assert shared in changed and set(changed) <= {shared, *own}
+        assert torch.equal(results[-1], results[0])
+    assert gc.status() == 0
+    # the summary is a build's: nearly all bytes, or in fp32 the basis up to its signs
+    built = summ.reshape(old.shape)[shared]
+    if fmt == "f32":
+        mu = [x.view(torch.float32).reshape(Hkv, -1)[:, :128] for x in (results[0][shared], built)]
+        assert torch.allclose(mu[0], mu[1], rtol=0, atol=1e-5)   # fp32 sums of 16 keys of a few units
+    else:
+        assert (results[0][shared] != built).float().mean() <= 2e-2
+
+
 # The splits of a problem merge through the shared memory of their cluster (16, 8, 4 or 2 CTAs, by the number of problems; the last
 # case has one CTA each): slices of whole heads, of parts of heads and across heads, lists shorter than their row, an output buffer
 # that is aligned to its elements only.  Tolerance: P and the result in bf16 (see test_gpu_parity.py).

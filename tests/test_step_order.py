@@ -64,6 +64,6 @@ def test_a_step_follows_all_of_the_step_before(program, early, append, call, nth
     for j in second:
         assert set(first) <= before[j], (ops[j], [ops[i] for i in first if i not in before[j]])
     # arrivals that a broken-off step may have counted in part are cleared when nothing is left that counts
-    if early and append and call != "none":
+    if early and call != "none":
         clear = [i for i in first if ops[i][1] == "clear"]
         assert clear and all(i in before[clear[-1]] for i in first if ops[i][1] in ("build", "select"))
