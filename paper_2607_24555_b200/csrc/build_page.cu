@@ -200,7 +200,11 @@ __global__ void __launch_bounds__(page_threads(B) * page_ctas(B)) build_page_ker
   const int sub = threadIdx.x / NT, tid = threadIdx.x % NT, lane = tid & 31, warp = tid >> 5, r = p.r;
   PageShared<B> &sh = reinterpret_cast<PageShared<B> *>(smem_raw)[sub];
   auto sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(sub + 1), "n"(NT) : "memory"); };   // the page's threads
-  if (p.hint && blockIdx.x == 0 && threadIdx.x < 32)
+  if (p.stage) {
+    // Beside the scan the lengths are about to change, and the suggestion does not depend on them: a tensor scan that leaves room
+    // has a warp for every group, and then the strided partition takes one round.
+    if (p.hint && blockIdx.x == 0 && threadIdx.x == 0) *p.hint = LOCKS_PARTITION_STRIDED;
+  } else if (p.hint && blockIdx.x == 0 && threadIdx.x < 32)
     locks_update_partition_hint(p.hint, p.seq_lens, p.batch, p.Hkv, p.kpages, p.hint_wpp, p.hint_rounds, p.hint_W, lane);
   const int prob = blockIdx.x * PPC + sub;
   if (prob >= p.batch * p.Hkv) return;

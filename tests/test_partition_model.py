@@ -82,6 +82,33 @@ def test_balanced_partition_invariants(seed):
         assert all(rs[w][0] > s for w in touching[1:])
 
 
+def scan_geometry(nprob, max_groups, sms=148):
+    """CTAs, warps, warps per problem, problems in flight and rounds of a tensor scan, and whether a step's build fits beside it."""
+    need = max(1, -(-nprob * max_groups // 8))
+    grid = min(2 * sms, need)
+    W = 8 * grid
+    wpp = max(1, W // nprob)
+    nslots = W // wpp
+    return grid, W, wpp, nslots, -(-nprob // nslots), grid + -(-nprob // 4) <= 2 * sms
+
+
+def test_beside_a_build_the_strided_partition_is_always_suggested():
+    """A step's build that runs beside the scan writes this suggestion without a look at the lengths: with a warp for every group of
+    the longest possible sequence, one round of strides is never slower than the balanced partition."""
+    seen = 0
+    for nprob in range(1, 600):
+        for max_groups in list(range(1, 70)) + [127, 128, 255, 256, 511, 1056, 2048, 2367, 2368, 2400]:
+            grid, W, wpp, nslots, rounds, room = scan_geometry(nprob, max_groups)
+            if not room:
+                continue
+            seen += 1
+            assert wpp >= max_groups and rounds == 1
+            for most in {0, 1, max_groups // 2, max_groups}:             # groups of the longest sequence, of all of them
+                for units in {most, most * nprob}:
+                    assert not rounds * -(-most // wpp) * 16 > -(-units // W) * 17 + 8
+    assert seen > 1000
+
+
 def test_partition_suggestion_rule():
     """Iterations of the longest warp: strided = rounds * ceil(max groups / wpp), balanced = ceil(U / W); the
     balanced partition is suggested only when it wins by more than 1/16 plus half an iteration."""
