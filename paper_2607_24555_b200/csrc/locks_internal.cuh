@@ -131,30 +131,6 @@ locks_scan_geom locks_scan_geometry(const locks_ctx *c, int batch);
 // Whether the CTAs of a step's build fit beside this step's scan
 bool locks_scan_leaves_room(const locks_ctx *c, int batch);
 
-// Which partition suits these lengths: iterations of the longest warp, strided = rounds * ceil(max groups / wpp)
-// against balanced = ceil(units / warps); the balanced one has to win by more than its set-up costs.
-// Called by one warp; lane 0 writes *hint.
-__device__ __forceinline__ void locks_update_partition_hint(int32_t *hint, const int32_t *seq_lens, int batch, int Hkv,
-                                                            int k, int wpp, int rounds, int W, int lane) {
-  int sum = 0, mx = 0;
-  for (int b = lane; b < batch; b += 32) {
-    const int P = (seq_lens[b] + LOCKS_B - 1) / LOCKS_B;   // (the hint serves the tensor scan: 16-token pages)
-    const int ng = P <= k ? 0 : (P - 1 + LOCKS_GROUP - 1) / LOCKS_GROUP;
-    sum += ng;
-    mx = max(mx, ng);
-  }
-#pragma unroll
-  for (int o = 16; o; o >>= 1) {
-    sum += __shfl_xor_sync(0xffffffffu, sum, o);
-    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  }
-  if (lane == 0) {
-    const int strided = rounds * ((mx + wpp - 1) / wpp);
-    const int even = (int)(((int64_t)sum * Hkv + W - 1) / W);
-    *hint = (strided * 16 > even * 17 + 8) ? LOCKS_PARTITION_BALANCED : LOCKS_PARTITION_STRIDED;
-  }
-}
-
 // launchers (each returns LOCKS_OK or LOCKS_ERR_CUDA and adds to ctx->last_launches)
 // seq_inc = 1: lengths are taken one token longer than kv->seq_lens says and published in ctx->seq_eff
 int locks_launch_scan(locks_ctx *c, const void *q, const void *summaries, const locks_kv *kv, int batch,
@@ -268,6 +244,30 @@ __host__ __device__ constexpr int locks_fmt_stride(int fmt, int r, int B = LOCKS
 }
 
 #ifdef __CUDACC__
+
+// Which partition suits these lengths: iterations of the longest warp, strided = rounds * ceil(max groups / wpp)
+// against balanced = ceil(units / warps); the balanced one has to win by more than its set-up costs.
+// Called by one warp; lane 0 writes *hint.
+__device__ __forceinline__ void locks_update_partition_hint(int32_t *hint, const int32_t *seq_lens, int batch, int Hkv,
+                                                            int k, int wpp, int rounds, int W, int lane) {
+  int sum = 0, mx = 0;
+  for (int b = lane; b < batch; b += 32) {
+    const int P = (seq_lens[b] + LOCKS_B - 1) / LOCKS_B;   // (the hint serves the tensor scan: 16-token pages)
+    const int ng = P <= k ? 0 : (P - 1 + LOCKS_GROUP - 1) / LOCKS_GROUP;
+    sum += ng;
+    mx = max(mx, ng);
+  }
+#pragma unroll
+  for (int o = 16; o; o >>= 1) {
+    sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  }
+  if (lane == 0) {
+    const int strided = rounds * ((mx + wpp - 1) / wpp);
+    const int even = (int)(((int64_t)sum * Hkv + W - 1) / W);
+    *hint = (strided * 16 > even * 17 + 8) ? LOCKS_PARTITION_BALANCED : LOCKS_PARTITION_STRIDED;
+  }
+}
 
 __device__ __forceinline__ void set_status(int32_t *status, int code) { atomicCAS(status, 0, code); }
 

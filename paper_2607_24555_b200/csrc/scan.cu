@@ -18,6 +18,7 @@
 //                         per page, after an 8x8 movmatrix transpose of the fp16 hi/lo projection:
 //                           MMA#2  L[heads, tokens] = (P_hi | P_lo)[heads x 16] . codesC^T          (2 x m16n8k16 fp16)
 //                         and per 8 pages the centroid dots a[heads, pages] (8 x m16n8k16 fp16).
+#include <algorithm>
 #include <cstring>
 #include <cuda.h>            // CUtensorMap (types only; the encoder is fetched from the driver at run time)
 #include <cudaTypedefs.h>
@@ -1393,7 +1394,8 @@ int locks_launch_scan(locks_ctx *c, const void *q, const void *summaries, const 
     p.wpp = geo.wpp; p.nslots = geo.nslots; p.cta_reduce = geo.cta_reduce;
     // strided partition: one partial per (problem, warp), or per (problem, CTA) with the CTA-level merge;
     // balanced partition: the kernel counts the partials of each problem itself (part_cnt)
-    c->part_slots = geo.cta_reduce ? geo.wpp / kScanWarps : geo.wpp;
+    // (a problem can have more warps than groups; the selector reads this many of a row of max_groups before it knows the length)
+    c->part_slots = geo.cta_reduce ? geo.wpp / kScanWarps : std::min(geo.wpp, c->max_groups);
     int mode = c->scan_partition;
     if (mode == LOCKS_PARTITION_AUTO)
       mode = (c->hint_host && *reinterpret_cast<volatile int32_t *>(c->hint_host) == LOCKS_PARTITION_BALANCED)
@@ -1403,7 +1405,7 @@ int locks_launch_scan(locks_ctx *c, const void *q, const void *summaries, const 
     const bool balanced = LOCKS_SCAN_BALANCED && mode == LOCKS_PARTITION_BALANCED;
     if (balanced) {
       p.cta_reduce = 0;
-      c->part_slots = geo.wpp;
+      c->part_slots = c->max_groups;
     }
     c->part_balanced = balanced ? 1 : 0;
     c->last_partition = balanced ? LOCKS_PARTITION_BALANCED : LOCKS_PARTITION_STRIDED;

@@ -1,0 +1,41 @@
+"""What the scan's launcher decides on the host, from the library's own code with the CUDA runtime replaced by fakes
+(tests/fakes/scan_launch.cpp)."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
+FORMAT = {"f32": 0, "i4": 1, "i8": 2, "bf16": 3}
+STRIDED, BALANCED = 1, 2
+
+
+@pytest.fixture(scope="module")
+def decide(tmp_path_factory):
+    """decide([(B, Hq, Hkv, rank, format, query bits, batch, pages, partition), ..]) -> [(partials, slots, CTAs, early build), ..]"""
+    if not (shutil.which(NVCC) and shutil.which("g++")):
+        pytest.skip("no compiler")
+    d = tmp_path_factory.mktemp("scan_launch")
+    csrc, inc = os.path.join(ROOT, "paper_2607_24555_b200", "csrc"), os.path.join(ROOT, "include")
+    scan, exe = str(d / "scan.o"), str(d / "scan_launch")
+    subprocess.run([NVCC, "-gencode", "arch=compute_100a,code=sm_100a", "-std=c++17", "-O0", "-Xcicc", "-O0", "-Xptxas", "-O0", "-I", inc, "-I", csrc,
+                    "-c", os.path.join(csrc, "scan.cu"), "-o", scan], check=True, capture_output=True)
+    subprocess.run(["g++", "-std=c++17", "-I", inc, "-I", csrc, "-I", os.path.join(os.path.dirname(os.path.dirname(NVCC)), "include"), "-o", exe,
+                    os.path.join(ROOT, "tests", "fakes", "scan_launch.cpp"), scan, "-Wl,--unresolved-symbols=ignore-all"], check=True, capture_output=True)
+
+    def run(cases):
+        text = "\n".join(" ".join(str(x) for x in (*c[:4], FORMAT[c[4]], 1 if c[5] == 16 else 0, *c[6:])) for c in cases)
+        out = subprocess.run([exe], input=text, check=True, capture_output=True, text=True, timeout=60).stdout.split("\n")[:-1]
+        assert len(out) == len(cases)
+        return [tuple(int(x) for x in line.split()) for line in out]
+    return run
+
+
+def test_partials_fit_their_row(decide):
+    """The selector reads a problem's partials before it knows how many of them this sequence has."""
+    cases = [(16, 4 * Hkv, Hkv, rank, "i4", 16, batch, pages, part) for Hkv in (1, 2, 3, 8) for rank in (8, 4, 2) for batch in (1, 2, 3, 5, 40)
+             for pages in (1, 8, 9, 24, 40, 100, 1000) for part in (STRIDED, BALANCED)]
+    for case, (partials, slots, _, _) in zip(cases, decide(cases)):
+        assert 1 <= partials <= slots, (case, partials, slots)
