@@ -128,7 +128,7 @@ struct locks_scan_geom {
   int cta_reduce;            // all warps of a CTA share one problem for the whole launch
 };
 locks_scan_geom locks_scan_geometry(const locks_ctx *c, int batch);
-// Whether the CTAs of a step's build fit beside this step's scan
+// Whether a step's build had better start beside this step's scan than behind it
 bool locks_scan_leaves_room(const locks_ctx *c, int batch);
 
 // launchers (each returns LOCKS_OK or LOCKS_ERR_CUDA and adds to ctx->last_launches)

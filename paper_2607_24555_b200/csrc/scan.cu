@@ -1359,10 +1359,29 @@ locks_scan_geom locks_scan_geometry(const locks_ctx *c, int batch) {
   return g;
 }
 
-// Only the tensor scan fills every SM for as long as it lasts; of two slots on an SM a build CTA (four page-heads) takes one.
+namespace {
+// The scan that a step launches: the tensor kernel, that of wide pages, or one of the plain ones
+bool tensor_scan(const locks_ctx *c) {
+  return c->cfg.summary_fmt == LOCKS_FMT_I4 && c->cfg.q_dtype == LOCKS_BF16 && c->scorer == LOCKS_SCORER_SUMMARY && c->B == LOCKS_B;   // ranks 2, 4, 8
+}
+dim3 plain_scan_grid(const locks_ctx *c, int batch) { return dim3((c->max_groups + 3) / 4, c->cfg.num_kv_heads, batch); }
+}  // namespace
+
+// 16-token pages: the build (22 us) is shorter than most scans and has to fit beside it; both together take at most two CTAs on an SM.
+// The tensor scan has two slots on an SM, of which a build CTA (four page-heads) takes one, and a CTA that had to wait for a build
+// would end last.  The plain scans have more slots, but lose beyond the same number.  Steps of batch x 8K tokens, 8 KV heads, behind a copy of the lengths, a page filled / none; CTAs of the
+// scan, build after the scan -> beside it:
+//   fp32   144: 39.0 -> 31.6 / 30.8 -> 30.8 us   288: 43.4 -> 41.0 / 35.3 -> 37.3   576: 57.1 -> 61.8 / 55.6 -> 61.3   1152: 93.7 -> 99.9 / 95.4 -> 98.9
+//   int8   144: 98.4 -> 88.2 / 86.1 -> 92.2      288: 105 -> 96.3 / 94.2 -> 96.3    576: 123 -> 121 / 115 -> 119       1152: 158 -> 160 / 158 -> 160
+//   bf16   144: 93.3 -> 79.9 / 82.0 -> 79.9      288: 102 -> 92.2 / 92.3 -> 92.2    576: 117 -> 111 / 111 -> 111       1152: 146 -> 146 / 146 -> 146
+// (behind a kernel instead of a copy a step that fills no page takes the same time either way, to 2 us.)  32- and 64-token pages:
+// the build (47 and 180 us) is what such a step waits for (4 x 16K tokens of 32: 63.6 -> 55.3 / 32.8 -> 33.1; of 64, 8 x 8K: 215 ->
+// 202 / 36.9 -> 44.8; int8, 4 x 8K of 64: 285 -> 197 / 106 -> 115; 32 x 8K of 32: 116 -> 113 / 112 -> 113).
 bool locks_scan_leaves_room(const locks_ctx *c, int batch) {
-  if (!(c->cfg.summary_fmt == LOCKS_FMT_I4 && c->cfg.q_dtype == LOCKS_BF16 && c->B == LOCKS_B)) return true;
-  return locks_scan_geometry(c, batch).grid + (batch * c->cfg.num_kv_heads + 3) / 4 <= kScanCtasPerSm * c->num_sms;
+  if (c->B != LOCKS_B) return true;
+  const dim3 plain = plain_scan_grid(c, batch);
+  const int64_t ctas = tensor_scan(c) ? locks_scan_geometry(c, batch).grid : (int64_t)plain.x * plain.y * plain.z;
+  return ctas + (batch * c->cfg.num_kv_heads + 3) / 4 <= kScanCtasPerSm * c->num_sms;
 }
 
 int locks_launch_scan(locks_ctx *c, const void *q, const void *summaries, const locks_kv *kv, int batch,
@@ -1383,12 +1402,10 @@ int locks_launch_scan(locks_ctx *c, const void *q, const void *summaries, const 
   p.Pmax = c->Pmax; p.max_groups = c->max_groups; p.num_blocks = kv->num_blocks; p.k = c->k;
   p.S = c->S; p.r = c->cfg.rank; p.sm_scale = c->cfg.sm_scale; p.B = c->B;
   p.scorer = c->scorer;
-  const bool tensor = c->cfg.summary_fmt == LOCKS_FMT_I4 && c->cfg.q_dtype == LOCKS_BF16 &&
-                      c->scorer == LOCKS_SCORER_SUMMARY && c->B == LOCKS_B;   // ranks 2, 4, 8
   c->part_slots = c->max_groups;   // generic kernel: one partial per 8-page group
   c->part_balanced = 0;
   c->last_partition = 0;
-  if (tensor) {
+  if (tensor_scan(c)) {
     const locks_scan_geom geo = locks_scan_geometry(c, batch);
     const int grid = geo.grid;
     p.wpp = geo.wpp; p.nslots = geo.nslots; p.cta_reduce = geo.cta_reduce;
@@ -1483,7 +1500,7 @@ int locks_launch_scan(locks_ctx *c, const void *q, const void *summaries, const 
 #undef LOCKS_WIDE_LAUNCH
 #undef LOCKS_WIDE_SPLIT
   } else {
-    dim3 grid((c->max_groups + 3) / 4, p.Hkv, batch);
+    const dim3 grid = plain_scan_grid(c, batch);
     const bool qbf = c->cfg.q_dtype == LOCKS_BF16;
     if (c->cfg.summary_fmt == LOCKS_FMT_F32 && c->B == LOCKS_B && p.scorer == LOCKS_SCORER_SUMMARY && (p.r == 2 || p.r == 4 || p.r == 8)) {
 #define LOCKS_F32_LAUNCH(R_)                                                                        \

@@ -39,3 +39,17 @@ def test_partials_fit_their_row(decide):
              for pages in (1, 8, 9, 24, 40, 100, 1000) for part in (STRIDED, BALANCED)]
     for case, (partials, slots, _, _) in zip(cases, decide(cases)):
         assert 1 <= partials <= slots, (case, partials, slots)
+
+
+def test_builds_start_beside_scans_that_leave_room(decide):
+    """16-token pages: the CTAs of the scan that is launched, whichever it is, and those of the build (four page-heads each) take at
+    most two places on an SM.  Wider pages: always, since the build lasts several times as long as the rest of the step."""
+    cases = [(B, 4 * Hkv, Hkv, rank, fmt, 16 if dtype == "bf16" else 32, batch, pages, STRIDED) for B in (16, 32, 64) for Hkv in (1, 2, 8)
+             for rank in (8, 2) for fmt, dtype in (("i4", "bf16"), ("i4", "f32"), ("i8", "bf16"), ("bf16", "bf16"), ("f32", "f32")) for batch in (1, 2, 4, 9, 40)
+             for pages in (8, 100, 300, 576, 1100)]
+    rooms = set()
+    for case, (_, _, ctas, room) in zip(cases, decide(cases)):
+        fits = ctas + -(-case[6] * case[2] // 4) <= 2 * 148
+        assert room == (case[0] != 16 or fits), (case, ctas, room)
+        rooms.add((case[0], case[4], case[5], room))
+    assert {(16, f, d, r) for f, d in (("i4", 16), ("i4", 32), ("i8", 16), ("bf16", 16), ("f32", 32)) for r in (0, 1)} <= rooms
