@@ -526,12 +526,12 @@ def test_selection_from_chunk_lists(pages, Hq, Hkv, k):
 # stores the length.  Requests before, at and after a page boundary, and one without room for the token; KV heads that fill the
 # build's CTAs (4, 2 or 1 page-heads) and that do not; three steps, so that what one step leaves behind shows in the next.
 @pytest.mark.parametrize("Hkv", [1, 3, 4])
-@pytest.mark.parametrize("B,dtype", [(16, "bf16"), (32, "bf16"), (64, "bf16"), (16, "f32")])
-def test_lengths_of_steps_whose_build_starts_at_once(B, dtype, Hkv):
+@pytest.mark.parametrize("B,dtype,fmt", [(16, "bf16", "i4"), (32, "bf16", "i4"), (64, "bf16", "i4"), (16, "f32", "f32"), (16, "bf16", "i8"), (32, "bf16", "bf16")])
+def test_lengths_of_steps_whose_build_starts_at_once(B, dtype, fmt, Hkv):
     from gpu_util import GpuCase
     rows = 24
     w = locks_synth.Workload("lengths", [B * rows, B * 9 - 1, B * 9 - 2, B * 9, 1, B * 20 - 3], Hq=4 * Hkv, Hkv=Hkv, B=B, dtype=dtype,
-                             fmt="i4" if dtype == "bf16" else "f32", rank=8, budget=4 * B, seed=B + Hkv)
+                             fmt=fmt, rank=8, budget=4 * B, seed=B + Hkv)
     gc = GpuCase(w)
     want = gc.case.seq_lens.clone()
     summ = gc.gpu_build()
@@ -598,7 +598,8 @@ def test_summary_of_a_shared_page_changes_after_the_scores(B, fmt, dtype, rank, 
 
 # The splits of a problem merge through the shared memory of their cluster (16, 8, 4 or 2 CTAs, by the number of problems; the last
 # case has one CTA each): slices of whole heads, of parts of heads and across heads, lists shorter than their row, an output buffer
-# that is aligned to its elements only.  Tolerance: P and the result in bf16 (see test_gpu_parity.py).
+# that is aligned to its elements only.  Tolerance: P and the result are rounded to bf16, each by at most 2^-9 of itself, and the
+# weighted mean of |v| is no smaller than |out|.
 @pytest.mark.parametrize("n,Hkv,G", [(1, 3, 5), (1, 2, 16), (3, 4, 1), (2, 4, 12), (5, 8, 7), (10, 4, 9), (5, 8, 16), (25, 4, 4), (25, 4, 3), (50, 4, 5), (64, 4, 8)])
 def test_splits_merge_in_their_cluster(n, Hkv, G):
     from gpu_util import GpuCase
@@ -606,11 +607,69 @@ def test_splits_merge_in_their_cluster(n, Hkv, G):
     gc = GpuCase(w)
     ids, cnt, _, _ = gc.gpu_select(gc.gpu_build())
     want, want_lse = oracle.attend(gc.cache, t2np(gc.case.q), gc.sm, ids, cnt)
+    gc.cache.v &= 0x7FFF   # |v|, as bf16 bits
+    bound = oracle.attend(gc.cache, t2np(gc.case.q), gc.sm, ids, cnt)[0] * 2.0**-8 + 1e-5
     d_ids, d_cnt = torch.from_numpy(ids).cuda(), torch.from_numpy(cnt).cuda()
     for shift in (0, 1):
         out = torch.empty(w.n * w.Hq * w.d + 1, dtype=torch.bfloat16, device="cuda:0")[shift:][:w.n * w.Hq * w.d].view(w.n, w.Hq, w.d)
         lse = torch.empty(w.n, w.Hq, dtype=torch.float32, device="cuda:0")
         gc.ctx.locks_sparse_attend(gc.case.q, gc.kv, w.n, d_ids, d_cnt, out, lse)
         torch.cuda.synchronize()
-        assert np.abs(out.float().cpu().numpy() - want).max() <= 2e-2 and np.abs(lse.cpu().numpy() - want_lse).max() <= 1e-3
+        assert (np.abs(out.float().cpu().numpy() - want) <= bound).all() and np.abs(lse.cpu().numpy() - want_lse).max() <= 1e-3
     assert gc.status() == 0
+
+
+# Infinite and undefined values pass the same merge: they reach the outputs of their dimension and no other.
+@pytest.mark.parametrize("n,Hkv,G", [(1, 3, 5), (1, 2, 16), (5, 8, 7), (10, 4, 9), (25, 4, 4), (64, 4, 8)])
+def test_infinite_values_pass_the_cluster_merge(n, Hkv, G):
+    from gpu_util import GpuCase
+    w = locks_synth.Workload("merge", [900 + 7 * i % 60 for i in range(n)], Hq=G * Hkv, Hkv=Hkv, budget=768, seed=n + G)
+    gc = GpuCase(w)
+    ids, cnt, _, _ = gc.gpu_select(gc.gpu_build())
+    want = oracle.attend(gc.cache, t2np(gc.case.q), gc.sm, ids, cnt)[0]
+    for b in range(n):
+        for h in range(Hkv):
+            for at, dim, v in ((0, 3, "inf"), (cnt[b, h] // 2, 64, "nan"), (cnt[b, h] - 1, 127, "-inf")):
+                gc.case.v[int(gc.case.block_table[b, int(ids[b, h, at])]), h, 0, dim] = float(v)
+                want[b, h * G:(h + 1) * G, dim] = float(v)
+    out, lse = gc.gpu_attend(ids, cnt)
+    assert np.array_equal(np.isnan(out), np.isnan(want)) and np.array_equal(np.isinf(out), np.isinf(want))
+    assert np.array_equal(np.sign(out[np.isinf(out)]), np.sign(want[np.isinf(want)])) and np.isfinite(lse).all()
+    there = np.isfinite(want)
+    assert np.abs(out[there] - want[there]).max() <= 2e-2
+
+
+# log Z from many partials, whole slices of them (32 of every warps-per-head x 32) and single ones at minus infinity, and scores at
+# minus infinity for some of a group's heads.  The expected shares in fp64; scores and log Z of a few units, sums in fp32.
+@pytest.mark.parametrize("Hq,Hkv", [(8, 2), (6, 1), (16, 2), (16, 1)])
+@pytest.mark.parametrize("pages", [3000, 20000])
+def test_log_shares_with_empty_slices_of_partials(pages, Hq, Hkv):
+    import paper_2607_24555_b200 as locks
+    from paper_2607_24555_b200.binding import KVView, make_config
+    rng = np.random.default_rng(pages + Hq)
+    G, k = Hq // Hkv, 64
+    ctx = locks.Context(make_config(Hq, Hkv, 8, "i4", "bf16", 1, pages, k * 16))
+    dummy = torch.zeros(1, Hkv, 16, 128, dtype=torch.bfloat16, device="cuda:0")
+    kv = KVView(dummy, dummy, (Hkv * 2048, 2048, 128), 1, torch.zeros(1, pages, dtype=torch.int32, device="cuda:0"),
+                torch.tensor([pages * 16 - 3], dtype=torch.int32, device="cuda:0"))
+    mass = (3.0 * rng.standard_normal((1, Hq, pages))).astype(np.float32)
+    mass[:, ::max(2, G), ::7] = -np.inf
+    for nparts in (1, 33, 200, 360):
+        parts = (2.0 * rng.standard_normal((nparts, 1, Hq))).astype(np.float32)
+        parts[32:64] = -np.inf
+        parts[96:128] = -np.inf
+        parts[1::5] = -np.inf
+        parts[:, 0, Hq - 1] = -np.inf
+        parts[nparts - 1 if nparts < 33 else 20, 0, Hq - 1] = 0.5
+        ids = torch.full((1, Hkv, k), -7, dtype=torch.int32, device="cuda:0")
+        cnt = torch.full((1, Hkv), -7, dtype=torch.int32, device="cuda:0")
+        share = torch.full((1, Hkv, pages), float("nan"), device="cuda:0")
+        ctx.locks_select_scored(torch.from_numpy(parts).cuda(), kv, 1, ids, cnt, share, torch.from_numpy(mass).cuda())
+        with np.errstate(divide="ignore"):
+            logz = np.log(np.exp(parts.astype(np.float64)).sum(0))[0]
+            want = np.log(np.exp(mass[0].astype(np.float64) - logz[:, None]).reshape(Hkv, G, pages).mean(1))
+        got = share[0].cpu().numpy()[:, 1:-1]
+        assert np.abs(got - want[:, 1:-1]).max() <= 1e-4
+        for h in range(Hkv):
+            best = 1 + np.sort(np.argsort(-got[h], kind="stable")[:k - 2])
+            assert np.array_equal(ids[0, h].cpu().numpy(), np.concatenate([[0], best, [pages - 1]]))
