@@ -267,9 +267,9 @@ int locks_sparse_attend(locks_ctx *ctx, const void *q, const locks_kv *kv, int b
  *      reads it, not even that of another request of the batch that holds the same block.  Its bytes may differ
  *      from those that locks_build_summaries gives for the same page, in about one of ten thousand (another solver,
  *      as accurate).
- * These are the results; inside, the token is counted from the first kernel on, its rows are written by
- * the selector's kernel (no page summary depends on them) and seq_lens is stored back there, so the
- * append costs no launch of its own.  k_new / v_new: device, 16-byte aligned.  A sequence whose
+ * These are the results; inside, the token is counted from the first kernel on and its rows are written by
+ * the selector's kernel, so the append costs no launch of its own.  seq_lens is stored back there, or by the build
+ * of the page summaries where that runs beside the whole step; the build takes the token from k_new.  k_new / v_new: device, 16-byte aligned.  A sequence whose
  * block-table row is full keeps its length, nothing is written for it and LOCKS_ERR_BAD_BLOCK is
  * recorded in the status word.
  * page_ids / page_count may be NULL (kept in the workspace). */

@@ -465,8 +465,8 @@ int locks_decode_step(locks_ctx *ctx, const void *q, const void *k_new, const vo
     else cudaEventRecord(pe[i], st);
   };
   // The new token is counted from the scan on (lengths one longer, published in the workspace); its K/V
-  // rows are written by the selector's kernel, beside the ranking, which is early enough for the two
-  // readers of the last page (attention, and the summary build when the token completes a page).
+  // rows are written by the selector's kernel, beside the ranking, which is early enough for attention.  The build of
+  // a page that the token completes runs at the same time and takes it from k_new.
   locks_append app;
   locks_kv kv_step = *kv;
   if (k_new) {

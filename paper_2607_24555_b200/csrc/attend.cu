@@ -566,8 +566,9 @@ __global__ void __launch_bounds__(LOCKS_ATT_WARPS * 32, LOCKS_ATT_CTAS_PER_SM) a
 // Steps with fp32 caches, before (a warp per head, token after token, each with a warp reduction of its own) and after this
 // kernel and scan_f32_kernel: 30 requests x 32 pages, 4 heads, 226 -> 70 us; 25 x 169..666 tokens, all pages, 122 -> 41; 48 x
 // 237..968, 5 heads, 377 -> 114; 3 x 31K, 8 heads, 357 -> 99.
+constexpr int kF32CtasPerSm = 3;
 template <int NH>
-__global__ void __launch_bounds__(128, 3) attend_f32_kernel(AttParams p) {
+__global__ void __launch_bounds__(128, kF32CtasPerSm) attend_f32_kernel(AttParams p) {
   constexpr int kTok = 8, NV = kTok * NH, kDup = 32 / NV;   // kDup lanes hold the same score
   static_assert(NH == 1 || NH == 4, "scores have to fill or divide a warp");
   __shared__ float so[4][NH][LOCKS_D];
@@ -840,9 +841,18 @@ AttGeom attend_geometry(locks_ctx *c, int batch, int Hkv, int G, bool dense) {
 
 }  // namespace
 
+// Called at once, attention's CTAs wait in their slots while the selector works, and a build that starts when the scan ends has what
+// they leave.  Worth it between about 7/8 and 19/20 of the slots.  Steps that append, called when the keys are there -> at once; CTAs
+// of attention + of the build, of 592 slots: 512 + 16 (8 x 24K) 50.0 -> 53.0 us, (8 x 32K) 53.7 ->
+// 53.5; 512 + 32 (16 x 8K) 51.6 -> 51.7; 528 + 17 (11 x 8K, 6 KV heads) 41.0 -> 38.4; 528 + 33 (33 x 8K, 4) 55.3 -> 56.7; 532 + 34 (19 x 8K,
+// 7) 55.4 -> 53.0; 544 + 34 (17 x 8K) 58.5 -> 53.6, when all 17 fill a page 61.1 -> 75.3; 560 + 18 (10 x 8K, 7) 43.0 -> 42.4; 560 + 35
+// (20 x 8K, 7) 60.8 -> 54.9; 576 + 18 (9 x
+// 32K) 56.0 -> 57.0; 576 + 36 (18 x 8K) 55.8 -> 58.4, (18 x 30K) 87.5 -> 90.8; 592 + 37 (37 x 8K, 4) 66.4 -> 77.6.  fp32 caches (three CTAs on
+// an SM, always more than fit): 8 x 8K 91.4 -> 94.5, 16 x 8K 144.6 -> 148.8.
 bool locks_attend_fills(locks_ctx *c, int batch) {
-  const int Hkv = c->cfg.num_kv_heads;
-  return 8 * attend_geometry(c, batch, Hkv, c->G, false).splits * Hkv * batch > 7 * c->num_sms * LOCKS_ATT_CTAS_PER_SM;
+  const int Hkv = c->cfg.num_kv_heads, slots = c->num_sms * (c->cfg.kv_dtype == LOCKS_BF16 ? LOCKS_ATT_CTAS_PER_SM : kF32CtasPerSm);
+  const int ctas = attend_geometry(c, batch, Hkv, c->G, false).splits * Hkv * batch;
+  return 8 * ctas > 7 * slots && 20 * ctas <= 19 * slots;
 }
 
 int locks_launch_attend(locks_ctx *c, const void *q, const locks_kv *kv, int batch, const int32_t *ids,

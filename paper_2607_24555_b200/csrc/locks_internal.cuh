@@ -15,7 +15,8 @@
 #define LOCKS_SEL_MAX_EPT 16 // pages per thread a selector CTA ranks at most (512 threads: 8192 pages or list entries)
 #define LOCKS_ATT_WARPS 3        // warps per attend CTA
 #define LOCKS_ATT_STAGES 2       // pages (4 KB of K + 4 KB of V each) in each warp's ring
-#define LOCKS_ATT_CTAS_PER_SM 4  // 4 x 48 KB of shared memory
+#define LOCKS_ATT_CTAS_PER_SM 4  // 4 x 48 KB of shared memory; as clusters up to 56 KB each, which with 1 KB reserved per CTA is all of an
+                                 // SM's 228 KB: no static shared memory in attend_bf16_kernel
 #define LOCKS_ATT_MAX_SPLITS 128
 #define LOCKS_ATT_SLOT_BOUND 1024 // upper bound on resident attend CTAs of any supported GPU (148 SMs x 4 on B200)
 #ifndef LOCKS_SCAN_GATHER
@@ -88,7 +89,7 @@ struct locks_ctx {
   int32_t *arrivals;       // [max_batch] readers of a request's length that are done (zero between steps; see BuildParams)
   int32_t *staged;         // [max_batch][Hkv], behind arrivals: which of a staged summary's two parties have come (zero between steps)
   char *stage_summ;        // [max_batch][Hkv][S] summaries of a step that were ready before its scores
-  cudaStream_t side;       // build of freshly filled pages runs beside attend
+  cudaStream_t side;       // build of freshly filled pages, beside the whole step or from the end of the scan on
   cudaEvent_t ev_fork, ev_join;
   int last_launches;
   locks_host_graph hg[LOCKS_HOST_GRAPHS];

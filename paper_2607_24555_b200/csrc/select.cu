@@ -3,7 +3,7 @@
 //   log m_bar_j = log( (1/G) sum_g exp(s^_j(q_g) - log Z_g) )
 //   S = {0, P-1}  U  top-(k-2) candidates by log m_bar_j (ties: lower page index), ids ascending.
 // One 512-thread CTA ranks a chunk of 512 .. 8192 pages of a (request, KV head): it turns the chunk's scores into
-// order-preserving 32-bit keys in shared memory and emits the K = k-2 largest in page order (select_emit: a histogram that
+// order-preserving 32-bit keys in shared memory and emits the K = k-2 largest in page order (emit_winners: a histogram that
 // finds the bin of the K-th largest key, an exact ranking of that bin's few keys, and a bit map of the winners, whose prefix
 // counts are the output positions).  With one chunk per problem that is the final table.  With several, each chunk emits
 // its own top-(k-2) (key, page) list, and the CTA of a problem that finishes last ranks the lists the same way in the same
@@ -13,7 +13,7 @@
 // coalesced and every thread is busy whatever the context length.
 // The kernel runs once through its code on at most a few dozen SMs, so instruction fetch is a visible part
 // of its latency: loops over a thread's elements stay rolled (keys live in shared memory, not in
-// registers), and the two routines used by both rounds are real calls.
+// registers), and the ranking is a real call (select_emit) in the kernels that need it twice.
 #include "locks_internal.cuh"
 
 namespace {
@@ -48,7 +48,8 @@ struct SelParams {
 // cache (one warp, a few independent loads and stores beside the ranking's own loads), and the CTA of
 // head 0 stores the step's length back to the caller's array.  Nothing reads the caller's array between
 // the scan (complete before this kernel passes its wait) and the end of the step, except a build that started
-// beside the scan (a.arrivals): the step's other kernels take lengths from the published copy.
+// beside the scan: the step's other kernels take lengths from the published copy.  With such a build (a.arrivals) the
+// last to arrive of this CTA and the request's page-heads stores the length.
 __device__ __noinline__ void append_token(const SelParams &p, int b, int h, int lane, int T) {
   const locks_append &a = p.app;
   const int batch = p.batch, Hkv = p.Hkv, Pmax = p.Pmax, Bshift = p.Bshift;
@@ -120,8 +121,8 @@ struct SelShared {
 };
 
 extern __shared__ __align__(16) uint8_t sel_smem[];
-// The routines below are real calls; each takes the block's shared state from the symbol itself (a
-// reference argument would turn every access into a generic one) and its inputs by value (no stack).
+// Routines that are real calls take the block's shared state from the symbol itself (a reference argument would turn every
+// access into a generic one) and their inputs by value (no stack).
 __device__ __forceinline__ SelShared &shared_state() { return *reinterpret_cast<SelShared *>(sel_smem); }
 
 __device__ __forceinline__ float ex2f(float x) {
@@ -139,7 +140,7 @@ __device__ __forceinline__ uint32_t order_key(float f) {
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-// smallest and largest valid key of this thread -> sh.red (read by select_emit after its first barrier)
+// smallest and largest valid key of this thread -> sh.red (read by emit_winners after its first barrier)
 __device__ __forceinline__ void publish_range(SelShared &sh, uint32_t kmin, uint32_t kmax) {
   kmin = __reduce_min_sync(0xffffffffu, kmin);
   kmax = __reduce_max_sync(0xffffffffu, kmax);
@@ -553,7 +554,7 @@ __global__ void __launch_bounds__(LOCKS_SEL_THREADS, 2) select_kernel(const __gr
   }, p.logshare ? p.logshare + (int64_t)prob * p.Pmax : nullptr);
   // Attention's CTAs are called when the keys are there, not at once: waiting, they would hold the slots in which the step's build
   // starts when the scan ends (32 x 16K tokens, budget 16 pages: 59.4 -> 53.3 us a step, 8 x 24K 59.2 -> 52.9).  Where attention
-  // itself needs more than 7/8 of the slots it comes first (17 x 8K tokens, 544 of 592: 55.7 us; the build first 61.6).
+  // itself needs most of the slots, but leaves some, it comes first (locks_attend_fills).
   pdl_trigger();
   if (P <= p.k) return;
   if (nslab == 0) {  // chunk past the candidates: an empty list
