@@ -38,16 +38,14 @@ template <int B> struct PageShared {
   float sig[16];                      // singular values with the sign of their mode
   float mx[4], kn[4];
   uint8_t codes[16 * LOCKS_D];        // int4 codes before packing
-  int early, pad[3];                  // the summary has to wait (BuildParams::stage); a CTA's pages start on 16 bytes
+  int early, solved, pad[2];          // the summary has to wait (BuildParams::stage); the modes are there; a CTA's pages start on 16 bytes
 };
 
 static_assert(sizeof(PageShared<16>) % 16 == 0 && sizeof(PageShared<32>) % 16 == 0, "");
 
 // Eigenvectors and eigenvalues of the symmetric matrix m0 * 2^-ex (unit scale), by one warp: sh.us[mode][token] and
 // sh.lam[mode] of the modes in descending order (the first min(r, B) are accurate, the rest are not needed).
-// sh.early: whether the selector has yet to come to `staged` (BuildParams::stage).  In the usual case it has long been there; asked for
-// here, the answer arrives while the modes are put in order.
-template <int B> __device__ __forceinline__ void solve_modes(PageShared<B> &sh, float scale, float unscale, int r, int lane, const int32_t *staged) {
+template <int B> __device__ __forceinline__ void solve_modes(PageShared<B> &sh, float scale, float unscale, int r, int lane) {
   constexpr int L = 64 / B, R = B / L, R2 = R / 2;   // lanes per pair of columns; rows, and packed pairs of rows, per lane
   const int pair = lane / L, row0 = (lane % L) * R;
   const float *m0 = sh.m[0];
@@ -177,8 +175,6 @@ template <int B> __device__ __forceinline__ void solve_modes(PageShared<B> &sh, 
     }
     if (!__any_sync(0xffffffffu, bad != 0)) break;
   }
-  int come = 1;
-  if (staged && lane == 0) asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(come) : "l"(staged) : "memory");
   ranks();
 #pragma unroll
   for (int c = 0; c < 2; ++c) {
@@ -190,7 +186,6 @@ template <int B> __device__ __forceinline__ void solve_modes(PageShared<B> &sh, 
         *reinterpret_cast<float4 *>(sh.us + rank[c] * B + row0 + 2 * i) =
             make_float4(w[c][i].x * inv, w[c][i].y * inv, w[c][i + 1].x * inv, w[c][i + 1].y * inv);
   }
-  if (lane == 0) sh.early = come == 0;
 }
 
 template <int B>
@@ -200,8 +195,8 @@ __global__ void __launch_bounds__(page_threads(B) * page_ctas(B)) build_page_ker
   const int sub = threadIdx.x / NT, tid = threadIdx.x % NT, lane = tid & 31, warp = tid >> 5, r = p.r;
   PageShared<B> &sh = reinterpret_cast<PageShared<B> *>(smem_raw)[sub];
   auto sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(sub + 1), "n"(NT) : "memory"); };   // the page's threads
-  if (p.stage) {
-    // Beside the scan the lengths are about to change, and the suggestion does not depend on them: a tensor scan that leaves room
+  if (p.seq_commit) {
+    // The lengths are about to change, and the suggestion does not depend on them: a tensor scan that leaves room for this kernel
     // has a warp for every group, and then the strided partition takes one round.
     if (p.hint && blockIdx.x == 0 && threadIdx.x == 0) *p.hint = LOCKS_PARTITION_STRIDED;
   } else if (p.hint && blockIdx.x == 0 && threadIdx.x < 32)
@@ -257,6 +252,7 @@ __global__ void __launch_bounds__(page_threads(B) * page_ctas(B)) build_page_ker
     }
     kn = warp_sum(kn);
     if (lane == 0) sh.kn[warp] = kn;
+    if (tid == 0) sh.solved = 0;
   }
   sync();
   float knorm2 = 0.f;
@@ -315,7 +311,16 @@ __global__ void __launch_bounds__(page_threads(B) * page_ctas(B)) build_page_ker
       scale = __uint_as_float((uint32_t)(127 - ex) << 23);
       unscale = __uint_as_float((uint32_t)(127 + ex) << 23);
     }
-    solve_modes<B>(sh, scale, unscale, r, lane, p.stage ? p.staged + prob : nullptr);
+    solve_modes<B>(sh, scale, unscale, r, lane);
+    if (lane == 0) *reinterpret_cast<volatile int *>(&sh.solved) = 1;
+  } else if (warp == 1 && lane == 0) {
+    // Has the selector come (BuildParams::stage)?  It usually does long before the modes are there; asked here, the answer costs them
+    // no time (asked by the warp that solves, at its end, 4 x 16K tokens with 32-token pages: 57.9 us a step, now 56.5).
+    int come = 1;
+    if (p.stage) do {
+      asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(come) : "l"(p.staged + prob) : "memory");
+    } while (!come && !*reinterpret_cast<volatile int *>(&sh.solved));
+    sh.early = !come;
   }
   sync();
   // ---- modes kept

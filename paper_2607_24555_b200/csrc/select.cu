@@ -40,6 +40,7 @@ struct SelParams {
   int combine;       // LOCKS_COMBINE_*
   int attend_first;  // let the next kernel be scheduled at once
   int Bshift;        // log2 of the page size (4, 5 or 6)
+  int place;         // `staged` is given (asked for in a line of parameters that is read anyway)
   locks_append app;  // decode step only: the new token's K/V rows, written here beside the ranking
   locks_staged staged;  // decode step only: summaries that were ready before the scores
 };
@@ -542,7 +543,7 @@ __global__ void __launch_bounds__(LOCKS_SEL_THREADS, 2) select_kernel(const __gr
     P = np;
     if (p.app.k_new && chunk == 0 && tid >= LOCKS_SEL_THREADS - 32)
       append_token(p, b, h, tid & 31, T);
-    if (p.staged.stage && chunk == 0 && tid >= LOCKS_SEL_THREADS - 32) place_staged(p, b, h, tid & 31, T);
+    if (p.place && (T & ((1 << p.Bshift) - 1)) == 0 && chunk == 0 && tid >= LOCKS_SEL_THREADS - 32) place_staged(p, b, h, tid & 31, T);
     if (P <= p.k) {  // every page is kept
       if (chunk == 0) {
         for (int j = tid; j < p.k; j += LOCKS_SEL_THREADS) ids[j] = j < P ? j : -1;
@@ -706,6 +707,7 @@ int locks_launch_select(locks_ctx *c, const float *shat, const locks_kv *kv, int
   else p.app.k_new = nullptr;
   if (staged) p.staged = *staged;
   else p.staged.stage = nullptr;
+  p.place = p.staged.stage != nullptr;
   p.status = c->status;
   p.shat = shat; p.part = c->part; p.seq_lens = kv->seq_lens; p.ids = ids; p.cnt = cnt; p.logshare = logshare;
   p.cand_key = reinterpret_cast<uint32_t *>(c->cand_val); p.cand_idx = c->cand_idx; p.sel_done = c->sel_done;
