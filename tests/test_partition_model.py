@@ -93,8 +93,8 @@ def scan_geometry(nprob, max_groups, sms=148):
 
 
 def test_beside_a_build_the_strided_partition_is_always_suggested():
-    """A step's build that runs beside the scan writes this suggestion without a look at the lengths: with a warp for every group of
-    the longest possible sequence, one round of strides is never slower than the balanced partition."""
+    """The build of a step that appends, beside the scan, writes this suggestion without a look at the lengths: with a warp for every
+    group of the longest possible sequence, one round of strides is never slower than the balanced partition."""
     seen = 0
     for nprob in range(1, 600):
         for max_groups in list(range(1, 70)) + [127, 128, 255, 256, 511, 1056, 2048, 2367, 2368, 2400]:
