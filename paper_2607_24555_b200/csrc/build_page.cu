@@ -316,10 +316,11 @@ __global__ void __launch_bounds__(page_threads(B) * page_ctas(B)) build_page_ker
   } else if (warp == 1 && lane == 0) {
     // Has the selector come (BuildParams::stage)?  It usually does long before the modes are there; asked here, the answer costs them
     // no time (asked by the warp that solves, at its end, 4 x 16K tokens with 32-token pages: 57.9 us a step, now 56.5).
-    int come = 1;
-    if (p.stage) do {
+    int come = p.stage == nullptr;
+    for (int i = 0; !come && i < LOCKS_SPIN_LIMIT; ++i) {   // (until the modes are there: nothing waits for the selector)
       asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(come) : "l"(p.staged + prob) : "memory");
-    } while (!come && !*reinterpret_cast<volatile int *>(&sh.solved));
+      if (*reinterpret_cast<volatile int *>(&sh.solved)) break;
+    }
     sh.early = !come;
   }
   sync();
